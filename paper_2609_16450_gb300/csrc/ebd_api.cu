@@ -174,11 +174,23 @@ bool encode_bf16(CUtensorMap* m, const void* base, int rank, const uint64_t* dim
   return r == CUDA_SUCCESS;
 }
 
+// Tensor map of a row-major [rows][d] matrix, d a multiple of 64, as (column
+// within the k-box, row, k-box): one box holds box_rows rows of kbs k-boxes,
+// k-box by k-box, as the LM head's MMAs read them.
+bool encode_k_boxes(CUtensorMap* m, const void* base, int rows, int d, int box_rows, int kbs) {
+  const uint64_t dims[3] = {64ull, static_cast<uint64_t>(rows), static_cast<uint64_t>(d) / 64};
+  const uint64_t str[2] = {static_cast<uint64_t>(d) * 2, 128ull};
+  const uint32_t box[3] = {64, static_cast<uint32_t>(box_rows), static_cast<uint32_t>(kbs)};
+  return encode_bf16(m, base, 3, dims, str, box);
+}
+
 // Tensor map of W_lm in boxes of 64 columns by 64 rows: row-major [V][d], or
 // the packed layout ([unit][k-box][64 rows][64 columns], ebd_pack_lm_head).
 // For CTA pairs (pair_kbs > 0 k-boxes per stage) the packed layout is read as
 // a 4-D tensor (column, row, unit, k-box) in boxes of two units by pair_kbs
 // k-boxes: one box is a CTA's 128 W rows of a whole pipeline stage.
+// A row-major W whose d is a multiple of 64 is read by CTA pairs as a 3-D
+// tensor (column within the k-box, row, k-box), box 128 rows by pair_kbs.
 bool encode_w_lm(CUtensorMap* m, const void* w, int V, int d, bool packed, int pair_kbs) {
   const uint64_t units = (static_cast<uint64_t>(V) + kUnit - 1) / kUnit;
   const uint64_t nkb = (static_cast<uint64_t>(d) + 63) / 64;
@@ -188,6 +200,7 @@ bool encode_w_lm(CUtensorMap* m, const void* w, int V, int d, bool packed, int p
     const uint32_t box[4] = {64, 64, 2, static_cast<uint32_t>(pair_kbs)};
     return encode_bf16(m, w, 4, dims, str, box);
   }
+  if (pair_kbs > 0) return encode_k_boxes(m, w, V, d, 2 * kUnit, pair_kbs);
   const uint64_t dims[2] = {packed ? 64ull : static_cast<uint64_t>(d),
                             packed ? units * nkb * 64 : static_cast<uint64_t>(V)};
   const uint64_t str[1] = {packed ? 128ull : static_cast<uint64_t>(d) * 2};
@@ -781,6 +794,7 @@ ebd_status run_lm(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, bool p
     if (p.stages < 2) return fail(h, EBD_ERR_UNSUPPORTED, "LM head: shared memory plan failed");
     p.row0 = g0;
     p.packed = packed ? 1 : 0;
+    p.boxed = (p.pair && c.d_model % 64 == 0) ? 1 : 0;
     p.part_f = h->part_f;
     p.part_i = h->part_i;
     p.status = h->d_status;
@@ -788,16 +802,22 @@ ebd_status run_lm(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, bool p
     p.force_timeout = (c.debug_flags & EBD_DEBUG_FORCE_TIMEOUT) ? 1 : 0;
     p.pdl = (g0 == 0 && pdl_first) ? 1 : 0;
     CUtensorMap th;
-    const uint64_t dims[2] = {static_cast<uint64_t>(c.d_model), static_cast<uint64_t>(a->rows)};
-    const uint64_t str[1] = {static_cast<uint64_t>(c.d_model) * 2};
-    // a CTA of a pair loads half of each N sub-tile of hidden rows
-    const uint32_t box[2] = {64, static_cast<uint32_t>(p.pair ? p.nb / 2 : p.nb)};
-    if (!encode_bf16(&th, a->hidden, 2, dims, str, box))
-      return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (hidden) failed");
-    CUtensorMap tw4;  // the paired launches' view of packed W: one box per stage
-    if (p.pair && packed && !encode_w_lm(&tw4, a->w_lm, V, c.d_model, packed, p.kbs))
+    if (p.boxed) {
+      if (!encode_k_boxes(&th, a->hidden, a->rows, c.d_model, p.nb / 2, p.kbs))
+        return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (hidden) failed");
+    } else {
+      const uint64_t dims[2] = {static_cast<uint64_t>(c.d_model), static_cast<uint64_t>(a->rows)};
+      const uint64_t str[1] = {static_cast<uint64_t>(c.d_model) * 2};
+      // a CTA of a pair loads half of each N sub-tile of hidden rows
+      const uint32_t box[2] = {64, static_cast<uint32_t>(p.pair ? p.nb / 2 : p.nb)};
+      if (!encode_bf16(&th, a->hidden, 2, dims, str, box))
+        return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (hidden) failed");
+    }
+    CUtensorMap twp;  // the paired launches' view of W: one box per stage
+    const bool w_box = p.pair && (packed || p.boxed);
+    if (w_box && !encode_w_lm(&twp, a->w_lm, V, c.d_model, packed, p.kbs))
       return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (W_lm) failed");
-    cudaError_t e = launch_lm_stats(p.pair && packed ? tw4 : tw, th, p, st);
+    cudaError_t e = launch_lm_stats(w_box ? twp : tw, th, p, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "LM-head launch");
     h->lm_ctas = p.grid;
   }

@@ -187,8 +187,9 @@ __device__ __forceinline__ bool epilogue_buffer(uint32_t taddr0, int wg, int nwg
 
 }  // namespace
 
-// PAIR (p.pair) and PACKED (p.packed) are template parameters: a runtime
-// branch in the single-thread producer or MMA loop costs measurable time.
+// PAIR (p.pair), PACKED (p.packed) and BOXED (p.boxed) are template
+// parameters: a runtime branch in the single-thread producer or MMA loop
+// costs measurable time.
 //
 // PAIR: the CTAs of a cluster of 2 form a pair that runs cta_group::2 MMAs
 // of M = 256 vocabulary rows.  A vocabulary chunk is 4 units: the even CTA
@@ -201,11 +202,11 @@ __device__ __forceinline__ bool epilogue_buffer(uint32_t taddr0, int wg, int nwg
 // Each SM thus receives half of the hidden rows per MMA, which halves the
 // operand bytes per flop against a 128-row tile over the same rows.
 //
-// Row groups (p.rgroups = 2, paired launches of more than 432 rows): pair q
+// Row groups (p.rgroups = 2, paired launches of more than 256 rows): pair q
 // serves rows [row0 + g nb, row0 + (g + 1) nb) of group g = q / nwork over
 // the vocabulary range of owner q % nwork, and writes its partials to
 // columns [0, grp_cols) of those rows.
-template <bool PAIR, bool PACKED>
+template <bool PAIR, bool PACKED, bool BOXED>
 __global__ void __launch_bounds__(kLmThreads, 1)
     lm_stats_kernel(const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ CUtensorMap tmap_h, const LmParams p) {
@@ -305,9 +306,13 @@ __global__ void __launch_bounds__(kLmThreads, 1)
         else
           tma_load_2d(dst, map, &full[s], x, y, pol);
       };
+      auto load3 = [&](void* dst, const CUtensorMap* map, int s, int y, int z, uint64_t pol) {
+        tma_load_3d_pair(dst, map, mapa_shared(smem_u32(&full[s]), 0), 0, y, z, pol);
+      };
       auto load4 = [&](void* dst, const CUtensorMap* map, int s, int z, int w, uint64_t pol) {
         tma_load_4d_pair(dst, map, mapa_shared(smem_u32(&full[s]), 0), 0, 0, z, w, pol);
       };
+      constexpr bool W_BOX = PAIR && (PACKED || BOXED);  // a stage's W rows in one box
       // stage fill: vocabulary chunk u (kChunkUnits units), k-stage ks; the
       // leader arms the stage for the W and hidden bytes of both CTAs.
       // A pair reads packed W as a 4-D tensor (column, row, unit, k-box):
@@ -315,7 +320,12 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       // rows of the whole stage in one copy, laid out as the MMAs read it
       // (the copies, not L2, set the paired kernel's operand feed: at 64 x 32
       // rows the LM head took 1522 us with two 8 KB boxes per k-box, 1394 us
-      // with one 16 KB box, 1317 us with one box per stage).  A CTA with one
+      // with one 16 KB box, 1317 us with one box per stage).  Row-major W is
+      // read the same way through a 3-D view (column, row, k-box): 512 rows
+      // 397 -> 325 us, 390 rows 346 -> 290 us, 153 rows 204 -> 194 us against
+      // one 8 KB box per unit and k-box.  BOXED also takes the stage's hidden
+      // rows as one box; it wants d % 64 == 0, since the last k-box of a row
+      // would otherwise run into the next row.  A CTA with one
       // unit of the chunk still reads two (the second is the next pair's, or
       // zeros past the last unit) and its epilogue ignores the second.
       // Unpaired, HBM-bound launches read one unit at a time.
@@ -324,14 +334,20 @@ __global__ void __launch_bounds__(kLmThreads, 1)
         const int nsubk = min(p.kbs, p.nkb - ks * p.kbs);
         // W bytes of the stage: one box of kbs k-boxes by two units per CTA
         // with units in the chunk (a stage past the last k-box reads zeros)
-        const uint32_t w_bytes = (PACKED && PAIR)
+        const uint32_t w_bytes = W_BOX
                                      ? (nu > 2 ? 2u : 1u) * static_cast<uint32_t>(p.kbs) * kATile
                                      : static_cast<uint32_t>(nsubk * nu) * kUnit * 128u;
+        const uint32_t h_boxes = static_cast<uint32_t>(BOXED ? p.kbs : nsubk);
         if (leader)
-          mbar_arrive_expect_tx(&full[s], w_bytes + static_cast<uint32_t>(nsubk * p.n_pad) * 128u);
+          mbar_arrive_expect_tx(&full[s], w_bytes + h_boxes * static_cast<uint32_t>(p.n_pad) * 128u);
         uint8_t* a_st = sA + static_cast<size_t>(s) * a_stage;
-        if (PACKED && PAIR) {
-          if (nu > ulo) load4(a_st, &tmap_w, s, u + ulo, ks * p.kbs, pol_w);
+        if (W_BOX) {
+          if (nu > ulo) {
+            if (PACKED)
+              load4(a_st, &tmap_w, s, u + ulo, ks * p.kbs, pol_w);
+            else
+              load3(a_st, &tmap_w, s, (u + ulo) * kUnit, ks * p.kbs, pol_w);
+          }
         } else {
           // one unit at a time, its k-boxes back to back: each W row is
           // requested as one contiguous run of nsubk * 128 bytes
@@ -347,6 +363,10 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       auto issue_h = [&](int ks, int s) {
         const int nsubk = min(p.kbs, p.nkb - ks * p.kbs);
         uint8_t* b_st = sB + static_cast<size_t>(s) * b_stage;
+        if (BOXED) {  // one N sub-tile: the stage's k-boxes of this CTA's rows in one copy
+          load3(b_st, &tmap_h, s, rbase + static_cast<int>(crank) * hrows, ks * p.kbs, pol_h);
+          return;
+        }
         for (int j = 0; j < nsubk; ++j)
           for (int sb = 0; sb < p.nsub; ++sb)
             load(b_st + j * b_sub + sb * hrows * 128, &tmap_h, s, (ks * p.kbs + j) * 64,
@@ -443,7 +463,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
           const int nsubk = min(p.kbs, p.nkb - ks * p.kbs);
           const uint32_t a_addr = smem_u32(sA + static_cast<size_t>(s) * a_stage);
           const uint32_t b_addr = smem_u32(sB + static_cast<size_t>(s) * b_stage);
-          if (p.nsub <= 2 && nsubk >= 1 && nsubk <= 5) {
+          if ((PAIR || p.nsub <= 2) && nsubk >= 1 && nsubk <= 5) {
             // the unrolled issue path
             const uint32_t a_lo = static_cast<uint32_t>(umma_desc_sw128(a_addr));
             const uint32_t b_lo = static_cast<uint32_t>(umma_desc_sw128(b_addr));
@@ -453,7 +473,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
             const uint32_t acc0 = ks != 0 ? 1u : 0u;
 #define EBD_STAGE(K, S) \
   mma_stage<K, S, PAIR>(d0, a_lo, b_lo, b_step, sub_desc, sub_cols, desc_hi, idesc, acc0)
-            if (p.nsub == 1) {
+            if (PAIR || p.nsub == 1) {
               switch (nsubk) {
                 case 1: EBD_STAGE(1, 1); break;
                 case 2: EBD_STAGE(2, 1); break;
@@ -621,17 +641,16 @@ void lm_plan(LmParams& p, int rows, int V, int d, int num_sms, bool pair) {
   p.d = d;
   p.rows = rows;
   p.pair = pair ? 1 : 0;
-  // Paired launches of more than 432 rows split the rows into two groups of
+  // Paired launches of more than 256 rows split the rows into two groups of
   // at most 256, each served by half the pairs over the whole vocabulary:
   // every CTA's accumulator then fits twice in TMEM, so the epilogue of one
-  // chunk overlaps the MMAs of the next, and LLaDA-8B's 494 chunks split
-  // evenly over 38 pairs (6.5 per pair otherwise), at the cost of each W tile
-  // being read by two pairs (the second read from L2) and ~33 % more operand
-  // bytes per flop.  Measured (LM head): 512 rows 401 -> 378 us, 1024 rows
-  // 796 -> 751 us, 4096 rows 3188 -> 3021 us; but Dream-7B's 390 rows (groups
-  // of 208) 361 -> 396 us, hence the threshold.
-  p.rgroups = pair && rows > 432 ? (rows + 255) / 256 : 1;
-  if (const char* env = getenv("EBD_LM_RGROUPS")) p.rgroups = pair && atoi(env) > 1 ? (rows + 255) / 256 : 1;
+  // chunk overlaps the MMAs of the next, at the cost of each W tile being
+  // read by two pairs (the second read from L2) and ~33 % more operand bytes
+  // per flop.  Against one group of two N sub-tiles (one accumulator buffer,
+  // its epilogue exposed), packed W: LLaDA-8B 257 rows 285 -> 246 us, 300
+  // rows 301 -> 266, 390 rows 322 -> 291, 512 rows 384 -> 324; Dream-7B 390
+  // rows 333 -> 311.  Below 257 rows one group already has two buffers.
+  p.rgroups = pair ? (rows + 255) / 256 : 1;
   p.nsub = p.rgroups > 1 ? 1 : (rows + 255) / 256;
   if (p.nsub < 1) p.nsub = 1;
   p.nb = p.rgroups > 1 ? ((rows + p.rgroups - 1) / p.rgroups + 15) / 16 * 16
@@ -670,14 +689,14 @@ void lm_plan(LmParams& p, int rows, int V, int d, int num_sms, bool pair) {
   const uint32_t b_box = static_cast<uint32_t>(pair ? p.n_pad / 2 : p.n_pad) * 128u;
   // k-boxes (64 columns each) per pipeline stage, while keeping at least two
   // stages in flight.  Unpaired (few rows, HBM bound): up to 5, for longer
-  // contiguous runs of each W row per request.  Paired: about 512 / N, so
-  // that a stage's MMAs keep the tensor cores busy for about as long at any
-  // N: measured at 128 rows 4 k-boxes x 2 stages 172 us, 2 x 4 197 us; 256
-  // rows 2 x 3 214 us, 3 x 2 223 us, 1 x 6 272 us; 390 rows 1 x 4 360 us,
-  // 2 x 2 367 us.  Smaller stages cost more in hand-offs than their depth
-  // gains (one k-box per stage in separate W and hidden-row rings: 256 rows
-  // 434 us).
-  int kbs = pair ? 512 / p.n_pad : 5;
+  // contiguous runs of each W row per request.  Paired: three stages of two
+  // k-boxes fit at N = 256, and more of them below; three k-boxes (still
+  // three stages) up to N = 96.  Measured (LLaDA-8B, packed W, us at 1 / 2 /
+  // 3 / 4 k-boxes): 80 rows 191 / 162 / 160 / 164, 128 rows 193 / 164 / 183 /
+  // 168, 153 rows 197 / 175 / 189 / 190, 256 rows 214 / 201 / 219 / 226, 512
+  // rows 371 / 323 / 352 / 352.  One k-box pays a barrier round trip and a
+  // commit per 64 columns; four leave two stages in flight.
+  int kbs = !pair ? 5 : p.n_pad <= 96 ? 3 : 2;
   if (const char* env = getenv("EBD_LM_KBS")) kbs = atoi(env);
   if (kbs < 1) kbs = 1;
   if (kbs > 5) kbs = 5;
@@ -737,13 +756,19 @@ cudaError_t launch_pack_lm(const __nv_bfloat16* w, __nv_bfloat16* out, int V, in
   return cudaGetLastError();
 }
 
+using LmKernel = void (*)(CUtensorMap, CUtensorMap, LmParams);
+static LmKernel lm_kernel(bool pair, bool packed, bool boxed) {
+  if (!pair) return packed ? lm_stats_kernel<false, true, false> : lm_stats_kernel<false, false, false>;
+  if (boxed) return packed ? lm_stats_kernel<true, true, true> : lm_stats_kernel<true, false, true>;
+  return packed ? lm_stats_kernel<true, true, false> : lm_stats_kernel<true, false, false>;
+}
+
 cudaError_t lm_configure() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(lm_stats_kernel<true, true>, a, 232448)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(lm_stats_kernel<true, false>, a, 232448)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(lm_stats_kernel<false, true>, a, 232448)) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(lm_stats_kernel<false, false>, a, 232448);
+  for (int i = 0; i < 6; ++i)
+    if ((e = cudaFuncSetAttribute(lm_kernel(i > 1, i & 1, i > 3), a, 232448)) != cudaSuccess) return e;
+  return cudaSuccess;
 }
 
 cudaError_t launch_lm_stats(const CUtensorMap& tmap_w, const CUtensorMap& tmap_h,
@@ -769,11 +794,7 @@ cudaError_t launch_lm_stats(const CUtensorMap& tmap_w, const CUtensorMap& tmap_h
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  if (p.pair)
-    return p.packed ? cudaLaunchKernelEx(&cfg, lm_stats_kernel<true, true>, tmap_w, tmap_h, p)
-                    : cudaLaunchKernelEx(&cfg, lm_stats_kernel<true, false>, tmap_w, tmap_h, p);
-  return p.packed ? cudaLaunchKernelEx(&cfg, lm_stats_kernel<false, true>, tmap_w, tmap_h, p)
-                  : cudaLaunchKernelEx(&cfg, lm_stats_kernel<false, false>, tmap_w, tmap_h, p);
+  return cudaLaunchKernelEx(&cfg, lm_kernel(p.pair, p.packed, p.boxed), tmap_w, tmap_h, p);
 }
 
 }  // namespace ebd

@@ -16,11 +16,13 @@ struct LmParams {
   int nkb;                  // ceil(d / 64) k-blocks of 64 columns
   int kbs, nks;             // k-blocks per pipeline stage, stages per vocabulary chunk
   int packed;               // W is tiled: tile (unit, k-block) at row (unit*nkb + kb)*64
+  int boxed;                // CTA pairs: a stage's hidden rows (and row-major W rows) come in
+                            // as one 3-D box (d a multiple of 64)
   int stages, nbuf, acc_stride, tmem_cols;
   int nwg;                  // epilogue warpgroups in use (2 with a single accumulator buffer)
   int pair;                 // CTA pairs (clusters of 2) running cta_group::2 MMAs, M = 256
   int nwork;                // owners of vocabulary ranges per row group: CTAs, or pairs
-  int rgroups;              // row groups (paired launches of more than 256 rows: 2), each
+  int rgroups;              // row groups of at most 256 rows (paired launches: 1 or 2), each
                             // of nb rows, served by its own nwork owners
   int grp_cols;             // CTAs per row group (the partial columns a row gets here)
   int ncols;                // partial states per row written (>= grid; extra ones neutral)

@@ -78,3 +78,14 @@ def test_small_vocabulary_shards(rows, shards):
     of the one-CTA-per-SM launch."""
     _run(_shape(rows, 4096), "packed", shards=shards)
     _run(_shape(rows, 4096), "rowmajor", shards=shards)
+
+
+@pytest.mark.parametrize("rows", [65, 97, 256, 300])
+@pytest.mark.parametrize("layout", ["packed", "rowmajor"])
+@pytest.mark.parametrize("d_model", [264, 320])
+def test_paired_stage_boxes(rows, layout, d_model):
+    """CTA pairs: 320 columns are five k-boxes, so the last stage of two or
+    three reads past the matrix (zeros); 264 columns are not whole k-boxes,
+    so the hidden rows (and a row-major W) come in one box per k-box."""
+    rep = _run(_shape(rows, 4000).with_(d_model=d_model), layout)
+    assert rep["conf"] <= 2e-3
