@@ -13,7 +13,7 @@
 
 #include "ebd.h"
 #include "internal.h"
-#include "router_image.h"
+#include "rows_image.h"
 
 namespace {
 // An NVTX range around the host side of an entry point (visible in Nsight
@@ -25,8 +25,6 @@ struct NvtxRange {
 }  // namespace
 
 namespace ebd {
-cudaError_t decide_configure();
-cudaError_t decide_cta_configure();
 cudaError_t attn_configure();
 cudaError_t lm_configure();
 cudaError_t launch_merge_stats(const float4* part_f, const int* part_i, int rows, int grid,
@@ -230,8 +228,6 @@ struct ebd_handle {
   std::vector<TensorDesc> layout;
   std::vector<uint16_t> h_blob;
   uint16_t* d_blob = nullptr;
-  uint8_t* d_image = nullptr;
-  RouterImage img{};
   float* d_tok = nullptr;
   const uint16_t* w_emb = nullptr;
   float4* part_f = nullptr;
@@ -247,11 +243,11 @@ struct ebd_handle {
   int* d_status = nullptr;
   uint8_t* staging = nullptr;
   size_t staging_bytes = 0;
-  // the grid-wide decision (max_window > kMaxWindow)
-  float* d_seqw = nullptr;   // SeqWeights image
-  SeqWeights seqw{};
-  uint8_t* seq_scratch = nullptr;
-  SeqParams seqp{};          // scratch pointers, filled at create
+  // the decision
+  uint8_t* d_rows = nullptr;        // its router image (rows_image.h)
+  uint8_t* rows_scratch = nullptr;
+  int rows_slots[2] = {0, 0};       // its clusters of 8 and of 4 CTAs that fit the GPU
+  RowsParams rowsp{};               // image and scratch pointers, filled at create
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   int profile = 0;
   int prof_mode = 0, prof_attn = 0;  // what the last ebd_step recorded
@@ -339,312 +335,107 @@ ebd_status check_device(ebd_handle* h) {
   return EBD_OK;
 }
 
-// fp32 image of the router weights for the grid-wide decision: matrices
-// [in][out], vectors as they are (SeqWeights).
-ebd_status upload_seq_weights(ebd_handle* h) {
-  // element (r, c) of a blob tensor, its offset resolved once per name
-  std::string last;
-  size_t last_off = 0, last_cols = 0;
-  auto atf = [&](const std::string& name, int r, int c) -> float {
-    if (name != last) {
-      size_t off = 0;
-      bool found = false;
-      for (const auto& t : h->layout) {
-        if (t.name == name) {
-          last_cols = static_cast<size_t>(t.cols);
-          found = true;
-          break;
-        }
-        off += static_cast<size_t>(t.rows) * t.cols;
-      }
-      last = name;
-      last_off = found ? off : 0;
-    }
-    return bf16_to_f32(h->h_blob[last_off + static_cast<size_t>(r) * last_cols + c]);
-  };
-  SeqWeights& o = h->seqw;
-  int n = 0;
-  auto take = [&](int count) {
-    const int at = n;
-    n += (count + 3) / 4 * 4;
-    return at;
-  };
+// The router weights to the device: the blob, and the decision's image of it
+// (rows_image.h).
+ebd_status upload_router(ebd_handle* h) {
+  using namespace rowimg;
   const int L = h->cfg.gen_len;
-  o.ent1_w = take(64); o.ent1_b = take(64); o.ent2_t = take(64 * 64); o.ent2_b = take(64);
-  o.entln_g = take(64); o.entln_b = take(64); o.tok_b = take(64);
-  o.comb_t = take(128 * 128); o.comb_b = take(128); o.pos = take(L * 128);
-  for (int l = 0; l < 2; ++l) {
-    SeqLayer& q = o.l[l];
-    q.qkv_t = take(128 * 384); q.qkv_b = take(384); q.out_t = take(128 * 128); q.out_b = take(128);
-    q.ln1_g = take(128); q.ln1_b = take(128); q.ff1_t = take(128 * 256); q.ff1_b = take(256);
-    q.ff2_t = take(256 * 128); q.ff2_b = take(128); q.ln2_g = take(128); q.ln2_b = take(128);
-  }
-  o.head_w = take(128); o.head_b = take(1);
-  o.in_t = take(5 * 32); o.in_b = take(32); o.inln_g = take(32); o.inln_b = take(32);
-  for (int l = 0; l < 2; ++l) {
-    SeqBlock& q = o.p[l];
-    q.ln1_g = take(32); q.ln1_b = take(32); q.qkv_t = take(32 * 96); q.qkv_b = take(96);
-    q.out_t = take(32 * 32); q.out_b = take(32); q.ln2_g = take(32); q.ln2_b = take(32);
-    q.ff1_t = take(32 * 64); q.ff1_b = take(64); q.ff2_t = take(64 * 32); q.ff2_b = take(32);
-  }
-  o.phead_w = take(32); o.phead_b = take(1);
-  o.total = n;
-  std::vector<float> w(static_cast<size_t>(n), 0.f);
-  // [in][out] copy of a [out][in] matrix, and a vector
-  auto mat = [&](int at, const std::string& name, int nin, int nout) {
-    for (int k = 0; k < nin; ++k)
-      for (int c = 0; c < nout; ++c) w[at + static_cast<size_t>(k) * nout + c] = atf(name, c, k);
+  const size_t b_mat = static_cast<size_t>(M_TOTAL) * 16;
+  const size_t n_vec = static_cast<size_t>(V_POS) + static_cast<size_t>(L) * 128;
+  std::vector<uint16_t> mat(b_mat / 2, 0);
+  std::vector<float> vec(n_vec, 0.f);
+  auto tensor = [&](const std::string& name) -> const uint16_t* {
+    size_t off = 0;
+    for (const auto& t : h->layout) {
+      if (t.name == name) break;
+      off += static_cast<size_t>(t.rows) * t.cols;
+    }
+    return h->h_blob.data() + off;
   };
-  auto vec = [&](int at, const std::string& name, int count) {
-    for (int c = 0; c < count; ++c) w[at + c] = atf(name, 0, c);
+  auto put_mat = [&](int at, const std::string& name, int N, int K, bool natural) {
+    const uint16_t* w = tensor(name);
+    uint16_t* o = mat.data() + static_cast<size_t>(at) * 8;
+    for (int m = 0; m < N / 16; ++m)
+      for (int ks = 0; ks < K / 16; ++ks)
+        for (int lane = 0; lane < 32; ++lane)
+          for (int e = 0; e < 8; ++e) {  // register e / 2, half e % 2
+            const int g = lane / 4, t = lane % 4, up = (e / 2) & 1, hi = e / 4;
+            const int n = 16 * m + (natural ? g + 8 * up : 2 * g + up);
+            const int k = natural ? 16 * ks + 2 * t + 8 * hi + e % 2
+                                  : 32 * (ks / 2) + 8 * t + 4 * (ks % 2) + 2 * hi + e % 2;
+            o[((m * (K / 16) + ks) * 32 + lane) * 8 + e] = w[static_cast<size_t>(n) * K + k];
+          }
   };
-  for (int c = 0; c < 64; ++c) w[o.ent1_w + c] = atf("lbs.ent1.w", c, 0);
-  vec(o.ent1_b, "lbs.ent1.b", 64);
-  mat(o.ent2_t, "lbs.ent2.w", 64, 64);
-  vec(o.ent2_b, "lbs.ent2.b", 64);
-  vec(o.entln_g, "lbs.ent_ln.g", 64);
-  vec(o.entln_b, "lbs.ent_ln.b", 64);
-  vec(o.tok_b, "lbs.tok.b", 64);
-  mat(o.comb_t, "lbs.comb.w", 128, 128);
-  vec(o.comb_b, "lbs.comb.b", 128);
-  for (int j = 0; j < L; ++j)
-    for (int c = 0; c < 128; ++c) w[o.pos + static_cast<size_t>(j) * 128 + c] = atf("lbs.pos", j, c);
+  auto put_vec = [&](int at, const std::string& name, int count) {
+    const uint16_t* w = tensor(name);
+    for (int i = 0; i < count; ++i) vec[at + i] = bf16_to_f32(w[i]);
+  };
+  put_mat(M_ENT2, "lbs.ent2.w", 64, 64, false);
+  put_mat(M_COMB, "lbs.comb.w", 128, 128, false);
+  put_vec(V_ENT1W, "lbs.ent1.w", 64);
+  put_vec(V_ENT1B, "lbs.ent1.b", 64);
+  put_vec(V_ENT2B, "lbs.ent2.b", 64);
+  put_vec(V_ENTLNG, "lbs.ent_ln.g", 64);
+  put_vec(V_ENTLNB, "lbs.ent_ln.b", 64);
+  put_vec(V_TOKB, "lbs.tok.b", 64);
+  put_vec(V_COMBB, "lbs.comb.b", 128);
+  put_vec(V_POS, "lbs.pos", L * 128);
   for (int l = 0; l < 2; ++l) {
     const std::string pre = "lbs.l" + std::to_string(l);
-    const SeqLayer& q = o.l[l];
-    mat(q.qkv_t, pre + ".qkv.w", 128, 384); vec(q.qkv_b, pre + ".qkv.b", 384);
-    mat(q.out_t, pre + ".out.w", 128, 128); vec(q.out_b, pre + ".out.b", 128);
-    vec(q.ln1_g, pre + ".ln1.g", 128); vec(q.ln1_b, pre + ".ln1.b", 128);
-    mat(q.ff1_t, pre + ".ff1.w", 128, 256); vec(q.ff1_b, pre + ".ff1.b", 256);
-    mat(q.ff2_t, pre + ".ff2.w", 256, 128); vec(q.ff2_b, pre + ".ff2.b", 128);
-    vec(q.ln2_g, pre + ".ln2.g", 128); vec(q.ln2_b, pre + ".ln2.b", 128);
+    const int m = M_LAYER + l * ML_STRIDE, v = V_LAYER + l * VL_STRIDE;
+    put_mat(m + ML_QKV, pre + ".qkv.w", 384, 128, false);
+    put_mat(m + ML_OUT, pre + ".out.w", 128, 128, false);
+    put_mat(m + ML_FF1, pre + ".ff1.w", 256, 128, false);
+    put_mat(m + ML_FF2, pre + ".ff2.w", 128, 256, false);
+    put_vec(v + VL_QKVB, pre + ".qkv.b", 384);
+    put_vec(v + VL_OUTB, pre + ".out.b", 128);
+    put_vec(v + VL_LN1G, pre + ".ln1.g", 128);
+    put_vec(v + VL_LN1B, pre + ".ln1.b", 128);
+    put_vec(v + VL_FF1B, pre + ".ff1.b", 256);
+    put_vec(v + VL_FF2B, pre + ".ff2.b", 128);
+    put_vec(v + VL_LN2G, pre + ".ln2.g", 128);
+    put_vec(v + VL_LN2B, pre + ".ln2.b", 128);
   }
-  vec(o.head_w, "lbs.head.w", 128);
-  vec(o.head_b, "lbs.head.b", 1);
-  mat(o.in_t, "lps.in.w", 5, 32);
-  vec(o.in_b, "lps.in.b", 32);
-  vec(o.inln_g, "lps.in_ln.g", 32);
-  vec(o.inln_b, "lps.in_ln.b", 32);
+  put_vec(V_HEADW, "lbs.head.w", 128);
+  put_vec(V_HEADB, "lbs.head.b", 1);
+  {
+    const uint16_t* w = tensor("lps.in.w");  // [32][5] -> [5][32]
+    for (int o = 0; o < 32; ++o)
+      for (int k = 0; k < 5; ++k) vec[V_INT + 32 * k + o] = bf16_to_f32(w[5 * o + k]);
+  }
+  put_vec(V_INB, "lps.in.b", 32);
+  put_vec(V_INLNG, "lps.in_ln.g", 32);
+  put_vec(V_INLNB, "lps.in_ln.b", 32);
   for (int l = 0; l < 2; ++l) {
     const std::string pre = "lps.l" + std::to_string(l);
-    const SeqBlock& q = o.p[l];
-    vec(q.ln1_g, pre + ".ln1.g", 32); vec(q.ln1_b, pre + ".ln1.b", 32);
-    mat(q.qkv_t, pre + ".qkv.w", 32, 96); vec(q.qkv_b, pre + ".qkv.b", 96);
-    mat(q.out_t, pre + ".out.w", 32, 32); vec(q.out_b, pre + ".out.b", 32);
-    vec(q.ln2_g, pre + ".ln2.g", 32); vec(q.ln2_b, pre + ".ln2.b", 32);
-    mat(q.ff1_t, pre + ".ff1.w", 32, 64); vec(q.ff1_b, pre + ".ff1.b", 64);
-    mat(q.ff2_t, pre + ".ff2.w", 64, 32); vec(q.ff2_b, pre + ".ff2.b", 32);
+    const int m = M_BLOCK + l * MB_STRIDE, v = V_BLOCK + l * VB_STRIDE;
+    put_mat(m + MB_QKV, pre + ".qkv.w", 96, 32, true);
+    put_mat(m + MB_OUT, pre + ".out.w", 32, 32, true);
+    put_mat(m + MB_FF1, pre + ".ff1.w", 64, 32, true);
+    put_mat(m + MB_FF2, pre + ".ff2.w", 32, 64, true);
+    put_vec(v + VB_LN1G, pre + ".ln1.g", 32);
+    put_vec(v + VB_LN1B, pre + ".ln1.b", 32);
+    put_vec(v + VB_QKVB, pre + ".qkv.b", 96);
+    put_vec(v + VB_OUTB, pre + ".out.b", 32);
+    put_vec(v + VB_LN2G, pre + ".ln2.g", 32);
+    put_vec(v + VB_LN2B, pre + ".ln2.b", 32);
+    put_vec(v + VB_FF1B, pre + ".ff1.b", 64);
+    put_vec(v + VB_FF2B, pre + ".ff2.b", 32);
   }
-  vec(o.phead_w, "lps.head.w", 32);
-  vec(o.phead_b, "lps.head.b", 1);
-  if (h->d_seqw == nullptr) {
-    cudaError_t e = cudaMalloc(&h->d_seqw, w.size() * sizeof(float));
-    if (e != cudaSuccess) return cuda_fail(h, e, "cudaMalloc(router fp32 image)");
-  }
-  cudaError_t e = cudaMemcpy(h->d_seqw, w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemcpy(router fp32 image)");
-  return EBD_OK;
-}
-
-// Builds the decision kernel's weight image (router_image.h) from the blob.
-ebd_status upload_router(ebd_handle* h) {
-  using namespace rimg;
-  const auto& L = h->layout;
-  std::vector<size_t> off(L.size());
-  {
-    size_t o = 0;
-    for (size_t i = 0; i < L.size(); ++i) {
-      off[i] = o;
-      o += static_cast<size_t>(L[i].rows) * L[i].cols;
-    }
-  }
-  auto T = [&](const std::string& n) -> const TensorDesc& {
-    for (size_t i = 0; i < L.size(); ++i)
-      if (L[i].name == n) return L[i];
-    return L[0];
-  };
-  auto idx = [&](const std::string& n) -> size_t {
-    for (size_t i = 0; i < L.size(); ++i)
-      if (L[i].name == n) return i;
-    return 0;
-  };
-  // element (r, c) of tensor n as bf16 bits / float
-  auto at = [&](const std::string& n, int r, int c) -> uint16_t {
-    const size_t i = idx(n);
-    return h->h_blob[off[i] + static_cast<size_t>(r) * L[i].cols + c];
-  };
-  auto atf = [&](const std::string& n, int r, int c) { return bf16_to_f32(at(n, r, c)); };
-  (void)T;
-  std::vector<uint16_t> lbs(static_cast<size_t>(kRanks) * LBS_W_ELEMS, 0);
-  std::vector<uint16_t> lps(LPS_W_ELEMS, 0);
-  std::vector<float> vec(static_cast<size_t>(kRanks) * V_ELEMS, 0.f);
-  const int gen_len = h->cfg.gen_len;
-  for (int r = 0; r < kRanks; ++r) {
-    uint16_t* w = lbs.data() + static_cast<size_t>(r) * LBS_W_ELEMS;
-    float* v = vec.data() + static_cast<size_t>(r) * V_ELEMS;
-    for (int k = 0; k < 64; ++k)
-      for (int o = 0; o < 64; ++o) w[W_ENT2 + k * 64 + swz_col(k, o, 64)] = at("lbs.ent2.w", o, k);
-    for (int k = 0; k < 128; ++k)
-      for (int o = 0; o < kCombSlice; ++o)
-        w[W_COMB + k * kCombSlice + swz_col(k, o, kCombSlice)] = at("lbs.comb.w", kCombSlice * r + o, k);
-    for (int j = 0; j < kPosRows; ++j)
-      for (int o = 0; o < kCombSlice; ++o)
-        w[W_POS + j * kCombSlice + o] = j < gen_len ? at("lbs.pos", j, kCombSlice * r + o) : 0;
-    for (int l = 0; l < 2; ++l) {
-      const std::string pre = "lbs.l" + std::to_string(l);
-      uint16_t* wl = w + W_LAYER0 + l * W_LAYER_STRIDE;
-      float* vl = v + V_LAYER0 + l * V_LAYER_STRIDE;
-      for (int k = 0; k < 128; ++k) {
-        for (int o = 0; o < kQkvSlice; ++o)
-          wl[WL_QKV + k * kQkvSlice + swz_col(k, o, kQkvSlice)] = at(pre + ".qkv.w", kQkvSlice * r + o, k);
-        for (int o = 0; o < kOutSlice; ++o)
-          wl[WL_OUT + k * kOutSlice + swz_col(k, o, kOutSlice)] = at(pre + ".out.w", kOutSlice * r + o, k);
-        for (int o = 0; o < kFf1Slice; ++o)
-          wl[WL_FF1 + k * kFf1Slice + swz_col(k, o, kFf1Slice)] = at(pre + ".ff1.w", kFf1Slice * r + o, k);
-      }
-      for (int hh = 0; hh < kFf1Slice; ++hh)
-        for (int o = 0; o < 128; ++o)
-          wl[WL_FF2 + hh * 128 + swz_col(hh, o, 128)] = at(pre + ".ff2.w", o, kFf1Slice * r + hh);
-      for (int o = 0; o < kQkvSlice; ++o) vl[VL_QKVB + o] = atf(pre + ".qkv.b", 0, kQkvSlice * r + o);
-      for (int o = 0; o < kOutSlice; ++o) vl[VL_OUTB + o] = atf(pre + ".out.b", 0, kOutSlice * r + o);
-      for (int o = 0; o < kFf1Slice; ++o) vl[VL_FF1B + o] = atf(pre + ".ff1.b", 0, kFf1Slice * r + o);
-      for (int o = 0; o < kOutSlice; ++o) vl[VL_FF2B + o] = atf(pre + ".ff2.b", 0, kOutSlice * r + o);
-      for (int o = 0; o < 128; ++o) {
-        vl[VL_LN1G + o] = atf(pre + ".ln1.g", 0, o);
-        vl[VL_LN1B + o] = atf(pre + ".ln1.b", 0, o);
-        vl[VL_LN2G + o] = atf(pre + ".ln2.g", 0, o);
-        vl[VL_LN2B + o] = atf(pre + ".ln2.b", 0, o);
-      }
-    }
-    for (int o = 0; o < 64; ++o) {
-      v[V_ENT1W + o] = atf("lbs.ent1.w", o, 0);
-      v[V_ENT1B + o] = atf("lbs.ent1.b", 0, o);
-      v[V_ENT2B + o] = atf("lbs.ent2.b", 0, o);
-      v[V_ENTLNG + o] = atf("lbs.ent_ln.g", 0, o);
-      v[V_ENTLNB + o] = atf("lbs.ent_ln.b", 0, o);
-      v[V_TOKB + o] = atf("lbs.tok.b", 0, o);
-    }
-    for (int o = 0; o < 128; ++o) v[V_HEADW + o] = atf("lbs.head.w", 0, o);
-    v[V_HEADB] = atf("lbs.head.b", 0, 0);
-    for (int o = 0; o < kCombSlice; ++o) v[V_COMBB + o] = atf("lbs.comb.b", 0, kCombSlice * r + o);
-    // LPS vectors (every rank holds them; rank 0 uses them)
-    float* vp = v + V_LPS;
-    for (int k = 0; k < 5; ++k)
-      for (int o = 0; o < 32; ++o) vp[VP_INT + k * 32 + o] = atf("lps.in.w", o, k);
-    for (int o = 0; o < 32; ++o) {
-      vp[VP_INB + o] = atf("lps.in.b", 0, o);
-      vp[VP_INLNG + o] = atf("lps.in_ln.g", 0, o);
-      vp[VP_INLNB + o] = atf("lps.in_ln.b", 0, o);
-      vp[VP_HEADW + o] = atf("lps.head.w", 0, o);
-    }
-    vp[VP_HEADB] = atf("lps.head.b", 0, 0);
-    for (int l = 0; l < 2; ++l) {
-      const std::string pre = "lps.l" + std::to_string(l);
-      float* vl = vp + VP_LAYER0 + l * VP_LAYER_STRIDE;
-      for (int o = 0; o < 32; ++o) {
-        vl[VPL_LN1G + o] = atf(pre + ".ln1.g", 0, o);
-        vl[VPL_LN1B + o] = atf(pre + ".ln1.b", 0, o);
-        vl[VPL_OUTB + o] = atf(pre + ".out.b", 0, o);
-        vl[VPL_LN2G + o] = atf(pre + ".ln2.g", 0, o);
-        vl[VPL_LN2B + o] = atf(pre + ".ln2.b", 0, o);
-        vl[VPL_FF2B + o] = atf(pre + ".ff2.b", 0, o);
-      }
-      for (int o = 0; o < 96; ++o) vl[VPL_QKVB + o] = atf(pre + ".qkv.b", 0, o);
-      for (int o = 0; o < 64; ++o) vl[VPL_FF1B + o] = atf(pre + ".ff1.b", 0, o);
-    }
-  }
-  for (int l = 0; l < 2; ++l) {
-    const std::string pre = "lps.l" + std::to_string(l);
-    uint16_t* wl = lps.data() + l * PL_STRIDE;
-    for (int k = 0; k < 32; ++k) {
-      for (int o = 0; o < 96; ++o) wl[PL_QKV + k * PL_LDQKV + o] = at(pre + ".qkv.w", o, k);
-      for (int o = 0; o < 32; ++o) wl[PL_OUT + k * PL_LDOUT + o] = at(pre + ".out.w", o, k);
-      for (int o = 0; o < 64; ++o) wl[PL_FF1 + k * PL_LDFF1 + o] = at(pre + ".ff1.w", o, k);
-    }
-    for (int k = 0; k < 64; ++k)
-      for (int o = 0; o < 32; ++o) wl[PL_FF2 + k * PL_LDFF2 + o] = at(pre + ".ff2.w", o, k);
-  }
-  // the one-CTA kernel's image (rcta): 128 x 64 swizzled A tiles of W [out][in]
-  std::vector<uint16_t> cw(static_cast<size_t>(rcta::kChunks) * rcta::kChunkElems, 0);
-  std::vector<float> cv(rcta::S_ELEMS, 0.f);
-  {
-    using namespace rcta;
-    auto chunk = [&](int c) { return cw.data() + static_cast<size_t>(c) * kChunkElems; };
-    // chunks c0 + t * nkb + kb: rows [128 t, 128 t + 128) (< outs), inputs [64 kb, 64 kb + 64)
-    auto tiles = [&](int c0, const std::string& n, int outs, int ins) {
-      const int nt = (outs + 127) / 128, nkb = ins / 64;
-      for (int t = 0; t < nt; ++t)
-        for (int kb = 0; kb < nkb; ++kb)
-          for (int m = 0; m < 128 && 128 * t + m < outs; ++m)
-            for (int k = 0; k < 64; ++k)
-              chunk(c0 + t * nkb + kb)[tile_off(m, k)] = at(n, 128 * t + m, 64 * kb + k);
-    };
-    tiles(C_ENT, "lbs.ent2.w", 64, 64);
-    tiles(C_COMB, "lbs.comb.w", 128, 128);
-    for (int l = 0; l < 2; ++l) {
-      const std::string pre = "lbs.l" + std::to_string(l);
-      const int base = C_LAYER0 + l * CL_CHUNKS;
-      tiles(base + CL_QKV, pre + ".qkv.w", 384, 128);
-      tiles(base + CL_OUT, pre + ".out.w", 128, 128);
-      tiles(base + CL_FF1, pre + ".ff1.w", 256, 128);
-      tiles(base + CL_FF2, pre + ".ff2.w", 128, 256);
-      float* vl = cv.data() + S_LAYER0 + l * S_LAYER_STRIDE;
-      for (int o = 0; o < 384; ++o) vl[SL_QKVB + o] = atf(pre + ".qkv.b", 0, o);
-      for (int o = 0; o < 256; ++o) vl[SL_FF1B + o] = atf(pre + ".ff1.b", 0, o);
-      for (int o = 0; o < 128; ++o) {
-        vl[SL_OUTB + o] = atf(pre + ".out.b", 0, o);
-        vl[SL_FF2B + o] = atf(pre + ".ff2.b", 0, o);
-        vl[SL_LN1G + o] = atf(pre + ".ln1.g", 0, o);
-        vl[SL_LN1B + o] = atf(pre + ".ln1.b", 0, o);
-        vl[SL_LN2G + o] = atf(pre + ".ln2.g", 0, o);
-        vl[SL_LN2B + o] = atf(pre + ".ln2.b", 0, o);
-      }
-    }
-    uint16_t* pos = reinterpret_cast<uint16_t*>(cv.data() + S_POS);
-    for (int j = 0; j < rcta::kPosRows; ++j)
-      for (int o = 0; o < 128; ++o) pos[j * 128 + o] = j < gen_len ? at("lbs.pos", j, o) : 0;
-    std::copy(lps.begin(), lps.end(), chunk(C_LPS));
-    for (int o = 0; o < 64; ++o) {
-      cv[S_ENT1W + o] = atf("lbs.ent1.w", o, 0);
-      cv[S_ENT1B + o] = atf("lbs.ent1.b", 0, o);
-      cv[S_ENT2B + o] = atf("lbs.ent2.b", 0, o);
-      cv[S_ENTLNG + o] = atf("lbs.ent_ln.g", 0, o);
-      cv[S_ENTLNB + o] = atf("lbs.ent_ln.b", 0, o);
-      cv[S_TOKB + o] = atf("lbs.tok.b", 0, o);
-    }
-    for (int o = 0; o < 128; ++o) {
-      cv[S_COMBB + o] = atf("lbs.comb.b", 0, o);
-      cv[S_HEADW + o] = atf("lbs.head.w", 0, o);
-    }
-    cv[S_HEADB] = atf("lbs.head.b", 0, 0);
-    // the LPS vectors: the same as every rank's copy above
-    std::copy(vec.begin() + V_LPS, vec.begin() + V_ELEMS, cv.begin() + S_LPS);
-  }
-  const size_t b_lbs = lbs.size() * 2, b_lps = lps.size() * 2, b_vec = vec.size() * 4;
-  const size_t o_lps = (b_lbs + 255) / 256 * 256;
-  const size_t o_vec = o_lps + (b_lps + 255) / 256 * 256;
-  const size_t o_cw = o_vec + (b_vec + 255) / 256 * 256;
-  const size_t o_cv = o_cw + (cw.size() * 2 + 255) / 256 * 256;
-  const size_t total = o_cv + cv.size() * 4;
-  if (h->d_image) cudaFree(h->d_image);
-  h->d_image = nullptr;
-  cudaError_t e = cudaMalloc(&h->d_image, total);
-  if (e != cudaSuccess) return cuda_fail(h, e, "cudaMalloc(router image)");
-  if ((e = cudaMemcpy(h->d_image, lbs.data(), b_lbs, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(h->d_image + o_lps, lps.data(), b_lps, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(h->d_image + o_vec, vec.data(), b_vec, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(h->d_image + o_cw, cw.data(), cw.size() * 2, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(h->d_image + o_cv, cv.data(), cv.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
-    return cuda_fail(h, e, "cudaMemcpy(router image)");
-  e = cudaMemcpy(h->d_blob, h->h_blob.data(), h->h_blob.size() * 2, cudaMemcpyHostToDevice);
+  put_vec(V_PHEADW, "lps.head.w", 32);
+  put_vec(V_PHEADB, "lps.head.b", 1);
+  cudaError_t e = cudaMemcpy(h->d_blob, h->h_blob.data(), h->h_blob.size() * 2, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemcpy(router blob)");
-  h->img.lbs_w = reinterpret_cast<const __nv_bfloat16*>(h->d_image);
-  h->img.lps_w = reinterpret_cast<const __nv_bfloat16*>(h->d_image + o_lps);
-  h->img.vec = reinterpret_cast<const float*>(h->d_image + o_vec);
-  h->img.tok_table = h->d_tok;
-  h->img.cta_w = reinterpret_cast<const __nv_bfloat16*>(h->d_image + o_cw);
-  h->img.cta_vec = reinterpret_cast<const float*>(h->d_image + o_cv);
-  return upload_seq_weights(h);
+  if (h->d_rows == nullptr &&
+      (e = cudaMalloc(&h->d_rows, b_mat + n_vec * sizeof(float))) != cudaSuccess)
+    return cuda_fail(h, e, "cudaMalloc(router image)");
+  if ((e = cudaMemcpy(h->d_rows, mat.data(), b_mat, cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (e = cudaMemcpy(h->d_rows + b_mat, vec.data(), n_vec * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess)
+    return cuda_fail(h, e, "cudaMemcpy(router image)");
+  h->rowsp.mat = reinterpret_cast<const uint4*>(h->d_rows);
+  h->rowsp.vec = reinterpret_cast<const float*>(h->d_rows + b_mat);
+  h->rowsp.tok_table = h->d_tok;
+  return EBD_OK;
 }
 
 ebd_status fold(ebd_handle* h, cudaStream_t st) {
@@ -824,38 +615,24 @@ ebd_status run_lm(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, bool p
   return EBD_OK;
 }
 
-// Which kernel decides a launch of `batch` sequences with windows of up to
-// kCtaWindow rows: the one-CTA kernel from kCtaMinBatch sequences on, the
-// cluster kernel below.  Measured on the LLaDA-8B head shape (µs per step,
-// one-CTA against cluster): 1 x 32 rows 209 / 197, 4 x 32 245 / 214,
-// 16 x 8 200 / 212, 16 x 32 454 / 465, 64 x 8 464 / 515, 64 x 32 1638 /
-// 1749: one sequence decides faster on eight SMs, while many sequences
-// need several waves of 8-CTA clusters.  EBD_DECIDE_KERNEL=cta or cluster
-// overrides the rule (a measurement knob).
-constexpr int kCtaMinBatch = 16;
-bool cta_decision(const ebd_handle* h, int batch) {
-  if (h->cfg.max_window > kCtaWindow) return false;
-  if (const char* env = getenv("EBD_DECIDE_KERNEL")) {
-    if (strcmp(env, "cta") == 0) return true;
-    if (strcmp(env, "cluster") == 0) return false;
-  }
-  return batch >= kCtaMinBatch;
-}
-
-DecideParams decide_params(ebd_handle* h, const ebd_step_args* a, int features_in) {
+// features_in: a's statistics are inputs (device), else the LM head's
+// partial states are merged into them
+RowsParams rows_params(ebd_handle* h, const ebd_step_args* a, bool features_in) {
   const ebd_config& c = h->cfg;
-  DecideParams p{};
+  RowsParams p = h->rowsp;  // image and scratch
   p.B = a->batch;
+  p.R = a->rows;
   p.V = c.vocab;
   p.grid_lm = h->grid_lm;
-  p.features_in = features_in;
+  p.features_in = features_in ? 1 : 0;
+  p.strict = c.max_window <= kMaxWindow ? 1 : 0;
+  p.mode = c.decode_mode;
+  p.top_m = c.top_m;
   p.gen_len = c.gen_len;
   p.g_max = c.g_max;
   p.l_min = c.l_min;
   p.l_b = c.l_b;
   p.eos_id = c.eos_id;
-  p.mode = c.decode_mode;
-  p.top_m = c.top_m;
   p.lps_enabled = c.decode_mode == EBD_DECODE_EB ? c.lps_enabled : 0;
   p.tau = c.tau;
   p.tau_psi = c.tau_psi;
@@ -864,26 +641,34 @@ DecideParams decide_params(ebd_handle* h, const ebd_step_args* a, int features_i
   p.row_pos = a->row_pos;
   p.part_f = h->part_f;
   p.part_i = h->part_i;
-  p.tokens = a->tokens;
-  p.mask = a->mask;
-  p.in_block = a->in_block;
-  p.blk_meta = a->blk_meta;
-  p.tokens_out = a->tokens;
-  p.mask_out = a->mask;
-  p.in_block_out = a->in_block;
-  p.blk_meta_out = a->blk_meta;
-  p.conf = a->conf;
-  p.entropy = a->entropy;
-  p.ent_norm = a->ent_norm;
-  p.gap = a->gap;
-  p.argmax = a->argmax;
+  p.tokens = p.tokens_out = a->tokens;
+  p.mask = p.mask_out = a->mask;
+  p.in_block = p.in_block_out = a->in_block;
+  p.blk_meta = p.blk_meta_out = a->blk_meta;
+  if (features_in) {
+    p.s_conf = a->conf;
+    p.s_ent = a->ent_norm;
+    p.s_gap = a->gap;
+    p.s_arg = a->argmax;
+  } else {
+    p.conf = a->conf;
+    p.entropy = a->entropy;
+    p.ent_norm = a->ent_norm;
+    p.gap = a->gap;
+    p.argmax = a->argmax;
+  }
   p.lbs_logit = a->lbs_logit;
   p.lps_prob = a->lps_prob;
   p.accepted = a->accepted;
   p.status = h->d_status;
-  p.rows_expected = a->rows;
-  p.w = h->img;
   return p;
+}
+// Rows that the decision's launch holds per sequence.  Windows of up to 32
+// rows take half the CTAs per sequence where the batch is large (below that,
+// a sequence may bring more rows than the handle announced).
+int rows_cap(const ebd_handle* h, int batch) {
+  if (h->cfg.max_window > kMaxWindow) return kMaxSeqRows;
+  return h->cfg.max_window <= 32 && batch >= 16 ? 32 : 64;
 }
 
 }  // namespace
@@ -993,7 +778,7 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     return bail(fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable"));
   if ((e = lm_configure()) != cudaSuccess) return bail(cuda_fail(h, e, "LM-head attributes"));
   if ((e = attn_configure()) != cudaSuccess) return bail(cuda_fail(h, e, "attention attributes"));
-  if ((e = decide_configure()) != cudaSuccess || (e = decide_cta_configure()) != cudaSuccess)
+  if ((e = decide_rows_configure(h->rows_slots)) != cudaSuccess)
     return bail(cuda_fail(h, e, "decision attributes"));
 
   h->layout = router_layout(cfg->d_base, cfg->gen_len);
@@ -1088,45 +873,33 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
   // the copy stream of ebd_step_host, set up here rather than at its first
   // call, which may come while a stream is being captured into a graph
   if (cfg->max_window <= kMaxWindow) (void)copy_route_ready(h);
-  if (cfg->max_window > kMaxWindow) {  // scratch of the grid-wide decision
-    const size_t R = cfg->max_rows, B = cfg->max_batch;
+  {  // scratch of the decision
+    const int planes = cfg->max_window > kMaxWindow ? 3 : 2;
+    const size_t cap = static_cast<size_t>((cfg->max_rows + 31) / 32 * 32) + 32 * (static_cast<size_t>(cfg->max_batch) + 1);
+    const size_t R = cfg->max_rows;
     size_t bytes = 0;
     auto add = [&](size_t n) {
       const size_t at = bytes;
       bytes += (n + 255) / 256 * 256;
       return at;
     };
-    const size_t o_conf = add(R * 4), o_entn = add(R * 4), o_gap = add(R * 4), o_arg = add(R * 4);
-    const size_t o_seq = add(R * 4), o_mr = add(R * 4), o_mrows = add(R * 4), o_bmr = add(R * 4),
-                 o_bmrows = add(R * 4), o_bad = add(R), o_ib = add(R), o_sq = add((B + 1) * 8 * 4),
-                 o_O = add(R * 4), o_P = add(R * 4), o_f = add(R * 8 * 4), o_Z = add(R * 128 * 4),
-                 o_QKV = add(R * 384 * 4), o_A = add(R * 128 * 4), o_Zp = add(R * 32 * 4),
-                 o_QKVp = add(R * 96 * 4), o_Ap = add(R * 32 * 4);
-    if ((e = cudaMalloc(&h->seq_scratch, bytes)) != cudaSuccess)
+    const size_t o_kv = add(4 * planes * cap * 128 * 2), o_kvp = add(4 * planes * cap * 32 * 2), o_O = add(cap * 4),
+                 o_P = add(cap * 4), o_c = add((R + 1) * 4), o_e = add((R + 1) * 4), o_g = add((R + 1) * 4),
+                 o_a = add((R + 1) * 4);
+    if ((e = cudaMalloc(&h->rows_scratch, bytes)) != cudaSuccess)
       return bail(cuda_fail(h, e, "cudaMalloc(decision scratch)"));
-    uint8_t* b0 = h->seq_scratch;
-    SeqParams& q = h->seqp;
-    q.conf = reinterpret_cast<float*>(b0 + o_conf);
-    q.ent_norm = reinterpret_cast<float*>(b0 + o_entn);
-    q.gap = reinterpret_cast<float*>(b0 + o_gap);
-    q.argmax = reinterpret_cast<int*>(b0 + o_arg);
-    q.seq_of = reinterpret_cast<int*>(b0 + o_seq);
-    q.mrank = reinterpret_cast<int*>(b0 + o_mr);
-    q.mrows = reinterpret_cast<int*>(b0 + o_mrows);
-    q.bmrank = reinterpret_cast<int*>(b0 + o_bmr);
-    q.bmrows = reinterpret_cast<int*>(b0 + o_bmrows);
-    q.bad = b0 + o_bad;
-    q.ib = b0 + o_ib;
-    q.sq = reinterpret_cast<int*>(b0 + o_sq);
+    uint8_t* b0 = h->rows_scratch;
+    RowsParams& q = h->rowsp;
+    q.cap_rows = static_cast<int>(cap);
+    q.spare_row = cfg->max_rows;
+    q.kv = reinterpret_cast<__nv_bfloat16*>(b0 + o_kv);
+    q.kvp = reinterpret_cast<__nv_bfloat16*>(b0 + o_kvp);
     q.O = reinterpret_cast<float*>(b0 + o_O);
     q.P = reinterpret_cast<float*>(b0 + o_P);
-    q.feats = reinterpret_cast<float*>(b0 + o_f);
-    q.Z = reinterpret_cast<float*>(b0 + o_Z);
-    q.QKV = reinterpret_cast<float*>(b0 + o_QKV);
-    q.A = reinterpret_cast<float*>(b0 + o_A);
-    q.Zp = reinterpret_cast<float*>(b0 + o_Zp);
-    q.QKVp = reinterpret_cast<float*>(b0 + o_QKVp);
-    q.Ap = reinterpret_cast<float*>(b0 + o_Ap);
+    q.s_conf = reinterpret_cast<float*>(b0 + o_c);
+    q.s_ent = reinterpret_cast<float*>(b0 + o_e);
+    q.s_gap = reinterpret_cast<float*>(b0 + o_g);
+    q.s_arg = reinterpret_cast<int*>(b0 + o_a);
   }
   for (int i = 0; i < 4; ++i)
     if ((e = cudaEventCreate(&h->ev[i])) != cudaSuccess)
@@ -1147,7 +920,6 @@ void ebd_destroy(ebd_handle* h) {
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   cudaFree(h->d_ready);
   cudaFree(h->d_blob);
-  cudaFree(h->d_image);
   cudaFree(h->d_tok);
   cudaFree(h->part_f);
   cudaFree(h->part_i);
@@ -1155,8 +927,8 @@ void ebd_destroy(ebd_handle* h) {
   cudaFree(h->tickets);
   cudaFree(h->d_status);
   cudaFree(h->staging);
-  cudaFree(h->d_seqw);
-  cudaFree(h->seq_scratch);
+  cudaFree(h->d_rows);
+  cudaFree(h->rows_scratch);
   for (int i = 0; i < 4; ++i)
     if (h->ev[i]) cudaEventDestroy(h->ev[i]);
   if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
@@ -1324,44 +1096,7 @@ namespace {
 // windows of more than kMaxWindow rows per sequence: the grid-wide decision
 bool seq_mode(const ebd_handle* h) { return h->cfg.max_window > kMaxWindow; }
 
-SeqParams seq_params(ebd_handle* h, const ebd_step_args* a, const float* conf,
-                     const float* ent_norm, const float* gap, const int* argmax) {
-  const ebd_config& c = h->cfg;
-  SeqParams p = h->seqp;  // scratch
-  p.B = a->batch;
-  p.R = a->rows;
-  p.V = c.vocab;
-  p.gen_len = c.gen_len;
-  p.g_max = c.g_max;
-  p.l_min = c.l_min;
-  p.l_b = c.l_b;
-  p.eos_id = c.eos_id;
-  p.mode = c.decode_mode;
-  p.top_m = c.top_m;
-  p.lps_enabled = c.decode_mode == EBD_DECODE_EB ? c.lps_enabled : 0;
-  p.tau = c.tau;
-  p.tau_psi = c.tau_psi;
-  p.cu_rows = a->cu_rows;
-  p.row_pos = a->row_pos;
-  p.tokens = a->tokens;
-  p.mask = a->mask;
-  p.in_block = a->in_block;
-  p.blk_meta = a->blk_meta;
-  p.conf = conf;
-  p.ent_norm = ent_norm;
-  p.gap = gap;
-  p.argmax = argmax;
-  p.accepted = a->accepted;
-  p.lbs_logit = a->lbs_logit;
-  p.lps_prob = a->lps_prob;
-  p.w = h->d_seqw;
-  p.o = h->seqw;
-  p.tok_table = h->d_tok;
-  p.status = h->d_status;
-  return p;
-}
-
-// LM head, merge into the statistics, grid-wide decision
+// LM head and decision
 ebd_status step_seq(ebd_handle* h, const ebd_step_args* a, cudaStream_t st) {
   if (a->attn_out != nullptr || a->kv_append)
     return fail(h, EBD_ERR_UNSUPPORTED,
@@ -1369,23 +1104,12 @@ ebd_status step_seq(ebd_handle* h, const ebd_step_args* a, cudaStream_t st) {
                 "(this handle has max_window > 64)");
   const int prof = h->profile;
   cudaError_t e;
-  float* conf = a->conf ? a->conf : const_cast<float*>(h->seqp.conf);
-  float* entn = a->ent_norm ? a->ent_norm : const_cast<float*>(h->seqp.ent_norm);
-  float* gap = a->gap ? a->gap : const_cast<float*>(h->seqp.gap);
-  int* arg = a->argmax ? a->argmax : const_cast<int*>(h->seqp.argmax);
-  const SeqParams sp = seq_params(h, a, conf, entn, gap, arg);
-  // the decision's scratch reset first: from the LM head on, every kernel is
-  // a programmatic dependent of the one before it (unless profiled)
-  if ((e = launch_decide_seq_init(sp, st)) != cudaSuccess) return cuda_fail(h, e, "decision reset");
   if (prof && (e = record(h->ev[0], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
   ebd_status s = run_lm(h, a, st);
   if (s != EBD_OK) return s;
   if (prof && (e = record(h->ev[1], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
-  const float inv = static_cast<float>(1.0 / std::log(static_cast<double>(h->cfg.vocab)));
-  if ((e = launch_merge_stats(h->part_f, h->part_i, a->rows, h->grid_lm, h->cfg.vocab, inv, conf,
-                              a->entropy, entn, gap, arg, h->d_status, st, prof == 0)) != cudaSuccess)
-    return cuda_fail(h, e, "merge launch");
-  if ((e = launch_decide_seq(sp, st, true)) != cudaSuccess) return cuda_fail(h, e, "decision launch");
+  if ((e = launch_decide_rows(rows_params(h, a, false), kMaxSeqRows, h->rows_slots, st, prof == 0)) != cudaSuccess)
+    return cuda_fail(h, e, "decision launch");
   if (prof && (e = record(h->ev[2], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
   if (prof && (e = record(h->ev[3], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
   h->prof_mode = prof;
@@ -1412,19 +1136,15 @@ ebd_status step_run(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, cons
   if (prof && (e0 = record(h->ev[0], st)) != cudaSuccess) return cuda_fail(h, e0, "profile event");
   if ((s = run_lm(h, a, st, rt != nullptr && rt->lm_pdl && prof == 0)) != EBD_OK) return s;
   if (prof && (e0 = record(h->ev[1], st)) != cudaSuccess) return cuda_fail(h, e0, "profile event");
-  DecideParams p = decide_params(h, a, 0);
-  p.pdl = prof == 0 ? 1 : 0;  // no event between the LM head and the decision
+  RowsParams p = rows_params(h, a, false);
+  p.warm = prof == 0 ? 1 : 0;  // no event between the LM head and the decision
   if (rt != nullptr) {
     p.tokens_out = rt->tokens_out;
     p.mask_out = rt->mask_out;
     p.in_block_out = rt->in_block_out;
     p.blk_meta_out = rt->blk_meta_out;
   }
-  const bool cta = cta_decision(h, a->batch);
-  // the LM head's CTAs hold one SM each: the decision's CTAs are placed while
-  // it runs if enough SMs are left, and then warm up on a stand-in window
-  p.warm = (p.pdl && cta && h->num_sms - h->lm_ctas >= a->batch) ? 1 : 0;
-  cudaError_t e = cta ? launch_decide_cta(p, st) : launch_decide(p, st);
+  cudaError_t e = launch_decide_rows(p, rows_cap(h, a->batch), h->rows_slots, st, prof == 0);
   if (e != cudaSuccess) return cuda_fail(h, e, "decision launch");
   if (prof == 1 && (e0 = record(h->ev[2], st)) != cudaSuccess)
     return cuda_fail(h, e0, "profile event");
@@ -1472,17 +1192,8 @@ ebd_status ebd_decide(ebd_handle* h, const ebd_step_args* a, void* stream) {
     return fail(h, EBD_ERR_INVALID_ARG, "conf/ent_norm/gap/argmax inputs must be set");
   if (h->w_emb == nullptr) return fail(h, EBD_ERR_STATE, "bind the token embedding first");
   if (a->rows == 0 || a->batch == 0) return EBD_OK;
-  if (seq_mode(h)) {
-    const SeqParams sp = seq_params(h, a, a->conf, a->ent_norm, a->gap, a->argmax);
-    cudaError_t e = launch_decide_seq_init(sp, static_cast<cudaStream_t>(stream));
-    if (e == cudaSuccess) e = launch_decide_seq(sp, static_cast<cudaStream_t>(stream), false);
-    if (e != cudaSuccess) return cuda_fail(h, e, "decision launch");
-    return EBD_OK;
-  }
-  DecideParams p = decide_params(h, a, 1);
-  p.entropy = nullptr;
-  cudaError_t e = cta_decision(h, a->batch) ? launch_decide_cta(p, static_cast<cudaStream_t>(stream))
-                                  : launch_decide(p, static_cast<cudaStream_t>(stream));
+  cudaError_t e = launch_decide_rows(rows_params(h, a, true), rows_cap(h, a->batch), h->rows_slots,
+                                     static_cast<cudaStream_t>(stream), false);
   if (e != cudaSuccess) return cuda_fail(h, e, "decision launch");
   return EBD_OK;
 }
@@ -1499,7 +1210,7 @@ ebd_status ebd_lm_stats(ebd_handle* h, const ebd_step_args* a, void* stream) {
   const float inv = static_cast<float>(1.0 / std::log(static_cast<double>(h->cfg.vocab)));
   cudaError_t e = launch_merge_stats(h->part_f, h->part_i, a->rows, h->grid_lm, h->cfg.vocab, inv,
                                      a->conf, a->entropy, a->ent_norm, a->gap, a->argmax,
-                                     h->d_status, st);
+                                     h->d_status, st, true);
   if (e != cudaSuccess) return cuda_fail(h, e, "merge launch");
   return EBD_OK;
 }

@@ -28,15 +28,12 @@ __device__ __forceinline__ bool in_bounds(long long i, long long n, int* status)
 #endif
 }
 
-constexpr int kMaxWindow = 64;        // window rows per sequence of the cluster decision
-constexpr int kMaxSeqRows = 512;      // window rows per sequence of the grid-wide decision
+constexpr int kMaxWindow = 64;        // window rows per sequence in the block-window setting
+constexpr int kMaxSeqRows = 512;      // in the full-sequence setting
 constexpr int kUnit = 64;             // vocabulary rows per work unit of the LM head
 constexpr int kLmThreads = 320;  // TMA warp, MMA warp, two epilogue warpgroups of 4 warps
 constexpr int kMaxGroupRows = 512;    // rows per LM-head launch (TMEM: 512 columns)
-constexpr int kDecideCluster = 8;     // CTAs per sequence in the decision kernel
-constexpr int kDecideThreads = 256;
-constexpr int kCtaWindow = 32;        // window rows per sequence of the one-CTA decision
-constexpr int kCtaThreads = 512;
+constexpr int kRowsThreads = 256;
 constexpr int kAttnThreads = 128;
 constexpr int kAttnChunk = 64;        // keys per K/V tile
 constexpr int kAttnStages = 3;
@@ -66,104 +63,39 @@ struct AttnParams {
   unsigned ready_ticket;    // another stream, which then writes ready_ticket to *ready
 };
 
-// ------------------------------------------------------------------ routers
-// Device image of the router weights (layout in router_image.h).
-struct RouterImage {
-  const __nv_bfloat16* lbs_w;  // [8 ranks][LBS_W_ELEMS]
-  const __nv_bfloat16* lps_w;  // [LPS_W_ELEMS]
-  const float* vec;            // [8 ranks][V_ELEMS]
-  const float* tok_table;      // [V][64] = W_tok W_e[v] (no bias)
-  const __nv_bfloat16* cta_w;  // [rcta::kChunks][rcta::kChunkElems] (one-CTA kernel)
-  const float* cta_vec;        // [rcta::S_ELEMS]
-};
-
-struct DecideParams {
-  int B, V, grid_lm;        // grid_lm: LM-head partials per row
-  int features_in;          // 1: conf/ent_norm/gap/argmax are inputs
-  int pdl;                  // launched as a programmatic dependent of the LM head
-  int warm;                 // one-CTA kernel: its CTAs find free SMs while the LM head
-                            // runs, and each runs the decision once on a stand-in window
-                            // before it waits for the LM head
-  int mode, top_m;          // EBD_DECODE_*; commits per step of the Top-m rule
-  int gen_len, g_max, l_min, l_b, eos_id, lps_enabled;
+// ------------------------------------------------------------------ decision
+struct RowsParams {
+  int B, R, V, grid_lm;     // grid_lm: LM-head partials per row
+  int features_in;          // 1: s_conf/s_ent/s_gap/s_arg are inputs
+  int strict;               // cu_rows[B] has to be R
+  int warm;                 // launched behind the LM head: first passes on stand-in rows
+  int spare_row;            // a row of s_* that no window row uses
+  int mode, top_m, gen_len, g_max, l_min, l_b, eos_id, lps_enabled;
   float tau, tau_psi, inv_log_v;
   const int* cu_rows;
   const int* row_pos;
   const float4* part_f;
   const int* part_i;
-  const int* tokens;         // decode state in: read before the LM head's grid completes
+  const int* tokens;        // decode state in: read before the LM head's grid completes
   const uint8_t* mask;
   const uint8_t* in_block;
   const int* blk_meta;
-  int* tokens_out;           // decode state out: the same buffers as the state in,
-  uint8_t* mask_out;         // unless the state in is a staged copy of the caller's
+  int* tokens_out;          // decode state out: the same buffers as the state in,
+  uint8_t* mask_out;        // unless the state in is a staged copy of the caller's
   uint8_t* in_block_out;
   int* blk_meta_out;
-  float *conf, *entropy, *ent_norm, *gap, *lbs_logit, *lps_prob;
+  float *conf, *entropy, *ent_norm, *gap, *lbs_logit, *lps_prob;  // outputs, may be null
   int* argmax;
   uint8_t* accepted;
-  int* status;
-  int rows_expected;
-  RouterImage w;
-};
-
-// ------------------------------------------------------------------ grid-wide decision
-// fp32 copy of the router weights for the grid-wide decision (windows of up
-// to kMaxSeqRows rows per sequence): float offsets into one allocation;
-// matrices are stored [in][out] (consecutive outputs contiguous).
-struct SeqLayer {                // one LBS encoder layer
-  int qkv_t, qkv_b, out_t, out_b, ln1_g, ln1_b, ff1_t, ff1_b, ff2_t, ff2_b, ln2_g, ln2_b;
-};
-struct SeqBlock {                // one LPS block
-  int ln1_g, ln1_b, qkv_t, qkv_b, out_t, out_b, ln2_g, ln2_b, ff1_t, ff1_b, ff2_t, ff2_b;
-};
-struct SeqWeights {
-  int ent1_w, ent1_b, ent2_t, ent2_b, entln_g, entln_b, tok_b, comb_t, comb_b, pos;
-  SeqLayer l[2];
-  int head_w, head_b;
-  int in_t, in_b, inln_g, inln_b;  // LPS input layer
-  SeqBlock p[2];
-  int phead_w, phead_b;
-  int total;
-};
-
-struct SeqParams {
-  int B, R, V, gen_len, g_max, l_min, l_b, eos_id, lps_enabled, mode, top_m;
-  float tau, tau_psi;
-  const int* cu_rows;
-  const int* row_pos;
-  int* tokens;
-  uint8_t* mask;
-  uint8_t* in_block;
-  int* blk_meta;
-  const float* conf;        // statistics of every row (inputs)
-  const float* ent_norm;
-  const float* gap;
-  const int* argmax;
-  uint8_t* accepted;        // outputs, may be null
-  float* lbs_logit;
-  float* lps_prob;
-  const float* w;           // SeqWeights image
-  SeqWeights o;
+  float *s_conf, *s_ent, *s_gap;  // statistics of every row [R]: scratch, or inputs
+  int* s_arg;
+  const uint4* mat;         // router image (rows_image.h)
+  const float* vec;
   const float* tok_table;   // [V][64]
-  // scratch, [R] or [R][k] unless noted
-  int* seq_of;
-  int* mrank;               // rank of a masked row within its sequence's M, else -1
-  int* mrows;               // sequence b's masked rows at [cu_rows[b], cu_rows[b] + |M|)
-  int* bmrank;              // rank within B n M (rows the LPS scores), else -1
-  int* bmrows;
-  uint8_t* bad;
-  uint8_t* ib;              // block membership after the selection
-  int* sq;                  // [B + 1][8] per-sequence state (kSq* indices), then step flags
-  float* O;                 // LBS logit
-  float* P;                 // LPS probability
-  float* feats;             // [R][8]
-  float* Z;                 // [R][128]
-  float* QKV;               // [R][384]
-  float* A;                 // [R][128]
-  float* Zp;                // [R][32]
-  float* QKVp;              // [R][96]
-  float* Ap;                // [R][32]
+  int cap_rows;             // rows of the scratch below: R rounded up to 32, and 32 per sequence
+  __nv_bfloat16* kv;        // LBS keys and values [2 layers][2][planes][cap_rows][128]
+  __nv_bfloat16* kvp;       // LPS keys and values [2 blocks][2][planes][cap_rows][32]
+  float *O, *P;             // [cap_rows] LBS logits by rank in M, p_psi by rank in B n M
   int* status;
 };
 
@@ -181,23 +113,18 @@ void lm_plan(LmParams& p, int rows, int V, int d, int num_sms, bool pair = false
 cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const CUtensorMap& kw,
                              const CUtensorMap& vw, const AttnParams& p, cudaStream_t st,
                              bool pdl = false);
-cudaError_t launch_decide(const DecideParams& p, cudaStream_t st);
-// the same decision with one CTA per sequence, for windows of up to
-// kCtaWindow rows (k_decide_cta.cu)
-cudaError_t launch_decide_cta(const DecideParams& p, cudaStream_t st);
+// the decision, the rows of a sequence split over a cluster of CTAs
+// (k_decide.cu); cap: rows per sequence the launch has to hold (32, 64
+// or kMaxSeqRows).  slots: clusters of 8 and of 4 CTAs that fit the GPU at once
+cudaError_t decide_rows_configure(int (&slots)[2]);
+cudaError_t launch_decide_rows(const RowsParams& p, int cap, const int (&slots)[2], cudaStream_t st, bool pdl);
 // vocabulary-parallel LM head: one state per row from a launch's partials,
-// and the statistics from the states of several shards (k_decide.cu)
+// and the statistics from the states of several shards (k_stats.cu)
 cudaError_t launch_shard_state(const float4* part_f, const int* part_i, int rows, int grid,
                                float* state, cudaStream_t st);
 cudaError_t launch_merge_shards(const float* states, int shards, int rows, int V, float inv_log_v,
                                 float* conf, float* entropy, float* ent_norm, float* gap,
                                 int* argmax, int* status, cudaStream_t st);
-// the grid-wide decision: a chain of kernels on `st` (k_decide_seq.cu)
-// the grid-wide decision: the scratch reset (before the LM head, so that the
-// chain from the LM head on is unbroken), then the kernel chain; pdl_first:
-// its first kernel is a programmatic dependent of the kernel before it
-cudaError_t launch_decide_seq_init(const SeqParams& p, cudaStream_t st);
-cudaError_t launch_decide_seq(const SeqParams& p, cudaStream_t st, bool pdl_first);
 // prefix-cache append on commit: window row r of sequence b with mask[r] == 0
 // is copied (K and V, Hkv * D bf16 each) to cache position row_pos[r] < Pmax
 cudaError_t launch_kv_append(uint16_t* k_cache, uint16_t* v_cache, const uint16_t* k_win,

@@ -1,996 +1,1384 @@
-// The EB decision for every sequence of a step (App. E, algorithm
-// "Inference with LBS Block Selection and LPS Parallel Commit"):
-//   1. merge the LM-head partial states of each window row into
-//      kappa, H, H~ = H / ln|V|, Delta and x_hat (App. B, Sec. 5.1, Sec. 5.2);
-//   2. with no active block and |M| > L_min: the LBS router (Sec. 5.1,
-//      App. C.1) over the masked rows, then EOS removal, MaxGapFilter and the
-//      min-tokens fallback; with |M| <= L_min: B = M;
-//   3. the LPS router (Sec. 5.2, App. D.1) over the masked rows of B with
-//      features (kappa, H~, Delta, rho, pos);
-//   4. union accept, anti-stall fallback, parallel commit, block resolution.
+// The EB decision of a step (App. E algorithm "Inference with LBS Block
+// Selection and LPS Parallel Commit"; LBS, Sec. 5.1 and App. C.1; LPS,
+// Sec. 5.2 and App. D.1; baseline rules, App. B Eq. prelim-update), one
+// cluster of CTAs per sequence, the rows of a sequence split over the CTAs.
 //
-// One thread-block cluster of 8 CTAs per sequence.  The LBS encoder is split
-// across the cluster by output features (and, for attention, by head and
-// query half); every CTA keeps a full copy of the residual stream and the
-// slices are exchanged through distributed shared memory.  The LPS router
-// and the decision run in rank 0.
+// Everything but attention and the selection is local to a row, so a CTA
+// takes groups of 8 rows (the masked rows by rank) through whole LBS encoder
+// layers on its own; the CTAs of a cluster meet only where attention needs
+// every row's keys and values (once per layer) and before the selection:
+// three cluster barriers.  Keys and values travel through an L2-resident
+// scratch.  The LPS router is small enough for a warp to take 8 rows of
+// B n M through it in registers; its warps meet for the keys and values of
+// its two attentions only.
 //
-// Matrix products run on the tensor cores (mma.sync m16n8k16, bf16 weights,
-// fp32 accumulation).  Every activation that feeds a product is stored once,
-// by the phase that produces it, as a bf16 high part and a bf16 remainder
-// (x = hi + lo to ~16 mantissa bits), so that a product loads its A fragments
-// with ldmatrix and runs two MMAs per k-step.  The kernel is short and
-// latency-bound: phases are kept few and their per-warp chains short.
-#include <cooperative_groups.h>
-
+// Products run on mma.sync (m16n8k16) with the weights as the M = 16 operand
+// and the rows as N = 8.  The weights are bf16 values; an activation x is held
+// as NP bf16 planes, x = x0 + x1 (+ x2), so that a product has the
+// activation's ~16 (24) bits, and two activations multiply as the products of
+// planes i, j with i + j < NP.  NP = 2 for windows of up to 64 rows, 3 (fp32
+// accuracy) above.
 #include <climits>
 
-#include "decide_common.cuh"
-
-namespace cg = cooperative_groups;
+#include "decide_math.cuh"
+#include "internal.h"
+#include "ptx.cuh"
+#include "rows_image.h"
 
 namespace ebd {
 
 namespace {
 
-// activation pool (floats), LBS phase
-constexpr int P_Z = 0;                       // [64][132] fp32 residual stream z
-constexpr int P_ZH = P_Z + W * LDZ;          // [64][136] bf16 x2: z as GEMM input (hi, lo)
-constexpr int P_XH = P_ZH + W * LDH;         // [64][136] bf16 x2: [e;t] | concat ; fp32 FFN inbox [8][64][16]
-constexpr int P_KV = P_XH + W * LDH;         // [64][68]  fp32 k,v of this CTA's head | bf16 x2 FFN hidden / F_ent
-constexpr int P_Q = P_KV + W * LDKV;         // [32][36]  fp32 queries of this CTA's half
-constexpr int P_S = P_Q + 32 * LDQ;          // [32][68]  fp32 attention scores
-constexpr int POOL = P_S + 32 * LDS;
-static_assert(8 * W * 16 <= W * LDH, "FFN partial inbox");
-static_assert(W * 72 <= POOL - P_KV, "F_ent hidden hi/lo (spans k/v, q and scores)");
-static_assert(W * LDZ <= W * LDH, "ent2 output scratch in the z hi/lo region");
-static_assert(L_PROB + W <= POOL, "LPS pool layout");
+using namespace rowimg;
 
-struct __align__(16) Smem {
-  __nv_bfloat16 w[LBS_W_ELEMS];  // this rank's LBS weight slices; later the LPS weights
-  float v[V_ELEMS];              // vectors
-  float pool[POOL];
-  float f_conf[W], f_ent[W], f_gap[W], f_O[W], f_p[W];
-  int f_arg[W], f_pos[W], f_tok[W], Mrows[W], Brows[W], BMrows[W];
-  uint8_t f_mask[W], f_ib[W], f_acc[W], f_bad[W];
-  int nM, nBM, meta_b, meta_s, n_rows, r0, run_lbs, bad_seq, lps_loaded;
-  uint64_t bar;   // vectors (+ LBS weights)
-  uint64_t bar2;  // LPS weights
+constexpr int kT = kRowsThreads;  // 256
+constexpr int kNW = kT / 32;
+constexpr int kVecs = V_POS;  // floats of the vectors staged in shared memory
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// byte stride of a row of K bf16: 64 mod 128, so that the 16-byte reads of
+// two consecutive rows by 8 lanes fall in different banks
+__device__ __host__ constexpr int row_bytes(int K) { return K == 32 ? 64 : 2 * K + 64; }
+
+template <int NR, int NP>
+struct Lay {  // shared memory, byte offsets
+  static constexpr int R = 8 * NR;                  // rows of a CTA
+  static constexpr int P128 = R * row_bytes(128);   // one plane of R rows x 128
+  static constexpr int P256 = R * row_bytes(256);
+  static constexpr int kLdF = 132;                  // fp32 row stride of F
+  static constexpr int kLdO = 36;                   // partial attention output
+  static constexpr int V = 0;                       // vectors of the image
+  static constexpr int U = V + kVecs * 4;
+  // LBS activations ...
+  static constexpr int A = U;
+  static constexpr int Y = A + NP * P128;
+  static constexpr int Q = Y + NP * P128;
+  static constexpr int H = Q + NP * P128;           // FFN hidden, or attention partials
+  static constexpr int kPart = NR * kNW * 8 * kLdO * 4;
+  static constexpr int kH = NP * P256 > kPart ? NP * P256 : kPart;
+  static constexpr int ML = H + kH;                 // [NR][warp][8] (max, sum)
+  static constexpr int F = ML + NR * kNW * 8 * 8;
+  static constexpr int kLbsEnd = F + R * kLdF * 4;
+  // ... and, once they are dead, the LPS weights and (windows of up to 64
+  // rows) the keys and values of both blocks
+  static constexpr int W = U;
+  static constexpr int kLpsMat = 2 * MB_STRIDE;     // 16-byte units
+  static constexpr int KV = W + kLpsMat * 16;
+  static constexpr int kKvBlock = 64 * 64 * NP;     // elements of a block
+  static constexpr int kLpsEnd = KV + (NP == 2 ? 2 * kKvBlock * 2 : 0);
+  static constexpr int SLOT = kLbsEnd > kLpsEnd ? kLbsEnd : kLpsEnd;
+  static constexpr int ROW = SLOT + 3 * 32 * 4;     // per-row arrays
 };
-static_assert(sizeof(Smem) + 16 <= 232448, "dynamic shared memory of one CTA");
 
-// ------------------------------------------------------------------ LBS attention
-// This CTA's query rows [qa, qa + nq) of head hd (width 32) over the n rows'
-// keys/values: softmax(q k^T / sqrt(32)) v on the tensor cores.  q, k, v and
-// the probabilities are split into bf16 high and low parts (three products
-// per pair).  The work is spread over the warps: a warp takes one 16-query
-// tile, one block of 16 keys and (when tiles x blocks leave warps idle) a
-// group of the 8-column output tiles, and leaves its block's row max m, sum l
-// and unnormalised output o in shared memory (the z hi/lo region, free
-// between the QKV product and the next LayerNorm).  The whole CTA then
-// combines the blocks, out = sum_b e^(m_b - M) o_b / sum_b e^(m_b - M) l_b,
-// and writes the result as hi/lo, 16 bytes per store, into every rank's
-// concat buffer.
-constexpr int kAttLdp = 40;  // row stride of a partial output tile (floats)
+// the rows of this CTA's groups
+struct Slots {
+  int mrow[32];   // window row of a masked-rank slot, -1: none
+  float ent[32];
+  int arg[32];
+};
 
-__device__ __forceinline__ void lbs_attention(cg::cluster_group& cluster, float* P, int nq, int n,
-                                              int qa, int hd) {
-  const float* Q = P + P_Q;
-  const float* KV = P + P_KV;
-  float* part_o = P + P_ZH;                    // [unit][16][kAttLdp]
-  float* part_ml = part_o + 8 * 16 * kAttLdp;  // [unit][16][2]
-  static_assert(8 * 16 * (kAttLdp + 2) <= W * LDH, "attention partials fit the z hi/lo region");
-  __nv_bfloat16* X = reinterpret_cast<__nv_bfloat16*>(P + P_XH);
+template <int CAP>
+struct RowState {
+  int pos[CAP];
+  float conf[CAP];
+  float prob[CAP];
+  float feat[CAP][5];
+  int bpos[CAP];
+  int cnt[CAP / 32];
+  int urow[CAP];  // unmasked rows whose statistics this CTA merges
+  int cut, first, any, best, open;
+};
+
+__device__ __forceinline__ uint32_t pack2(float x, float y) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float lo_f(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float hi_f(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
+__device__ __forceinline__ float rcp(float x) {  // at most 1 ulp off
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// (x, y) as NP packed planes; every remainder is exact
+template <int NP>
+__device__ __forceinline__ void split2(float x, float y, uint32_t (&p)[NP]) {
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    p[i] = pack2(x, y);
+    x -= lo_f(p[i]);
+    y -= hi_f(p[i]);
+  }
+}
+
+// stores columns (c, c + 1) of a row into NP planes
+template <int NP>
+__device__ __forceinline__ void put2(uint8_t* base, int plane, int rb, int row, int c, float x, float y) {
+  uint32_t p[NP];
+  split2<NP>(x, y, p);
+#pragma unroll
+  for (int i = 0; i < NP; ++i)
+    *reinterpret_cast<uint32_t*>(base + i * plane + row * rb + 2 * c) = p[i];
+}
+
+// transpose of an 8 x 8 bf16 matrix, lane 4 g + t holding (row g, columns
+// 2 t, 2 t + 1): turns a product's accumulators (output g, rows 2 t, 2 t + 1)
+// into the next product's B fragment (row g, inputs 2 t, 2 t + 1)
+__device__ __forceinline__ uint32_t trans8(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+
+__device__ __forceinline__ uint4 ld_w(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// A fragments of the m16 tiles tile0 + 8 i of a matrix with K inputs
+template <int K, int NT>
+__device__ __forceinline__ void load_w(uint4 (&w)[NT * (K / 16)], const uint4* m, int tile0) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < NT; ++i)
+#pragma unroll
+    for (int ks = 0; ks < K / 16; ++ks)
+      w[i * (K / 16) + ks] = ld_w(m + ((tile0 + 8 * i) * (K / 16) + ks) * 32 + lane);
+}
+
+__device__ __forceinline__ void mma4(float (&d)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  const uint32_t r[4] = {a.x, a.y, a.z, a.w};
+  mma_bf16(d, r, b0, b1);
+}
+
+// acc[r][i]: outputs 16 tile_i + 2 g (elements 0, 1) and + 1 (2, 3) of rows
+// 8 r + 2 t, 8 r + 2 t + 1 of A W^T, A in NP planes.  The first plane has its
+// own accumulators; with NP = 3 they are added up in fp32 every 32 inputs,
+// since the tensor cores truncate where they align a sum's terms.
+template <int K, int NT, int NR, int NP>
+__device__ __forceinline__ void gemm(const uint8_t* A, int plane, const uint4 (&w)[NT * (K / 16)], int nr,
+                                     float (&acc)[NR][NT][4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  float al[NR][NT][4];
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int i = 0; i < NT; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[r][i][e] = al[r][i][e] = 0.f;
+#pragma unroll
+  for (int kb = 0; kb < K / 32; ++kb)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (NR > 1 && r >= nr) continue;
+      uint4 x[NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+        x[p] = *reinterpret_cast<const uint4*>(A + p * plane + (8 * r + g) * row_bytes(K) + 64 * kb + 16 * t);
+#pragma unroll
+      for (int i = 0; i < NT; ++i) {
+        const uint4 &a = w[i * (K / 16) + 2 * kb], &b = w[i * (K / 16) + 2 * kb + 1];
+#pragma unroll
+        for (int p = NP - 1; p > 0; --p) {
+          mma4(al[r][i], a, x[p].x, x[p].y);
+          mma4(al[r][i], b, x[p].z, x[p].w);
+        }
+        if (NP == 3) {
+          float d[4] = {0.f, 0.f, 0.f, 0.f};
+          mma4(d, a, x[0].x, x[0].y);
+          mma4(d, b, x[0].z, x[0].w);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[r][i][e] += d[e];
+        } else {
+          mma4(acc[r][i], a, x[0].x, x[0].y);
+          mma4(acc[r][i], b, x[0].z, x[0].w);
+        }
+      }
+    }
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int i = 0; i < NT; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[r][i][e] += al[r][i][e];
+}
+
+// LayerNorm (eps 1e-5) of a warp's row of 32 * N values, lane holding
+// columns lane * N .. + N
+template <int N>
+__device__ __forceinline__ void norm_row(float (&v)[N], const float* g, const float* b) {
+  const int lane = threadIdx.x & 31;
+  float s = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) s += v[i];
+  const float mean = warp_sum(s) * (1.0f / (32 * N));
+  float q = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) q += (v[i] - mean) * (v[i] - mean);
+  const float inv = rsqrtf(warp_sum(q) * (1.0f / (32 * N)) + 1e-5f);
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = (v[i] - mean) * inv * g[lane * N + i] + b[lane * N + i];
+}
+
+// Ranks of 0/1 flags over the rows j = 32 c + lane, chunk c = warp + 8 i:
+// rank[i] = flags set before row j; returns the total.  All threads.
+template <int CAP>
+__device__ __forceinline__ int rank_rows(RowState<CAP>& rs, const bool* flag, int* rank) {
+  constexpr int NC = CAP / 32, RPT = (NC + kNW - 1) / kNW;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t bal[RPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {
+    const int c = warp + kNW * i;
+    bal[i] = __ballot_sync(0xffffffffu, c < NC && flag[i]);
+    if (lane == 0 && c < NC) rs.cnt[c] = __popc(bal[i]);
+  }
+  __syncthreads();
+  int total = 0;
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) rank[i] = __popc(bal[i] & ((1u << lane) - 1u));
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const int n = rs.cnt[c];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+      if (c < warp + kNW * i) rank[i] += n;
+    total += n;
+  }
+  __syncthreads();
+  return total;
+}
+
+// reductions over the lanes of equal t (the 8 values of g)
+__device__ __forceinline__ float gsum(float v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 8);
+  return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+__device__ __forceinline__ float gmax(float v) {
+  v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 4));
+  v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
+  return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
+}
+
+// One block's online softmax: s = scores (in log2 units) of TL tiles of 16
+// keys (elements 0, 2: query 2 t; 1, 3: query 2 t + 1) becomes the probabilities against the
+// updated running maxima m; returns the old values' factors in c.
+template <int TL>
+__device__ __forceinline__ void softmax_block(float (&s)[TL][4], float (&m)[2], float (&l)[2], float (&c)[2]) {
+  float a0 = -INFINITY, a1 = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < TL; ++j) {
+    a0 = fmaxf(a0, fmaxf(s[j][0], s[j][2]));
+    a1 = fmaxf(a1, fmaxf(s[j][1], s[j][3]));
+  }
+  const float n0 = fmaxf(m[0], gmax(a0)), n1 = fmaxf(m[1], gmax(a1));  // finite: a block holds a key
+  c[0] = exp2f(m[0] - n0);
+  c[1] = exp2f(m[1] - n1);
+  m[0] = n0;
+  m[1] = n1;
+  float b0 = 0.f, b1 = 0.f;
+#pragma unroll
+  for (int j = 0; j < TL; ++j) {
+    s[j][0] = exp2f(s[j][0] - n0);
+    s[j][2] = exp2f(s[j][2] - n0);
+    s[j][1] = exp2f(s[j][1] - n1);
+    s[j][3] = exp2f(s[j][3] - n1);
+    b0 += s[j][0] + s[j][2];
+    b1 += s[j][1] + s[j][3];
+  }
+  l[0] = l[0] * c[0] + b0;
+  l[1] = l[1] * c[1] + b1;
+}
+
+// LBS attention of this CTA's groups of 8 queries over n keys in blocks of
+// 32, warp = (head, half of the blocks): running maximum and sum per warp,
+// the unnormalised output to `part`, (max, sum) to `ml`.  Q (scaled) in
+// planes in shared memory; Kp planes [key][128], Vp planes [dim][capk].
+// Scores are K Q^T (keys as M), outputs V^T P^T.  Row r of key tile s of a
+// block is key 8 (r / 2 % 4) + r % 2 + 2 (r / 8) + 4 s, so that lane t's keys
+// of the second product are 8 consecutive ones.
+template <int NR, int NP>
+__device__ __forceinline__ void attend(const uint8_t* Q, const __nv_bfloat16* Kp, const __nv_bfloat16* Vp,
+                                       size_t plane, int capk, int n, int nr, float* part, float* ml) {
+  using L = Lay<NR, NP>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const float scale = 0.17677669529663687f;  // 1/sqrt(32)
-  const int mtq = (nq + 15) >> 4, nkb = (n + 15) >> 4;
-  const int units = mtq * nkb;  // <= 2 x 4
-  const int nsplit = units <= 2 ? 4 : (units <= 4 ? 2 : 1);
-  if (warp < units * nsplit) {
-    const int u = warp / nsplit, part = warp % nsplit;
-    const int qt = u / nkb, kb = u % nkb;
-    const int nt0 = part * (4 / nsplit), nt1 = nt0 + 4 / nsplit;
-    const int r_lo = qt * 16 + g, r_hi = r_lo + 8;
-    uint32_t qh[2][4], ql[2][4];
+  const int head = warp & 3, half = warp >> 2;
+  const int n8 = (n + 7) & ~7;  // rows written
+  float o[NR][2][4], m[NR][2], l[NR][2];
 #pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      const float2 z = make_float2(0.f, 0.f);
-      const float* ql0 = Q + r_lo * LDQ + 16 * ks + 2 * t;
-      const float* qh0 = Q + r_hi * LDQ + 16 * ks + 2 * t;
-      const float2 a0 = r_lo < nq ? *reinterpret_cast<const float2*>(ql0) : z;
-      const float2 a1 = r_hi < nq ? *reinterpret_cast<const float2*>(qh0) : z;
-      const float2 a2 = r_lo < nq ? *reinterpret_cast<const float2*>(ql0 + 8) : z;
-      const float2 a3 = r_hi < nq ? *reinterpret_cast<const float2*>(qh0 + 8) : z;
-      split_bf16x2(a0.x, a0.y, qh[ks][0], ql[ks][0]);
-      split_bf16x2(a1.x, a1.y, qh[ks][1], ql[ks][1]);
-      split_bf16x2(a2.x, a2.y, qh[ks][2], ql[ks][2]);
-      split_bf16x2(a3.x, a3.y, qh[ks][3], ql[ks][3]);
-    }
-    const int k0 = 16 * kb;
-    float s[2][4];
+  for (int r = 0; r < NR; ++r) {
+    m[r][0] = m[r][1] = -INFINITY;
+    l[r][0] = l[r][1] = 0.f;
 #pragma unroll
-    for (int hb = 0; hb < 2; ++hb) {
-      const int key = k0 + 8 * hb + g;
-      float a[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int d = 0; d < 2; ++d)
 #pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        const float2 z = make_float2(0.f, 0.f);
-        const float* kp = KV + key * LDKV + 16 * ks + 2 * t;
-        const float2 k0v = key < n ? *reinterpret_cast<const float2*>(kp) : z;
-        const float2 k1v = key < n ? *reinterpret_cast<const float2*>(kp + 8) : z;
-        uint32_t bh0, bl0, bh1, bl1;
-        split_bf16x2(k0v.x, k0v.y, bh0, bl0);
-        split_bf16x2(k1v.x, k1v.y, bh1, bl1);
-        mma_bf16(a, qh[ks], bh0, bh1);
-        mma_bf16(a, qh[ks], bl0, bl1);
-        mma_bf16(a, ql[ks], bh0, bh1);
+      for (int e = 0; e < 4; ++e) o[r][d][e] = 0.f;
+  }
+  uint4 kf[2][2][NP];  // [tile][row half][plane]
+  auto load_k = [&](int blk) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        int key = 32 * blk + 8 * (g >> 1) + (g & 1) + 2 * u + 4 * s;
+        key = key < n8 ? key : 0;
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+          kf[s][u][p] = __ldcg(reinterpret_cast<const uint4*>(Kp + p * plane + static_cast<size_t>(key) * 128 +
+                                                              32 * head + 8 * t));
       }
-      const int c = k0 + 8 * hb + 2 * t;
-      s[hb][0] = c < n ? a[0] * scale : -INFINITY;
-      s[hb][1] = c + 1 < n ? a[1] * scale : -INFINITY;
-      s[hb][2] = c < n ? a[2] * scale : -INFINITY;
-      s[hb][3] = c + 1 < n ? a[3] * scale : -INFINITY;
-    }
-    float m0 = fmaxf(fmaxf(s[0][0], s[0][1]), fmaxf(s[1][0], s[1][1]));
-    float m1 = fmaxf(fmaxf(s[0][2], s[0][3]), fmaxf(s[1][2], s[1][3]));
-    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1));
-    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2));
-    m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 1));
-    m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 2));  // finite: key k0 is valid
+  };
+  if (32 * half < n) load_k(half);
+  for (int blk = half; 32 * blk < n; blk += 2) {
+    uint4 vf[2][2][NP];  // [dim tile][row half][plane]
+    const bool vok = 32 * blk + 8 * t < n8;
 #pragma unroll
-    for (int hb = 0; hb < 2; ++hb) {
-      s[hb][0] = expf(s[hb][0] - m0);
-      s[hb][1] = expf(s[hb][1] - m0);
-      s[hb][2] = expf(s[hb][2] - m1);
-      s[hb][3] = expf(s[hb][3] - m1);
-    }
-    uint32_t ph[4], pl[4];
-    split_bf16x2(s[0][0], s[0][1], ph[0], pl[0]);
-    split_bf16x2(s[0][2], s[0][3], ph[1], pl[1]);
-    split_bf16x2(s[1][0], s[1][1], ph[2], pl[2]);
-    split_bf16x2(s[1][2], s[1][3], ph[3], pl[3]);
-    float* po = part_o + u * 16 * kAttLdp;
+    for (int d = 0; d < 2; ++d)
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      if (nt < nt0 || nt >= nt1) continue;
-      float o[4] = {0.f, 0.f, 0.f, 0.f};
-      float v[4];
+      for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int key = k0 + (e >> 1) * 8 + 2 * t + (e & 1);
-        v[e] = key < n ? KV[key * LDKV + 32 + 8 * nt + g] : 0.f;
+        for (int p = 0; p < NP; ++p)
+          vf[d][u][p] = vok ? __ldcg(reinterpret_cast<const uint4*>(
+                                  Vp + p * plane + static_cast<size_t>(32 * head + 16 * d + 2 * g + u) * capk +
+                                  32 * blk + 8 * t))
+                            : make_uint4(0u, 0u, 0u, 0u);
+    uint32_t pb[NR][2][NP][2];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (NR > 1 && r >= nr) continue;
+      uint4 x[NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+        x[p] = *reinterpret_cast<const uint4*>(Q + p * L::P128 + (8 * r + g) * row_bytes(128) + 64 * head + 16 * t);
+      float s[2][4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[j][e] = 0.f;
+#pragma unroll
+        for (int sum = NP - 1; sum >= 0; --sum)
+#pragma unroll
+          for (int a = 0; a <= sum; ++a) {
+            const uint4 &u = kf[j][0][a], &v = kf[j][1][a], &q = x[sum - a];
+            mma4(s[j], make_uint4(u.x, v.x, u.y, v.y), q.x, q.y);
+            mma4(s[j], make_uint4(u.z, v.z, u.w, v.w), q.z, q.w);
+          }
+        const int key = 32 * blk + 8 * (g >> 1) + (g & 1) + 4 * j;
+        if (key >= n) s[j][0] = s[j][1] = -INFINITY;
+        if (key + 2 >= n) s[j][2] = s[j][3] = -INFINITY;
       }
-      uint32_t v0h, v0l, v1h, v1l;
-      split_bf16x2(v[0], v[1], v0h, v0l);
-      split_bf16x2(v[2], v[3], v1h, v1l);
-      mma_bf16(o, ph, v0h, v1h);
-      mma_bf16(o, ph, v0l, v1l);
-      mma_bf16(o, pl, v0h, v1h);
-      *reinterpret_cast<float2*>(po + g * kAttLdp + 8 * nt + 2 * t) = make_float2(o[0], o[1]);
-      *reinterpret_cast<float2*>(po + (g + 8) * kAttLdp + 8 * nt + 2 * t) = make_float2(o[2], o[3]);
+      float c[2];
+      softmax_block<2>(s, m[r], l[r], c);
+#pragma unroll
+      for (int d = 0; d < 2; ++d)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[r][d][e] *= c[e & 1];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          uint32_t q[NP];
+          split2<NP>(s[j][2 * u], s[j][2 * u + 1], q);
+#pragma unroll
+          for (int p = 0; p < NP; ++p) pb[r][j][p][u] = trans8(q[p]);
+        }
     }
-    if (part == 0) {
-      float l0 = (s[0][0] + s[0][1]) + (s[1][0] + s[1][1]);
-      float l1 = (s[0][2] + s[0][3]) + (s[1][2] + s[1][3]);
-      l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-      l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-      l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-      l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-      if (t == 0) {
-        float* pm = part_ml + u * 32;
-        *reinterpret_cast<float2*>(pm + 2 * g) = make_float2(m0, l0);
-        *reinterpret_cast<float2*>(pm + 2 * (g + 8)) = make_float2(m1, l1);
+    if (32 * (blk + 2) < n) load_k(blk + 2);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (NR > 1 && r >= nr) continue;
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int sum = NP - 1; sum >= 0; --sum)
+#pragma unroll
+          for (int a = 0; a <= sum; ++a) {
+            const uint4 &u = vf[d][0][a], &v = vf[d][1][a];
+            mma4(y, make_uint4(u.x, v.x, u.y, v.y), pb[r][0][sum - a][0], pb[r][0][sum - a][1]);
+            mma4(y, make_uint4(u.z, v.z, u.w, v.w), pb[r][1][sum - a][0], pb[r][1][sum - a][1]);
+          }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[r][d][e] += y[e];
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    if (NR > 1 && r >= nr) continue;
+    float* po = part + (r * kNW + warp) * 8 * L::kLdO;
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      *reinterpret_cast<float2*>(po + 2 * t * L::kLdO + 16 * d + 2 * g) = make_float2(o[r][d][0], o[r][d][2]);
+      *reinterpret_cast<float2*>(po + (2 * t + 1) * L::kLdO + 16 * d + 2 * g) = make_float2(o[r][d][1], o[r][d][3]);
+    }
+    const float l0 = gsum(l[r][0]), l1 = gsum(l[r][1]);
+    if (g == 0)
+      *reinterpret_cast<float4*>(ml + (r * kNW + warp) * 16 + 4 * t) = make_float4(m[r][0], l0, m[r][1], l1);
+  }
+}
+
+// The two halves' partial outputs merged and normalised, as NP planes of the
+// concatenated heads.  All threads.
+template <int NR, int NP>
+__device__ __forceinline__ void attend_merge(const float* part, const float* ml, uint8_t* A, int nr) {
+  using L = Lay<NR, NP>;
+  for (int it = threadIdx.x; it < 8 * nr * 64; it += kT) {
+    const int row = it >> 6, c = 2 * (it & 63), r = row >> 3, rr = row & 7, h = c >> 5, d = c & 31;
+    const float2 u = *reinterpret_cast<const float2*>(ml + (r * kNW + h) * 16 + 2 * rr);
+    const float2 v = *reinterpret_cast<const float2*>(ml + (r * kNW + 4 + h) * 16 + 2 * rr);
+    const float M = fmaxf(u.x, v.x);
+    const float e0 = exp2f(u.x - M), e1 = exp2f(v.x - M);  // an empty half has max -inf
+    const float2 x = *reinterpret_cast<const float2*>(part + ((r * kNW + h) * 8 + rr) * L::kLdO + d);
+    const float2 y = *reinterpret_cast<const float2*>(part + ((r * kNW + 4 + h) * 8 + rr) * L::kLdO + d);
+    const float il = rcp(e0 * u.y + e1 * v.y);
+    put2<NP>(A, L::P128, row_bytes(128), row, c, (e0 * x.x + e1 * y.x) * il, (e0 * x.y + e1 * y.y) * il);
+  }
+}
+
+// ------------------------------------------------------------------ LBS
+struct LbsArgs {
+  const uint4* mat;
+  const float* vec;
+  const float* tok_table;
+  __nv_bfloat16* kv;
+  float* O;
+  int V, gen_len, cap_rows, kbase, capk, nM;
+  int nr, first, step;  // this CTA's groups of 8 masked rows: first, first + step, ..
+
+  template <int NP>
+  __device__ __forceinline__ __nv_bfloat16* keys(int l) const {
+    return kv + (static_cast<size_t>(2 * l) * NP * cap_rows + kbase) * 128;
+  }
+  template <int NP>
+  __device__ __forceinline__ __nv_bfloat16* values(int l) const {
+    return kv + (static_cast<size_t>(2 * l + 1) * NP * cap_rows + kbase) * 128;
+  }
+};
+
+// epi(row, column c, values of columns c, c + 1) over a product's outputs
+template <class Epi>
+__device__ __forceinline__ void each(const float (&a)[4], int r, int tile, Epi epi) {
+  const int lane = threadIdx.x & 31, row = 8 * r + 2 * (lane & 3), c = 16 * tile + 2 * (lane >> 2);
+  epi(row, c, a[0], a[2]);
+  epi(row + 1, c, a[1], a[3]);
+}
+// F += a + bias
+__device__ __forceinline__ void add_f(float* F, int ld, const float (&a)[4], int r, int tile, const float* bias) {
+  each(a, r, tile, [&](int row, int c, float x, float y) {
+    float2* z = reinterpret_cast<float2*>(F + row * ld + c);
+    *z = make_float2(z->x + (x + bias[c]), z->y + (y + bias[c + 1]));
+  });
+}
+
+// LBS input z (Eq. lbs_feat) of the CTA's rows: fp32 in F, planes in Y.  Not
+// inlined, like the QKV product: run once on stand-in rows before the
+// statistics are there, its instructions are on the SM when they are.
+template <int NR, int NP>
+__device__ __noinline__ void lbs_input(const LbsArgs a) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  float* const F = reinterpret_cast<float*>(smem + L::F);
+  const float* const sv = reinterpret_cast<const float*>(smem + L::V);
+  const Slots& sl = *reinterpret_cast<const Slots*>(smem + L::SLOT);
+  uint8_t* const sA = smem + L::A;
+  uint8_t* const sY = smem + L::Y;
+  constexpr int LDF = L::kLdF;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nr = a.nr;
+  uint4 wc[8];
+  // F_ent hidden, rows without a masked row as zeros
+  for (int it = tid; it < 8 * nr * 32; it += kT) {
+    const int row = it >> 5, c = 2 * (it & 31);
+    const bool ok = sl.mrow[row] >= 0;
+    const float h = ok ? sl.ent[row] : 0.f;
+    // the token branch W_tok W_e[x_hat] + b (folded table): columns 64..127
+    const int tok = ok ? sl.arg[row] : -1;
+    float2 tv = make_float2(0.f, 0.f);
+    if (tok >= 0 && tok < a.V)
+      tv = __ldg(reinterpret_cast<const float2*>(a.tok_table + static_cast<size_t>(tok) * 64 + c));
+    put2<NP>(sY, L::P128, row_bytes(64), row, c, gelu(fmaf(sv[V_ENT1W + c], h, sv[V_ENT1B + c])),
+             gelu(fmaf(sv[V_ENT1W + c + 1], h, sv[V_ENT1B + c + 1])));
+    put2<NP>(sA, L::P128, row_bytes(128), row, 64 + c, tv.x + sv[V_TOKB + c], tv.y + sv[V_TOKB + c + 1]);
+  }
+  {
+    uint4 w[4];
+    load_w<64, 1>(w, a.mat + M_ENT2, warp & 3);
+    load_w<128, 1>(wc, a.mat + M_COMB, warp);
+    __syncthreads();
+    if (warp < 4) {
+      float acc[NR][1][4];
+      gemm<64, 1, NR, NP>(sY, L::P128, w, nr, acc);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        if (r >= nr) continue;
+        each(acc[r][0], r, warp, [&](int row, int c, float x, float y) {
+          *reinterpret_cast<float2*>(F + row * LDF + c) = make_float2(x + sv[V_ENT2B + c], y + sv[V_ENT2B + c + 1]);
+        });
       }
     }
   }
   __syncthreads();
-  // combine: one thread per (query row, 8 output columns), both planes to
-  // every rank (this one included)
-#pragma unroll 1
-  for (int it = threadIdx.x; it < nq * 4; it += blockDim.x) {
-    const int r = it >> 2, c8 = it & 3, qt = r >> 4, rr = r & 15;
-    float M = -INFINITY;
-#pragma unroll 1
-    for (int kb = 0; kb < nkb; ++kb) M = fmaxf(M, part_ml[(qt * nkb + kb) * 32 + 2 * rr]);
-    float L = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int u = qt * nkb + kb;
-      const float2 ml = *reinterpret_cast<const float2*>(part_ml + u * 32 + 2 * rr);
-      const float e = expf(ml.x - M);
-      L = fmaf(e, ml.y, L);
-      const float4* src = reinterpret_cast<const float4*>(part_o + (u * 16 + rr) * kAttLdp + 8 * c8);
-      const float4 x0 = src[0], x1 = src[1];
-      acc[0] = fmaf(e, x0.x, acc[0]);
-      acc[1] = fmaf(e, x0.y, acc[1]);
-      acc[2] = fmaf(e, x0.z, acc[2]);
-      acc[3] = fmaf(e, x0.w, acc[3]);
-      acc[4] = fmaf(e, x1.x, acc[4]);
-      acc[5] = fmaf(e, x1.y, acc[5]);
-      acc[6] = fmaf(e, x1.z, acc[6]);
-      acc[7] = fmaf(e, x1.w, acc[7]);
-    }
-    const float iL = 1.0f / L;
-    uint4 hi, lo;
-    split_bf16x2(acc[0] * iL, acc[1] * iL, hi.x, lo.x);
-    split_bf16x2(acc[2] * iL, acc[3] * iL, hi.y, lo.y);
-    split_bf16x2(acc[4] * iL, acc[5] * iL, hi.z, lo.z);
-    split_bf16x2(acc[6] * iL, acc[7] * iL, hi.w, lo.w);
-    const int off = (qa + r) * LDH + 32 * hd + 8 * c8;
-#pragma unroll 1
-    for (int rk = 0; rk < kDecideCluster; ++rk) {
-      __nv_bfloat16* dst = cluster.map_shared_rank(X, rk);
-      *reinterpret_cast<uint4*>(dst + off) = hi;
-      *reinterpret_cast<uint4*>(dst + W * LDH + off) = lo;
+  for (int row = warp; row < 8 * nr; row += kNW) {
+    const float2 x = *reinterpret_cast<const float2*>(F + row * LDF + 2 * lane);
+    float v[2] = {x.x, x.y};
+    norm_row<2>(v, sv + V_ENTLNG, sv + V_ENTLNB);
+    put2<NP>(sA, L::P128, row_bytes(128), row, 2 * lane, v[0], v[1]);
+  }
+  __syncthreads();
+  {
+    // fusion W_combine [e; t] + b + E_pos[rank]
+    float acc[NR][1][4];
+    gemm<128, 1, NR, NP>(sA, L::P128, wc, nr, acc);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (r >= nr) continue;
+      each(acc[r][0], r, warp, [&](int row, int c, float x, float y) {
+        const int k = 8 * (a.first + a.step * r) + (row & 7);
+        float2 pe = make_float2(0.f, 0.f);
+        if (k < a.gen_len)
+          pe = __ldg(reinterpret_cast<const float2*>(a.vec + V_POS + static_cast<size_t>(k) * 128 + c));
+        x += sv[V_COMBB + c] + pe.x;
+        y += sv[V_COMBB + c + 1] + pe.y;
+        *reinterpret_cast<float2*>(F + row * LDF + c) = make_float2(x, y);
+        put2<NP>(sY, L::P128, row_bytes(128), row, c, x, y);
+      });
     }
   }
 }
 
+// q, k and v of the CTA's rows in layer l: q (scaled) to planes in Q, k and v
+// to the scratch
+template <int NR, int NP>
+__device__ __noinline__ void lbs_qkv(const LbsArgs a, int l) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const float* const sv = reinterpret_cast<const float*>(smem + L::V);
+  uint8_t* const sY = smem + L::Y;
+  uint8_t* const sQ = smem + L::Q;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, nr = a.nr;
+  const size_t plane = static_cast<size_t>(a.cap_rows) * 128;  // elements of a K (V) plane
+  const uint4* const wl = a.mat + M_LAYER + l * ML_STRIDE;
+  const float* const vl = sv + V_LAYER + l * VL_STRIDE;
+  __nv_bfloat16* const Kp = a.template keys<NP>(l);
+  __nv_bfloat16* const Vp = a.template values<NP>(l);
+  // QKV: tiles warp + 8 i, i = 0 the queries, 1 the keys, 2 the values
+  constexpr int NQ = NR <= 2 ? 3 : 1;
+#pragma unroll
+  for (int i0 = 0; i0 < 3; i0 += NQ) {
+    uint4 w[NQ * 8];
+    load_w<128, NQ>(w, wl + ML_QKV, warp + 8 * i0);
+    if (i0 == 0) __syncthreads();
+    float acc[NR][NQ][4];
+    gemm<128, NQ, NR, NP>(sY, L::P128, w, nr, acc);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (r >= nr) continue;
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) {
+        const int kind = i0 + i, c = 16 * warp + 2 * g, k = 8 * (a.first + a.step * r) + 2 * t;
+        const float b0 = vl[VL_QKVB + 128 * kind + c], b1 = vl[VL_QKVB + 128 * kind + c + 1];
+        const float x0 = acc[r][i][0] + b0, x1 = acc[r][i][1] + b0;  // column c of rows 2 t, 2 t + 1
+        const float y0 = acc[r][i][2] + b1, y1 = acc[r][i][3] + b1;  // column c + 1
+        if (kind == 0) {
+          const float sc = 0.2550348616f;  // log2(e) / sqrt(32)
+          put2<NP>(sQ, L::P128, row_bytes(128), 8 * r + 2 * t, c, x0 * sc, y0 * sc);
+          put2<NP>(sQ, L::P128, row_bytes(128), 8 * r + 2 * t + 1, c, x1 * sc, y1 * sc);
+        } else {
+          uint32_t u[NP], v[NP];
+          if (kind == 1) {
+            split2<NP>(x0, y0, u);
+            split2<NP>(x1, y1, v);
+          } else {
+            split2<NP>(x0, x1, u);
+            split2<NP>(y0, y1, v);
+          }
+          __nv_bfloat16* const d0 = kind == 1 ? Kp + static_cast<size_t>(k) * 128 + c : Vp + static_cast<size_t>(c) * a.capk + k;
+          const size_t step = kind == 1 ? 128 : a.capk;
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            *reinterpret_cast<uint32_t*>(d0 + q * plane) = u[q];
+            *reinterpret_cast<uint32_t*>(d0 + q * plane + step) = v[q];
+          }
+        }
+      }
+    }
+  }
+}
+
+// the rest of layer l: attention, output projection, FFN; z of the next
+// layer in F and Y, or the LBS logits
+template <int NR, int NP>
+__device__ __forceinline__ void lbs_layer(const LbsArgs& a, int l) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  float* const F = reinterpret_cast<float*>(smem + L::F);
+  const float* const sv = reinterpret_cast<const float*>(smem + L::V);
+  uint8_t* const sA = smem + L::A;
+  uint8_t* const sY = smem + L::Y;
+  uint8_t* const sQ = smem + L::Q;
+  uint8_t* const sH = smem + L::H;
+  float* const part = reinterpret_cast<float*>(sH);
+  float* const ml = reinterpret_cast<float*>(smem + L::ML);
+  constexpr int LDF = L::kLdF;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nr = a.nr;
+  const size_t plane = static_cast<size_t>(a.cap_rows) * 128;
+  const uint4* const wl = a.mat + M_LAYER + l * ML_STRIDE;
+  const float* const vl = sv + V_LAYER + l * VL_STRIDE;
+  const __nv_bfloat16* const Kp = a.template keys<NP>(l);
+  const __nv_bfloat16* const Vp = a.template values<NP>(l);
+  attend<NR, NP>(sQ, Kp, Vp, plane, a.capk, a.nM, nr, part, ml);
+  uint4 wo[8];
+  load_w<128, 1>(wo, wl + ML_OUT, warp);
+  __syncthreads();
+  attend_merge<NR, NP>(part, ml, sA, nr);
+  __syncthreads();
+  {  // output projection + residual
+    float acc[NR][1][4];
+    gemm<128, 1, NR, NP>(sA, L::P128, wo, nr, acc);
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (r < nr) add_f(F, LDF, acc[r][0], r, warp, vl + VL_OUTB);
+  }
+  uint4 w1[16];
+  load_w<128, 2>(w1, wl + ML_FF1, warp);
+  __syncthreads();
+  auto norm = [&](const float* gm, const float* bt) {
+    for (int row = warp; row < 8 * nr; row += kNW) {
+      float4* z = reinterpret_cast<float4*>(F + row * LDF) + lane;
+      float v[4] = {z->x, z->y, z->z, z->w};
+      norm_row<4>(v, gm, bt);
+      *z = make_float4(v[0], v[1], v[2], v[3]);
+      put2<NP>(sY, L::P128, row_bytes(128), row, 4 * lane, v[0], v[1]);
+      put2<NP>(sY, L::P128, row_bytes(128), row, 4 * lane + 2, v[2], v[3]);
+    }
+  };
+  norm(vl + VL_LN1G, vl + VL_LN1B);
+  __syncthreads();
+  {  // h = GELU(W_1 z + b_1)
+    float acc[NR][2][4];
+    gemm<128, 2, NR, NP>(sY, L::P128, w1, nr, acc);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (r >= nr) continue;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        each(acc[r][i], r, warp + 8 * i, [&](int row, int c, float x, float y) {
+          put2<NP>(sH, L::P256, row_bytes(256), row, c, gelu(x + vl[VL_FF1B + c]), gelu(y + vl[VL_FF1B + c + 1]));
+        });
+    }
+  }
+  uint4 w2[16];
+  load_w<256, 1>(w2, wl + ML_FF2, warp);
+  __syncthreads();
+  {
+    float acc[NR][1][4];
+    gemm<256, 1, NR, NP>(sH, L::P256, w2, nr, acc);
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (r < nr) add_f(F, LDF, acc[r][0], r, warp, vl + VL_FF2B);
+  }
+  __syncthreads();
+  if (l == 0) {
+    norm(vl + VL_LN2G, vl + VL_LN2B);
+  } else {  // the last LayerNorm and the head O = w . z + b
+    for (int row = warp; row < 8 * nr; row += kNW) {
+      const float4 z = reinterpret_cast<const float4*>(F + row * LDF)[lane];
+      float v[4] = {z.x, z.y, z.z, z.w};
+      norm_row<4>(v, vl + VL_LN2G, vl + VL_LN2B);
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s = fmaf(v[i], sv[V_HEADW + 4 * lane + i], s);
+      s = warp_sum(s) + sv[V_HEADB];
+      const int k = 8 * (a.first + a.step * (row >> 3)) + (row & 7);
+      if (lane == 0 && k < a.nM) a.O[a.kbase + k] = s;
+    }
+  }
+}
+
+// ------------------------------------------------------------------ LPS
+// A warp's 8 rows: z[i], features 16 i + g (elements 0, 1: rows 2 t, 2 t + 1)
+// and 16 i + 8 + g (2, 3).
+
+// B fragments (rows as N) of T tiles of 16 features in NP planes
+template <int T, int NP>
+__device__ __forceinline__ void frags(const float (&v)[T][4], uint32_t (&f)[T][NP][2]) {
+#pragma unroll
+  for (int i = 0; i < T; ++i)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      uint32_t q[NP];
+      split2<NP>(v[i][2 * u], v[i][2 * u + 1], q);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) f[i][p][u] = trans8(q[p]);
+    }
+}
+
+// y = W x + b for MT tiles of outputs, KT tiles of inputs; w: A fragments in
+// shared memory
+template <int MT, int KT, int NP>
+__device__ __forceinline__ void lps_gemm(const uint4* w, const uint32_t (&f)[KT][NP][2], const float* b,
+                                         float (&y)[MT][4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2;
+  uint4 a[MT][KT];
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int k = 0; k < KT; ++k) a[i][k] = w[(i * KT + k) * 32 + lane];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < KT; ++k) {
+#pragma unroll
+      for (int p = NP - 1; p > 0; --p) mma4(lo, a[i][k], f[k][p][0], f[k][p][1]);
+      mma4(hi, a[i][k], f[k][0][0], f[k][0][1]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) y[i][e] = (hi[e] + lo[e]) + b[16 * i + g + 8 * (e >> 1)];
+  }
+}
+
+// LayerNorm over the 32 features of each row
+__device__ __forceinline__ void lps_norm(const float (&z)[2][4], const float* gm, const float* bt, float (&y)[2][4]) {
+  const int g = (threadIdx.x & 31) >> 2;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const float mean = gsum((z[0][c] + z[0][2 + c]) + (z[1][c] + z[1][2 + c])) * (1.0f / 32);
+    float q = 0.f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) q += (z[i][c] - mean) * (z[i][c] - mean) + (z[i][2 + c] - mean) * (z[i][2 + c] - mean);
+    const float inv = rsqrtf(gsum(q) * (1.0f / 32) + 1e-5f);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        y[i][2 * u + c] = (z[i][2 * u + c] - mean) * inv * gm[16 * i + 8 * u + g] + bt[16 * i + 8 * u + g];
+  }
+}
+
+// a lane's words of a key (or of a pair of keys' values): [head][plane]
+template <int NP, bool GLOBAL>
+__device__ __forceinline__ void ld_kv(const __nv_bfloat16* p, uint32_t (&w)[4 * NP]) {
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    const uint4* q = reinterpret_cast<const uint4*>(p) + i;
+    const uint4 v = GLOBAL ? __ldcg(q) : *q;
+    w[4 * i] = v.x;
+    w[4 * i + 1] = v.y;
+    w[4 * i + 2] = v.z;
+    w[4 * i + 3] = v.w;
+  }
+}
+
+// The router of one sequence's B n M (nb rows), 8 rows per warp: group
+// `grp` of 8 rows (idle if 8 * grp >= nb).  feat, prob: by rank in B n M.
+// wm: the weights in shared memory.  Keys and values of both blocks at kv +
+// block * kv_stride: K [key][dim pair][head][plane][2 dims] and, v_off
+// further, V [key pair][dim][head][plane][2 keys], so that a lane reads all
+// heads and planes of its key (pair) in NP 16-byte loads.  `meet` lets every
+// warp of the sequence see the others' keys and values.
+template <int NP, bool GLOBAL, class Feat, class Prob, class Meet>
+__device__ __forceinline__ void lps_router(const uint4* wm, const float* sv, int nb, int grp, int blocks,
+                                           __nv_bfloat16* kv, size_t kv_stride, size_t v_off, Feat feat,
+                                           Prob prob, Meet meet) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const bool on = 8 * grp < nb;
+  float z[2][4];
+  if (on) {  // Linear(5 -> 32), LayerNorm, GELU
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int row = 8 * grp + 2 * t + (e & 1), f = 16 * i + 8 * (e >> 1) + g;
+        float y = sv[V_INB + f];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) y = fmaf(row < nb ? feat(row, k) : 0.f, sv[V_INT + 32 * k + f], y);
+        z[i][e] = y;
+      }
+    lps_norm(z, sv + V_INLNG, sv + V_INLNB, z);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) z[i][e] = gelu(z[i][e]);
+  }
+#pragma unroll 1
+  for (int l = 0; l < blocks; ++l) {
+    const uint4* const wl = wm + l * MB_STRIDE;
+    const float* const vl = sv + V_BLOCK + l * VB_STRIDE;
+    __nv_bfloat16* const K = kv + l * kv_stride;
+    __nv_bfloat16* const V = K + v_off;
+    uint32_t qf[4][NP];  // queries of each head: dims 2 t, 2 t + 1 of row g
+    if (on) {
+      float y[2][4], q[6][4];
+      uint32_t f[2][NP][2];
+      lps_norm(z, vl + VB_LN1G, vl + VB_LN1B, y);
+      frags<2, NP>(y, f);
+      lps_gemm<6, 2, NP>(wl + MB_QKV, f, vl + VB_QKVB, q);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int i = h >> 1, u = 2 * (h & 1);
+        const float sc = 0.5100697233f;  // log2(e) / sqrt(8)
+        uint32_t a[NP], b[NP], c[NP];
+        split2<NP>(q[i][u] * sc, q[i][u + 1] * sc, a);
+        split2<NP>(q[2 + i][u], q[2 + i][u + 1], b);
+        split2<NP>(q[4 + i][u], q[4 + i][u + 1], c);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          qf[h][p] = trans8(a[p]);
+          *reinterpret_cast<uint32_t*>(K + (((8 * grp + g) * 4 + t) * (4 * NP) + h * NP + p) * 2) = trans8(b[p]);
+          *reinterpret_cast<uint32_t*>(V + (((4 * grp + t) * 8 + g) * (4 * NP) + h * NP + p) * 2) = c[p];
+        }
+      }
+    }
+    meet();
+    if (!on) continue;
+    // the four heads side by side: each block's chain of two products, a
+    // maximum, exponentials and transposes is latency
+    const int n8 = (nb + 7) & ~7;
+    float o[4][4], m[4][2], sum[4][2];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[h][e] = 0.f;
+      m[h][0] = m[h][1] = -INFINITY;
+      sum[h][0] = sum[h][1] = 0.f;
+    }
+#pragma unroll 1
+    for (int k0 = 0; k0 < nb; k0 += 32) {
+      float s[4][2][4], c[4][2], y[4][4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int key = k0 + 16 * j + g;
+        uint32_t k0w[4 * NP], k1w[4 * NP];  // keys key, key + 8: dims 2 t, 2 t + 1
+        ld_kv<NP, GLOBAL>(K + ((key < n8 ? key : 0) * 4 + t) * (8 * NP), k0w);
+        ld_kv<NP, GLOBAL>(K + ((key + 8 < n8 ? key + 8 : 0) * 4 + t) * (8 * NP), k1w);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          float(&x)[4] = s[h][j];
+          const uint32_t *u = k0w + h * NP, *v = k1w + h * NP;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[e] = 0.f;
+          // 8 dims fill half a k16 step: two products of planes per MMA
+          if (NP == 3) {
+            mma4(x, make_uint4(u[NP - 1], v[NP - 1], u[0], v[0]), qf[h][0], qf[h][NP - 1]);
+            mma4(x, make_uint4(u[1], v[1], u[1], v[1]), qf[h][0], qf[h][1]);
+          } else {
+            mma4(x, make_uint4(u[1], v[1], 0u, 0u), qf[h][0], 0u);
+          }
+          mma4(x, make_uint4(u[0], v[0], u[0], v[0]), qf[h][0], qf[h][1]);
+          if (key >= nb) x[0] = x[1] = -INFINITY;
+          if (key + 8 >= nb) x[2] = x[3] = -INFINITY;
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        softmax_block<2>(s[h], m[h], sum[h], c[h]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[h][e] = 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        uint32_t va[2][4 * NP];  // keys 16 j + 8 u + 2 t, + 1: dim g
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int key = k0 + 16 * j + 8 * u;
+          ld_kv<NP, GLOBAL>(V + (((key < n8 ? key : 0) / 2 + t) * 8 + g) * (8 * NP), va[u]);
+          if (key >= n8)
+#pragma unroll
+            for (int i = 0; i < 4 * NP; ++i) va[u][i] = 0u;
+        }
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          uint32_t pb[NP][2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            uint32_t q[NP];
+            split2<NP>(s[h][j][2 * u], s[h][j][2 * u + 1], q);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) pb[p][u] = trans8(q[p]);
+          }
+          const uint32_t *v0 = va[0] + h * NP, *v1 = va[1] + h * NP;
+          // 8 dims fill half of M: planes 0 and 1 of the values on top of each other
+          if (NP == 3) mma4(y[h], make_uint4(v0[NP - 1], 0u, v1[NP - 1], 0u), pb[0][0], pb[0][1]);
+#pragma unroll
+          for (int p = NP - 1; p >= 0; --p)
+            mma4(y[h], make_uint4(v0[0], v0[1], v1[0], v1[1]), pb[p][0], pb[p][1]);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[h][e] = fmaf(o[h][e], c[h][e & 1], y[h][e]);
+    }
+    float a[2][4];  // attention output, heads concatenated
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      a[h >> 1][2 * (h & 1)] = (o[h][0] + o[h][2]) * rcp(gsum(sum[h][0]));
+      a[h >> 1][2 * (h & 1) + 1] = (o[h][1] + o[h][3]) * rcp(gsum(sum[h][1]));
+    }
+    float y[2][4];
+    uint32_t f[2][NP][2];
+    frags<2, NP>(a, f);
+    lps_gemm<2, 2, NP>(wl + MB_OUT, f, vl + VB_OUTB, y);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) z[i][e] += y[i][e];
+    lps_norm(z, vl + VB_LN2G, vl + VB_LN2B, y);
+    frags<2, NP>(y, f);
+    float hd[4][4];
+    lps_gemm<4, 2, NP>(wl + MB_FF1, f, vl + VB_FF1B, hd);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) hd[i][e] = gelu(hd[i][e]);
+    uint32_t fh[4][NP][2];
+    frags<4, NP>(hd, fh);
+    lps_gemm<2, 4, NP>(wl + MB_FF2, fh, vl + VB_FF2B, y);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) z[i][e] += y[i][e];
+  }
+  if (on) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) s = fmaf(z[i][2 * u + c], sv[V_PHEADW + 16 * i + 8 * u + g], s);
+      s = gsum(s) + sv[V_PHEADB];
+      const int row = 8 * grp + 2 * t + c;
+      if (g == 0 && row < nb) prob(row, 1.0f / (1.0f + expf(-s)));
+    }
+  }
+}
+
+// The router of up to 64 rows by one CTA, in shared memory.  Not inlined, for
+// the same reason as lbs_input: a run on stand-in rows comes first.
+template <int CAP, int NR, int NP>
+__device__ __noinline__ void lps_local(int nb, int blocks) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
+  lps_router<NP, false>(reinterpret_cast<const uint4*>(smem + L::W), reinterpret_cast<const float*>(smem + L::V), nb,
+                        threadIdx.x >> 5, blocks, reinterpret_cast<__nv_bfloat16*>(smem + L::KV), L::kKvBlock,
+                        64 * 32 * NP, [&](int row, int k) { return rs.feat[row][k]; },
+                        [&](int row, float v) { rs.prob[row] = v; }, [] { __syncthreads(); });
+}
 
 }  // namespace
 
-__global__ void __cluster_dims__(kDecideCluster, 1, 1) __launch_bounds__(kDecideThreads, 1)
-    decide_kernel(const DecideParams p) {
-  extern __shared__ uint8_t smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 15) & ~static_cast<uintptr_t>(15));
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = static_cast<int>(cluster.block_rank());
-  const int seq = blockIdx.x / kDecideCluster;
+template <int C, int NR, int NP>
+__global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) {
+  using L = Lay<NR, NP>;
+  constexpr int CAP = 8 * NR * C;
+  constexpr int NC = CAP / 32, RPT = (NC + kNW - 1) / kNW;
+  extern __shared__ __align__(16) uint8_t smem[];
+  float* const sv = reinterpret_cast<float*>(smem + L::V);
+  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
+  Slots& sl = *reinterpret_cast<Slots*>(smem + L::SLOT);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  float* const P = sm.pool;
-  // a kernel launched after this one as a programmatic dependent (the window
-  // attention, which shares no data with the decision) may start on the SMs
-  // this grid leaves free once every CTA of it is resident
+  const int rank = static_cast<int>(cluster_ctarank());
+  const int b = blockIdx.x / C;
+  // the window attention, which shares no data with the decision, may start
+  // on the SMs this grid leaves free once every CTA of it is resident
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
+  for (int i = tid; i < kVecs / 4; i += kT)
+    reinterpret_cast<float4*>(sv)[i] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
+
+  // ------------------------------------------------------------ decode state
+  const int r0 = p.cu_rows[b];
+  int n = p.cu_rows[b + 1] - r0;
+  const bool bad_seq = n < 0 || n > CAP || r0 < 0 || r0 + n > p.R ||
+                       (p.strict ? p.cu_rows[p.B] != p.R : n > p.gen_len);
+  if (bad_seq) {
+    if (rank == 0 && tid == 0) atomicCAS(p.status, 0, EBD_ERR_INVALID_ARG);
+    n = 0;
+  }
+  const int kbase = ((r0 + 31) & ~31) + 32 * b;  // this sequence's rows of the scratch
+  const int capk = (n + 31) & ~31;
+  int meta_b = p.blk_meta[2 * b], meta_s = p.blk_meta[2 * b + 1];
+  bool m[RPT], inb[RPT], f[RPT];
+  int pos[RPT], mrank[RPT], urank[RPT];
+  if (tid < 32) {
+    sl.mrow[tid] = -1;
+    sl.ent[tid] = 0.f;
+    sl.arg[tid] = -1;
+  }
   if (tid == 0) {
-    // weights and vectors of this rank: bulk copies issued first, so they
-    // land while the statistics are merged.  With no active block the LBS
-    // weights are needed (every rank); otherwise only rank 0 needs the LPS
-    // weights, which then go straight into the weight region.
-    mbar_init(&sm.bar, 1);
-    mbar_init(&sm.bar2, 1);
-    fence_mbar_init();
-    sm.meta_b = p.blk_meta[2 * seq];
-    sm.meta_s = p.blk_meta[2 * seq + 1];
-    const bool lbs_possible = p.mode == EBD_DECODE_EB && sm.meta_s == 0;
-    const uint32_t wb = LBS_W_ELEMS * 2u, vb = V_ELEMS * 4u;
-    mbar_arrive_expect_tx(&sm.bar, vb + (lbs_possible ? wb : 0u));
-    bulk_copy(sm.v, p.w.vec + static_cast<size_t>(rank) * V_ELEMS, vb, &sm.bar);
-    if (lbs_possible)
-      bulk_copy(sm.w, p.w.lbs_w + static_cast<size_t>(rank) * LBS_W_ELEMS, wb, &sm.bar);
-    sm.lps_loaded = 0;
-    if (!lbs_possible && rank == 0 && p.lps_enabled) {
-      mbar_arrive_expect_tx(&sm.bar2, LPS_W_ELEMS * 2u);
-      bulk_copy(sm.w, p.w.lps_w, LPS_W_ELEMS * 2u, &sm.bar2);
-      sm.lps_loaded = 1;
+    rs.cut = INT_MAX;
+    rs.first = INT_MAX;
+    rs.any = 0;
+    rs.best = -1;
+    rs.open = 0;
+  }
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {
+    const int j = 32 * (warp + kNW * i) + lane;
+    const bool row = j < n;
+    m[i] = row && p.mask[r0 + j] != 0;
+    inb[i] = row && p.in_block[r0 + j] != 0;
+    pos[i] = row ? p.row_pos[r0 + j] : 0;
+    if (row) rs.pos[j] = pos[i];
+    f[i] = row && !m[i];
+  }
+  const int nM = rank_rows<CAP>(rs, m, mrank);
+  const int nU = rank_rows<CAP>(rs, f, urank);
+  // Windows of up to 64 rows: CTA 0 makes the decision.  Eight CTAs with a
+  // group to spare leave all rows to the other seven, so that CTA 0 can bring
+  // in the LPS and its weights meanwhile.
+  constexpr bool kWide = CAP > 64;
+  const int groups = (nM + 7) >> 3;
+  const bool apart = C == 8 && !kWide && groups < C;
+  const int nw = apart ? C - 1 : C, wk = apart ? rank - 1 : rank;
+  // group k of 8 rows of M belongs to worker k % nw, its slot k / nw; the
+  // statistics of the other rows are merged by the workers without a group
+  const int u0 = groups < nw ? groups : 0, nuw = nw - u0;
+  if (wk >= 0) {
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const int j = 32 * (warp + kNW * i) + lane, grp = mrank[i] >> 3;
+      if (m[i] && grp % nw == wk) sl.mrow[8 * (grp / nw) + (mrank[i] & 7)] = j;
+      if (f[i] && u0 + urank[i] % nuw == wk) rs.urow[urank[i] / nuw] = j;
     }
-    const int r0 = p.cu_rows[seq], r1 = p.cu_rows[seq + 1];
-    const int n = r1 - r0;
-    sm.bad_seq = 0;
-    if (p.cu_rows[p.B] != p.rows_expected || n < 0 || n > W || r0 < 0) {
-      sm.bad_seq = 1;
-      if (rank == 0) atomicCAS(p.status, 0, EBD_ERR_INVALID_ARG);
-    }
-    sm.r0 = r0;
-    sm.n_rows = sm.bad_seq ? 0 : n;
   }
-  // every CTA of the cluster must be running before any distributed
-  // shared-memory access; this also orders the block-level setup above
-  cluster.sync();
-  const int r0 = sm.r0, nr = sm.n_rows;
+  const bool run_lbs = p.mode == EBD_DECODE_EB && meta_s == 0 && nM > p.l_min;
+  const int nr = wk >= 0 && groups > wk ? (groups - wk + nw - 1) / nw : 0;  // groups of this CTA
+  const int nu = wk >= u0 && nU > wk - u0 ? (nU - (wk - u0) + nuw - 1) / nuw : 0;
+  const LbsArgs la{p.mat, p.vec, p.tok_table, p.kv, p.O, p.V, p.gen_len, p.cap_rows, kbase, capk, nM, nr, wk, nw};
+  __syncthreads();
 
-#pragma unroll 1
-  for (int j = tid; j < nr; j += blockDim.x) {
-    sm.f_mask[j] = p.mask[r0 + j];
-    sm.f_ib[j] = p.in_block[r0 + j];
-    sm.f_tok[j] = p.tokens[r0 + j];
-    sm.f_pos[j] = p.row_pos[r0 + j];
-    sm.f_acc[j] = 0;
-    sm.f_O[j] = __int_as_float(0x7fc00000);
-    sm.f_p[j] = __int_as_float(0x7fc00000);
+  // The LM head has streamed its weight through L2: bring the router's back
+  // while its last CTAs run.
+  if (b == 0) {
+    const char* w = reinterpret_cast<const char*>(p.mat);
+    for (int i = (run_lbs ? 0 : M_BLOCK / 8) + rank * kT + tid; i < M_TOTAL / 8; i += C * kT)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 128 * static_cast<size_t>(i)));
   }
-
-  // Every step starts with this kernel's code out of every cache.  While the
-  // LM head finishes, ranks 1..5 each run one stretch of the LPS router on a
-  // stand-in block in their own shared memory (the pool, unused until the
-  // statistics are merged; the results are discarded), so that the
-  // instructions rank 0 runs there after the LBS come from L2.
-  if (rank >= 1 && rank <= 5 && p.lps_enabled && p.mode == EBD_DECODE_EB) {
-    const int from = rank == 1 ? 0 : rank == 2 ? 1 : rank == 3 ? 3 : rank == 4 ? 4 : 6;
-    const int to = rank == 1 ? 0 : rank == 2 ? 2 : rank == 3 ? 3 : rank == 4 ? 5 : 7;
-    lps_forward(P, 32, sm.w, sm.v + V_LPS, from, to);
+  auto copy_lps = [&]() {
+    for (int i = tid; i < L::kLpsMat; i += kT)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem + L::W + 16 * i)), "l"(p.mat + M_BLOCK + i)
+                   : "memory");
+  };
+  // Launched behind the LM head, this grid waits some microseconds for its
+  // last CTAs, with code that no SM has cached (a first pass through it costs
+  // about as much again as the work itself): meanwhile CTA 0 runs the LPS
+  // router, the others the LBS input layers and the first QKV product, on
+  // stand-in rows.
+  const bool warm = p.warm != 0 && C == 8 && !kWide && p.mode == EBD_DECODE_EB;
+  if (!kWide && apart && rank == 0 && p.lps_enabled) {
+    copy_lps();
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (warm) lps_local<CAP, NR, NP>(32, 1);
+  } else if (warm && run_lbs && nr > 0) {
+    lbs_input<NR, NP>(la);
+    lbs_qkv<NR, NP>(la, 0);
   }
 
-  // ---------------------------------------------------------------- 1. statistics
-  // Launched as a programmatic dependent of the LM head, the kernel may start
-  // while the LM head's last CTAs run: everything above (weights in flight,
-  // decode state loaded) overlaps them; the partial states are read only
-  // after the LM head's grid has completed and its writes are visible.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // ------------------------------------------------------------ statistics
+  // everything above overlaps the LM head's last CTAs; the partial states
+  // are read only after its grid completed.  A masked row is merged by the
+  // CTA that holds it in the LBS, the others are spread over the cluster.
   if (p.features_in) {
-#pragma unroll 1
-    for (int j = tid; j < nr; j += blockDim.x) {
-      const float c = p.conf[r0 + j], e = p.ent_norm[r0 + j], g = p.gap[r0 + j];
-      const int a = p.argmax[r0 + j];
-      sm.f_conf[j] = c;
-      sm.f_ent[j] = e;
-      sm.f_gap[j] = g;
-      sm.f_arg[j] = a;
-      sm.f_bad[j] = !(isfinite(c) && isfinite(e) && isfinite(g)) || a < 0 || a >= p.V;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tid < 8 * NR && sl.mrow[tid] >= 0) {
+      sl.ent[tid] = p.s_ent[r0 + sl.mrow[tid]];
+      sl.arg[tid] = p.s_arg[r0 + sl.mrow[tid]];
     }
   } else {
-    // row j is merged by warp (j / 8) of rank (j % 8) and broadcast
-#pragma unroll 1
-    for (int j = warp * kDecideCluster + rank; j < nr; j += kDecideCluster * (blockDim.x >> 5)) {
+    bool waited = false;
+    // the first pass, it < 0, merges no states into a row of its own
+    for (int it = warm && nr + nu > 0 ? warp - kNW : warp; it < 8 * nr + nu; it += kNW) {
+      const bool real = it >= 0;
+      if (real && !waited) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+      }
+      const int j = !real ? 0 : it < 8 * nr ? sl.mrow[it] : rs.urow[it - 8 * nr];
+      if (j < 0 || (real && !in_bounds(r0 + j, p.R, p.status))) continue;
       const size_t base = static_cast<size_t>(r0 + j) * p.grid_lm;
-      float m = -INFINITY, s = 0.f, t = 0.f, l2 = -INFINITY;
-      int idx = INT_MAX;
-      float4 fv[8];
-      int iv[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {  // independent loads first (partials per lane <= 8)
-        const int g = lane + 32 * c;
-        fv[c] = g < p.grid_lm ? p.part_f[base + g] : make_float4(-INFINITY, 0.f, 0.f, -INFINITY);
-        iv[c] = g < p.grid_lm ? p.part_i[base + g] : INT_MAX;
-      }
-#pragma unroll
-      for (int c = 0; c < 8; ++c)
-        merge_state(m, s, t, l2, idx, fv[c].x, fv[c].y, fv[c].z, fv[c].w, iv[c]);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float bm = __shfl_xor_sync(0xffffffffu, m, off);
-        const float bs = __shfl_xor_sync(0xffffffffu, s, off);
-        const float bt = __shfl_xor_sync(0xffffffffu, t, off);
-        const float bl = __shfl_xor_sync(0xffffffffu, l2, off);
-        const int bi = __shfl_xor_sync(0xffffffffu, idx, off);
-        merge_state(m, s, t, l2, idx, bm, bs, bt, bl, bi);
-      }
-      const float conf = 1.0f / s;
-      const float ent = logf(s) - t / s;
-      const float entn = ent * p.inv_log_v;
-      const float gap = (1.0f - expf(l2 - m)) / s;
-      const bool bad = !(isfinite(m) && isfinite(s) && isfinite(t) && s >= 1.0f) || idx < 0 ||
-                       idx >= p.V;
-      if (lane == 0 && in_bounds(r0 + j, p.rows_expected, p.status)) {
-        const int r = r0 + j;
-        if (p.conf) p.conf[r] = conf;
-        if (p.entropy) p.entropy[r] = ent;
-        if (p.ent_norm) p.ent_norm[r] = entn;
-        if (p.gap) p.gap[r] = gap;
-        if (p.argmax) p.argmax[r] = bad ? -1 : idx;
-        if (bad) atomicCAS(p.status, 0, EBD_ERR_NONFINITE);
-      }
-      if (lane < kDecideCluster) {
-        Smem* dst = cluster.map_shared_rank(&sm, lane);
-        dst->f_conf[j] = conf;
-        dst->f_ent[j] = entn;
-        dst->f_gap[j] = gap;
-        dst->f_arg[j] = bad ? -1 : idx;
-        dst->f_bad[j] = bad ? 1 : 0;
+      const RowStats st = merge_row(p.part_f + base, p.part_i + base, real ? p.grid_lm : 0);
+      if (lane == 0) {
+        const int r = r0 + j, sr = real ? r : p.spare_row;
+        const float conf = 1.0f / st.s, ent = logf(st.s) - st.t * conf, entn = ent * p.inv_log_v;
+        const float gap = (1.0f - expf(st.l2 - st.m)) * conf;
+        const bool bad = !(isfinite(st.m) && isfinite(st.s) && isfinite(st.t) && st.s >= 1.0f) || st.idx < 0 ||
+                         st.idx >= p.V;
+        const int arg = bad ? -1 : st.idx;
+        p.s_conf[sr] = conf;
+        p.s_ent[sr] = entn;
+        p.s_gap[sr] = gap;
+        p.s_arg[sr] = arg;
+        if (real) {
+          if (p.conf) p.conf[r] = conf;
+          if (p.entropy) p.entropy[r] = ent;
+          if (p.ent_norm) p.ent_norm[r] = entn;
+          if (p.gap) p.gap[r] = gap;
+          if (p.argmax) p.argmax[r] = arg;
+          if (bad) atomicCAS(p.status, 0, EBD_ERR_NONFINITE);
+          if (it < 8 * nr) {
+            sl.ent[it] = entn;
+            sl.arg[it] = arg;
+          }
+        }
       }
     }
-  }
-  // the weight copy must have landed before any use (and before exit)
-  if (!mbar_wait(&sm.bar, 0, 1000ull * 1000 * 1000, nullptr) && tid == 0)
-    atomicCAS(p.status, 0, EBD_ERR_TIMEOUT);
-  cluster.sync();
-
-  // ---------------------------------------------------------------- 2. masked set
-  if (warp == 0) {
-    int base = 0;
-#pragma unroll 1
-    for (int j0 = 0; j0 < nr; j0 += 32) {
-      const int j = j0 + lane;
-      const bool m = j < nr && sm.f_mask[j];
-      const uint32_t bal = __ballot_sync(0xffffffffu, m);
-      if (m) sm.Mrows[base + __popc(bal & ((1u << lane) - 1u))] = j;
-      base += __popc(bal);
-    }
-    if (lane == 0) {
-      sm.nM = base;
-      sm.run_lbs = (p.mode == EBD_DECODE_EB && sm.meta_s == 0 && base > p.l_min) ? 1 : 0;
-    }
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
   }
   __syncthreads();
-  const int nM = sm.nM;
 
-  // ---------------------------------------------------------------- 3. LBS router
-  if (sm.run_lbs) {
-    const int n = nM;
-    float* Z = P + P_Z;
-    const HL Zh = hl_at(P + P_ZH, LDH);
-    const HL Xh = hl_at(P + P_XH, LDH);
-    float* Xin = P + P_XH;  // fp32 FFN partial inbox [8][64][16] (aliases Xh)
-    const HL Fh = hl_at(P + P_KV, 72);  // F_ent hidden (hi/lo)
-    const HL Hh = hl_at(P + P_KV, 40);  // FFN hidden slice (hi/lo)
-    float* KV = P + P_KV;
-    float* Q = P + P_Q;
-    const float* Vv = sm.v;
-    // 3a. entropy branch F_ent and token branch, every rank for all rows.
-    // The token branch's gathers from the folded table are issued first and
-    // stored only after the entropy branch, which hides their latency.
-    static_assert(kDecideThreads * 8 >= W * 32, "token-branch items per thread");
-    float2 tv[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int it = tid + k * kDecideThreads;
-      tv[k] = make_float2(0.f, 0.f);
-      if (it < n * 32) {
-        const int tok = sm.f_arg[sm.Mrows[it >> 5]];
-        if (tok >= 0 && tok < p.V)
-          tv[k] = __ldg(reinterpret_cast<const float2*>(p.w.tok_table + static_cast<size_t>(tok) * 64 +
-                                                       2 * (it & 31)));
-      }
-    }
-#pragma unroll 1
-    for (int it = tid; it < n * 32; it += blockDim.x) {
-      const int j = it >> 5, o = 2 * (it & 31);
-      const float h = sm.f_ent[sm.Mrows[j]];
-      hl_store2(Fh, j, o, gelu(fmaf(Vv[V_ENT1W + o], h, Vv[V_ENT1B + o])),
-                gelu(fmaf(Vv[V_ENT1W + o + 1], h, Vv[V_ENT1B + o + 1])));
-    }
-    __syncthreads();
-    // the ent2 output goes to the z hi/lo region: z itself receives the
-    // other ranks' fusion outputs as soon as they get there
-    float* E2 = P + P_ZH;
-    gemm_hl<true>(Fh, n, 64, sm.w + W_ENT2, 64, 64, [&](int j, int o, float a, float b) {
-      *reinterpret_cast<float2*>(E2 + j * LDZ + o) = make_float2(a + Vv[V_ENT2B + o], b + Vv[V_ENT2B + o + 1]);
-    });
-    __syncthreads();
-    ln_rows<64, false>(E2, LDZ, nullptr, 0, Xh, n, Vv + V_ENTLNG, Vv + V_ENTLNB);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {  // the token branch into columns 64..127
-      const int it = tid + k * kDecideThreads;
-      if (it < n * 32) {
-        const int o = 2 * (it & 31);
-        hl_store2(Xh, it >> 5, 64 + o, tv[k].x + Vv[V_TOKB + o], tv[k].y + Vv[V_TOKB + o + 1]);
-      }
-    }
-    __syncthreads();
-    // 3b. fusion W_combine [e; t] + E_pos[rank of the row]: this CTA's 16 outputs
-    {
-      const int o0 = kCombSlice * rank;
-      gemm_hl<true>(Xh, n, 128, sm.w + W_COMB, kCombSlice, kCombSlice, [&](int j, int o, float a, float b) {
-        const float2 pe = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(sm.w + W_POS + j * kCombSlice + o));
-        const float2 val = make_float2(a + Vv[V_COMBB + o] + pe.x, b + Vv[V_COMBB + o + 1] + pe.y);
-#pragma unroll 1
-        for (int r = 0; r < kDecideCluster; ++r)
-          *reinterpret_cast<float2*>(cluster.map_shared_rank(Z, r) + j * LDZ + o0 + o) = val;
-      });
-    }
-    cluster.sync();
-    // z as the first QKV input (hi/lo), every rank for all rows
-#pragma unroll 1
-    for (int it = tid; it < n * 64; it += blockDim.x) {
-      const int j = it >> 6, o = 2 * (it & 63);
-      hl_store2(Zh, j, o, Z[j * LDZ + o], Z[j * LDZ + o + 1]);
-    }
-    __syncthreads();
-    // 3c. two post-norm encoder layers
-    const int hd = rank >> 1, half = rank & 1;
-    const int nh = (n + 1) >> 1;
-    const int qa = half == 0 ? 0 : nh, qb = half == 0 ? nh : n;
+  // ------------------------------------------------------------ LBS
+  if (run_lbs) {
+    if (nr > 0) lbs_input<NR, NP>(la);
 #pragma unroll 1
     for (int l = 0; l < 2; ++l) {
-      const __nv_bfloat16* Wl = sm.w + W_LAYER0 + l * W_LAYER_STRIDE;
-      const float* Vl = Vv + V_LAYER0 + l * V_LAYER_STRIDE;
-      // QKV: this CTA's 48 features for every row, scattered to the CTAs
-      // that attend with them (head h lives in ranks 2h and 2h+1)
-      gemm_hl<true>(Zh, n, 128, Wl + WL_QKV, kQkvSlice, kQkvSlice, [&](int j, int o, float a, float b) {
-        const int f = kQkvSlice * rank + o;  // even; f and f+1 share part and head
-        const int part = f >> 7, h = (f >> 5) & 3, dd = f & 31;
-        const float2 val = make_float2(a + Vl[VL_QKVB + o], b + Vl[VL_QKVB + o + 1]);
-        if (part == 0) {
-          const int dst = 2 * h + (j >= nh ? 1 : 0);
-          const int jj = j >= nh ? j - nh : j;
-          *reinterpret_cast<float2*>(cluster.map_shared_rank(Q, dst) + jj * LDQ + dd) = val;
-        } else {
-          const int col = (part == 1 ? 0 : 32) + dd;
-          *reinterpret_cast<float2*>(cluster.map_shared_rank(KV, 2 * h) + j * LDKV + col) = val;
-          *reinterpret_cast<float2*>(cluster.map_shared_rank(KV, 2 * h + 1) + j * LDKV + col) = val;
-        }
-      });
-      cluster.sync();
-      lbs_attention(cluster, P, qb - qa, n, qa, hd);
-      cluster.sync();
-      {  // output projection + residual, 16 outputs, written in place into z
-        const int o0 = kOutSlice * rank;
-        gemm_hl<true>(Xh, n, 128, Wl + WL_OUT, kOutSlice, kOutSlice, [&](int j, int o, float a, float b) {
-          const float2 zz = *reinterpret_cast<const float2*>(Z + j * LDZ + o0 + o);
-          const float2 val = make_float2(zz.x + (a + Vl[VL_OUTB + o]), zz.y + (b + Vl[VL_OUTB + o + 1]));
-#pragma unroll 1
-          for (int r = 0; r < kDecideCluster; ++r)
-            *reinterpret_cast<float2*>(cluster.map_shared_rank(Z, r) + j * LDZ + o0 + o) = val;
-        });
-      }
-      cluster.sync();
-      ln_rows<128, true>(Z, LDZ, Z, LDZ, Zh, n, Vl + VL_LN1G, Vl + VL_LN1B);
-      __syncthreads();
-      // FFN: hidden units [32r, 32r+32) locally, then the partial second
-      // linear of those units sent to the owners of each 16-output slice
-      gemm_hl<true>(Zh, n, 128, Wl + WL_FF1, kFf1Slice, kFf1Slice, [&](int j, int o, float a, float b) {
-        hl_store2(Hh, j, o, gelu(a + Vl[VL_FF1B + o]), gelu(b + Vl[VL_FF1B + o + 1]));
-      });
-      __syncthreads();
-      gemm_hl<true>(Hh, n, kFf1Slice, Wl + WL_FF2, 128, 128, [&](int j, int o, float a, float b) {
-        *reinterpret_cast<float2*>(cluster.map_shared_rank(Xin, o >> 4) + (rank * W + j) * 16 + (o & 15)) =
-            make_float2(a, b);
-      });
-      cluster.sync();
-      {  // owner: sum the 8 partials + bias + residual, broadcast its slice
-        const int o0 = kOutSlice * rank;
-#pragma unroll 1
-        for (int it = tid; it < n * 8; it += blockDim.x) {
-          const int j = it >> 3, oo = 2 * (it & 7);
-          float2 a = *reinterpret_cast<const float2*>(Z + j * LDZ + o0 + oo);
-          a.x += Vl[VL_FF2B + oo];
-          a.y += Vl[VL_FF2B + oo + 1];
-#pragma unroll
-          for (int src = 0; src < kDecideCluster; ++src) {
-            const float2 q = *reinterpret_cast<const float2*>(Xin + (src * W + j) * 16 + oo);
-            a.x += q.x;
-            a.y += q.y;
-          }
-#pragma unroll 1
-          for (int rr = 0; rr < kDecideCluster; ++rr)
-            *reinterpret_cast<float2*>(cluster.map_shared_rank(Z, rr) + j * LDZ + o0 + oo) = a;
-        }
-      }
-      cluster.sync();
-      ln_rows<128, true>(Z, LDZ, Z, LDZ, Zh, n, Vl + VL_LN2G, Vl + VL_LN2B);
-      __syncthreads();
-      if (l == 0 && rank == 0 && tid == 0 && p.lps_enabled) {
-        // the first layer's weights (and everything before them) are dead:
-        // fetch the LPS weights into that region behind the second layer
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive_expect_tx(&sm.bar2, LPS_W_ELEMS * 2u);
-        bulk_copy(sm.w, p.w.lps_w, LPS_W_ELEMS * 2u, &sm.bar2);
-        sm.lps_loaded = 1;
-      }
+      if (nr > 0) lbs_qkv<NR, NP>(la, l);
+      cluster_barrier();  // every row's keys and values (l = 0: and statistics) are visible
+      if (nr > 0) lbs_layer<NR, NP>(la, l);
     }
-    // 3d. head Linear(128 -> 1), needed by rank 0
-    if (rank == 0) {
-#pragma unroll 1
-      for (int j = warp; j < n; j += (blockDim.x >> 5)) {
-        float a = 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) a += Z[j * LDZ + lane + 32 * c] * Vv[V_HEADW + lane + 32 * c];
-        a = warp_sum(a) + Vv[V_HEADB];
-        if (lane == 0) sm.f_O[sm.Mrows[j]] = a;
-      }
-    }
-    __syncthreads();
   }
-  // No distributed shared-memory access after this point.  Rank 0 makes the
-  // decision.  Ranks 1..7 make none: each runs a part of the LPS router, or
-  // the accept step, on a stand-in block of its own shared memory, skipping
-  // the block selection and writing nothing to global memory.  Every step
-  // starts with this kernel's code out of every cache; ahead of rank 0 and in
-  // parallel, those runs bring the code rank 0 is about to execute into L2.
-  const bool shadow = rank != 0;
+  cluster_barrier();  // every row's statistics and LBS logit are visible
 
-  // ---------------------------------------------------------------- 4. block selection
-  if (tid == 0 && !sm.lps_loaded && p.lps_enabled) {
-    // no LBS ran: the weight region is free now
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive_expect_tx(&sm.bar2, LPS_W_ELEMS * 2u);
-    bulk_copy(sm.w, p.w.lps_w, LPS_W_ELEMS * 2u, &sm.bar2);
-    sm.lps_loaded = 1;
+  if (!kWide && rank != 0) return;
+  if (!apart && p.lps_enabled) copy_lps();  // behind the selection, over the dead LBS activations
+
+  // ------------------------------------------------------------ block selection
+  // (Readings R8, R9)
+  float conf[RPT], ent[RPT], gap[RPT], lbs[RPT];
+  int arg[RPT], brank[RPT];
+  bool bad[RPT], sel[RPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {
+    const int j = 32 * (warp + kNW * i) + lane, r = r0 + j;
+    conf[i] = ent[i] = gap[i] = 0.f;
+    arg[i] = -1;
+    bad[i] = false;
+    lbs[i] = __int_as_float(0x7fc00000);
+    if (j < n) {
+      conf[i] = __ldcg(p.s_conf + r);
+      ent[i] = __ldcg(p.s_ent + r);
+      gap[i] = __ldcg(p.s_gap + r);
+      arg[i] = __ldcg(p.s_arg + r);
+      bad[i] = !(isfinite(conf[i]) && isfinite(ent[i]) && isfinite(gap[i])) || arg[i] < 0 || arg[i] >= p.V;
+      if (run_lbs && m[i]) lbs[i] = __ldcg(p.O + kbase + mrank[i]);
+    }
   }
-  if (warp == 0) {
-    if (shadow) {
-      // stand-in block: the first min(32, |M|) masked rows
-      const int nB = nM < 32 ? nM : 32;
-      for (int j = lane; j < nr; j += 32) sm.f_ib[j] = 0;
-      __syncwarp();
-      for (int k = lane; k < nB; k += 32) sm.f_ib[sm.Mrows[k]] = 1;
-      if (lane == 0 && nB > 0) {
-        sm.meta_b = sm.f_pos[sm.Mrows[0]];
-        sm.meta_s = nB;
+  if (p.mode != EBD_DECODE_EB) {
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) sel[i] = 32 * (warp + kNW * i) + lane < n;  // the window is the block
+  } else if (meta_s != 0) {
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) sel[i] = inb[i];
+  } else {
+    int nB = nM;
+    if (nM <= p.l_min) {
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) sel[i] = m[i];
+    } else {
+      bool cand[RPT];
+      int cr[RPT];
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) cand[i] = m[i] && lbs[i] > 0.f && arg[i] != p.eos_id && !bad[i];
+      const int nC = rank_rows<CAP>(rs, cand, cr);
+#pragma unroll
+      for (int i = 0; i < RPT; ++i)
+        if (cand[i]) rs.bpos[cr[i]] = pos[i];
+      __syncthreads();
+      // MaxGapFilter: cut at the first candidate farther than g_max from its predecessor
+#pragma unroll
+      for (int i = 0; i < RPT; ++i)
+        if (cand[i] && cr[i] >= 1 && pos[i] - rs.bpos[cr[i] - 1] > p.g_max) atomicMin(&rs.cut, cr[i]);
+      __syncthreads();
+      nB = min(rs.cut, nC);
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) sel[i] = cand[i] && cr[i] < nB;
+      if (nB < p.l_min) {  // min-tokens fallback: the first min(L_B, |M|) masked rows
+        nB = nM < p.l_b ? nM : p.l_b;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) sel[i] = m[i] && mrank[i] < nB;
       }
-      __syncwarp();
-    } else if (p.mode != EBD_DECODE_EB) {
-      // baselines: the window is the active fixed block; no block state
-    } else if (sm.meta_s == 0) {
-      for (int j = lane; j < nr; j += 32) sm.f_ib[j] = 0;
-      __syncwarp();
-      int nB = 0;
-      if (nM <= p.l_min) {
-        for (int k = lane; k < nM; k += 32) sm.Brows[k] = sm.Mrows[k];
-        nB = nM;
-      } else {
-        // candidates (router O > 0, not EOS) compacted in ascending position
-        int nC = 0;
-        for (int k0 = 0; k0 < nM; k0 += 32) {
-          const int k = k0 + lane;
-          int j = -1;
-          bool c = false;
-          if (k < nM) {
-            j = sm.Mrows[k];
-            c = sm.f_O[j] > 0.f && sm.f_arg[j] != p.eos_id && !sm.f_bad[j];
-          }
-          const uint32_t bal = __ballot_sync(0xffffffffu, c);
-          if (c) sm.Brows[nC + __popc(bal & ((1u << lane) - 1u))] = j;
-          nC += __popc(bal);
-        }
-        __syncwarp();
-        // MaxGapFilter: cut at the first candidate farther than g_max from its predecessor
-        int cut = nC;
-        for (int c0 = 1; c0 < nC; c0 += 32) {
-          const int c = c0 + lane;
-          const bool gap = c < nC && sm.f_pos[sm.Brows[c]] - sm.f_pos[sm.Brows[c - 1]] > p.g_max;
-          const uint32_t bal = __ballot_sync(0xffffffffu, gap);
-          if (bal) {
-            cut = c0 + __ffs(bal) - 1;
-            break;
-          }
-        }
-        nB = cut;
-        if (nB < p.l_min) {  // min-tokens fallback: first min(L_B, |M|) masked rows
-          nB = nM < p.l_b ? nM : p.l_b;
-          __syncwarp();
-          for (int k = lane; k < nB; k += 32) sm.Brows[k] = sm.Mrows[k];
-        }
-      }
-      __syncwarp();
-      for (int k = lane; k < nB; k += 32) sm.f_ib[sm.Brows[k]] = 1;
-      if (lane == 0 && nB > 0) {
-        sm.meta_b = sm.f_pos[sm.Brows[0]];
-        sm.meta_s = nB;
-      }
-      __syncwarp();
     }
-    int base = 0;
-    for (int j0 = 0; j0 < nr; j0 += 32) {
-      const int j = j0 + lane;
-      const bool inb = p.mode != EBD_DECODE_EB || sm.f_ib[j];
-      const bool m = j < nr && inb && sm.f_mask[j] && !sm.f_bad[j];
-      const uint32_t bal = __ballot_sync(0xffffffffu, m);
-      if (m) sm.BMrows[base + __popc(bal & ((1u << lane) - 1u))] = j;
-      base += __popc(bal);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+      if (sel[i]) atomicMin(&rs.first, 32 * (warp + kNW * i) + lane);
+    __syncthreads();
+    if (nB > 0) {
+      meta_b = rs.pos[rs.first];
+      meta_s = nB;
     }
-    if (lane == 0) sm.nBM = base;
+  }
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) f[i] = sel[i] && m[i] && !bad[i];
+  const int nBM = rank_rows<CAP>(rs, f, brank);
+  const bool run_lps = p.mode == EBD_DECODE_EB && p.lps_enabled && nBM > 0;
+
+  // ------------------------------------------------------------ LPS
+  if (run_lps) {
+    const float rho = static_cast<float>(nBM) / static_cast<float>(meta_s);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      if (!f[i]) continue;
+      float* ft = rs.feat[brank[i]];
+      ft[0] = conf[i];
+      ft[1] = ent[i];
+      ft[2] = gap[i];
+      ft[3] = rho;
+      ft[4] = static_cast<float>(pos[i] - meta_b) / static_cast<float>(meta_s);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (kWide) {
+      const size_t block = static_cast<size_t>(p.cap_rows) * 64 * NP;  // K and V of a block
+      lps_router<NP, true>(reinterpret_cast<const uint4*>(smem + L::W), sv, nBM, rank + C * warp, 2,
+                           p.kvp + static_cast<size_t>(kbase) * 64 * NP, block, static_cast<size_t>(capk) * 32 * NP,
+                           [&](int row, int k) { return rs.feat[row][k]; },
+                           [&](int row, float v) { p.P[kbase + row] = v; }, [] { cluster_barrier(); });
+      cluster_barrier();  // every row's p_psi is visible
+    } else {
+      lps_local<CAP, NR, NP>(nBM, 2);
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (rank != 0 || bad_seq) return;
+
+  // ------------------------------------------------------------ accept, commit
+  // union accept (Reading R14), anti-stall fallback, parallel commit, block
+  // resolution; the baselines' rules (Reading R20) in their modes
+  float prob[RPT];
+  bool acc[RPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {
+    prob[i] = __int_as_float(0x7fc00000);
+    acc[i] = false;
+    if (!f[i]) continue;
+    if (run_lps && kWide) prob[i] = __ldcg(p.P + kbase + brank[i]);
+    rs.conf[brank[i]] = conf[i];
+    rs.bpos[brank[i]] = pos[i];
   }
   __syncthreads();
-
-  // ---------------------------------------------------------------- 5. LPS + accept + commit
-  // the LPS weight copy must have landed before use and before exit
-  if (sm.lps_loaded && !mbar_wait(&sm.bar2, 0, 1000ull * 1000 * 1000, nullptr))
-    atomicCAS(p.status, 0, EBD_ERR_TIMEOUT);
-  const int nBM = sm.nBM;
-  // phase of the LPS router where a stand-in run starts (-1: accept only)
-  const int lps_from = !shadow ? 0 : (rank <= 4 ? rank - 1 : (rank == 5 ? 4 : (rank == 6 ? 6 : -1)));
-  if (nBM > 0 && p.lps_enabled && lps_from >= 0) {
-    float* feats = P + L_FEAT;
-    const float rho = static_cast<float>(nBM) / static_cast<float>(sm.meta_s);
-#pragma unroll 1
-    for (int i = tid; i < nBM; i += blockDim.x) {
-      const int r = sm.BMrows[i];
-      feats[i * 8 + 0] = sm.f_conf[r];
-      feats[i * 8 + 1] = sm.f_ent[r];
-      feats[i * 8 + 2] = sm.f_gap[r];
-      feats[i * 8 + 3] = rho;
-      feats[i * 8 + 4] = static_cast<float>(sm.f_pos[r] - sm.meta_b) / static_cast<float>(sm.meta_s);
-    }
-    __syncthreads();
-    const float* prob = P + L_PROB;
-    lps_forward(P, nBM, sm.w, sm.v + V_LPS, lps_from, 8);
-#pragma unroll 1
-    for (int i = tid; i < nBM; i += blockDim.x) sm.f_p[sm.BMrows[i]] = prob[i];
-    __syncthreads();
-  }
-  if (warp == 0 && p.mode == EBD_DECODE_TOPM) {
-    // Top-m (App. B, Eq. prelim-update): the rank of a row is the number of
-    // rows ahead of it (higher kappa, or equal kappa and lower position)
-    for (int i = lane; i < nBM; i += 32) {
-      const int j = sm.BMrows[i];
-      const float c = sm.f_conf[j];
-      int rank = 0;
-      for (int k = 0; k < nBM; ++k) {
-        const int jk = sm.BMrows[k];
-        const float ck = sm.f_conf[jk];
-        rank += (ck > c || (ck == c && jk < j)) ? 1 : 0;
-      }
-      if (rank < p.top_m) sm.f_acc[j] = 1;
-    }
-    __syncwarp();
-    for (int j = lane; j < nr; j += 32)
-      if (sm.f_acc[j]) {
-        sm.f_tok[j] = sm.f_arg[j];
-        sm.f_mask[j] = 0;
-      }
-  } else if (warp == 0) {
-    // union accept rule, anti-stall fallback, parallel commit, resolution
-    bool any = false;
-    for (int i0 = 0; i0 < nBM; i0 += 32) {
-      const int i = i0 + lane;
-      bool a = false;
-      if (i < nBM) {
-        const int j = sm.BMrows[i];
-        a = sm.f_conf[j] >= p.tau || (p.lps_enabled && sm.f_p[j] > p.tau_psi);
-        if (a) sm.f_acc[j] = 1;
-      }
-      any |= __ballot_sync(0xffffffffu, a) != 0;
-    }
-    if (!any && nBM > 0) {
-      // highest confidence; the lowest position among equal confidences
-      float best = -INFINITY;
-      int bj = INT_MAX;
-      for (int i = lane; i < nBM; i += 32) {
-        const int j = sm.BMrows[i];
-        const float c = sm.f_conf[j];
-        if (c > best || (c == best && j < bj)) {
-          best = c;
-          bj = j;
-        }
-      }
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, off);
-        const int oj = __shfl_xor_sync(0xffffffffu, bj, off);
-        if (ob > best || (ob == best && oj < bj)) {
-          best = ob;
-          bj = oj;
-        }
-      }
-      if (lane == 0) sm.f_acc[bj] = 1;
+  for (int i = 0; i < RPT; ++i) {
+    if (!f[i]) continue;
+    if (run_lps && !kWide) prob[i] = rs.prob[brank[i]];
+    if (p.mode == EBD_DECODE_TOPM) {
+      int ahead = 0;  // rows ahead: higher kappa, or equal kappa and lower position
+      for (int k = 0; k < nBM; ++k)
+        ahead += (rs.conf[k] > conf[i] || (rs.conf[k] == conf[i] && rs.bpos[k] < pos[i])) ? 1 : 0;
+      acc[i] = ahead < p.top_m;
+    } else {
+      acc[i] = conf[i] >= p.tau || prob[i] > p.tau_psi;  // NaN where the LPS did not run
     }
-    __syncwarp();
-    bool open = false;
-    for (int j0 = 0; j0 < nr; j0 += 32) {
-      const int j = j0 + lane;
-      if (j < nr) {
-        if (sm.f_acc[j]) {
-          sm.f_tok[j] = sm.f_arg[j];
-          sm.f_mask[j] = 0;
-        }
-        open |= sm.f_ib[j] && sm.f_mask[j];
-      }
-    }
-    open = __ballot_sync(0xffffffffu, open) != 0;
-    if (p.mode == EBD_DECODE_EB && sm.meta_s > 0 && !open) {
-      for (int j = lane; j < nr; j += 32) sm.f_ib[j] = 0;
-      if (lane == 0) {
-        sm.meta_b = 0;
-        sm.meta_s = 0;
-      }
-    }
+    if (acc[i]) rs.any = 1;
   }
   __syncthreads();
-
-  // ---------------------------------------------------------------- 6. write back
-  if (shadow) return;
-  for (int j = tid; j < nr; j += blockDim.x) {
-    const int r = r0 + j;
-    if (!in_bounds(r, p.rows_expected, p.status)) continue;
-    p.tokens_out[r] = sm.f_tok[j];
-    p.mask_out[r] = sm.f_mask[j];
-    p.in_block_out[r] = sm.f_ib[j];
-    if (p.accepted) p.accepted[r] = sm.f_acc[j];
-    if (p.lbs_logit) p.lbs_logit[r] = sm.f_O[j];
-    if (p.lps_prob) p.lps_prob[r] = sm.f_p[j];
-  }
-  if (tid == 0 && !sm.bad_seq) {
-    p.blk_meta_out[2 * seq] = sm.meta_b;
-    p.blk_meta_out[2 * seq + 1] = sm.meta_s;
-  }
-}
-
-// ----------------------------------------------------------------- token-branch fold
-// table[v][j] = sum_k W_tok[j][k] W_e[v][k]  (fp32 accumulation)
-__global__ void __launch_bounds__(256) fold_tok_kernel(const __nv_bfloat16* __restrict__ w_tok,
-                                                        const __nv_bfloat16* __restrict__ w_emb,
-                                                        float* __restrict__ table, int V,
-                                                        int d_base) {
-  __shared__ float sE[64][33];
-  __shared__ float sW[64][33];
-  const int v0 = blockIdx.x * 64;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads, 4x4 outputs
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < d_base; k0 += 32) {
-    for (int it = threadIdx.x; it < 64 * 32; it += 256) {
-      const int r = it >> 5, c = it & 31;
-      const int k = k0 + c;
-      const int v = v0 + r;
-      sE[r][c] = (v < V && k < d_base) ? __bfloat162float(w_emb[static_cast<size_t>(v) * d_base + k]) : 0.f;
-      sW[r][c] = (k < d_base) ? __bfloat162float(w_tok[static_cast<size_t>(r) * d_base + k]) : 0.f;
+  if (!rs.any && nBM > 0) {  // anti-stall: the highest kappa, lowest position on ties
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      if (!f[i]) continue;
+      bool best = true;
+      for (int k = 0; k < nBM; ++k)
+        if (rs.conf[k] > conf[i] || (rs.conf[k] == conf[i] && rs.bpos[k] < pos[i])) best = false;
+      if (best) rs.best = brank[i];
     }
     __syncthreads();
-    for (int c = 0; c < 32; ++c) {
-      float e[4], ww[4];
-      for (int i = 0; i < 4; ++i) e[i] = sE[ty * 4 + i][c];
-      for (int i = 0; i < 4; ++i) ww[i] = sW[tx * 4 + i][c];
-      for (int i = 0; i < 4; ++i)
-        for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(e[i], ww[jj], acc[i][jj]);
-    }
-    __syncthreads();
-  }
-  for (int i = 0; i < 4; ++i) {
-    const int v = v0 + ty * 4 + i;
-    if (v >= V) continue;
-    for (int jj = 0; jj < 4; ++jj) table[static_cast<size_t>(v) * 64 + tx * 4 + jj] = acc[i][jj];
-  }
-}
-
-// Merge of the LM-head partial states into the statistics, one warp per row
-// (the statistics-only entry point).
-__global__ void __launch_bounds__(256) merge_stats_kernel(const float4* __restrict__ part_f,
-                                                          const int* __restrict__ part_i, int rows,
-                                                          int grid, int V, float inv_log_v,
-                                                          float* conf, float* entropy,
-                                                          float* ent_norm, float* gap, int* argmax,
-                                                          int* status) {
-  // as a programmatic dependent of the LM head: its partial states are read
-  // only after its grid completed; the grid-wide decision's chain follows
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  const size_t base = static_cast<size_t>(r) * grid;
-  float m = -INFINITY, s = 0.f, t = 0.f, l2 = -INFINITY;
-  int idx = INT_MAX;
-  for (int g = lane; g < grid; g += 32) {
-    const float4 f = part_f[base + g];
-    merge_state(m, s, t, l2, idx, f.x, f.y, f.z, f.w, part_i[base + g]);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) acc[i] = f[i] && brank[i] == rs.best;
   }
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float bm = __shfl_xor_sync(0xffffffffu, m, off);
-    const float bs = __shfl_xor_sync(0xffffffffu, s, off);
-    const float bt = __shfl_xor_sync(0xffffffffu, t, off);
-    const float bl = __shfl_xor_sync(0xffffffffu, l2, off);
-    const int bi = __shfl_xor_sync(0xffffffffu, idx, off);
-    merge_state(m, s, t, l2, idx, bm, bs, bt, bl, bi);
+  for (int i = 0; i < RPT; ++i) {
+    m[i] = m[i] && !acc[i];
+    if (p.mode != EBD_DECODE_EB) sel[i] = inb[i];  // no block state
+    if (sel[i] && m[i]) rs.open = 1;
   }
-  if (lane != 0) return;
-  const float ent = logf(s) - t / s;
-  const bool bad = !(isfinite(m) && isfinite(s) && isfinite(t) && s >= 1.0f) || idx < 0 || idx >= V;
-  if (conf) conf[r] = 1.0f / s;
-  if (entropy) entropy[r] = ent;
-  if (ent_norm) ent_norm[r] = ent * inv_log_v;
-  if (gap) gap[r] = (1.0f - expf(l2 - m)) / s;
-  if (argmax) argmax[r] = bad ? -1 : idx;
-  if (bad) atomicCAS(status, 0, EBD_ERR_NONFINITE);
+  __syncthreads();
+  const bool resolve = p.mode == EBD_DECODE_EB && meta_s > 0 && !rs.open;
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {
+    const int j = 32 * (warp + kNW * i) + lane, r = r0 + j;
+    if (j >= n || !in_bounds(r, p.R, p.status)) continue;
+    p.tokens_out[r] = acc[i] ? arg[i] : p.tokens[r];
+    p.mask_out[r] = m[i] ? 1 : 0;
+    p.in_block_out[r] = (sel[i] && !resolve) ? 1 : 0;
+    if (p.accepted) p.accepted[r] = acc[i] ? 1 : 0;
+    if (p.lbs_logit) p.lbs_logit[r] = lbs[i];
+    if (p.lps_prob) p.lps_prob[r] = prob[i];
+  }
+  if (tid == 0) {
+    if (resolve) meta_b = meta_s = 0;
+    p.blk_meta_out[2 * b] = meta_b;
+    p.blk_meta_out[2 * b + 1] = meta_s;
+  }
 }
 
-cudaError_t launch_merge_stats(const float4* part_f, const int* part_i, int rows, int grid, int V,
-                               float inv_log_v, float* conf, float* entropy, float* ent_norm,
-                               float* gap, int* argmax, int* status, cudaStream_t st, bool pdl) {
+namespace {
+template <int C, int NR, int NP>
+constexpr int smem_bytes() {
+  return Lay<NR, NP>::ROW + static_cast<int>(sizeof(RowState<8 * NR * C>));
+}
+template <int C, int NR, int NP>
+cudaError_t configure_one() {
+  cudaError_t e = cudaFuncSetAttribute(decide_rows_kernel<C, NR, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_bytes<C, NR, NP>());
+  if (e == cudaSuccess && C > 8)
+    e = cudaFuncSetAttribute(decide_rows_kernel<C, NR, NP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+template <int C, int NR, int NP>
+cudaError_t launch_one(const RowsParams& p, cudaStream_t st, bool pdl, int* slots) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>((rows + 7) / 8));
-  cfg.blockDim = dim3(256);
+  cfg.gridDim = dim3(static_cast<unsigned>(slots != nullptr ? C : p.B * C));
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = smem_bytes<C, NR, NP>();
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, merge_stats_kernel, part_f, part_i, rows, grid, V, inv_log_v, conf,
-                            entropy, ent_norm, gap, argmax, status);
+  cfg.numAttrs = pdl ? 2 : 1;
+  if (slots != nullptr) return cudaOccupancyMaxActiveClusters(slots, decide_rows_kernel<C, NR, NP>, &cfg);
+  return cudaLaunchKernelEx(&cfg, decide_rows_kernel<C, NR, NP>, p);
+}
+}  // namespace
+
+cudaError_t decide_rows_configure(int (&slots)[2]) {
+  cudaError_t e;
+  const RowsParams none{};
+  if ((e = configure_one<8, 1, 2>()) != cudaSuccess || (e = configure_one<4, 2, 2>()) != cudaSuccess ||
+      (e = configure_one<2, 4, 2>()) != cudaSuccess || (e = configure_one<4, 1, 2>()) != cudaSuccess ||
+      (e = configure_one<2, 2, 2>()) != cudaSuccess || (e = configure_one<1, 4, 2>()) != cudaSuccess ||
+      (e = configure_one<16, 4, 3>()) != cudaSuccess ||
+      (e = launch_one<8, 1, 2>(none, nullptr, false, &slots[0])) != cudaSuccess ||
+      (e = launch_one<4, 2, 2>(none, nullptr, false, &slots[1])) != cudaSuccess)
+    return e;
+  return cudaSuccess;
 }
 
-// Vocabulary-parallel LM head (several GPUs, each holding a range of W's
-// rows).  The softmax statistics of App. B (Eq. app-confidence), Sec. 5.1
-// and Sec. 5.2 are functions of the whole vocabulary; each shard reduces its
-// range to one online-softmax state per row (m, S, T, l2, x_hat), and the
-// merge of states is associative, so the states of the shards, gathered on
-// every GPU, merge into the statistics of the whole vocabulary.
-//
-// shard_state_kernel: one warp per row merges the row's `grid` LM-head
-// partials into one state, stored as 8 words: m, S, T, l2, idx (int32 bits),
-// and three zero words (32-byte rows).
-__global__ void __launch_bounds__(256) shard_state_kernel(const float4* __restrict__ part_f,
-                                                          const int* __restrict__ part_i, int rows,
-                                                          int grid, float* __restrict__ state) {
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  const size_t base = static_cast<size_t>(r) * grid;
-  float m = -INFINITY, s = 0.f, t = 0.f, l2 = -INFINITY;
-  int idx = INT_MAX;
-  for (int g = lane; g < grid; g += 32) {
-    const float4 f = part_f[base + g];
-    merge_state(m, s, t, l2, idx, f.x, f.y, f.z, f.w, part_i[base + g]);
+cudaError_t launch_decide_rows(const RowsParams& p, int cap, const int (&slots)[2], cudaStream_t st, bool pdl) {
+  if (p.B <= 0 || p.R <= 0) return cudaSuccess;
+  if (cap > 64) return launch_one<16, 4, 3>(p, st, pdl, nullptr);
+  if (cap > 32) {
+    if (p.B <= slots[0]) return launch_one<8, 1, 2>(p, st, pdl, nullptr);
+    return p.B <= slots[1] ? launch_one<4, 2, 2>(p, st, pdl, nullptr) : launch_one<2, 4, 2>(p, st, pdl, nullptr);
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float bm = __shfl_xor_sync(0xffffffffu, m, off);
-    const float bs = __shfl_xor_sync(0xffffffffu, s, off);
-    const float bt = __shfl_xor_sync(0xffffffffu, t, off);
-    const float bl = __shfl_xor_sync(0xffffffffu, l2, off);
-    const int bi = __shfl_xor_sync(0xffffffffu, idx, off);
-    merge_state(m, s, t, l2, idx, bm, bs, bt, bl, bi);
-  }
-  if (lane != 0) return;
-  float4* o = reinterpret_cast<float4*>(state + static_cast<size_t>(r) * 8);
-  o[0] = make_float4(m, s, t, l2);
-  o[1] = make_float4(__int_as_float(idx), 0.f, 0.f, 0.f);
-}
-
-// merge_shards_kernel: one warp per row merges the row's state from each of
-// `shards` shards (states[shard][row][8]) and writes the statistics as the
-// merge of the single-GPU path does (kappa = 1/S, H = ln S - T/S,
-// H~ = H / ln V with V the whole vocabulary, Delta = (1 - exp(l2 - m)) / S,
-// x_hat = idx); a non-finite state records EBD_ERR_NONFINITE.
-__global__ void __launch_bounds__(256) merge_shards_kernel(const float* __restrict__ states,
-                                                           int shards, int rows, int V,
-                                                           float inv_log_v, float* conf,
-                                                           float* entropy, float* ent_norm,
-                                                           float* gap, int* argmax, int* status) {
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  float m = -INFINITY, s = 0.f, t = 0.f, l2 = -INFINITY;
-  int idx = INT_MAX;
-  for (int g = lane; g < shards; g += 32) {
-    const float4* q = reinterpret_cast<const float4*>(
-        states + (static_cast<size_t>(g) * rows + r) * 8);
-    const float4 f = q[0];
-    const float4 i4 = q[1];
-    merge_state(m, s, t, l2, idx, f.x, f.y, f.z, f.w, __float_as_int(i4.x));
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float bm = __shfl_xor_sync(0xffffffffu, m, off);
-    const float bs = __shfl_xor_sync(0xffffffffu, s, off);
-    const float bt = __shfl_xor_sync(0xffffffffu, t, off);
-    const float bl = __shfl_xor_sync(0xffffffffu, l2, off);
-    const int bi = __shfl_xor_sync(0xffffffffu, idx, off);
-    merge_state(m, s, t, l2, idx, bm, bs, bt, bl, bi);
-  }
-  if (lane != 0) return;
-  const float ent = logf(s) - t / s;
-  const bool bad = !(isfinite(m) && isfinite(s) && isfinite(t) && s >= 1.0f) || idx < 0 || idx >= V;
-  if (conf) conf[r] = 1.0f / s;
-  if (entropy) entropy[r] = ent;
-  if (ent_norm) ent_norm[r] = ent * inv_log_v;
-  if (gap) gap[r] = (1.0f - expf(l2 - m)) / s;
-  if (argmax) argmax[r] = bad ? -1 : idx;
-  if (bad) atomicCAS(status, 0, EBD_ERR_NONFINITE);
-}
-
-cudaError_t launch_shard_state(const float4* part_f, const int* part_i, int rows, int grid,
-                               float* state, cudaStream_t st) {
-  shard_state_kernel<<<static_cast<unsigned>((rows + 7) / 8), 256, 0, st>>>(part_f, part_i, rows,
-                                                                            grid, state);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_merge_shards(const float* states, int shards, int rows, int V, float inv_log_v,
-                                float* conf, float* entropy, float* ent_norm, float* gap,
-                                int* argmax, int* status, cudaStream_t st) {
-  merge_shards_kernel<<<static_cast<unsigned>((rows + 7) / 8), 256, 0, st>>>(
-      states, shards, rows, V, inv_log_v, conf, entropy, ent_norm, gap, argmax, status);
-  return cudaGetLastError();
-}
-
-cudaError_t decide_configure() {
-  return cudaFuncSetAttribute(decide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(sizeof(Smem) + 16));
-}
-
-cudaError_t launch_decide(const DecideParams& p, cudaStream_t st) {
-  if (p.B <= 0) return cudaSuccess;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(p.B * kDecideCluster, 1, 1);
-  cfg.blockDim = dim3(kDecideThreads, 1, 1);
-  cfg.dynamicSmemBytes = sizeof(Smem) + 16;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = p.pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, decide_kernel, p);
-}
-
-cudaError_t launch_fold_tok(const __nv_bfloat16* w_tok, const __nv_bfloat16* w_emb, float* table,
-                            int V, int d_base, cudaStream_t st) {
-  fold_tok_kernel<<<(V + 63) / 64, 256, 0, st>>>(w_tok, w_emb, table, V, d_base);
-  return cudaGetLastError();
+  if (p.B <= slots[1]) return launch_one<4, 1, 2>(p, st, pdl, nullptr);
+  return p.B <= 2 * slots[1] ? launch_one<2, 2, 2>(p, st, pdl, nullptr) : launch_one<1, 4, 2>(p, st, pdl, nullptr);
 }
 
 }  // namespace ebd
