@@ -68,7 +68,9 @@ struct Lay {  // shared memory, byte offsets
   static constexpr int kLpsMat = 2 * MB_STRIDE;     // 16-byte units
   static constexpr int KV = W + kLpsMat * 16;
   static constexpr int kKvBlock = 64 * 64 * NP;     // elements of a block
-  static constexpr int kLpsEnd = KV + (NP == 2 ? 2 * kKvBlock * 2 : 0);
+  static constexpr int ST = KV + (NP == 2 ? 2 * kKvBlock * 2 : 0);  // a warp's values between the parts
+  static constexpr int GL = ST + kNW * (16 + 4 * NP) * 32 * 4;      // LpsGlobal
+  static constexpr int kLpsEnd = GL + 32;
   static constexpr int SLOT = kLbsEnd > kLpsEnd ? kLbsEnd : kLpsEnd;
   static constexpr int ROW = SLOT + 3 * 32 * 4;     // per-row arrays
 };
@@ -779,21 +781,43 @@ __device__ __forceinline__ void ld_kv(const __nv_bfloat16* p, uint32_t (&w)[4 * 
   }
 }
 
-// The router of one sequence's B n M (nb rows), 8 rows per warp: group
-// `grp` of 8 rows (idle if 8 * grp >= nb).  feat, prob: by rank in B n M.
-// wm: the weights in shared memory.  Keys and values of both blocks at kv +
-// block * kv_stride: K [key][dim pair][head][plane][2 dims] and, v_off
-// further, V [key pair][dim][head][plane][2 keys], so that a lane reads all
-// heads and planes of its key (pair) in NP 16-byte loads.  `meet` lets every
-// warp of the sequence see the others' keys and values.
-template <int NP, bool GLOBAL, class Feat, class Prob, class Meet>
-__device__ __forceinline__ void lps_router(const uint4* wm, const float* sv, int nb, int grp, int blocks,
-                                           __nv_bfloat16* kv, size_t kv_stride, size_t v_off, Feat feat,
-                                           Prob prob, Meet meet) {
+// The LPS router of one sequence's B n M, 8 rows per warp, in three parts that
+// hand a warp's values over in shared memory (ST): z, the queries, the
+// attention output.  They are not inlined, so that each part's instructions
+// can be brought in by a warp of its own, on stand-in rows, while the
+// statistics are not there yet: with the code out of L2 as well (a step on
+// buffers of its own, after other work), one warp running through all of it
+// took 45k cycles, 29k of them after the LM head had ended; the parts side by
+// side end before it.  (One function whose parts are skipped by branches ran
+// 1.5 times as long.)
+// Keys and values of both blocks at kv + block * kv_stride (GLOBAL, else in
+// shared memory): K [key][dim pair][head][plane][2 dims] and, v_off further, V
+// [key pair][dim][head][plane][2 keys], so that a lane reads all heads and
+// planes of its key (pair) in NP 16-byte loads.
+struct LpsGlobal {  // (GLOBAL; in shared memory, for all warps)
+  __nv_bfloat16* kv;
+  size_t kv_stride, v_off;
+  float* prob;  // by rank in B n M
+};
+template <int NP>
+constexpr int kLpsWords = 8 + 4 * NP + 8;  // z, queries, attention output
+
+// Linear(5 -> 32), LayerNorm, GELU (block 0); LN1, QKV
+template <int CAP, int NR, int NP, bool GLOBAL>
+__device__ __noinline__ void lps_qkv(int nb, int grp, int l) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const float* const sv = reinterpret_cast<const float*>(smem + L::V);
+  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
+  float* const st = reinterpret_cast<float*>(smem + L::ST) + (threadIdx.x >> 5) * kLpsWords<NP> * 32 + (threadIdx.x & 31);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const bool on = 8 * grp < nb;
+  const uint4* const wl = reinterpret_cast<const uint4*>(smem + L::W) + l * MB_STRIDE;
+  const float* const vl = sv + V_BLOCK + l * VB_STRIDE;
+  const LpsGlobal& gl = *reinterpret_cast<const LpsGlobal*>(smem + L::GL);
+  __nv_bfloat16* const K = GLOBAL ? gl.kv + l * gl.kv_stride : reinterpret_cast<__nv_bfloat16*>(smem + L::KV) + l * L::kKvBlock;
+  __nv_bfloat16* const V = K + (GLOBAL ? gl.v_off : L::kKvBlock / 2);
   float z[2][4];
-  if (on) {  // Linear(5 -> 32), LayerNorm, GELU
+  if (l == 0) {
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -801,7 +825,7 @@ __device__ __forceinline__ void lps_router(const uint4* wm, const float* sv, int
         const int row = 8 * grp + 2 * t + (e & 1), f = 16 * i + 8 * (e >> 1) + g;
         float y = sv[V_INB + f];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) y = fmaf(row < nb ? feat(row, k) : 0.f, sv[V_INT + 32 * k + f], y);
+        for (int k = 0; k < 5; ++k) y = fmaf(row < nb ? rs.feat[row][k] : 0.f, sv[V_INT + 32 * k + f], y);
         z[i][e] = y;
       }
     lps_norm(z, sv + V_INLNG, sv + V_INLNB, z);
@@ -809,147 +833,185 @@ __device__ __forceinline__ void lps_router(const uint4* wm, const float* sv, int
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int e = 0; e < 4; ++e) z[i][e] = gelu(z[i][e]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) z[i >> 2][i & 3] = st[32 * i];
+  }
+  uint32_t qf[4][NP];  // queries of each head: dims 2 t, 2 t + 1 of row g
+  float y[2][4], q[6][4];
+  uint32_t f[2][NP][2];
+  lps_norm(z, vl + VB_LN1G, vl + VB_LN1B, y);
+  frags<2, NP>(y, f);
+  lps_gemm<6, 2, NP>(wl + MB_QKV, f, vl + VB_QKVB, q);
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int i = h >> 1, u = 2 * (h & 1);
+    const float sc = 0.5100697233f;  // log2(e) / sqrt(8)
+    uint32_t qp[NP], kp[NP], vp[NP];
+    split2<NP>(q[i][u] * sc, q[i][u + 1] * sc, qp);
+    split2<NP>(q[2 + i][u], q[2 + i][u + 1], kp);
+    split2<NP>(q[4 + i][u], q[4 + i][u + 1], vp);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      qf[h][p] = trans8(qp[p]);
+      *reinterpret_cast<uint32_t*>(K + (((8 * grp + g) * 4 + t) * (4 * NP) + h * NP + p) * 2) = trans8(kp[p]);
+      *reinterpret_cast<uint32_t*>(V + (((4 * grp + t) * 8 + g) * (4 * NP) + h * NP + p) * 2) = vp[p];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) st[32 * i] = z[i >> 2][i & 3];
+#pragma unroll
+  for (int h = 0; h < 4; ++h)
+#pragma unroll
+    for (int p = 0; p < NP; ++p) st[32 * (8 + h * NP + p)] = __uint_as_float(qf[h][p]);
+}
+
+// softmax(q k^T / sqrt(8)) v
+template <int CAP, int NR, int NP, bool GLOBAL>
+__device__ __noinline__ void lps_attend(int nb, int grp, int l) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  float* const st = reinterpret_cast<float*>(smem + L::ST) + (threadIdx.x >> 5) * kLpsWords<NP> * 32 + (threadIdx.x & 31);
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const LpsGlobal& gl = *reinterpret_cast<const LpsGlobal*>(smem + L::GL);
+  const __nv_bfloat16* const K = GLOBAL ? gl.kv + l * gl.kv_stride : reinterpret_cast<const __nv_bfloat16*>(smem + L::KV) + l * L::kKvBlock;
+  const __nv_bfloat16* const V = K + (GLOBAL ? gl.v_off : L::kKvBlock / 2);
+  uint32_t qf[4][NP];
+#pragma unroll
+  for (int h = 0; h < 4; ++h)
+#pragma unroll
+    for (int p = 0; p < NP; ++p) qf[h][p] = __float_as_uint(st[32 * (8 + h * NP + p)]);
+  // the four heads side by side: each block's chain of two products, a
+  // maximum, exponentials and transposes is latency
+  const int n8 = (nb + 7) & ~7;
+  float o[4][4], m[4][2], sum[4][2];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[h][e] = 0.f;
+    m[h][0] = m[h][1] = -INFINITY;
+    sum[h][0] = sum[h][1] = 0.f;
   }
 #pragma unroll 1
-  for (int l = 0; l < blocks; ++l) {
-    const uint4* const wl = wm + l * MB_STRIDE;
-    const float* const vl = sv + V_BLOCK + l * VB_STRIDE;
-    __nv_bfloat16* const K = kv + l * kv_stride;
-    __nv_bfloat16* const V = K + v_off;
-    uint32_t qf[4][NP];  // queries of each head: dims 2 t, 2 t + 1 of row g
-    if (on) {
-      float y[2][4], q[6][4];
-      uint32_t f[2][NP][2];
-      lps_norm(z, vl + VB_LN1G, vl + VB_LN1B, y);
-      frags<2, NP>(y, f);
-      lps_gemm<6, 2, NP>(wl + MB_QKV, f, vl + VB_QKVB, q);
+  for (int k0 = 0; k0 < nb; k0 += 32) {
+    float s[4][2][4], c[4][2], y[4][4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int key = k0 + 16 * j + g;
+      uint32_t k0w[4 * NP], k1w[4 * NP];  // keys key, key + 8: dims 2 t, 2 t + 1
+      ld_kv<NP, GLOBAL>(K + ((key < n8 ? key : 0) * 4 + t) * (8 * NP), k0w);
+      ld_kv<NP, GLOBAL>(K + ((key + 8 < n8 ? key + 8 : 0) * 4 + t) * (8 * NP), k1w);
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
-        const int i = h >> 1, u = 2 * (h & 1);
-        const float sc = 0.5100697233f;  // log2(e) / sqrt(8)
-        uint32_t a[NP], b[NP], c[NP];
-        split2<NP>(q[i][u] * sc, q[i][u + 1] * sc, a);
-        split2<NP>(q[2 + i][u], q[2 + i][u + 1], b);
-        split2<NP>(q[4 + i][u], q[4 + i][u + 1], c);
+        float(&x)[4] = s[h][j];
+        const uint32_t *u = k0w + h * NP, *v = k1w + h * NP;
 #pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          qf[h][p] = trans8(a[p]);
-          *reinterpret_cast<uint32_t*>(K + (((8 * grp + g) * 4 + t) * (4 * NP) + h * NP + p) * 2) = trans8(b[p]);
-          *reinterpret_cast<uint32_t*>(V + (((4 * grp + t) * 8 + g) * (4 * NP) + h * NP + p) * 2) = c[p];
+        for (int e = 0; e < 4; ++e) x[e] = 0.f;
+        // 8 dims fill half a k16 step: two products of planes per MMA
+        if (NP == 3) {
+          mma4(x, make_uint4(u[NP - 1], v[NP - 1], u[0], v[0]), qf[h][0], qf[h][NP - 1]);
+          mma4(x, make_uint4(u[1], v[1], u[1], v[1]), qf[h][0], qf[h][1]);
+        } else {
+          mma4(x, make_uint4(u[1], v[1], 0u, 0u), qf[h][0], 0u);
         }
+        mma4(x, make_uint4(u[0], v[0], u[0], v[0]), qf[h][0], qf[h][1]);
+        if (key >= nb) x[0] = x[1] = -INFINITY;
+        if (key + 8 >= nb) x[2] = x[3] = -INFINITY;
       }
     }
-    meet();
-    if (!on) continue;
-    // the four heads side by side: each block's chain of two products, a
-    // maximum, exponentials and transposes is latency
-    const int n8 = (nb + 7) & ~7;
-    float o[4][4], m[4][2], sum[4][2];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
+      softmax_block<2>(s[h], m[h], sum[h], c[h]);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) o[h][e] = 0.f;
-      m[h][0] = m[h][1] = -INFINITY;
-      sum[h][0] = sum[h][1] = 0.f;
+      for (int e = 0; e < 4; ++e) y[h][e] = 0.f;
     }
-#pragma unroll 1
-    for (int k0 = 0; k0 < nb; k0 += 32) {
-      float s[4][2][4], c[4][2], y[4][4];
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int key = k0 + 16 * j + g;
-        uint32_t k0w[4 * NP], k1w[4 * NP];  // keys key, key + 8: dims 2 t, 2 t + 1
-        ld_kv<NP, GLOBAL>(K + ((key < n8 ? key : 0) * 4 + t) * (8 * NP), k0w);
-        ld_kv<NP, GLOBAL>(K + ((key + 8 < n8 ? key + 8 : 0) * 4 + t) * (8 * NP), k1w);
+    for (int j = 0; j < 2; ++j) {
+      uint32_t va[2][4 * NP];  // keys 16 j + 8 u + 2 t, + 1: dim g
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          float(&x)[4] = s[h][j];
-          const uint32_t *u = k0w + h * NP, *v = k1w + h * NP;
+      for (int u = 0; u < 2; ++u) {
+        const int key = k0 + 16 * j + 8 * u;
+        ld_kv<NP, GLOBAL>(V + (((key < n8 ? key : 0) / 2 + t) * 8 + g) * (8 * NP), va[u]);
+        if (key >= n8)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) x[e] = 0.f;
-          // 8 dims fill half a k16 step: two products of planes per MMA
-          if (NP == 3) {
-            mma4(x, make_uint4(u[NP - 1], v[NP - 1], u[0], v[0]), qf[h][0], qf[h][NP - 1]);
-            mma4(x, make_uint4(u[1], v[1], u[1], v[1]), qf[h][0], qf[h][1]);
-          } else {
-            mma4(x, make_uint4(u[1], v[1], 0u, 0u), qf[h][0], 0u);
-          }
-          mma4(x, make_uint4(u[0], v[0], u[0], v[0]), qf[h][0], qf[h][1]);
-          if (key >= nb) x[0] = x[1] = -INFINITY;
-          if (key + 8 >= nb) x[2] = x[3] = -INFINITY;
-        }
+          for (int i = 0; i < 4 * NP; ++i) va[u][i] = 0u;
       }
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
-        softmax_block<2>(s[h], m[h], sum[h], c[h]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) y[h][e] = 0.f;
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        uint32_t va[2][4 * NP];  // keys 16 j + 8 u + 2 t, + 1: dim g
+        uint32_t pb[NP][2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int key = k0 + 16 * j + 8 * u;
-          ld_kv<NP, GLOBAL>(V + (((key < n8 ? key : 0) / 2 + t) * 8 + g) * (8 * NP), va[u]);
-          if (key >= n8)
+          uint32_t q[NP];
+          split2<NP>(s[h][j][2 * u], s[h][j][2 * u + 1], q);
 #pragma unroll
-            for (int i = 0; i < 4 * NP; ++i) va[u][i] = 0u;
+          for (int p = 0; p < NP; ++p) pb[p][u] = trans8(q[p]);
         }
+        const uint32_t *v0 = va[0] + h * NP, *v1 = va[1] + h * NP;
+        // 8 dims fill half of M: planes 0 and 1 of the values on top of each other
+        if (NP == 3) mma4(y[h], make_uint4(v0[NP - 1], 0u, v1[NP - 1], 0u), pb[0][0], pb[0][1]);
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          uint32_t pb[NP][2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            uint32_t q[NP];
-            split2<NP>(s[h][j][2 * u], s[h][j][2 * u + 1], q);
-#pragma unroll
-            for (int p = 0; p < NP; ++p) pb[p][u] = trans8(q[p]);
-          }
-          const uint32_t *v0 = va[0] + h * NP, *v1 = va[1] + h * NP;
-          // 8 dims fill half of M: planes 0 and 1 of the values on top of each other
-          if (NP == 3) mma4(y[h], make_uint4(v0[NP - 1], 0u, v1[NP - 1], 0u), pb[0][0], pb[0][1]);
-#pragma unroll
-          for (int p = NP - 1; p >= 0; --p)
-            mma4(y[h], make_uint4(v0[0], v0[1], v1[0], v1[1]), pb[p][0], pb[p][1]);
-        }
+        for (int p = NP - 1; p >= 0; --p)
+          mma4(y[h], make_uint4(v0[0], v0[1], v1[0], v1[1]), pb[p][0], pb[p][1]);
       }
-#pragma unroll
-      for (int h = 0; h < 4; ++h)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) o[h][e] = fmaf(o[h][e], c[h][e & 1], y[h][e]);
     }
-    float a[2][4];  // attention output, heads concatenated
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      a[h >> 1][2 * (h & 1)] = (o[h][0] + o[h][2]) * rcp(gsum(sum[h][0]));
-      a[h >> 1][2 * (h & 1) + 1] = (o[h][1] + o[h][3]) * rcp(gsum(sum[h][1]));
-    }
-    float y[2][4];
-    uint32_t f[2][NP][2];
-    frags<2, NP>(a, f);
-    lps_gemm<2, 2, NP>(wl + MB_OUT, f, vl + VB_OUTB, y);
+    for (int h = 0; h < 4; ++h)
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) z[i][e] += y[i][e];
-    lps_norm(z, vl + VB_LN2G, vl + VB_LN2B, y);
-    frags<2, NP>(y, f);
-    float hd[4][4];
-    lps_gemm<4, 2, NP>(wl + MB_FF1, f, vl + VB_FF1B, hd);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) hd[i][e] = gelu(hd[i][e]);
-    uint32_t fh[4][NP][2];
-    frags<4, NP>(hd, fh);
-    lps_gemm<2, 4, NP>(wl + MB_FF2, fh, vl + VB_FF2B, y);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) z[i][e] += y[i][e];
+      for (int e = 0; e < 4; ++e) o[h][e] = fmaf(o[h][e], c[h][e & 1], y[h][e]);
   }
-  if (on) {
+  float x[2][4];  // heads concatenated
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    x[h >> 1][2 * (h & 1)] = (o[h][0] + o[h][2]) * rcp(gsum(sum[h][0]));
+    x[h >> 1][2 * (h & 1) + 1] = (o[h][1] + o[h][3]) * rcp(gsum(sum[h][1]));
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) st[32 * (8 + 4 * NP + i)] = x[i >> 2][i & 3];
+}
+
+// output projection, LN2, FFN; after block 1 the head and p_psi
+template <int CAP, int NR, int NP, bool GLOBAL>
+__device__ __noinline__ void lps_ffn(int nb, int grp, int l) {
+  using L = Lay<NR, NP>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const float* const sv = reinterpret_cast<const float*>(smem + L::V);
+  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
+  float* const st = reinterpret_cast<float*>(smem + L::ST) + (threadIdx.x >> 5) * kLpsWords<NP> * 32 + (threadIdx.x & 31);
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const uint4* const wl = reinterpret_cast<const uint4*>(smem + L::W) + l * MB_STRIDE;
+  const float* const vl = sv + V_BLOCK + l * VB_STRIDE;
+  float z[2][4], x[2][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    z[i >> 2][i & 3] = st[32 * i];
+    x[i >> 2][i & 3] = st[32 * (8 + 4 * NP + i)];
+  }
+  float hd[4][4];
+  float y[2][4];
+  uint32_t f[2][NP][2];
+  frags<2, NP>(x, f);
+  lps_gemm<2, 2, NP>(wl + MB_OUT, f, vl + VB_OUTB, y);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) z[i][e] += y[i][e];
+  lps_norm(z, vl + VB_LN2G, vl + VB_LN2B, y);
+  frags<2, NP>(y, f);
+  lps_gemm<4, 2, NP>(wl + MB_FF1, f, vl + VB_FF1B, hd);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) hd[i][e] = gelu(hd[i][e]);
+  uint32_t fh[4][NP][2];
+  frags<4, NP>(hd, fh);
+  lps_gemm<2, 4, NP>(wl + MB_FF2, fh, vl + VB_FF2B, y);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) z[i][e] += y[i][e];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) st[32 * i] = z[i >> 2][i & 3];
+  if (l == 1) {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       float s = 0.f;
@@ -959,22 +1021,25 @@ __device__ __forceinline__ void lps_router(const uint4* wm, const float* sv, int
         for (int u = 0; u < 2; ++u) s = fmaf(z[i][2 * u + c], sv[V_PHEADW + 16 * i + 8 * u + g], s);
       s = gsum(s) + sv[V_PHEADB];
       const int row = 8 * grp + 2 * t + c;
-      if (g == 0 && row < nb) prob(row, 1.0f / (1.0f + expf(-s)));
+      if (g == 0 && row < nb) (GLOBAL ? reinterpret_cast<const LpsGlobal*>(smem + L::GL)->prob : rs.prob)[row] = 1.0f / (1.0f + expf(-s));
     }
   }
 }
 
-// The router of up to 64 rows by one CTA, in shared memory.  Not inlined, for
-// the same reason as lbs_input: a run on stand-in rows comes first.
-template <int CAP, int NR, int NP>
-__device__ __noinline__ void lps_local(int nb, int blocks) {
-  using L = Lay<NR, NP>;
-  extern __shared__ __align__(16) uint8_t smem[];
-  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
-  lps_router<NP, false>(reinterpret_cast<const uint4*>(smem + L::W), reinterpret_cast<const float*>(smem + L::V), nb,
-                        threadIdx.x >> 5, blocks, reinterpret_cast<__nv_bfloat16*>(smem + L::KV), L::kKvBlock,
-                        64 * 32 * NP, [&](int row, int k) { return rs.feat[row][k]; },
-                        [&](int row, float v) { rs.prob[row] = v; }, [] { __syncthreads(); });
+// 8 rows of the nb per warp, group grp; meet(): every warp of the sequence
+// sees the others' keys and values
+template <int CAP, int NR, int NP, bool GLOBAL, class Meet>
+__device__ __forceinline__ void lps_router(int nb, int grp, Meet meet) {
+  const bool on = 8 * grp < nb;
+#pragma unroll 1
+  for (int l = 0; l < 2; ++l) {
+    if (on) lps_qkv<CAP, NR, NP, GLOBAL>(nb, grp, l);
+    meet();
+    if (on) {
+      lps_attend<CAP, NR, NP, GLOBAL>(nb, grp, l);
+      lps_ffn<CAP, NR, NP, GLOBAL>(nb, grp, l);
+    }
+  }
 }
 
 }  // namespace
@@ -1074,15 +1139,23 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   };
   // Launched behind the LM head, this grid waits some microseconds for its
   // last CTAs, with code that no SM has cached (a first pass through it costs
-  // about as much again as the work itself): meanwhile CTA 0 runs the LPS
-  // router, the others the LBS input layers and the first QKV product, on
+  // about as much again as the work itself, with the code out of L2 as well
+  // several times as much): meanwhile CTA 0 runs the LPS router, one part
+  // per warp, the others the LBS input layers and the first QKV product, on
   // stand-in rows.
   const bool warm = p.warm != 0 && C == 8 && !kWide && p.mode == EBD_DECODE_EB;
   if (!kWide && apart && rank == 0 && p.lps_enabled) {
     copy_lps();
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    if (warm) lps_local<CAP, NR, NP>(32, 1);
+    if (warm) {
+      if (warp % 3 == 0)
+        lps_qkv<CAP, NR, NP, false>(64, warp, 0);
+      else if (warp % 3 == 1)
+        lps_attend<CAP, NR, NP, false>(64, warp, 0);
+      else
+        lps_ffn<CAP, NR, NP, false>(64, warp, 0);
+    }
   } else if (warm && run_lbs && nr > 0) {
     lbs_input<NR, NP>(la);
     lbs_qkv<NR, NP>(la, 0);
@@ -1241,14 +1314,15 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (kWide) {
-      const size_t block = static_cast<size_t>(p.cap_rows) * 64 * NP;  // K and V of a block
-      lps_router<NP, true>(reinterpret_cast<const uint4*>(smem + L::W), sv, nBM, rank + C * warp, 2,
-                           p.kvp + static_cast<size_t>(kbase) * 64 * NP, block, static_cast<size_t>(capk) * 32 * NP,
-                           [&](int row, int k) { return rs.feat[row][k]; },
-                           [&](int row, float v) { p.P[kbase + row] = v; }, [] { cluster_barrier(); });
+      if (tid == 0)
+        *reinterpret_cast<LpsGlobal*>(smem + L::GL) =
+            LpsGlobal{p.kvp + static_cast<size_t>(kbase) * 64 * NP, static_cast<size_t>(p.cap_rows) * 64 * NP,
+                      static_cast<size_t>(capk) * 32 * NP, p.P + kbase};
+      __syncthreads();
+      lps_router<CAP, NR, NP, true>(nBM, rank + C * warp, [] { cluster_barrier(); });
       cluster_barrier();  // every row's p_psi is visible
     } else {
-      lps_local<CAP, NR, NP>(nBM, 2);
+      lps_router<CAP, NR, NP, false>(nBM, warp, [] { __syncthreads(); });
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
