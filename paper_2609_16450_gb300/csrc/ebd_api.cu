@@ -809,33 +809,37 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     // Both attention kernels take 64-row query tiles.  The tcgen05 kernel
     // holds an SM alone (one CTA per SM) and pays a fixed setup and drain
     // per CTA (TMEM, barriers, the query tile, its output), which long key
-    // ranges amortise; the mma.sync kernel runs two CTAs per SM and keeps
-    // launches of many short key ranges (measured, attention alone, LLaDA-8B
-    // heads, us, mma.sync against tcgen05: 16 x 256 x 32 rows 41.6 / 47.8,
-    // 64 x 1024 x 8 211.6 / 230.0; but 16 x 4096 x 32 305.8 / 203.4,
-    // 64 x 4096 x 32 1032.9 / 690.8, 4 x 1024 x 32 45.7 / 27.3, LLaDA-8B
-    // 21.2 / 17.1, Dream-7B 53.9 / 39.6).  EBD_ATTN_KERNEL=tc|mma forces one,
-    // EBD_ATTN_SPLITS the split count (measurement sweeps).
+    // ranges amortise; the mma.sync kernel runs two CTAs per SM, and with
+    // tiles of up to 32 rows it reads the cache as fast, its warps sharing
+    // each chunk's keys.  So, measured (attention alone, LLaDA-8B heads, us,
+    // mma.sync against tcgen05 in the better of their split counts):
+    //   more tiles than SMs: 64 x 1024 x 32 rows 190 / 235, 64 x 4096 x 32
+    //     637 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 58 / 53; but tiles
+    //     of 33 to 64 rows over 1024 keys and more 92 / 78 (16 x 1024 x 64),
+    //     1069 / 711 (64 x 4096 x 64), below that 113 / 150 (64 x 256 x 64);
+    //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
+    //     47.5, 1 x 4096 x 32 26.5 / 20.7; but at 256 keys 10.8 / 12.2.
+    // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count
+    // (measurement sweeps).
     const int tile = 64;
     const int group = cfg->n_heads_q / cfg->n_heads_kv;
     const int aw = cfg->max_window < kMaxWindow ? cfg->max_window : kMaxWindow;
     h->attn_max_qtiles = (aw * group + tile - 1) / tile;
     const int slots = cfg->max_batch * cfg->n_heads_kv * h->attn_max_qtiles;
     const int nch = (cfg->max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
-    h->attn_tc = (slots <= 2 * h->num_sms || nch >= 65 || (nch >= 17 && aw >= 32)) ? 1 : 0;
+    const bool one_wave = slots <= h->num_sms;
+    h->attn_tc = aw * group > 32 ? (one_wave || nch >= 17) : (one_wave && nch >= 9);
     if (const char* env = getenv("EBD_ATTN_KERNEL")) h->attn_tc = strcmp(env, "mma") == 0 ? 0 : 1;
-    int splits;
-    if (h->attn_tc) {
-      // one split, unless few tiles leave most SMs idle: then about one
-      // CTA per SM, but at least 8 key chunks per split
-      splits = 1;
-      if (2 * slots < h->num_sms) {
-        splits = (h->num_sms + slots - 1) / slots;
-        if (splits > nch / 8) splits = nch / 8;
-      }
-    } else {
-      splits = (2 * h->num_sms + slots - 1) / slots;
-    }
+    // key splits per tile: as many as keep one wave of CTAs, of at least 4
+    // chunks each (a CTA more than the SMs hold costs a second wave: 1 x 4096
+    // x 8 rows on tcgen05 28.7 us with 5 splits, 18.7 with 4)
+    int splits = (h->attn_tc ? h->num_sms : 2 * h->num_sms) / slots;
+    if (splits > nch / 4) splits = nch / 4;
+    // a little more than a wave of long ranges: half-length CTAs (10 x 4096
+    // x 8 rows 145 -> 130 us, 12 x 4096 x 32 183 -> 158)
+    const int wave = 2 * h->num_sms;
+    if (!h->attn_tc && nch >= 33 && slots > wave && 2 * ((slots + wave - 1) / wave) > (2 * slots + wave - 1) / wave)
+      splits = 2;
     if (const char* env = getenv("EBD_ATTN_SPLITS")) splits = atoi(env);
     if (splits > kMaxSplits) splits = kMaxSplits;
     if (splits > nch) splits = nch;

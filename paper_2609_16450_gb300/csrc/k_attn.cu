@@ -25,7 +25,9 @@ namespace ebd {
 
 namespace {
 
-constexpr int kStageBytes = 4 * 8192;  // K and V, two 64-dim halves each
+// a stage of the mma.sync kernel: a chunk's K and V, 64-dim halves
+constexpr int attn_stage_bytes(int D) { return 2 * (D / 64) * 8192; }
+constexpr int attn_smem_bytes(int D) { return kAttnStages * attn_stage_bytes(D) + 1024 + 64; }
 
 // byte offset of 16-byte chunk `c` (0..7) of row `r` in a 128B-swizzled tile
 __device__ __forceinline__ uint32_t swz(int r, int c) {
@@ -145,10 +147,18 @@ __device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const float (
 
 }  // namespace
 
-template <int D>
-__device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtensorMap& tm_vc,
+// KG key groups per 64-key chunk: a tile of at most 16 (32) rows has one (two)
+// 16-row blocks, and its 4 warps take a quarter (half) of every chunk's keys
+// each, with a running maximum, sum and output of their own that meet at the
+// end.  With the rows' blocks on one warp each instead, such a tile's MMAs
+// (8 cycles each on the one or two sub-partitions in use) bound it.
+template <int D, int KG>
+__device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtensorMap& tm_vc,
                                           const CUtensorMap& tm_kw, const CUtensorMap& tm_vw,
                                           const AttnParams& p) {
+  constexpr int RW = 4 / KG;   // warps along the rows
+  constexpr int KB = 4 / KG;   // 16-key blocks of a chunk per warp
+  constexpr int kStageBytes = attn_stage_bytes(D);
   constexpr int NH = D / 64;   // 64-dim halves
   constexpr int KS = D / 16;   // k-steps of Q K^T
   constexpr int NT = D / 8;    // n-tiles of the output
@@ -190,7 +200,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
     const int s = i % kAttnStages;
     const int c = c0 + i;
     uint8_t* kd = smem + s * kStageBytes;
-    uint8_t* vd = kd + 2 * 8192;
+    uint8_t* vd = kd + NH * 8192;
     mbar_arrive_expect_tx(&full[s], 2u * NH * 8192u);
 #pragma unroll
     for (int hf = 0; hf < NH; ++hf) {
@@ -211,7 +221,8 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
     for (int i = 0; i < nmy && i < kAttnStages; ++i) issue(i);
 
   // query fragments of this warp's 16 rows
-  const int mrow_lo = qt * 64 + warp * 16 + (lane >> 2);
+  const int rw = warp % RW, kg = warp / RW;
+  const int mrow_lo = qt * 64 + rw * 16 + (lane >> 2);
   const int mrow_hi = mrow_lo + 8;
   auto qptr = [&](int m) -> const __nv_bfloat16* {
     if (m >= m_total) return nullptr;
@@ -220,7 +231,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
   };
   const __nv_bfloat16* q_lo = qptr(mrow_lo);
   const __nv_bfloat16* q_hi = qptr(mrow_hi);
-  const bool warp_active = qt * 64 + warp * 16 < m_total;
+  const bool warp_active = qt * 64 + rw * 16 < m_total;
   uint32_t qf[KS][4];
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks) {
@@ -256,19 +267,19 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
     const int nvalid = c < ncc ? min(kAttnChunk, P - c * kAttnChunk)
                        : (c == ncc ? wb : min(kAttnChunk, S - (c - ncc - 1) * kAttnChunk));
     const uint32_t kbase = smem_u32(smem + s * kStageBytes);
-    const uint32_t vbase = kbase + 2 * 8192;
-    if (warp_active) {
-      float sc[8][4];
+    const uint32_t vbase = kbase + NH * 8192;
+    if (warp_active && 16 * KB * kg < nvalid) {  // the warp has a key
+      float sc[2 * KB][4];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) sc[t][0] = sc[t][1] = sc[t][2] = sc[t][3] = 0.f;
+      for (int t = 0; t < 2 * KB; ++t) sc[t][0] = sc[t][1] = sc[t][2] = sc[t][3] = 0.f;
       const int mi = lane >> 3, rr = lane & 7;
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
         const int hf = ks >> 2;
         const int cidx = (ks & 3) * 2;
 #pragma unroll
-        for (int np = 0; np < 4; ++np) {
-          const int key = np * 16 + (mi >> 1) * 8 + rr;
+        for (int np = 0; np < KB; ++np) {
+          const int key = (KB * kg + np) * 16 + (mi >> 1) * 8 + rr;
           const uint32_t addr = kbase + hf * 8192 + swz(key, cidx + (mi & 1));
           uint32_t b0, b1, b2, b3;
           ldsm_x4(addr, b0, b1, b2, b3);
@@ -278,8 +289,8 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
       }
       float mx_lo = -INFINITY, mx_hi = -INFINITY;
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int k0 = t * 8 + 2 * (lane & 3);
+      for (int t = 0; t < 2 * KB; ++t) {
+        const int k0 = 16 * KB * kg + t * 8 + 2 * (lane & 3);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int key = k0 + (e & 1);
@@ -300,7 +311,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
       m_hi = mn_hi;
       float sum_lo = 0.f, sum_hi = 0.f;
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
+      for (int t = 0; t < 2 * KB; ++t) {
         sc[t][0] = exp2f(sc[t][0] - mn_lo);
         sc[t][1] = exp2f(sc[t][1] - mn_lo);
         sc[t][2] = exp2f(sc[t][2] - mn_hi);
@@ -324,7 +335,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
       }
       // O += P V, P split into bf16 high and low parts
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
+      for (int kk = 0; kk < KB; ++kk) {
         uint32_t ah[4], al[4];
         split_bf16x2(sc[2 * kk][0], sc[2 * kk][1], ah[0], al[0]);
         split_bf16x2(sc[2 * kk][2], sc[2 * kk][3], ah[1], al[1]);
@@ -333,7 +344,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
 #pragma unroll
         for (int dp = 0; dp < D / 16; ++dp) {
           const int hf = dp >> 2;
-          const int key = kk * 16 + (mi & 1) * 8 + rr;
+          const int key = (KB * kg + kk) * 16 + (mi & 1) * 8 + rr;
           const int chunk = (dp & 3) * 2 + (mi >> 1);
           const uint32_t addr = vbase + hf * 8192 + swz(key, chunk);
           uint32_t b0, b1, b2, b3;
@@ -350,13 +361,50 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
   }
   if (failed) return;
 
+  if (KG > 1) {  // the key groups' states meet in the first one, through the ring
+    float4* const x = reinterpret_cast<float4*>(smem);
+    float2* const xl = reinterpret_cast<float2*>(smem + 3 * NT * 32 * 16);
+    if (kg > 0) {
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+        x[((warp - RW) * NT + t) * 32 + lane] = make_float4(o[t][0], o[t][1], o[t][2], o[t][3]);
+      xl[(2 * (warp - RW)) * 32 + lane] = make_float2(m_lo, l_lo);
+      xl[(2 * (warp - RW) + 1) * 32 + lane] = make_float2(m_hi, l_hi);
+    }
+    __syncthreads();
+    if (kg == 0) {
+#pragma unroll
+      for (int k = 1; k < KG; ++k) {
+        const int w = (k - 1) * RW + rw;
+        const float2 a = xl[2 * w * 32 + lane], c = xl[(2 * w + 1) * 32 + lane];
+        const float n_lo = fmaxf(m_lo, a.x), n_hi = fmaxf(m_hi, c.x);
+        // -inf - -inf where neither group saw a key
+        const float p_lo = m_lo == n_lo ? 1.f : exp2f(m_lo - n_lo), p_hi = m_hi == n_hi ? 1.f : exp2f(m_hi - n_hi);
+        const float q_lo = a.x == n_lo ? 1.f : exp2f(a.x - n_lo), q_hi = c.x == n_hi ? 1.f : exp2f(c.x - n_hi);
+        m_lo = n_lo;
+        m_hi = n_hi;
+        l_lo = l_lo * p_lo + a.y * q_lo;
+        l_hi = l_hi * p_hi + c.y * q_hi;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+          const float4 v = x[(w * NT + t) * 32 + lane];
+          o[t][0] = o[t][0] * p_lo + v.x * q_lo;
+          o[t][1] = o[t][1] * p_lo + v.y * q_lo;
+          o[t][2] = o[t][2] * p_hi + v.z * q_hi;
+          o[t][3] = o[t][3] * p_hi + v.w * q_hi;
+        }
+      }
+    }
+  }
+  const bool writer = warp_active && kg == 0;
+
   // ------------------------------------------------------------ output / partials
   auto out_row = [&](int m) -> float* {
     const int hl = m / wb, r = m - hl * wb;
     return p.out + (static_cast<size_t>(r0 + r) * p.Hq + g * p.group + hl) * D;
   };
   if (p.splits == 1) {
-    if (warp_active) {
+    if (writer) {
       const float il = l_lo > 0.f ? 1.0f / l_lo : 0.f, ih = l_hi > 0.f ? 1.0f / l_hi : 0.f;
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
@@ -373,8 +421,8 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
   // partials: O rows [slot][split][64][D] and (max, sum) [slot][split][64][2]
   float* po = p.part + (static_cast<size_t>(slot) * p.splits + split) * 64 * D;
   float* pml = p.part_ml + (static_cast<size_t>(slot) * p.splits + split) * 64 * 2;
-  if (warp_active) {
-    const int ml = warp * 16 + (lane >> 2), mh = ml + 8;
+  if (writer) {
+    const int ml = rw * 16 + (lane >> 2), mh = ml + 8;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
       const int d = t * 8 + 2 * (lane & 3);
@@ -394,7 +442,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
   __threadfence();
   // last CTA of the slot: per-row split weights, then a weighted sum of the
   // splits' O rows with independent vector loads
-  __shared__ float s_w[64][kMaxAttnSplits];
+  float(*const s_w)[kMaxAttnSplits] = reinterpret_cast<float(*)[kMaxAttnSplits]>(smem);  // the ring is free
   const float* bo = p.part + static_cast<size_t>(slot) * p.splits * 64 * D;
   const float* bml = p.part_ml + static_cast<size_t>(slot) * p.splits * 64 * 2;
   const int rows_here = min(64, m_total - qt * 64);
@@ -431,6 +479,21 @@ __device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtens
       *reinterpret_cast<float4*>(out_row(qt * 64 + r) + d) = acc;
   }
   if (tid == 0) p.tickets[slot] = 0;
+}
+
+// the tile's rows pick the split of its warps (uniform over the CTA)
+template <int D>
+__device__ __forceinline__ void attn_body(const CUtensorMap& tm_kc, const CUtensorMap& tm_vc,
+                                          const CUtensorMap& tm_kw, const CUtensorMap& tm_vw,
+                                          const AttnParams& p) {
+  const int b = blockIdx.z / p.Hkv;
+  const int rows = (p.cu_rows[b + 1] - p.cu_rows[b]) * p.group - static_cast<int>(blockIdx.y) * 64;
+  if (rows > 32)
+    attn_tile<D, 1>(tm_kc, tm_vc, tm_kw, tm_vw, p);
+  else if (rows > 16)
+    attn_tile<D, 2>(tm_kc, tm_vc, tm_kw, tm_vw, p);
+  else
+    attn_tile<D, 4>(tm_kc, tm_vc, tm_kw, tm_vw, p);
 }
 
 __device__ __forceinline__ bool named_barrier_and(uint32_t id, uint32_t n, bool pred) {
@@ -1026,10 +1089,9 @@ __global__ void __launch_bounds__(kAttnTcThreads, 1)
 
 cudaError_t attn_configure() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int bytes = kAttnStages * kStageBytes + 1024 + 64;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(attn_kernel<64>, a, bytes)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(attn_kernel<128>, a, bytes)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<64>, a, attn_smem_bytes(64))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<128>, a, attn_smem_bytes(128))) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attn_tc_kernel<64>, a, TcMap<64>::kDyn)) != cudaSuccess) return e;
   return cudaFuncSetAttribute(attn_tc_kernel<128>, a, TcMap<128>::kDyn);
 }
@@ -1041,7 +1103,7 @@ cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const
   cfg.gridDim = dim3(p.splits, p.max_qtiles, p.B * p.Hkv);
   cfg.blockDim = dim3(p.tc ? kAttnTcThreads : kAttnThreads, 1, 1);
   cfg.dynamicSmemBytes = p.tc ? (p.D == 64 ? TcMap<64>::kDyn : TcMap<128>::kDyn)
-                              : kAttnStages * kStageBytes + 1024 + 64;
+                              : attn_smem_bytes(p.D);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
