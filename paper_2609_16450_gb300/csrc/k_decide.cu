@@ -162,20 +162,25 @@ __device__ __forceinline__ void mma4(float (&d)[4], const uint4& a, uint32_t b0,
 }
 
 // acc[r][i]: outputs 16 tile_i + 2 g (elements 0, 1) and + 1 (2, 3) of rows
-// 8 r + 2 t, 8 r + 2 t + 1 of A W^T, A in NP planes.  The first plane has its
-// own accumulators; with NP = 3 they are added up in fp32 every 32 inputs,
+// 8 r + 2 t, 8 r + 2 t + 1 of A W^T, A in NP planes.  Each plane has its own
+// accumulators, and dependent MMAs (31 cycles apart, one every 8 otherwise)
+// stand as far apart as the tile allows; with NP = 3 they are added up in fp32 every 32 inputs,
 // since the tensor cores truncate where they align a sum's terms.
 template <int K, int NT, int NR, int NP>
 __device__ __forceinline__ void gemm(const uint8_t* A, int plane, const uint4 (&w)[NT * (K / 16)], int nr,
                                      float (&acc)[NR][NT][4]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  float al[NR][NT][4];
+  float al[NR][NT][NP - 1][4];
 #pragma unroll
   for (int r = 0; r < NR; ++r)
 #pragma unroll
     for (int i = 0; i < NT; ++i)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[r][i][e] = al[r][i][e] = 0.f;
+      for (int e = 0; e < 4; ++e) {
+        acc[r][i][e] = 0.f;
+#pragma unroll
+        for (int p = 0; p < NP - 1; ++p) al[r][i][p][e] = 0.f;
+      }
 #pragma unroll
   for (int kb = 0; kb < K / 32; ++kb)
 #pragma unroll
@@ -185,32 +190,30 @@ __device__ __forceinline__ void gemm(const uint8_t* A, int plane, const uint4 (&
 #pragma unroll
       for (int p = 0; p < NP; ++p)
         x[p] = *reinterpret_cast<const uint4*>(A + p * plane + (8 * r + g) * row_bytes(K) + 64 * kb + 16 * t);
+      float d[NT][4];
 #pragma unroll
-      for (int i = 0; i < NT; ++i) {
-        const uint4 &a = w[i * (K / 16) + 2 * kb], &b = w[i * (K / 16) + 2 * kb + 1];
+      for (int i = 0; i < NT; ++i)
 #pragma unroll
-        for (int p = NP - 1; p > 0; --p) {
-          mma4(al[r][i], a, x[p].x, x[p].y);
-          mma4(al[r][i], b, x[p].z, x[p].w);
-        }
-        if (NP == 3) {
-          float d[4] = {0.f, 0.f, 0.f, 0.f};
-          mma4(d, a, x[0].x, x[0].y);
-          mma4(d, b, x[0].z, x[0].w);
+        for (int e = 0; e < 4; ++e) d[i][e] = NP == 3 ? 0.f : acc[r][i][e];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) acc[r][i][e] += d[e];
-        } else {
-          mma4(acc[r][i], a, x[0].x, x[0].y);
-          mma4(acc[r][i], b, x[0].z, x[0].w);
-        }
-      }
+      for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+        for (int p = NP - 1; p >= 0; --p)
+#pragma unroll
+          for (int i = 0; i < NT; ++i)
+            mma4(p > 0 ? al[r][i][p - 1] : d[i], w[i * (K / 16) + 2 * kb + ks], ks == 0 ? x[p].x : x[p].z,
+                 ks == 0 ? x[p].y : x[p].w);
+#pragma unroll
+      for (int i = 0; i < NT; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[r][i][e] = NP == 3 ? acc[r][i][e] + d[i][e] : d[i][e];
     }
 #pragma unroll
   for (int r = 0; r < NR; ++r)
 #pragma unroll
     for (int i = 0; i < NT; ++i)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[r][i][e] += al[r][i][e];
+      for (int e = 0; e < 4; ++e) acc[r][i][e] += NP == 3 ? al[r][i][0][e] + al[r][i][NP - 2][e] : al[r][i][0][e];
 }
 
 // LayerNorm (eps 1e-5) of a warp's row of 32 * N values, lane holding
@@ -361,19 +364,27 @@ __device__ __forceinline__ void attend(const uint8_t* Q, const __nv_bfloat16* Kp
 #pragma unroll
       for (int p = 0; p < NP; ++p)
         x[p] = *reinterpret_cast<const uint4*>(Q + p * L::P128 + (8 * r + g) * row_bytes(128) + 64 * head + 16 * t);
-      float s[2][4];
+      float s[2][4], s1[2][4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[j][e] = s1[j][e] = 0.f;
+#pragma unroll
+      for (int sum = NP - 1; sum >= 0; --sum)
+#pragma unroll
+        for (int a = 0; a <= sum; ++a) {
+          const uint4& q = x[sum - a];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const uint4 &u = kf[j][0][a], &v = kf[j][1][a];
+            mma4(s[j], make_uint4(u.x, v.x, u.y, v.y), q.x, q.y);
+            mma4(s1[j], make_uint4(u.z, v.z, u.w, v.w), q.z, q.w);
+          }
+        }
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[j][e] = 0.f;
-#pragma unroll
-        for (int sum = NP - 1; sum >= 0; --sum)
-#pragma unroll
-          for (int a = 0; a <= sum; ++a) {
-            const uint4 &u = kf[j][0][a], &v = kf[j][1][a], &q = x[sum - a];
-            mma4(s[j], make_uint4(u.x, v.x, u.y, v.y), q.x, q.y);
-            mma4(s[j], make_uint4(u.z, v.z, u.w, v.w), q.z, q.w);
-          }
+        for (int e = 0; e < 4; ++e) s[j][e] += s1[j][e];
         const int key = 32 * blk + 8 * (g >> 1) + (g & 1) + 4 * j;
         if (key >= n) s[j][0] = s[j][1] = -INFINITY;
         if (key + 2 >= n) s[j][2] = s[j][3] = -INFINITY;
@@ -398,20 +409,25 @@ __device__ __forceinline__ void attend(const uint8_t* Q, const __nv_bfloat16* Kp
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       if (NR > 1 && r >= nr) continue;
+      float y[2][2][4];
 #pragma unroll
-      for (int d = 0; d < 2; ++d) {
-        float y[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int d = 0; d < 2; ++d)
 #pragma unroll
-        for (int sum = NP - 1; sum >= 0; --sum)
+        for (int e = 0; e < 4; ++e) y[d][0][e] = y[d][1][e] = 0.f;
 #pragma unroll
-          for (int a = 0; a <= sum; ++a) {
+      for (int sum = NP - 1; sum >= 0; --sum)
+#pragma unroll
+        for (int a = 0; a <= sum; ++a)
+#pragma unroll
+          for (int d = 0; d < 2; ++d) {
             const uint4 &u = vf[d][0][a], &v = vf[d][1][a];
-            mma4(y, make_uint4(u.x, v.x, u.y, v.y), pb[r][0][sum - a][0], pb[r][0][sum - a][1]);
-            mma4(y, make_uint4(u.z, v.z, u.w, v.w), pb[r][1][sum - a][0], pb[r][1][sum - a][1]);
+            mma4(y[d][0], make_uint4(u.x, v.x, u.y, v.y), pb[r][0][sum - a][0], pb[r][0][sum - a][1]);
+            mma4(y[d][1], make_uint4(u.z, v.z, u.w, v.w), pb[r][1][sum - a][0], pb[r][1][sum - a][1]);
           }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) o[r][d][e] += y[e];
-      }
+      for (int d = 0; d < 2; ++d)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[r][d][e] += y[d][0][e] + y[d][1][e];
     }
   }
 #pragma unroll
@@ -735,18 +751,21 @@ __device__ __forceinline__ void lps_gemm(const uint4* w, const uint32_t (&f)[KT]
   for (int i = 0; i < MT; ++i)
 #pragma unroll
     for (int k = 0; k < KT; ++k) a[i][k] = w[(i * KT + k) * 32 + lane];
+  float lo[MT][4], hi[MT][4];
 #pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int k = 0; k < KT; ++k) {
+    for (int e = 0; e < 4; ++e) lo[i][e] = hi[i][e] = 0.f;
 #pragma unroll
-      for (int p = NP - 1; p > 0; --p) mma4(lo, a[i][k], f[k][p][0], f[k][p][1]);
-      mma4(hi, a[i][k], f[k][0][0], f[k][0][1]);
-    }
+  for (int k = 0; k < KT; ++k)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) y[i][e] = (hi[e] + lo[e]) + b[16 * i + g + 8 * (e >> 1)];
-  }
+    for (int p = NP - 1; p >= 0; --p)
+#pragma unroll
+      for (int i = 0; i < MT; ++i) mma4(p > 0 ? lo[i] : hi[i], a[i][k], f[k][p][0], f[k][p][1]);
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) y[i][e] = (hi[i][e] + lo[i][e]) + b[16 * i + g + 8 * (e >> 1)];
 }
 
 // LayerNorm over the 32 features of each row
@@ -902,21 +921,28 @@ __device__ __noinline__ void lps_attend(int nb, int grp, int l) {
       ld_kv<NP, GLOBAL>(K + ((key < n8 ? key : 0) * 4 + t) * (8 * NP), k0w);
       ld_kv<NP, GLOBAL>(K + ((key + 8 < n8 ? key + 8 : 0) * 4 + t) * (8 * NP), k1w);
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        float(&x)[4] = s[h][j];
-        const uint32_t *u = k0w + h * NP, *v = k1w + h * NP;
+      for (int h = 0; h < 4; ++h)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x[e] = 0.f;
-        // 8 dims fill half a k16 step: two products of planes per MMA
-        if (NP == 3) {
-          mma4(x, make_uint4(u[NP - 1], v[NP - 1], u[0], v[0]), qf[h][0], qf[h][NP - 1]);
-          mma4(x, make_uint4(u[1], v[1], u[1], v[1]), qf[h][0], qf[h][1]);
-        } else {
-          mma4(x, make_uint4(u[1], v[1], 0u, 0u), qf[h][0], 0u);
+        for (int e = 0; e < 4; ++e) s[h][j][e] = 0.f;
+      // 8 dims fill half a k16 step: two products of planes per MMA
+#pragma unroll
+      for (int part = NP == 3 ? 0 : 1; part < 3; ++part)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const uint32_t *u = k0w + h * NP, *v = k1w + h * NP;
+          if (part == 0)
+            mma4(s[h][j], make_uint4(u[NP - 1], v[NP - 1], u[0], v[0]), qf[h][0], qf[h][NP - 1]);
+          else if (part == 1 && NP == 3)
+            mma4(s[h][j], make_uint4(u[1], v[1], u[1], v[1]), qf[h][0], qf[h][1]);
+          else if (part == 1)
+            mma4(s[h][j], make_uint4(u[1], v[1], 0u, 0u), qf[h][0], 0u);
+          else
+            mma4(s[h][j], make_uint4(u[0], v[0], u[0], v[0]), qf[h][0], qf[h][1]);
         }
-        mma4(x, make_uint4(u[0], v[0], u[0], v[0]), qf[h][0], qf[h][1]);
-        if (key >= nb) x[0] = x[1] = -INFINITY;
-        if (key + 8 >= nb) x[2] = x[3] = -INFINITY;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (key >= nb) s[h][j][0] = s[h][j][1] = -INFINITY;
+        if (key + 8 >= nb) s[h][j][2] = s[h][j][3] = -INFINITY;
       }
     }
 #pragma unroll
@@ -936,23 +962,27 @@ __device__ __noinline__ void lps_attend(int nb, int grp, int l) {
 #pragma unroll
           for (int i = 0; i < 4 * NP; ++i) va[u][i] = 0u;
       }
+      uint32_t pb[4][NP][2];
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        uint32_t pb[NP][2];
+      for (int h = 0; h < 4; ++h)
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           uint32_t q[NP];
           split2<NP>(s[h][j][2 * u], s[h][j][2 * u + 1], q);
 #pragma unroll
-          for (int p = 0; p < NP; ++p) pb[p][u] = trans8(q[p]);
+          for (int p = 0; p < NP; ++p) pb[h][p][u] = trans8(q[p]);
         }
-        const uint32_t *v0 = va[0] + h * NP, *v1 = va[1] + h * NP;
-        // 8 dims fill half of M: planes 0 and 1 of the values on top of each other
-        if (NP == 3) mma4(y[h], make_uint4(v0[NP - 1], 0u, v1[NP - 1], 0u), pb[0][0], pb[0][1]);
+      // 8 dims fill half of M: planes 0 and 1 of the values on top of each other
 #pragma unroll
-        for (int p = NP - 1; p >= 0; --p)
-          mma4(y[h], make_uint4(v0[0], v0[1], v1[0], v1[1]), pb[p][0], pb[p][1]);
-      }
+      for (int p = NP == 3 ? NP : NP - 1; p >= 0; --p)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const uint32_t *v0 = va[0] + h * NP, *v1 = va[1] + h * NP;
+          if (p == NP)
+            mma4(y[h], make_uint4(v0[NP - 1], 0u, v1[NP - 1], 0u), pb[h][0][0], pb[h][0][1]);
+          else
+            mma4(y[h], make_uint4(v0[0], v0[1], v1[0], v1[1]), pb[h][p][0], pb[h][p][1]);
+        }
     }
 #pragma unroll
     for (int h = 0; h < 4; ++h)
