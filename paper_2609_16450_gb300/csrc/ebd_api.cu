@@ -889,7 +889,8 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     };
     const size_t o_kv = add(4 * planes * cap * 128 * 2), o_kvp = add(4 * planes * cap * 32 * 2), o_O = add(cap * 4),
                  o_P = add(cap * 4), o_c = add((R + 1) * 4), o_e = add((R + 1) * 4), o_g = add((R + 1) * 4),
-                 o_a = add((R + 1) * 4);
+                 o_a = add((R + 1) * 4), o_z = add(planes == 3 ? cap * 128 * 4 : 0),
+                 o_q = add(planes == 3 ? 3 * cap * 128 * 2 : 0);
     if ((e = cudaMalloc(&h->rows_scratch, bytes)) != cudaSuccess)
       return bail(cuda_fail(h, e, "cudaMalloc(decision scratch)"));
     uint8_t* b0 = h->rows_scratch;
@@ -898,6 +899,8 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     q.spare_row = cfg->max_rows;
     q.kv = reinterpret_cast<__nv_bfloat16*>(b0 + o_kv);
     q.kvp = reinterpret_cast<__nv_bfloat16*>(b0 + o_kvp);
+    q.z = reinterpret_cast<float*>(b0 + o_z);
+    q.q = reinterpret_cast<__nv_bfloat16*>(b0 + o_q);
     q.O = reinterpret_cast<float*>(b0 + o_O);
     q.P = reinterpret_cast<float*>(b0 + o_P);
     q.s_conf = reinterpret_cast<float*>(b0 + o_c);

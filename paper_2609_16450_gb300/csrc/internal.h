@@ -95,6 +95,8 @@ struct RowsParams {
   int cap_rows;             // rows of the scratch below: R rounded up to 32, and 32 per sequence
   __nv_bfloat16* kv;        // LBS keys and values [2 layers][2][planes][cap_rows][128]
   __nv_bfloat16* kvp;       // LPS keys and values [2 blocks][2][planes][cap_rows][32]
+  float* z;                 // windows of more than 64 rows: LBS activations [cap_rows][128]
+  __nv_bfloat16* q;         // and queries [planes][cap_rows][128] between launches
   float *O, *P;             // [cap_rows] LBS logits by rank in M, p_psi by rank in B n M
   int* status;
 };

@@ -8,7 +8,8 @@
 // layers on its own; the CTAs of a cluster meet only where attention needs
 // every row's keys and values (once per layer) and before the selection:
 // three cluster barriers.  Keys and values travel through an L2-resident
-// scratch.  The LPS router is small enough for a warp to take 8 rows of
+// scratch.  Windows of more than 64 rows take their LBS through three launches
+// over the whole GPU instead (lbs_wide_kernel), ahead of the cluster.  The LPS router is small enough for a warp to take 8 rows of
 // B n M through it in registers; its warps meet for the keys and values of
 // its two attentions only.
 //
@@ -1072,12 +1073,166 @@ __device__ __forceinline__ void lps_router(int nb, int grp, Meet meet) {
   }
 }
 
+// The statistics of the CTA's rows merged from the LM head's partial states:
+// its groups' slots, then its share of the unmasked rows, a row per warp.
+// Waits for the grid before this one first.  With `warm` each warp starts
+// with a pass that merges no states, into a row of its own (before the wait).
+template <int CAP>
+__device__ __forceinline__ void merge_rows(const RowsParams& p, Slots& sl, const RowState<CAP>& rs, int r0, int nr,
+                                           int nu, bool warm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  bool waited = false;
+  for (int it = warm && nr + nu > 0 ? warp - kNW : warp; it < 8 * nr + nu; it += kNW) {
+    const bool real = it >= 0;
+    if (real && !waited) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      waited = true;
+    }
+    const int j = !real ? 0 : it < 8 * nr ? sl.mrow[it] : rs.urow[it - 8 * nr];
+    if (j < 0 || (real && !in_bounds(r0 + j, p.R, p.status))) continue;
+    const size_t base = static_cast<size_t>(r0 + j) * p.grid_lm;
+    const RowStats st = merge_row(p.part_f + base, p.part_i + base, real ? p.grid_lm : 0);
+    if (lane == 0) {
+      const int r = r0 + j, sr = real ? r : p.spare_row;
+      const float conf = 1.0f / st.s, ent = logf(st.s) - st.t * conf, entn = ent * p.inv_log_v;
+      const float gap = (1.0f - expf(st.l2 - st.m)) * conf;
+      const bool bad = !(isfinite(st.m) && isfinite(st.s) && isfinite(st.t) && st.s >= 1.0f) || st.idx < 0 ||
+                       st.idx >= p.V;
+      const int arg = bad ? -1 : st.idx;
+      p.s_conf[sr] = conf;
+      p.s_ent[sr] = entn;
+      p.s_gap[sr] = gap;
+      p.s_arg[sr] = arg;
+      if (real) {
+        if (p.conf) p.conf[r] = conf;
+        if (p.entropy) p.entropy[r] = ent;
+        if (p.ent_norm) p.ent_norm[r] = entn;
+        if (p.gap) p.gap[r] = gap;
+        if (p.argmax) p.argmax[r] = arg;
+        if (bad) atomicCAS(p.status, 0, EBD_ERR_NONFINITE);
+        if (it < 8 * nr) {
+          sl.ent[it] = entn;
+          sl.arg[it] = arg;
+        }
+      }
+    }
+  }
+  if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace
 
-template <int C, int NR, int NP>
+// The statistics and the LBS of windows of more than 64 rows, ahead of the
+// decision's kernel: a CTA per group of 8 masked rows (grid: groups, sequences)
+// over the whole GPU, one launch per stretch between two attentions, rows and
+// queries handed on through the scratch.
+//   PART 0: statistics; LBS input, QKV of layer 0
+//   PART 1: layer 0, QKV of layer 1      PART 2: layer 1, LBS logits
+// Bound by the chain of dependent phases of a CTA.  With the LBS in the
+// cluster's 16 CTAs, four groups each, an attention over 384 keys took 39k
+// cycles: the unrolled loop over a CTA's groups left the instruction caches, on
+// 16 SMs of 152.  ebd_decide, 384 masked rows of 512: 105 us so, 62 here; eight
+// such sequences 152.
+template <int PART>
+__global__ void __launch_bounds__(kT, 1) lbs_wide_kernel(const RowsParams p) {
+  constexpr int NP = 3, CAP = kMaxSeqRows;
+  using L = Lay<1, NP>;
+  constexpr int RPT = CAP / kT;
+  extern __shared__ __align__(16) uint8_t smem[];
+  float* const sv = reinterpret_cast<float*>(smem + L::V);
+  float* const F = reinterpret_cast<float*>(smem + L::F);
+  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
+  Slots& sl = *reinterpret_cast<Slots*>(smem + L::SLOT);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int b = blockIdx.y, wk = blockIdx.x, nw = gridDim.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int i = tid; i < kVecs / 4; i += kT)
+    reinterpret_cast<float4*>(sv)[i] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
+  const int r0 = p.cu_rows[b];
+  int n = p.cu_rows[b + 1] - r0;
+  if (n < 0 || n > CAP || r0 < 0 || r0 + n > p.R || n > p.gen_len) n = 0;  // reported by the decision
+  const int kbase = ((r0 + 31) & ~31) + 32 * b, capk = (n + 31) & ~31;
+  bool m[RPT], f[RPT];
+  int mrank[RPT], urank[RPT];
+  if (PART == 0 && tid < 32) {
+    sl.mrow[tid] = -1;
+    sl.ent[tid] = 0.f;
+    sl.arg[tid] = -1;
+  }
+  int nM = 0, nU = 0;
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) {
+    const int j = 32 * (warp + kNW * i) + lane;
+    m[i] = j < n && p.mask[r0 + j] != 0;
+    f[i] = j < n && !m[i];
+    if (PART != 0) nM += __syncthreads_count(m[i]);
+  }
+  if (PART == 0) {
+    nM = rank_rows<CAP>(rs, m, mrank);
+    nU = rank_rows<CAP>(rs, f, urank);
+  }
+  const bool run_lbs = p.mode == EBD_DECODE_EB && p.blk_meta[2 * b + 1] == 0 && nM > p.l_min;
+  const int groups = (nM + 7) >> 3;
+  const int nr = wk < groups ? 1 : 0;
+  const LbsArgs la{p.mat, p.vec, p.tok_table, p.kv, p.O, p.V, p.gen_len, p.cap_rows, kbase, capk, nM, nr, wk, nw};
+  float* const zg = p.z + static_cast<size_t>(kbase + 8 * wk) * 128;
+  uint8_t* const qg = reinterpret_cast<uint8_t*>(p.q + static_cast<size_t>(kbase + 8 * wk) * 128);
+  const size_t qplane = static_cast<size_t>(p.cap_rows) * 256;  // bytes
+  if (PART == 0) {
+    // as in the cluster: the rows without a group go to the CTAs without one
+    const int u0 = groups < nw ? groups : 0, nuw = nw - u0;
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const int j = 32 * (warp + kNW * i) + lane;
+      if (m[i] && (mrank[i] >> 3) == wk) sl.mrow[mrank[i] & 7] = j;
+      if (f[i] && u0 + urank[i] % nuw == wk) rs.urow[urank[i] / nuw] = j;
+    }
+    const int nu = wk >= u0 && nU > wk - u0 ? (nU - (wk - u0) + nuw - 1) / nuw : 0;
+    __syncthreads();
+    if (p.features_in) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (tid < 8 && sl.mrow[tid] >= 0) {
+        sl.ent[tid] = p.s_ent[r0 + sl.mrow[tid]];
+        sl.arg[tid] = p.s_arg[r0 + sl.mrow[tid]];
+      }
+    } else {
+      merge_rows<CAP>(p, sl, rs, r0, nr, nu, false);
+    }
+    __syncthreads();
+    if (!run_lbs || nr == 0) return;
+    lbs_input<1, NP>(la);
+  } else {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!run_lbs || nr == 0) return;
+    for (int i = tid; i < 8 * 32; i += kT)
+      reinterpret_cast<float4*>(F + (i >> 5) * L::kLdF)[i & 31] = __ldcg(reinterpret_cast<const float4*>(zg) + i);
+    for (int i = tid; i < NP * 8 * 16; i += kT) {
+      const int pl = i >> 7, row = (i >> 4) & 7, c = i & 15;
+      *reinterpret_cast<uint4*>(smem + L::Q + pl * L::P128 + row * row_bytes(128) + 16 * c) =
+          __ldcg(reinterpret_cast<const uint4*>(qg + pl * qplane + row * 256) + c);
+    }
+    __syncthreads();
+    lbs_layer<1, NP>(la, PART - 1);
+    if (PART == 2) return;
+  }
+  lbs_qkv<1, NP>(la, PART);
+  __syncthreads();
+  for (int i = tid; i < 8 * 32; i += kT)
+    reinterpret_cast<float4*>(zg)[i] = reinterpret_cast<const float4*>(F + (i >> 5) * L::kLdF)[i & 31];
+  for (int i = tid; i < NP * 8 * 16; i += kT) {
+    const int pl = i >> 7, row = (i >> 4) & 7, c = i & 15;
+    reinterpret_cast<uint4*>(qg + pl * qplane + row * 256)[c] =
+        *reinterpret_cast<const uint4*>(smem + L::Q + pl * L::P128 + row * row_bytes(128) + 16 * c);
+  }
+}
+
+template <int C, int NR, int NP, int CAP>
 __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) {
   using L = Lay<NR, NP>;
-  constexpr int CAP = 8 * NR * C;
+  // windows of more than 64 rows: the LBS and the statistics come from
+  // lbs_wide_kernel
+  constexpr bool kWide = CAP > 64;
+  static_assert(kWide || CAP == 8 * NR * C, "rows of the cluster's groups");
   constexpr int NC = CAP / 32, RPT = (NC + kNW - 1) / kNW;
   extern __shared__ __align__(16) uint8_t smem[];
   float* const sv = reinterpret_cast<float*>(smem + L::V);
@@ -1130,133 +1285,102 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     f[i] = row && !m[i];
   }
   const int nM = rank_rows<CAP>(rs, m, mrank);
-  const int nU = rank_rows<CAP>(rs, f, urank);
-  // Windows of up to 64 rows: CTA 0 makes the decision.  Eight CTAs with a
-  // group to spare leave all rows to the other seven, so that CTA 0 can bring
-  // in the LPS and its weights meanwhile.
-  constexpr bool kWide = CAP > 64;
-  const int groups = (nM + 7) >> 3;
-  const bool apart = C == 8 && !kWide && groups < C;
-  const int nw = apart ? C - 1 : C, wk = apart ? rank - 1 : rank;
-  // group k of 8 rows of M belongs to worker k % nw, its slot k / nw; the
-  // statistics of the other rows are merged by the workers without a group
-  const int u0 = groups < nw ? groups : 0, nuw = nw - u0;
-  if (wk >= 0) {
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int j = 32 * (warp + kNW * i) + lane, grp = mrank[i] >> 3;
-      if (m[i] && grp % nw == wk) sl.mrow[8 * (grp / nw) + (mrank[i] & 7)] = j;
-      if (f[i] && u0 + urank[i] % nuw == wk) rs.urow[urank[i] / nuw] = j;
-    }
-  }
+  const int nU = kWide ? 0 : rank_rows<CAP>(rs, f, urank);
   const bool run_lbs = p.mode == EBD_DECODE_EB && meta_s == 0 && nM > p.l_min;
-  const int nr = wk >= 0 && groups > wk ? (groups - wk + nw - 1) / nw : 0;  // groups of this CTA
-  const int nu = wk >= u0 && nU > wk - u0 ? (nU - (wk - u0) + nuw - 1) / nuw : 0;
-  const LbsArgs la{p.mat, p.vec, p.tok_table, p.kv, p.O, p.V, p.gen_len, p.cap_rows, kbase, capk, nM, nr, wk, nw};
-  __syncthreads();
-
-  // The LM head has streamed its weight through L2: bring the router's back
-  // while its last CTAs run.
-  if (b == 0) {
-    const char* w = reinterpret_cast<const char*>(p.mat);
-    for (int i = (run_lbs ? 0 : M_BLOCK / 8) + rank * kT + tid; i < M_TOTAL / 8; i += C * kT)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 128 * static_cast<size_t>(i)));
-  }
   auto copy_lps = [&]() {
     for (int i = tid; i < L::kLpsMat; i += kT)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem + L::W + 16 * i)), "l"(p.mat + M_BLOCK + i)
                    : "memory");
   };
-  // Launched behind the LM head, this grid waits some microseconds for its
-  // last CTAs, with code that no SM has cached (a first pass through it costs
-  // about as much again as the work itself, with the code out of L2 as well
-  // several times as much): meanwhile CTA 0 runs the LPS router, one part
-  // per warp, the others the LBS input layers and the first QKV product, on
-  // stand-in rows.
-  const bool warm = p.warm != 0 && C == 8 && !kWide && p.mode == EBD_DECODE_EB;
-  if (!kWide && apart && rank == 0 && p.lps_enabled) {
-    copy_lps();
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    if (warm) {
-      if (warp % 3 == 0)
-        lps_qkv<CAP, NR, NP, false>(64, warp, 0);
-      else if (warp % 3 == 1)
-        lps_attend<CAP, NR, NP, false>(64, warp, 0);
-      else
-        lps_ffn<CAP, NR, NP, false>(64, warp, 0);
-    }
-  } else if (warm && run_lbs && nr > 0) {
-    lbs_input<NR, NP>(la);
-    lbs_qkv<NR, NP>(la, 0);
-  }
-
-  // ------------------------------------------------------------ statistics
-  // everything above overlaps the LM head's last CTAs; the partial states
-  // are read only after its grid completed.  A masked row is merged by the
-  // CTA that holds it in the LBS, the others are spread over the cluster.
-  if (p.features_in) {
+  if (kWide) {
+    if (p.lps_enabled) copy_lps();
+    // the statistics and the LBS logits of every row
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (tid < 8 * NR && sl.mrow[tid] >= 0) {
-      sl.ent[tid] = p.s_ent[r0 + sl.mrow[tid]];
-      sl.arg[tid] = p.s_arg[r0 + sl.mrow[tid]];
-    }
+    __syncthreads();
   } else {
-    bool waited = false;
-    // the first pass, it < 0, merges no states into a row of its own
-    for (int it = warm && nr + nu > 0 ? warp - kNW : warp; it < 8 * nr + nu; it += kNW) {
-      const bool real = it >= 0;
-      if (real && !waited) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        waited = true;
-      }
-      const int j = !real ? 0 : it < 8 * nr ? sl.mrow[it] : rs.urow[it - 8 * nr];
-      if (j < 0 || (real && !in_bounds(r0 + j, p.R, p.status))) continue;
-      const size_t base = static_cast<size_t>(r0 + j) * p.grid_lm;
-      const RowStats st = merge_row(p.part_f + base, p.part_i + base, real ? p.grid_lm : 0);
-      if (lane == 0) {
-        const int r = r0 + j, sr = real ? r : p.spare_row;
-        const float conf = 1.0f / st.s, ent = logf(st.s) - st.t * conf, entn = ent * p.inv_log_v;
-        const float gap = (1.0f - expf(st.l2 - st.m)) * conf;
-        const bool bad = !(isfinite(st.m) && isfinite(st.s) && isfinite(st.t) && st.s >= 1.0f) || st.idx < 0 ||
-                         st.idx >= p.V;
-        const int arg = bad ? -1 : st.idx;
-        p.s_conf[sr] = conf;
-        p.s_ent[sr] = entn;
-        p.s_gap[sr] = gap;
-        p.s_arg[sr] = arg;
-        if (real) {
-          if (p.conf) p.conf[r] = conf;
-          if (p.entropy) p.entropy[r] = ent;
-          if (p.ent_norm) p.ent_norm[r] = entn;
-          if (p.gap) p.gap[r] = gap;
-          if (p.argmax) p.argmax[r] = arg;
-          if (bad) atomicCAS(p.status, 0, EBD_ERR_NONFINITE);
-          if (it < 8 * nr) {
-            sl.ent[it] = entn;
-            sl.arg[it] = arg;
-          }
-        }
+    // Windows of up to 64 rows: CTA 0 makes the decision.  Eight CTAs with a
+    // group to spare leave all rows to the other seven, so that CTA 0 can bring
+    // in the LPS and its weights meanwhile.
+    const int groups = (nM + 7) >> 3;
+    const bool apart = C == 8 && groups < C;
+    const int nw = apart ? C - 1 : C, wk = apart ? rank - 1 : rank;
+    // group k of 8 rows of M belongs to worker k % nw, its slot k / nw; the
+    // statistics of the other rows are merged by the workers without a group
+    const int u0 = groups < nw ? groups : 0, nuw = nw - u0;
+    if (wk >= 0) {
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const int j = 32 * (warp + kNW * i) + lane, grp = mrank[i] >> 3;
+        if (m[i] && grp % nw == wk) sl.mrow[8 * (grp / nw) + (mrank[i] & 7)] = j;
+        if (f[i] && u0 + urank[i] % nuw == wk) rs.urow[urank[i] / nuw] = j;
       }
     }
-    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
-  }
-  __syncthreads();
+    const int nr = wk >= 0 && groups > wk ? (groups - wk + nw - 1) / nw : 0;  // groups of this CTA
+    const int nu = wk >= u0 && nU > wk - u0 ? (nU - (wk - u0) + nuw - 1) / nuw : 0;
+    const LbsArgs la{p.mat, p.vec, p.tok_table, p.kv, p.O, p.V, p.gen_len, p.cap_rows, kbase, capk, nM, nr, wk, nw};
+    __syncthreads();
 
-  // ------------------------------------------------------------ LBS
-  if (run_lbs) {
-    if (nr > 0) lbs_input<NR, NP>(la);
+    // The LM head has streamed its weight through L2: bring the router's back
+    // while its last CTAs run.
+    if (b == 0) {
+      const char* w = reinterpret_cast<const char*>(p.mat);
+      for (int i = (run_lbs ? 0 : M_BLOCK / 8) + rank * kT + tid; i < M_TOTAL / 8; i += C * kT)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 128 * static_cast<size_t>(i)));
+    }
+    // Launched behind the LM head, this grid waits some microseconds for its
+    // last CTAs, with code that no SM has cached (a first pass through it costs
+    // about as much again as the work itself, with the code out of L2 as well
+    // several times as much): meanwhile CTA 0 runs the LPS router, one part
+    // per warp, the others the LBS input layers and the first QKV product, on
+    // stand-in rows.
+    const bool warm = p.warm != 0 && C == 8 && p.mode == EBD_DECODE_EB;
+    if (apart && rank == 0 && p.lps_enabled) {
+      copy_lps();
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+      if (warm) {
+        if (warp % 3 == 0)
+          lps_qkv<CAP, NR, NP, false>(64, warp, 0);
+        else if (warp % 3 == 1)
+          lps_attend<CAP, NR, NP, false>(64, warp, 0);
+        else
+          lps_ffn<CAP, NR, NP, false>(64, warp, 0);
+      }
+    } else if (warm && run_lbs && nr > 0) {
+      lbs_input<NR, NP>(la);
+      lbs_qkv<NR, NP>(la, 0);
+    }
+
+    // ------------------------------------------------------------ statistics
+    // everything above overlaps the LM head's last CTAs; the partial states
+    // are read only after its grid completed.  A masked row is merged by the
+    // CTA that holds it in the LBS, the others are spread over the cluster.
+    if (p.features_in) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (tid < 8 * NR && sl.mrow[tid] >= 0) {
+        sl.ent[tid] = p.s_ent[r0 + sl.mrow[tid]];
+        sl.arg[tid] = p.s_arg[r0 + sl.mrow[tid]];
+      }
+    } else {
+      merge_rows<CAP>(p, sl, rs, r0, nr, nu, warm);
+    }
+    __syncthreads();
+
+    // ------------------------------------------------------------ LBS
+    if (run_lbs) {
+      if (nr > 0) lbs_input<NR, NP>(la);
 #pragma unroll 1
-    for (int l = 0; l < 2; ++l) {
-      if (nr > 0) lbs_qkv<NR, NP>(la, l);
-      cluster_barrier();  // every row's keys and values (l = 0: and statistics) are visible
-      if (nr > 0) lbs_layer<NR, NP>(la, l);
+      for (int l = 0; l < 2; ++l) {
+        if (nr > 0) lbs_qkv<NR, NP>(la, l);
+        cluster_barrier();  // every row's keys and values (l = 0: and statistics) are visible
+        if (nr > 0) lbs_layer<NR, NP>(la, l);
+      }
     }
-  }
-  cluster_barrier();  // every row's statistics and LBS logit are visible
+    cluster_barrier();  // every row's statistics and LBS logit are visible
 
-  if (!kWide && rank != 0) return;
-  if (!apart && p.lps_enabled) copy_lps();  // behind the selection, over the dead LBS activations
+    if (rank != 0) return;
+    if (!apart && p.lps_enabled) copy_lps();  // behind the selection, over the dead LBS activations
+  }
 
   // ------------------------------------------------------------ block selection
   // (Readings R8, R9)
@@ -1429,19 +1553,25 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 
 namespace {
 template <int C, int NR, int NP>
-constexpr int smem_bytes() {
-  return Lay<NR, NP>::ROW + static_cast<int>(sizeof(RowState<8 * NR * C>));
+constexpr int rows_cap() {
+  return NP == 3 ? kMaxSeqRows : 8 * NR * C;
 }
 template <int C, int NR, int NP>
+constexpr int smem_bytes() {
+  return Lay<NR, NP>::ROW + static_cast<int>(sizeof(RowState<rows_cap<C, NR, NP>()>));
+}
+constexpr int kWideSmem = Lay<1, 3>::ROW + static_cast<int>(sizeof(RowState<kMaxSeqRows>));
+
+template <int C, int NR, int NP>
 cudaError_t configure_one() {
-  cudaError_t e = cudaFuncSetAttribute(decide_rows_kernel<C, NR, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes<C, NR, NP>());
-  if (e == cudaSuccess && C > 8)
-    e = cudaFuncSetAttribute(decide_rows_kernel<C, NR, NP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  const auto k = decide_rows_kernel<C, NR, NP, rows_cap<C, NR, NP>()>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<C, NR, NP>());
+  if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 template <int C, int NR, int NP>
 cudaError_t launch_one(const RowsParams& p, cudaStream_t st, bool pdl, int* slots) {
+  const auto k = decide_rows_kernel<C, NR, NP, rows_cap<C, NR, NP>()>;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(slots != nullptr ? C : p.B * C));
   cfg.blockDim = dim3(kT);
@@ -1456,27 +1586,62 @@ cudaError_t launch_one(const RowsParams& p, cudaStream_t st, bool pdl, int* slot
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2 : 1;
-  if (slots != nullptr) return cudaOccupancyMaxActiveClusters(slots, decide_rows_kernel<C, NR, NP>, &cfg);
-  return cudaLaunchKernelEx(&cfg, decide_rows_kernel<C, NR, NP>, p);
+  if (slots != nullptr) return cudaOccupancyMaxActiveClusters(slots, k, &cfg);
+  return cudaLaunchKernelEx(&cfg, k, p);
+}
+cudaError_t launch_wide(void (*k)(RowsParams), const RowsParams& p, int groups, cudaStream_t st, bool pdl) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(groups), static_cast<unsigned>(p.B));
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = kWideSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, p);
 }
 }  // namespace
 
 cudaError_t decide_rows_configure(int (&slots)[2]) {
   cudaError_t e;
   const RowsParams none{};
+  const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if ((e = configure_one<8, 1, 2>()) != cudaSuccess || (e = configure_one<4, 2, 2>()) != cudaSuccess ||
       (e = configure_one<2, 4, 2>()) != cudaSuccess || (e = configure_one<4, 1, 2>()) != cudaSuccess ||
       (e = configure_one<2, 2, 2>()) != cudaSuccess || (e = configure_one<1, 4, 2>()) != cudaSuccess ||
-      (e = configure_one<16, 4, 3>()) != cudaSuccess ||
+      (e = configure_one<16, 1, 3>()) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(lbs_wide_kernel<0>, smem, kWideSmem)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(lbs_wide_kernel<1>, smem, kWideSmem)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(lbs_wide_kernel<2>, smem, kWideSmem)) != cudaSuccess ||
       (e = launch_one<8, 1, 2>(none, nullptr, false, &slots[0])) != cudaSuccess ||
       (e = launch_one<4, 2, 2>(none, nullptr, false, &slots[1])) != cudaSuccess)
     return e;
   return cudaSuccess;
 }
 
+// Clusters per sequence: as many CTAs as leave all sequences resident at once
+// (ebd_decide, us, 8 CTAs of one group / 4 of two / 2 of four: 8 x 64 rows 35
+// / 42 / 55, 16 x 64 49 / 41 / 55, 36 x 64 68 / 43 / 53, 40 x 64 68 / 66 / 53;
+// windows of up to 32 rows, 4 of one / 2 of two / 1 of four: 16 x 32 33 / 41 /
+// 53, 40 x 32 48 / 40 / 52, 128 x 32 98 / 73 / 54).
 cudaError_t launch_decide_rows(const RowsParams& p, int cap, const int (&slots)[2], cudaStream_t st, bool pdl) {
   if (p.B <= 0 || p.R <= 0) return cudaSuccess;
-  if (cap > 64) return launch_one<16, 4, 3>(p, st, pdl, nullptr);
+  if (cap > 64) {
+    cudaError_t e = cudaSuccess;
+    const bool lbs = p.mode == EBD_DECODE_EB;
+    // a sequence may bring more rows than announced, up to all of the step's
+    const int most = p.gen_len < p.R ? p.gen_len : p.R, groups = ((most < kMaxSeqRows ? most : kMaxSeqRows) + 7) / 8;
+    if (lbs || !p.features_in) {
+      if ((e = launch_wide(lbs_wide_kernel<0>, p, groups, st, pdl)) != cudaSuccess) return e;
+      pdl = true;
+    }
+    if (lbs && ((e = launch_wide(lbs_wide_kernel<1>, p, groups, st, true)) != cudaSuccess ||
+                (e = launch_wide(lbs_wide_kernel<2>, p, groups, st, true)) != cudaSuccess))
+      return e;
+    return launch_one<16, 1, 3>(p, st, pdl, nullptr);
+  }
   if (cap > 32) {
     if (p.B <= slots[0]) return launch_one<8, 1, 2>(p, st, pdl, nullptr);
     return p.B <= slots[1] ? launch_one<4, 2, 2>(p, st, pdl, nullptr) : launch_one<2, 4, 2>(p, st, pdl, nullptr);

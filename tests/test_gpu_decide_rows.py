@@ -1,9 +1,9 @@
 """The decision's launch shapes at their boundaries, on statistics given to
 ebd_decide: clusters of 8, 4 and 2 CTAs for windows of up to 64 rows (picked by
-the batch), of 4, 2 and 1 for up to 32 rows in batches of 16 and more, of 16
-above 64 rows; windows of a row, of whole groups of 8 rows and one more or one
-less, with nothing masked, and blocks of every masked row (the LPS over the
-whole window)."""
+the batch), of 4, 2 and 1 for up to 32 rows in batches of 16 and more; a CTA
+per group of 8 rows above 64 rows; windows of a row, of whole groups of 8 rows
+and one more or one less, with nothing masked, and blocks of every masked row
+(the LPS over the whole window)."""
 import dataclasses
 
 import numpy as np
