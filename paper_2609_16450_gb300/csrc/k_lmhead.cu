@@ -17,6 +17,18 @@
 // warp 1 issues tcgen05.mma, warps 2..5 (and 6..9) drain TMEM and run the
 // statistics.  Where the rows make the tensor cores the bound, CTA pairs run
 // cta_group::2 MMAs with M = 256 (two SMs, one accumulator tile).
+//
+// Warps 0 and 1 run their loops with all lanes and elect one for the copies
+// and the MMAs: addresses, descriptors and trip counts then are the same in
+// every lane and stay in uniform registers.  With lane 0 alone in the loop,
+// each stage cost its issuing thread some 450 cycles besides 62 per MMA (8
+// MMAs of N = 160: 946 cycles against the 640 they take; now 45 + 40 each).
+// LLaDA-8B, us, lane 0 alone / elected: 64 rows 153 / 150, 80 rows 158 / 152,
+// 153 rows 172 / 168, 512 rows 326 / 317, 2048 rows 1330 / 1290; Dream-7B step
+// over 312 rows 335 / 319.  What is left above 256 rows is W out of HBM (with
+// W in L2 the MMAs are busy 97 % of the time) and the clock, which the power
+// limit takes from 2.07 to 1.5 GHz; neither a TMA nor a plain prefetch of W
+// into L2 helps (512 rows 317 -> 340..385 us).
 #include <climits>
 #include <cstdlib>
 
@@ -297,7 +309,8 @@ __global__ void __launch_bounds__(kLmThreads, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       const uint64_t pol_w = l2_policy_evict_first();
       const uint64_t pol_h = l2_policy_evict_last();
       auto load = [&](void* dst, const CUtensorMap* map, int s, int x, int y, uint64_t pol) {
@@ -392,11 +405,13 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       int it = 0;
       {
         const int ks0 = ks;
-        for (; it < p.stages && u < u1; ++it, advance()) issue_w(u, ks, it);  // stages start empty
+        for (; it < p.stages && u < u1; ++it, advance())  // stages start empty
+          if (one) issue_w(u, ks, it);
+        __syncwarp();
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         for (int i = 0, hk = ks0; i < it; ++i) {
-          issue_h(hk, i);
+          if (one) issue_h(hk, i);
           if (++hk == p.nks) hk = 0;
         }
       }
@@ -404,18 +419,19 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       uint32_t ph = it == p.stages ? 1u : 0u;  // its phase parity
       bool ok = true;
       for (; u < u1; ++it, advance()) {
-        if (!mbar_wait(&empty[s], ph ^ 1u, p.limit_ns, abort)) {
-          ok = false;
-          break;
+        ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], ph ^ 1u, p.limit_ns, abort));
+        if (!ok) break;
+        if (one) {
+          issue_w(u, ks, s);
+          issue_h(ks, s);
         }
-        issue_w(u, ks, s);
-        issue_h(ks, s);
+        __syncwarp();
         if (++s == p.stages) {
           s = 0;
           ph ^= 1u;
         }
       }
-      if (!ok) {
+      if (!ok && one) {
         if (!*abort) record_error(p.status, abort, EBD_ERR_TIMEOUT);
         if (leader) {
           // let the copies already in flight land before the CTA can exit
@@ -432,11 +448,13 @@ __global__ void __launch_bounds__(kLmThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && leader) {
+    if (leader) {
       const uint32_t idesc = umma_idesc_bf16(PAIR ? 256 : 128, static_cast<uint32_t>(p.nb));
       const uint32_t desc_hi = static_cast<uint32_t>(umma_desc_sw128(0) >> 32);
-      int it = 0, c = 0;
-      int s = 0;        // stage of iteration it, as in the producer
+      const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
+      const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+      int c = 0;
+      int s = 0;        // stage, as in the producer
       uint32_t ph = 0;
       bool ok = true;
       auto commit_stage = [&](int st) {
@@ -448,87 +466,91 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       for (int u = u0; u < u1 && ok; u += kChunkUnits, ++c) {
         const int buf = c % p.nbuf;
         const uint32_t bph = static_cast<uint32_t>(c / p.nbuf) & 1u;
-        if (!mbar_wait(&acc_empty[buf], bph ^ 1u, p.limit_ns, abort)) {
-          ok = false;
-          break;
-        }
+        ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[buf], bph ^ 1u, p.limit_ns, abort));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d0 = tmem_base + static_cast<uint32_t>(buf * p.acc_stride);
+        const uint32_t d0 = tmem_u + static_cast<uint32_t>(buf * p.acc_stride);
         for (int ks = 0; ks < p.nks; ++ks) {
-          if (!mbar_wait(&full[s], ph, p.limit_ns, abort)) {
-            ok = false;
-            break;
-          }
+          ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.limit_ns, abort));
+          if (!ok) break;
           tc_fence_after();
           const int nsubk = min(p.kbs, p.nkb - ks * p.kbs);
-          const uint32_t a_addr = smem_u32(sA + static_cast<size_t>(s) * a_stage);
-          const uint32_t b_addr = smem_u32(sB + static_cast<size_t>(s) * b_stage);
-          if ((PAIR || p.nsub <= 2) && nsubk >= 1 && nsubk <= 5) {
-            // the unrolled issue path
-            const uint32_t a_lo = static_cast<uint32_t>(umma_desc_sw128(a_addr));
-            const uint32_t b_lo = static_cast<uint32_t>(umma_desc_sw128(b_addr));
-            const uint32_t b_step = b_sub >> 4;
-            const uint32_t sub_desc = static_cast<uint32_t>(hrows) * 8u;  // hrows x 128 B >> 4
-            const uint32_t sub_cols = static_cast<uint32_t>(p.nb);
-            const uint32_t acc0 = ks != 0 ? 1u : 0u;
+          const uint32_t a_addr = a_base + static_cast<uint32_t>(s) * a_stage;
+          const uint32_t b_addr = b_base + static_cast<uint32_t>(s) * b_stage;
+          if (elect_one()) {
+            if ((PAIR || p.nsub <= 2) && nsubk >= 1 && nsubk <= 5) {
+              // the unrolled issue path
+              const uint32_t a_lo = static_cast<uint32_t>(umma_desc_sw128(a_addr));
+              const uint32_t b_lo = static_cast<uint32_t>(umma_desc_sw128(b_addr));
+              const uint32_t b_step = b_sub >> 4;
+              const uint32_t sub_desc = static_cast<uint32_t>(hrows) * 8u;  // hrows x 128 B >> 4
+              const uint32_t sub_cols = static_cast<uint32_t>(p.nb);
+              const uint32_t acc0 = ks != 0 ? 1u : 0u;
 #define EBD_STAGE(K, S) \
-  mma_stage<K, S, PAIR>(d0, a_lo, b_lo, b_step, sub_desc, sub_cols, desc_hi, idesc, acc0)
-            if (PAIR || p.nsub == 1) {
-              switch (nsubk) {
-                case 1: EBD_STAGE(1, 1); break;
-                case 2: EBD_STAGE(2, 1); break;
-                case 3: EBD_STAGE(3, 1); break;
-                case 4: EBD_STAGE(4, 1); break;
-                default: EBD_STAGE(5, 1); break;
+    mma_stage<K, S, PAIR>(d0, a_lo, b_lo, b_step, sub_desc, sub_cols, desc_hi, idesc, acc0)
+              if (PAIR || p.nsub == 1) {
+                switch (nsubk) {
+                  case 1: EBD_STAGE(1, 1); break;
+                  case 2: EBD_STAGE(2, 1); break;
+                  case 3: EBD_STAGE(3, 1); break;
+                  case 4: EBD_STAGE(4, 1); break;
+                  default: EBD_STAGE(5, 1); break;
+                }
+              } else {
+                switch (nsubk) {
+                  case 1: EBD_STAGE(1, 2); break;
+                  case 2: EBD_STAGE(2, 2); break;
+                  case 3: EBD_STAGE(3, 2); break;
+                  case 4: EBD_STAGE(4, 2); break;
+                  default: EBD_STAGE(5, 2); break;
+                }
               }
-            } else {
-              switch (nsubk) {
-                case 1: EBD_STAGE(1, 2); break;
-                case 2: EBD_STAGE(2, 2); break;
-                case 3: EBD_STAGE(3, 2); break;
-                case 4: EBD_STAGE(4, 2); break;
-                default: EBD_STAGE(5, 2); break;
-              }
-            }
 #undef EBD_STAGE
-          } else {
-            for (int j = 0; j < nsubk; ++j) {
+            } else {
+              for (int j = 0; j < nsubk; ++j) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t ad = umma_desc_sw128(a_addr + j * kATile + kk * 32);
-                for (int sb = 0; sb < p.nsub; ++sb) {
-                  const uint64_t bd = umma_desc_sw128(b_addr + j * b_sub + sb * hrows * 128 + kk * 32);
-                  const uint32_t acc = (ks | j | kk) != 0 ? 1u : 0u;
-                  const uint32_t dd = d0 + static_cast<uint32_t>(sb * p.nb);
-                  if (PAIR)
-                    umma_bf16_lo_pair(dd, static_cast<uint32_t>(ad), static_cast<uint32_t>(bd),
-                                      desc_hi, idesc, acc);
-                  else
-                    umma_bf16(dd, ad, bd, idesc, acc);
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t ad = umma_desc_sw128(a_addr + j * kATile + kk * 32);
+                  for (int sb = 0; sb < p.nsub; ++sb) {
+                    const uint64_t bd = umma_desc_sw128(b_addr + j * b_sub + sb * hrows * 128 + kk * 32);
+                    const uint32_t acc = (ks | j | kk) != 0 ? 1u : 0u;
+                    const uint32_t dd = d0 + static_cast<uint32_t>(sb * p.nb);
+                    if (PAIR)
+                      umma_bf16_lo_pair(dd, static_cast<uint32_t>(ad), static_cast<uint32_t>(bd),
+                                        desc_hi, idesc, acc);
+                    else
+                      umma_bf16(dd, ad, bd, idesc, acc);
+                  }
                 }
               }
             }
+            commit_stage(s);
           }
-          commit_stage(s);
-          ++it;
+          __syncwarp();
           if (++s == p.stages) {
             s = 0;
             ph ^= 1u;
           }
         }
         if (!ok) break;
-        if (PAIR)
-          umma_commit_pair_mc(&acc_full[buf], 0x3);
-        else
-          umma_commit(&acc_full[buf]);
+        if (elect_one()) {
+          if (PAIR)
+            umma_commit_pair_mc(&acc_full[buf], 0x3);
+          else
+            umma_commit(&acc_full[buf]);
+        }
+        __syncwarp();
       }
       if (!ok) {
-        if (!*abort) record_error(p.status, abort, EBD_ERR_TIMEOUT);
+        if (lane == 0 && !*abort) record_error(p.status, abort, EBD_ERR_TIMEOUT);
         // completes once every MMA issued so far is done
-        if (PAIR)
-          umma_commit_pair(drain);
-        else
-          umma_commit(drain);
+        if (elect_one()) {
+          if (PAIR)
+            umma_commit_pair(drain);
+          else
+            umma_commit(drain);
+        }
+        __syncwarp();
         mbar_wait(drain, 0, p.limit_ns, nullptr);
       }
     }
@@ -689,14 +711,13 @@ void lm_plan(LmParams& p, int rows, int V, int d, int num_sms, bool pair) {
   const uint32_t b_box = static_cast<uint32_t>(pair ? p.n_pad / 2 : p.n_pad) * 128u;
   // k-boxes (64 columns each) per pipeline stage, while keeping at least two
   // stages in flight.  Unpaired (few rows, HBM bound): up to 5, for longer
-  // contiguous runs of each W row per request.  Paired: three stages of two
-  // k-boxes fit at N = 256, and more of them below; three k-boxes (still
-  // three stages) up to N = 96.  Measured (LLaDA-8B, packed W, us at 1 / 2 /
-  // 3 / 4 k-boxes): 80 rows 191 / 162 / 160 / 164, 128 rows 193 / 164 / 183 /
-  // 168, 153 rows 197 / 175 / 189 / 190, 256 rows 214 / 201 / 219 / 226, 512
-  // rows 371 / 323 / 352 / 352.  One k-box pays a barrier round trip and a
-  // commit per 64 columns; four leave two stages in flight.
-  int kbs = !pair ? 5 : p.n_pad <= 96 ? 3 : 2;
+  // contiguous runs of each W row per request.  Paired: two, i.e. three stages
+  // at N = 256 and more below.  Measured (LLaDA-8B, packed W, us at 1 / 2 / 3 /
+  // 4 k-boxes): 80 rows 160 / 152 / 152 / 156, 128 rows 163 / 154 / 174 / 163,
+  // 153 rows 170 / 168 / 186 / 185, 256 rows 205 / 200 / 232 / 239, 512 rows
+  // 349 / 326 / 411 / 411.  One k-box takes twice the copies, each of half the
+  // size; four leave two stages in flight.
+  int kbs = pair ? 2 : 5;
   if (const char* env = getenv("EBD_LM_KBS")) kbs = atoi(env);
   if (kbs < 1) kbs = 1;
   if (kbs > 5) kbs = 5;
