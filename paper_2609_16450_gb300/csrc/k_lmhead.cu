@@ -2,7 +2,7 @@
 //
 // For each window row r and vocabulary entry v the logit is
 // l[r][v] = sum_k h[r][k] W[v][k]; the kernel never stores it.  Each CTA owns a
-// contiguous range of 64-row vocabulary units and keeps, per window row, the
+// share of the 64-row vocabulary units and keeps, per window row, the
 // online-softmax state over the vocabulary it has seen:
 //   m  = max logit,  S = sum exp(l - m),  T = sum exp(l - m) (l - m),
 //   l2 = second largest logit (duplicates count),  idx = argmax (lowest).
@@ -299,8 +299,18 @@ __global__ void __launch_bounds__(kLmThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
 
-  const int u0 = static_cast<int>((static_cast<long long>(owner) * p.n_units) / p.nwork);
-  const int u1 = static_cast<int>((static_cast<long long>(owner + 1) * p.n_units) / p.nwork);
+  // The owner's vocabulary chunks: a contiguous range of the units, or, from
+  // a row-major W of six chunks per owner and more, every nwork-th chunk.  A
+  // stage reads 256 bytes of each of its rows there, and owners on adjacent
+  // rows keep fewer memory pages open: LLaDA-8B (6.5 or 7 chunks per owner) 32
+  // rows 156 -> 154 us, 80 rows 170 -> 160, 153 rows 186 -> 174, 256 rows 216 ->
+  // 209, 512 rows as before.  With fewer chunks the uneven last one would
+  // weigh more.  Packed tiles are contiguous by themselves (80 rows 152 -> 153
+  // us; Dream-7B 32 rows 159 -> 161 us).
+  const bool spread = !PACKED && p.n_units >= 6 * kChunkUnits * p.nwork;
+  const int ustep = spread ? kChunkUnits * p.nwork : kChunkUnits;
+  const int u0 = spread ? kChunkUnits * owner : static_cast<int>((static_cast<long long>(owner) * p.n_units) / p.nwork);
+  const int u1 = spread ? p.n_units : static_cast<int>((static_cast<long long>(owner + 1) * p.n_units) / p.nwork);
   const uint32_t b_sub = static_cast<uint32_t>(p.nsub * hrows) * 128u;  // one k-box of hidden rows here
   const uint32_t a_stage = static_cast<uint32_t>(p.kbs) * kATile;
   const uint32_t b_stage = static_cast<uint32_t>(p.kbs) * b_sub;
@@ -389,7 +399,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
       auto advance = [&]() {
         if (++ks == p.nks) {
           ks = 0;
-          u += kChunkUnits;
+          u += ustep;
         }
       };
       // The first stages' W go out before anything else.  As a programmatic
@@ -463,7 +473,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
         else
           umma_commit(&empty[st]);
       };
-      for (int u = u0; u < u1 && ok; u += kChunkUnits, ++c) {
+      for (int u = u0; u < u1 && ok; u += ustep, ++c) {
         const int buf = c % p.nbuf;
         const uint32_t bph = static_cast<uint32_t>(c / p.nbuf) & 1u;
         ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[buf], bph ^ 1u, p.limit_ns, abort));
@@ -580,7 +590,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
         mbar_arrive(&acc_empty[buf]);
     };
     int c = 0;
-    for (int u = u0; u < u1 && ok; u += kChunkUnits, ++c) {
+    for (int u = u0; u < u1 && ok; u += ustep, ++c) {
       const int nu = min(kChunkUnits, u1 - u);
       const int buf = c % p.nbuf;
       const uint32_t bph = static_cast<uint32_t>(c / p.nbuf) & 1u;

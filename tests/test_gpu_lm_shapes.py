@@ -89,3 +89,12 @@ def test_paired_stage_boxes(rows, layout, d_model):
     so the hidden rows (and a row-major W) come in one box per k-box."""
     rep = _run(_shape(rows, 4000).with_(d_model=d_model), layout)
     assert rep["conf"] <= 2e-3
+
+
+@pytest.mark.parametrize("rows", [40, 100, 300])
+@pytest.mark.parametrize("units", [1823, 1825])
+def test_spread_vocabulary_chunks(rows, units):
+    """A row-major W of six chunks and more per owner (from 1824 units on for
+    76 pairs): every nwork-th chunk, the last one of a single row."""
+    rep = _run(_shape(rows, (units - 1) * 64 + 1).with_(d_model=128), "rowmajor")
+    assert rep["conf"] <= 2e-3
