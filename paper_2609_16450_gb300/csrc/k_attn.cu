@@ -650,7 +650,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
     // as soon as a slot is free.  A step's second chunk past the split's end
     // is a load from beyond the cache, which TMA fills with zeros (finite V
     // for the masked keys).
-    if (lane == 0 && nst > 0) {
+    if (nst > 0) {
       const bool is_k = warp == 0;
       const CUtensorMap* mc = is_k ? &tm_kc : &tm_vc;
       const CUtensorMap* mw = is_k ? &tm_kw : &tm_vw;
@@ -661,9 +661,11 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
       int n = 0;
       for (; n < nst; ++n) {
         const int s = n % kTcRing;
-        if (n >= kTcRing &&
-            !mbar_wait(&emptyb[s], static_cast<uint32_t>(n / kTcRing - 1) & 1u, p.limit_ns, abort))
+        if (n >= kTcRing && !__all_sync(0xffffffffu, mbar_wait(&emptyb[s], static_cast<uint32_t>(n / kTcRing - 1) & 1u,
+                                                               p.limit_ns, abort)))
           break;
+        __syncwarp();
+        if (!elect_one()) continue;
         uint64_t* bar = &fullb[s];
         mbar_arrive_expect_tx(bar, 2u * NB * L::kBox);
 #pragma unroll
@@ -685,7 +687,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
         }
       }
       if (n < nst) {
-        if (!*abort) {
+        if (lane == 0 && !*abort) {
           *abort = 1;
           atomicCAS(p.status, 0, EBD_ERR_TIMEOUT);
         }
@@ -696,7 +698,9 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA thread
-    if (lane == 0 && nst > 0) {
+    // (all lanes in the loop, one elected for the MMAs)
+    if (nst > 0) {
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
       const uint32_t idesc_s = umma_idesc_bf16(128, 128);
       const uint32_t idesc_o = umma_idesc_bf16(128, D) | (1u << 16);  // B (V) MN-major
       // descriptors as 32-bit low words (start address >> 4, leading byte
@@ -711,51 +715,56 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
       // softmax has read S(j - 2) out of that buffer
       auto qk = [&](int j) -> bool {
         const int s = j % kTcRing;
-        if (!mbar_wait(&kfull[s], static_cast<uint32_t>(j / kTcRing) & 1u, p.limit_ns, abort))
-          return false;
-        if (j >= 2 && !mbar_wait(&s_free[j & 1], static_cast<uint32_t>((j - 2) >> 1) & 1u,
-                                 p.limit_ns, abort))
-          return false;
+        bool w = mbar_wait(&kfull[s], static_cast<uint32_t>(j / kTcRing) & 1u, p.limit_ns, abort);
+        if (j >= 2)
+          w = w && mbar_wait(&s_free[j & 1], static_cast<uint32_t>((j - 2) >> 1) & 1u, p.limit_ns, abort);
+        if (!__all_sync(0xffffffffu, w)) return false;
         tc_fence_after();
         const uint32_t k_lo = k0_lo + static_cast<uint32_t>(s) * (L::kStep >> 4);
-        const uint32_t d = tmem + static_cast<uint32_t>((j & 1) * 128);
+        const uint32_t d = tm + static_cast<uint32_t>((j & 1) * 128);
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk)
-          umma_bf16_lo(d, q_lo + static_cast<uint32_t>((kk >> 2) * (16384 >> 4) + (kk & 3) * 2),
-                       k_lo + static_cast<uint32_t>((kk >> 2) * (16384 >> 4) + (kk & 3) * 2),
-                       desc_hi, idesc_s, kk > 0 ? 1u : 0u);
-        umma_commit(&s_full[j & 1]);
-        umma_commit(&kempty[s]);
+          for (int kk = 0; kk < D / 16; ++kk)
+            umma_bf16_lo(d, q_lo + static_cast<uint32_t>((kk >> 2) * (16384 >> 4) + (kk & 3) * 2),
+                         k_lo + static_cast<uint32_t>((kk >> 2) * (16384 >> 4) + (kk & 3) * 2),
+                         desc_hi, idesc_s, kk > 0 ? 1u : 0u);
+          umma_commit(&s_full[j & 1]);
+          umma_commit(&kempty[s]);
+        }
+        __syncwarp();
         return true;
       };
-      bool ok = mbar_wait(q_ready, 0, p.limit_ns, abort);
+      bool ok = __all_sync(0xffffffffu, mbar_wait(q_ready, 0, p.limit_ns, abort));
       for (int j = 0; j < 2 && j < nst && ok; ++j) ok = qk(j);
       for (int i = 0; i < nst && ok; ++i) {
         const int s = i % kTcRing;
-        if (!mbar_wait(p_full, static_cast<uint32_t>(i) & 1u, p.limit_ns, abort) ||
-            !mbar_wait(&vfull[s], static_cast<uint32_t>(i / kTcRing) & 1u, p.limit_ns, abort)) {
-          ok = false;
-          break;
-        }
+        ok = __all_sync(0xffffffffu,
+                        mbar_wait(&vfull[s], static_cast<uint32_t>(i / kTcRing) & 1u, p.limit_ns, abort) &&
+                            mbar_wait(p_full, static_cast<uint32_t>(i) & 1u, p.limit_ns, abort));
+        if (!ok) break;
         tc_fence_after();
         const uint32_t v_lo = v0_lo + static_cast<uint32_t>(s) * (L::kStep >> 4);
-        const uint32_t d = tmem + 256u;
+        const uint32_t d = tm + 256u;
         const uint32_t acc0 = i != 0 ? 1u : 0u;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kTcKeys / 16; ++kk)  // 16 keys per k-step
-          umma_bf16_lo(d, p_lo + static_cast<uint32_t>((kk >> 2) * (16384 >> 4) + (kk & 3) * 2),
-                       v_lo + static_cast<uint32_t>(kk * (2048 >> 4)), desc_hi, idesc_o,
-                       kk != 0 ? 1u : acc0);
-        umma_commit(pv_done);
-        umma_commit(&vempty[s]);
+          for (int kk = 0; kk < kTcKeys / 16; ++kk)  // 16 keys per k-step
+            umma_bf16_lo(d, p_lo + static_cast<uint32_t>((kk >> 2) * (16384 >> 4) + (kk & 3) * 2),
+                         v_lo + static_cast<uint32_t>(kk * (2048 >> 4)), desc_hi, idesc_o,
+                         kk != 0 ? 1u : acc0);
+          umma_commit(pv_done);
+          umma_commit(&vempty[s]);
+        }
+        __syncwarp();
         if (i + 2 < nst) ok = qk(i + 2);
       }
       if (!ok) {
-        if (!*abort) {
+        if (lane == 0 && !*abort) {
           *abort = 1;
           atomicCAS(p.status, 0, EBD_ERR_TIMEOUT);
         }
-        umma_commit(drain);  // completes once every MMA issued so far is done
+        if (elect_one()) umma_commit(drain);  // completes once every MMA issued so far is done
+        __syncwarp();
         mbar_wait(drain, 0, p.limit_ns, nullptr);
       }
     }
