@@ -505,22 +505,27 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   const uint64_t Pm = static_cast<uint64_t>(c.max_prefix > 0 ? c.max_prefix : 1);
   const void* kcp = c.max_prefix > 0 ? a->k_cache : a->k_win;  // any valid pointer if no cache
   const void* vcp = c.max_prefix > 0 ? a->v_cache : a->v_win;
-  {
-    const uint64_t dims[4] = {static_cast<uint64_t>(D), static_cast<uint64_t>(Hkv), Pm,
-                              static_cast<uint64_t>(c.max_prefix > 0 ? a->batch : 1)};
-    const uint64_t str[3] = {static_cast<uint64_t>(D) * 2, static_cast<uint64_t>(Hkv) * D * 2,
-                             Pm * Hkv * D * 2};
-    const uint32_t box[4] = {64, 1, 64, 1};
-    if (!encode_bf16(&kc, kcp, 4, dims, str, box) || !encode_bf16(&vc, vcp, 4, dims, str, box))
-      return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (K/V cache) failed");
+  const uint64_t Bc = static_cast<uint64_t>(c.max_prefix > 0 ? a->batch : 1);
+  const uint64_t H = static_cast<uint64_t>(Hkv), NB = static_cast<uint64_t>(D) / 64;
+  const uint64_t head = static_cast<uint64_t>(D) * 2, row = H * head;  // bytes
+  // boxes of 64 keys: 64 dims for the tcgen05 kernel (dim, head, key(, sequence)),
+  // all dims of a head for the mma.sync kernel, half by half (dim of the half,
+  // key, half, head(, sequence))
+  bool ok;
+  if (h->attn_tc) {
+    const uint64_t cdims[4] = {static_cast<uint64_t>(D), H, Pm, Bc}, wdims[3] = {static_cast<uint64_t>(D), H, R};
+    const uint64_t cstr[3] = {head, row, Pm * row}, wstr[2] = {head, row};
+    const uint32_t cbox[4] = {64, 1, 64, 1}, wbox[3] = {64, 1, 64};
+    ok = encode_bf16(&kc, kcp, 4, cdims, cstr, cbox) && encode_bf16(&vc, vcp, 4, cdims, cstr, cbox) &&
+         encode_bf16(&kw, a->k_win, 3, wdims, wstr, wbox) && encode_bf16(&vw, a->v_win, 3, wdims, wstr, wbox);
+  } else {
+    const uint64_t cdims[5] = {64, Pm, NB, H, Bc}, wdims[4] = {64, R, NB, H};
+    const uint64_t cstr[4] = {row, 128, head, Pm * row}, wstr[3] = {row, 128, head};
+    const uint32_t cbox[5] = {64, 64, static_cast<uint32_t>(NB), 1, 1}, wbox[4] = {64, 64, static_cast<uint32_t>(NB), 1};
+    ok = encode_bf16(&kc, kcp, 5, cdims, cstr, cbox) && encode_bf16(&vc, vcp, 5, cdims, cstr, cbox) &&
+         encode_bf16(&kw, a->k_win, 4, wdims, wstr, wbox) && encode_bf16(&vw, a->v_win, 4, wdims, wstr, wbox);
   }
-  {
-    const uint64_t dims[3] = {static_cast<uint64_t>(D), static_cast<uint64_t>(Hkv), R};
-    const uint64_t str[2] = {static_cast<uint64_t>(D) * 2, static_cast<uint64_t>(Hkv) * D * 2};
-    const uint32_t box[3] = {64, 1, 64};
-    if (!encode_bf16(&kw, a->k_win, 3, dims, str, box) || !encode_bf16(&vw, a->v_win, 3, dims, str, box))
-      return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (window K/V) failed");
-  }
+  if (!ok) return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (K/V) failed");
   AttnParams p{};
   p.B = a->batch;
   p.R = a->rows;

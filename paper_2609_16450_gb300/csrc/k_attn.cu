@@ -202,19 +202,14 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
     uint8_t* kd = smem + s * kStageBytes;
     uint8_t* vd = kd + NH * 8192;
     mbar_arrive_expect_tx(&full[s], 2u * NH * 8192u);
-#pragma unroll
-    for (int hf = 0; hf < NH; ++hf) {
-      if (c < ncc) {
-        tma_load_4d(kd + hf * 8192, &tm_kc, &full[s], hf * 64, g, c * kAttnChunk, b);
-        tma_load_4d(vd + hf * 8192, &tm_vc, &full[s], hf * 64, g, c * kAttnChunk, b);
-      } else if (c == ncc) {
-        tma_load_3d(kd + hf * 8192, &tm_kw, &full[s], hf * 64, g, r0);
-        tma_load_3d(vd + hf * 8192, &tm_vw, &full[s], hf * 64, g, r0);
-      } else {
-        const int y = S0 + (c - ncc - 1) * kAttnChunk;
-        tma_load_4d(kd + hf * 8192, &tm_kc, &full[s], hf * 64, g, y, b);
-        tma_load_4d(vd + hf * 8192, &tm_vc, &full[s], hf * 64, g, y, b);
-      }
+    // one copy each for K and V, both 64-dim halves
+    if (c == ncc) {
+      tma_load_4d(kd, &tm_kw, &full[s], 0, r0, 0, g);
+      tma_load_4d(vd, &tm_vw, &full[s], 0, r0, 0, g);
+    } else {
+      const int y = c < ncc ? c * kAttnChunk : S0 + (c - ncc - 1) * kAttnChunk;
+      tma_load_5d(kd, &tm_kc, &full[s], 0, y, 0, g, b);
+      tma_load_5d(vd, &tm_vc, &full[s], 0, y, 0, g, b);
     }
   };
   if (tid == 0)
