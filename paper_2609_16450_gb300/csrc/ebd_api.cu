@@ -239,6 +239,7 @@ struct ebd_handle {
   float* attn_part_ml = nullptr;
   int* tickets = nullptr;
   int attn_splits = 1, attn_max_qtiles = 1;
+  int attn_stages = kAttnStages;
   int attn_tc = 1;         // window attention on tcgen05 (else the mma.sync kernel)
   int* d_status = nullptr;
   uint8_t* staging = nullptr;
@@ -536,6 +537,7 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   p.max_prefix = c.max_prefix;
   p.max_qtiles = h->attn_max_qtiles;
   p.splits = h->attn_splits;
+  p.stages = h->attn_stages;
   p.tc = h->attn_tc;
   p.cu_rows = a->cu_rows;
   p.prefix_len = a->prefix_len;
@@ -814,18 +816,18 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     // Both attention kernels take 64-row query tiles.  The tcgen05 kernel
     // holds an SM alone (one CTA per SM) and pays a fixed setup and drain
     // per CTA (TMEM, barriers, the query tile, its output), which long key
-    // ranges amortise; the mma.sync kernel runs two CTAs per SM, and with
-    // tiles of up to 32 rows it reads the cache as fast, its warps sharing
-    // each chunk's keys.  So, measured (attention alone, LLaDA-8B heads, us,
-    // mma.sync against tcgen05 in the better of their split counts):
-    //   more tiles than SMs: 64 x 1024 x 32 rows 190 / 235, 64 x 4096 x 32
-    //     637 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 58 / 53; but tiles
-    //     of 33 to 64 rows over 1024 keys and more 92 / 78 (16 x 1024 x 64),
-    //     1069 / 711 (64 x 4096 x 64), below that 113 / 150 (64 x 256 x 64);
+    // ranges amortise; the mma.sync kernel runs two or three CTAs per SM, and
+    // with tiles of up to 32 rows it reads the cache as fast, its warps
+    // sharing each chunk's keys.  So, measured (attention alone, LLaDA-8B
+    // heads, us, mma.sync against tcgen05 in the better of their splits):
+    //   more tiles than SMs: 64 x 1024 x 32 rows 183 / 228, 64 x 4096 x 32
+    //     630 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 44 / 53; but tiles
+    //     of 33 to 64 rows over 1024 keys and more 103 / 74 (16 x 1024 x 64),
+    //     1087 / 653 (64 x 4096 x 64), below that 117 / 150 (64 x 256 x 64);
     //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
-    //     47.5, 1 x 4096 x 32 26.5 / 20.7; but at 256 keys 10.8 / 12.2.
-    // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count
-    // (measurement sweeps).
+    //     47, 1 x 4096 x 32 26.5 / 21; but at 256 keys 10.8 / 12.2.
+    // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count,
+    // EBD_ATTN_STAGES the ring's stages (measurement sweeps).
     const int tile = 64;
     const int group = cfg->n_heads_q / cfg->n_heads_kv;
     const int aw = cfg->max_window < kMaxWindow ? cfg->max_window : kMaxWindow;
@@ -840,16 +842,21 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     // x 8 rows on tcgen05 28.7 us with 5 splits, 18.7 with 4)
     int splits = (h->attn_tc ? h->num_sms : 2 * h->num_sms) / slots;
     if (splits > nch / 4) splits = nch / 4;
-    // a little more than a wave of long ranges: half-length CTAs (10 x 4096
-    // x 8 rows 145 -> 130 us, 12 x 4096 x 32 183 -> 158)
-    const int wave = 2 * h->num_sms;
-    if (!h->attn_tc && nch >= 33 && slots > wave && 2 * ((slots + wave - 1) / wave) > (2 * slots + wave - 1) / wave)
-      splits = 2;
     if (const char* env = getenv("EBD_ATTN_SPLITS")) splits = atoi(env);
     if (splits > kMaxSplits) splits = kMaxSplits;
     if (splits > nch) splits = nch;
     if (splits < 1) splits = 1;
     h->attn_splits = splits;
+    // CTAs per SM of the mma.sync kernel: two with a ring of three stages or
+    // three with two.  Three hide more of the CTAs' starts and ends and of the
+    // work between copies (us, two / three: 10 x 1024 x 8 rows 45 / 33, 12 x
+    // 4096 x 8 146 / 122, 24 x 1024 x 32 86 / 79, 64 x 256 x 32 81 / 69, 64 x
+    // 1024 x 32 193 / 183), but a wave of them takes longer: two where three
+    // would leave a last wave too empty (16 x 1024 x 8, 512 CTAs, 50 / 60; but
+    // 32 x 1024 x 8, 1024 CTAs, 94 / 95, x 32 rows 111 / 106).
+    auto waves = [&](int per_sm) { return (slots * splits + per_sm * h->num_sms - 1) / (per_sm * h->num_sms); };
+    h->attn_stages = 6 * waves(3) <= 5 * waves(2) ? 2 : kAttnStages;
+    if (const char* env = getenv("EBD_ATTN_STAGES")) h->attn_stages = atoi(env) == 2 ? 2 : kAttnStages;
     if (splits > 1) {
       const size_t bytes = static_cast<size_t>(slots) * splits * tile * (cfg->head_dim + 2) * 4;
       if ((e = cudaMalloc(&h->attn_part, bytes)) != cudaSuccess)

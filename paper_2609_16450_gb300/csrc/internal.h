@@ -36,7 +36,7 @@ constexpr int kMaxGroupRows = 512;    // rows per LM-head launch (TMEM: 512 colu
 constexpr int kRowsThreads = 256;
 constexpr int kAttnThreads = 128;
 constexpr int kAttnChunk = 64;        // keys per K/V tile
-constexpr int kAttnStages = 3;
+constexpr int kAttnStages = 3;        // at most
 constexpr int kMaxAttnSplits = 8;
 constexpr int kAttnTcThreads = 352;   // tcgen05 attention: K and V load warps, MMA warp, 8 softmax warps
 constexpr int kAttnTcRows = 64;       // query rows per tile of the tcgen05 attention
@@ -47,6 +47,7 @@ struct AttnParams {
   int R;                    // rows of the step (extent of q and out)
   int max_prefix;
   int max_qtiles, splits;
+  int stages;               // ring of the mma.sync kernel: kAttnStages, or 2 for three CTAs per SM
   int tc;                   // 1: the tcgen05 kernel, 0: the mma.sync kernel (64-row tiles)
   const int* cu_rows;
   const int* prefix_len;

@@ -13,8 +13,8 @@
 // a bf16 remainder, so that P V keeps ~16 mantissa bits.
 //   attn_tc_kernel: the 5th-generation tensor cores (S and O in TMEM); one
 //     CTA per SM; for long key ranges and launches of few tiles.
-//   attn_kernel: mma.sync, 4 warps of 16 query rows, a 3-stage K/V ring, two
-//     CTAs per SM; for launches of many tiles with short key ranges, where
+//   attn_kernel: mma.sync, 4 warps of 16 query rows, a K/V ring of two stages
+//     and three CTAs per SM, or of three and two; for launches of many tiles with short key ranges, where
 //     the tcgen05 kernel's per-CTA setup does not amortise.
 #include <type_traits>
 
@@ -27,7 +27,7 @@ namespace {
 
 // a stage of the mma.sync kernel: a chunk's K and V, 64-dim halves
 constexpr int attn_stage_bytes(int D) { return 2 * (D / 64) * 8192; }
-constexpr int attn_smem_bytes(int D) { return kAttnStages * attn_stage_bytes(D) + 1024 + 64; }
+constexpr int attn_smem_bytes(int D, int stages) { return stages * attn_stage_bytes(D) + 1024 + 64; }
 
 // byte offset of 16-byte chunk `c` (0..7) of row `r` in a 128B-swizzled tile
 __device__ __forceinline__ uint32_t swz(int r, int c) {
@@ -165,7 +165,7 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kAttnStages * kStageBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * kStageBytes);
   __shared__ int s_flag;
 
   const int split = blockIdx.x, qt = blockIdx.y, bg = blockIdx.z;
@@ -190,14 +190,13 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int s = 0; s < kAttnStages; ++s) mbar_init(&full[s], 1);
+    for (int s = 0; s < p.stages; ++s) mbar_init(&full[s], 1);
     fence_mbar_init();
     s_flag = 0;
   }
   __syncthreads();
 
-  auto issue = [&](int i) {
-    const int s = i % kAttnStages;
+  auto issue = [&](int i, int s) {  // chunk i of this split into stage s
     const int c = c0 + i;
     uint8_t* kd = smem + s * kStageBytes;
     uint8_t* vd = kd + NH * 8192;
@@ -213,7 +212,7 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
     }
   };
   if (tid == 0)
-    for (int i = 0; i < nmy && i < kAttnStages; ++i) issue(i);
+    for (int i = 0; i < nmy && i < p.stages; ++i) issue(i, i);
 
   // query fragments of this warp's 16 rows
   const int rw = warp % RW, kg = warp / RW;
@@ -244,17 +243,16 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
   const float sl2 = 1.4426950408889634f / sqrtf(static_cast<float>(D));  // log2(e)/sqrt(D)
 
   bool failed = false;
+  int s = 0;        // stage of chunk i, and the parity of its phase
+  uint32_t ph = 0;
   for (int i = 0; i < nmy; ++i) {
-    const int s = i % kAttnStages;
-    const bool ok = mbar_wait(&full[s], static_cast<uint32_t>(i / kAttnStages) & 1u, p.limit_ns,
-                              nullptr);
+    const bool ok = mbar_wait(&full[s], ph, p.limit_ns, nullptr);
     if (__syncthreads_or(!ok)) {
       failed = true;
       if (tid == 0) {
         atomicCAS(p.status, 0, EBD_ERR_TIMEOUT);
-        for (int j = i; j < nmy && j < i + kAttnStages; ++j)
-          mbar_wait(&full[j % kAttnStages], static_cast<uint32_t>(j / kAttnStages) & 1u,
-                    p.limit_ns, nullptr);
+        for (int j = i; j < nmy && j < i + p.stages; ++j)
+          mbar_wait(&full[j % p.stages], static_cast<uint32_t>(j / p.stages) & 1u, p.limit_ns, nullptr);
       }
       break;
     }
@@ -352,7 +350,11 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
       }
     }
     __syncthreads();
-    if (tid == 0 && i + kAttnStages < nmy) issue(i + kAttnStages);
+    if (tid == 0 && i + p.stages < nmy) issue(i + p.stages, s);
+    if (++s == p.stages) {
+      s = 0;
+      ph ^= 1u;
+    }
   }
   if (failed) return;
 
@@ -1073,8 +1075,9 @@ __device__ __forceinline__ bool wait_ready(const AttnParams& p) {
 // waits for the grid it is a programmatic dependent of (the decision) before
 // it exits, so that a kernel launched after this one as its dependent sees
 // that grid complete as well.
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads)
+// PER_SM CTAs per SM: three take 168 registers a thread, which spills a few.
+template <int D, int PER_SM>
+__global__ void __launch_bounds__(kAttnThreads, PER_SM)
     attn_kernel(const __grid_constant__ CUtensorMap tm_kc, const __grid_constant__ CUtensorMap tm_vc,
                 const __grid_constant__ CUtensorMap tm_kw, const __grid_constant__ CUtensorMap tm_vw,
                 const AttnParams p) {
@@ -1094,8 +1097,10 @@ __global__ void __launch_bounds__(kAttnTcThreads, 1)
 cudaError_t attn_configure() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(attn_kernel<64>, a, attn_smem_bytes(64))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(attn_kernel<128>, a, attn_smem_bytes(128))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<64, 2>, a, attn_smem_bytes(64, kAttnStages))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<64, 3>, a, attn_smem_bytes(64, 2))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<128, 2>, a, attn_smem_bytes(128, kAttnStages))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<128, 3>, a, attn_smem_bytes(128, 2))) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attn_tc_kernel<64>, a, TcMap<64>::kDyn)) != cudaSuccess) return e;
   return cudaFuncSetAttribute(attn_tc_kernel<128>, a, TcMap<128>::kDyn);
 }
@@ -1107,7 +1112,7 @@ cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const
   cfg.gridDim = dim3(p.splits, p.max_qtiles, p.B * p.Hkv);
   cfg.blockDim = dim3(p.tc ? kAttnTcThreads : kAttnThreads, 1, 1);
   cfg.dynamicSmemBytes = p.tc ? (p.D == 64 ? TcMap<64>::kDyn : TcMap<128>::kDyn)
-                              : attn_smem_bytes(p.D);
+                              : attn_smem_bytes(p.D, p.stages);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1117,8 +1122,9 @@ cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const
   if (p.tc)
     return p.D == 64 ? cudaLaunchKernelEx(&cfg, attn_tc_kernel<64>, kc, vc, kw, vw, p)
                      : cudaLaunchKernelEx(&cfg, attn_tc_kernel<128>, kc, vc, kw, vw, p);
-  if (p.D == 64) return cudaLaunchKernelEx(&cfg, attn_kernel<64>, kc, vc, kw, vw, p);
-  return cudaLaunchKernelEx(&cfg, attn_kernel<128>, kc, vc, kw, vw, p);
+  const auto k = p.stages == 2 ? (p.D == 64 ? attn_kernel<64, 3> : attn_kernel<128, 3>)
+                               : (p.D == 64 ? attn_kernel<64, 2> : attn_kernel<128, 2>);
+  return cudaLaunchKernelEx(&cfg, k, kc, vc, kw, vw, p);
 }
 
 }  // namespace ebd
