@@ -40,13 +40,11 @@
  *     sequence <= max_window <= 512, gen_len >= max_window, vocab >= 2,
  *     rows of a step <= max_rows <= 4096.  Anything else returns
  *     EBD_ERR_UNSUPPORTED.
- *   - max_window <= 64: the decision runs as one thread-block cluster per
- *     sequence; with max_window <= 32, a launch of 16 or more sequences runs
- *     it as one CTA per sequence instead (the same results; the environment
- *     variable EBD_DECIDE_KERNEL = "cta" or "cluster" forces either kernel
- *     for max_window <= 32).  max_window > 64 (the full-sequence setting, where every
- *     position of the response is a row, App. E with M = all masked
- *     positions): the decision runs as a chain of grid-wide kernels, and a
+ *   - The decision runs as one thread-block cluster per sequence, of as many
+ *     CTAs as suit the launch's sequences.  max_window > 64 (the
+ *     full-sequence setting, where every position of the response is a row,
+ *     App. E with M = all masked positions): the statistics and the LBS run
+ *     over the whole GPU ahead of it, and a
  *     step takes no window attention (attn_out and kv_append must be unset:
  *     EBD_ERR_UNSUPPORTED otherwise).
  *   - stream arguments are cudaStream_t values passed as void* (NULL = the
@@ -281,10 +279,11 @@ ebd_status ebd_merge_shard_states(ebd_handle* h, const float* states, int32_t sh
 /* Only step 1 (window attention): writes a->attn_out.  The handle picks one
  * of two kernels when it is created: the tcgen05 kernel (S and O in tensor
  * memory, one CTA per SM) for long key ranges with few tiles or with query
- * tiles of more than 32 rows, the mma.sync kernel (two CTAs per SM)
+ * tiles of more than 32 rows, the mma.sync kernel (two or three CTAs per SM)
  * otherwise; both compute the same attention.  The environment variables
- * EBD_ATTN_KERNEL = "tc" or "mma" and EBD_ATTN_SPLITS (key splits per query
- * tile, 1..8), read at ebd_create, override the choices. */
+ * EBD_ATTN_KERNEL = "tc" or "mma", EBD_ATTN_SPLITS (key splits per query
+ * tile, 1..8) and EBD_ATTN_STAGES (ring of the mma.sync kernel: 2, three
+ * CTAs per SM, or 3, two), read at ebd_create, override the choices. */
 ebd_status ebd_attention(ebd_handle* h, const ebd_step_args* a, void* stream);
 
 /* Synchronises `stream`, returns the first device-side failure recorded

@@ -29,6 +29,15 @@ namespace {
 constexpr int attn_stage_bytes(int D) { return 2 * (D / 64) * 8192; }
 constexpr int attn_smem_bytes(int D, int stages) { return stages * attn_stage_bytes(D) + 1024 + 64; }
 
+__device__ __forceinline__ void tma_load_5d(void* smem_dst, const void* tmap, uint64_t* bar, int32_t x,
+                                            int32_t y, int32_t z, int32_t w, int32_t v) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(smem_dst)),
+      "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(smem_u32(bar))
+      : "memory");
+}
+
 // byte offset of 16-byte chunk `c` (0..7) of row `r` in a 128B-swizzled tile
 __device__ __forceinline__ uint32_t swz(int r, int c) {
   return static_cast<uint32_t>(r * 128 + ((c ^ (r & 7)) << 4));
