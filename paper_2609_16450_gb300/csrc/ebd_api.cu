@@ -840,9 +840,13 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     if (const char* env = getenv("EBD_ATTN_KERNEL")) h->attn_tc = strcmp(env, "mma") == 0 ? 0 : 1;
     // key splits per tile: as many as keep one wave of CTAs, of at least 4
     // chunks each (a CTA more than the SMs hold costs a second wave: 1 x 4096
-    // x 8 rows on tcgen05 28.7 us with 5 splits, 18.7 with 4)
+    // x 8 rows on tcgen05 28.7 us with 5 splits, 18.7 with 4).  On tcgen05,
+    // with its longer steps, a split's partials cost as much as it saves below
+    // 16 chunks (2 x 452 x 50 rows 14.5 us unsplit, 16.4 with 2; 2 x 1024 x 50
+    // 18.6 either way, 2 x 2048 x 50 26.8 / 22.7).
     int splits = (h->attn_tc ? h->num_sms : 2 * h->num_sms) / slots;
     if (splits > nch / 4) splits = nch / 4;
+    if (h->attn_tc && nch < 16) splits = 1;
     if (const char* env = getenv("EBD_ATTN_SPLITS")) splits = atoi(env);
     if (splits > kMaxSplits) splits = kMaxSplits;
     if (splits > nch) splits = nch;
