@@ -1245,8 +1245,9 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   // on the SMs this grid leaves free once every CTA of it is resident
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  for (int i = tid; i < kVecs / 4; i += kT)
-    reinterpret_cast<float4*>(sv)[i] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
+  if (p.mode == EBD_DECODE_EB)  // the baselines' rules use no router
+    for (int i = tid; i < kVecs / 4; i += kT)
+      reinterpret_cast<float4*>(sv)[i] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
 
   // ------------------------------------------------------------ decode state
   const int r0 = p.cu_rows[b];
@@ -1322,7 +1323,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 
     // The LM head has streamed its weight through L2: bring the router's back
     // while its last CTAs run.
-    if (b == 0) {
+    if (b == 0 && p.mode == EBD_DECODE_EB) {
       const char* w = reinterpret_cast<const char*>(p.mat);
       for (int i = (run_lbs ? 0 : M_BLOCK / 8) + rank * kT + tid; i < M_TOTAL / 8; i += C * kT)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 128 * static_cast<size_t>(i)));
