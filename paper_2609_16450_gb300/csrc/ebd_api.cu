@@ -823,10 +823,14 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     // heads, us, mma.sync against tcgen05 in the better of their splits):
     //   more tiles than SMs: 64 x 1024 x 32 rows 183 / 228, 64 x 4096 x 32
     //     630 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 44 / 53; but tiles
-    //     of 33 to 64 rows over 1024 keys and more 103 / 74 (16 x 1024 x 64),
-    //     1087 / 653 (64 x 4096 x 64), below that 117 / 150 (64 x 256 x 64);
+    //     of 33 to 64 rows over more than 8 chunks 62 / 62 (16 x 640 x 64), 298
+    //     / 235 (64 x 900 x 64), Dream-7B heads 51 / 43 (36 x 640 x 21), 120 /
+    //     86 (64 x 900 x 21), at 8 chunks 167 / 168 (64 x 400 x 64), 40 / 37
+    //     (36 x 400 x 21), below that 117 / 153 (64 x 250 x 64);
     //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
-    //     47, 1 x 4096 x 32 26.5 / 21; but at 256 keys 10.8 / 12.2.
+    //     47, 1 x 4096 x 32 26.5 / 21, but at 256 keys 10.8 / 12.2; with tiles
+    //     of 33 to 64 rows 14 / 13 at 250 keys (8 x 250 x 21, Dream-7B heads),
+    //     10.8 / 12.2 at 120.
     // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count,
     // EBD_ATTN_STAGES the ring's stages (measurement sweeps).
     const int tile = 64;
@@ -836,7 +840,7 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     const int slots = cfg->max_batch * cfg->n_heads_kv * h->attn_max_qtiles;
     const int nch = (cfg->max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
     const bool one_wave = slots <= h->num_sms;
-    h->attn_tc = aw * group > 32 ? (one_wave || nch >= 17) : (one_wave && nch >= 9);
+    h->attn_tc = aw * group > 32 ? nch >= (one_wave ? 5 : 9) : (one_wave && nch >= 9);
     if (const char* env = getenv("EBD_ATTN_KERNEL")) h->attn_tc = strcmp(env, "mma") == 0 ? 0 : 1;
     // key splits per tile: as many as keep one wave of CTAs, of at least 4
     // chunks each (a CTA more than the SMs hold costs a second wave: 1 x 4096
