@@ -830,7 +830,7 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
     //     47, 1 x 4096 x 32 26.5 / 21, but at 256 keys 10.8 / 12.2; with tiles
     //     of 33 to 64 rows 14 / 13 at 250 keys (8 x 250 x 21, Dream-7B heads),
-    //     10.8 / 12.2 at 120.
+    //     12.3 / 12.3 at 180, 10.8 / 12.2 at 120.
     // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count,
     // EBD_ATTN_STAGES the ring's stages (measurement sweeps).
     const int tile = 64;
@@ -840,17 +840,20 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     const int slots = cfg->max_batch * cfg->n_heads_kv * h->attn_max_qtiles;
     const int nch = (cfg->max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
     const bool one_wave = slots <= h->num_sms;
-    h->attn_tc = aw * group > 32 ? nch >= (one_wave ? 5 : 9) : (one_wave && nch >= 9);
+    h->attn_tc = aw * group > 32 ? nch >= (one_wave ? 4 : 9) : (one_wave && nch >= 9);
     if (const char* env = getenv("EBD_ATTN_KERNEL")) h->attn_tc = strcmp(env, "mma") == 0 ? 0 : 1;
     // key splits per tile: as many as keep one wave of CTAs, of at least 4
     // chunks each (a CTA more than the SMs hold costs a second wave: 1 x 4096
     // x 8 rows on tcgen05 28.7 us with 5 splits, 18.7 with 4).  On tcgen05,
     // with its longer steps, a split's partials cost as much as it saves below
     // 16 chunks (2 x 452 x 50 rows 14.5 us unsplit, 16.4 with 2; 2 x 1024 x 50
-    // 18.6 either way, 2 x 2048 x 50 26.8 / 22.7).
+    // 18.6 either way, 2 x 2048 x 50 26.8 / 22.7); and five to seven are no
+    // better than four (Dream-7B heads 2 x 1600 x 16 16.5 with 4, 18.6 with 5 to
+    // 7; 2 x 2048 x 4 16.4 with 4, 14.5 with 8).
     int splits = (h->attn_tc ? h->num_sms : 2 * h->num_sms) / slots;
     if (splits > nch / 4) splits = nch / 4;
     if (h->attn_tc && nch < 16) splits = 1;
+    if (h->attn_tc && splits > 4 && splits < 8) splits = 4;
     if (const char* env = getenv("EBD_ATTN_SPLITS")) splits = atoi(env);
     if (splits > kMaxSplits) splits = kMaxSplits;
     if (splits > nch) splits = nch;
