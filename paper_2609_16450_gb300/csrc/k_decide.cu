@@ -1295,6 +1295,10 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   };
   if (kWide) {
     if (p.lps_enabled) copy_lps();
+    // Rank 0 commits in place, and where no LPS follows nothing else stands
+    // between a CTA's reads of the decode state above and that commit.  (In a
+    // step this meeting is over before the grids ahead are.)
+    cluster_barrier();
     // the statistics and the LBS logits of every row
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
