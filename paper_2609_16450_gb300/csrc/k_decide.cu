@@ -1073,10 +1073,39 @@ __device__ __forceinline__ void lps_router(int nb, int grp, Meet meet) {
   }
 }
 
-// The statistics of the CTA's rows merged from the LM head's partial states:
-// its groups' slots, then its share of the unmasked rows, a row per warp.
-// Waits for the grid before this one first.  With `warm` each warp starts
-// with a pass that merges no states, into a row of its own (before the wait).
+// The statistics of step row r, merged by a warp from the LM head's partial
+// states, to the scratch and the caller's outputs; lane 0 returns H~ and the
+// argmax in `ent` and `arg`.  With `real` false no states are merged and the
+// result goes to the scratch's spare row.
+__device__ __forceinline__ void merge_one(const RowsParams& p, int r, bool real, float& ent, int& arg) {
+  const size_t base = static_cast<size_t>(r) * p.grid_lm;
+  const RowStats st = merge_row(p.part_f + base, p.part_i + base, real ? p.grid_lm : 0);
+  if ((threadIdx.x & 31) != 0) return;
+  const int sr = real ? r : p.spare_row;
+  const float conf = 1.0f / st.s, h = logf(st.s) - st.t * conf, entn = h * p.inv_log_v;
+  const float gap = (1.0f - expf(st.l2 - st.m)) * conf;
+  const bool bad = !(isfinite(st.m) && isfinite(st.s) && isfinite(st.t) && st.s >= 1.0f) || st.idx < 0 ||
+                   st.idx >= p.V;
+  ent = entn;
+  arg = bad ? -1 : st.idx;
+  p.s_conf[sr] = conf;
+  p.s_ent[sr] = entn;
+  p.s_gap[sr] = gap;
+  p.s_arg[sr] = arg;
+  if (real) {
+    if (p.conf) p.conf[r] = conf;
+    if (p.entropy) p.entropy[r] = h;
+    if (p.ent_norm) p.ent_norm[r] = entn;
+    if (p.gap) p.gap[r] = gap;
+    if (p.argmax) p.argmax[r] = arg;
+    if (bad) atomicCAS(p.status, 0, EBD_ERR_NONFINITE);
+  }
+}
+
+// The statistics of the CTA's rows: its groups' slots, then its share of the
+// unmasked rows, a row per warp.  Waits for the grid before this one first.
+// With `warm` each warp starts with a pass that merges no states (before the
+// wait).
 template <int CAP>
 __device__ __forceinline__ void merge_rows(const RowsParams& p, Slots& sl, const RowState<CAP>& rs, int r0, int nr,
                                            int nu, bool warm) {
@@ -1090,31 +1119,12 @@ __device__ __forceinline__ void merge_rows(const RowsParams& p, Slots& sl, const
     }
     const int j = !real ? 0 : it < 8 * nr ? sl.mrow[it] : rs.urow[it - 8 * nr];
     if (j < 0 || (real && !in_bounds(r0 + j, p.R, p.status))) continue;
-    const size_t base = static_cast<size_t>(r0 + j) * p.grid_lm;
-    const RowStats st = merge_row(p.part_f + base, p.part_i + base, real ? p.grid_lm : 0);
-    if (lane == 0) {
-      const int r = r0 + j, sr = real ? r : p.spare_row;
-      const float conf = 1.0f / st.s, ent = logf(st.s) - st.t * conf, entn = ent * p.inv_log_v;
-      const float gap = (1.0f - expf(st.l2 - st.m)) * conf;
-      const bool bad = !(isfinite(st.m) && isfinite(st.s) && isfinite(st.t) && st.s >= 1.0f) || st.idx < 0 ||
-                       st.idx >= p.V;
-      const int arg = bad ? -1 : st.idx;
-      p.s_conf[sr] = conf;
-      p.s_ent[sr] = entn;
-      p.s_gap[sr] = gap;
-      p.s_arg[sr] = arg;
-      if (real) {
-        if (p.conf) p.conf[r] = conf;
-        if (p.entropy) p.entropy[r] = ent;
-        if (p.ent_norm) p.ent_norm[r] = entn;
-        if (p.gap) p.gap[r] = gap;
-        if (p.argmax) p.argmax[r] = arg;
-        if (bad) atomicCAS(p.status, 0, EBD_ERR_NONFINITE);
-        if (it < 8 * nr) {
-          sl.ent[it] = entn;
-          sl.arg[it] = arg;
-        }
-      }
+    float ent = 0.f;
+    int arg = -1;
+    merge_one(p, r0 + j, real, ent, arg);
+    if (lane == 0 && real && it < 8 * nr) {
+      sl.ent[it] = ent;
+      sl.arg[it] = arg;
     }
   }
   if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1197,6 +1207,18 @@ __global__ void __launch_bounds__(kT, 1) lbs_wide_kernel(const RowsParams p) {
       }
     } else {
       merge_rows<CAP>(p, sl, rs, r0, nr, nu, false);
+      // Statistics are every row's, also of a rejected sequence and of the
+      // rows before the first offset and past the last: from each offset up
+      // to the next, 0 and R in place of the first and the last, the spans
+      // that run forward hold every row.
+      const int lo = b == 0 ? 0 : min(max(r0, 0), p.R);
+      const int hi = b == p.B - 1 ? p.R : min(max(p.cu_rows[b + 1], 0), p.R);
+      for (int i = wk * kNW + warp; i < hi - lo - n; i += nw * kNW) {
+        const int r = lo + i < r0 ? lo + i : lo + i + n;
+        float ent;
+        int arg;
+        merge_one(p, r, true, ent, arg);
+      }
     }
     __syncthreads();
     if (!run_lbs || nr == 0) return;
