@@ -905,7 +905,7 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
   if (cfg->max_window <= kMaxWindow) (void)copy_route_ready(h);
   {  // scratch of the decision
     const int planes = cfg->max_window > kMaxWindow ? 3 : 2;
-    const size_t cap = static_cast<size_t>((cfg->max_rows + 31) / 32 * 32) + 32 * (static_cast<size_t>(cfg->max_batch) + 1);
+    const size_t cap = scratch_rows(cfg->max_rows, cfg->max_batch);
     const size_t R = cfg->max_rows;
     size_t bytes = 0;
     auto add = [&](size_t n) {
@@ -913,10 +913,11 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
       bytes += (n + 255) / 256 * 256;
       return at;
     };
-    const size_t o_kv = add(4 * planes * cap * 128 * 2), o_kvp = add(4 * planes * cap * 32 * 2), o_O = add(cap * 4),
-                 o_P = add(cap * 4), o_c = add((R + 1) * 4), o_e = add((R + 1) * 4), o_g = add((R + 1) * 4),
-                 o_a = add((R + 1) * 4), o_z = add(planes == 3 ? cap * 128 * 4 : 0),
-                 o_q = add(planes == 3 ? 3 * cap * 128 * 2 : 0);
+    const bool wide = planes == 3;
+    const size_t o_kv = add(4 * planes * cap * 128 * 2), o_O = add(cap * 4), o_P = add(cap * 4),
+                 o_c = add((R + 1) * 4), o_e = add((R + 1) * 4), o_g = add((R + 1) * 4), o_a = add((R + 1) * 4),
+                 o_kvp = add(wide ? 4 * planes * cap * 32 * 2 : 0), o_z = add(wide ? cap * 128 * 4 : 0),
+                 o_q = add(wide ? planes * cap * 128 * 2 : 0);
     if ((e = cudaMalloc(&h->rows_scratch, bytes)) != cudaSuccess)
       return bail(cuda_fail(h, e, "cudaMalloc(decision scratch)"));
     uint8_t* b0 = h->rows_scratch;

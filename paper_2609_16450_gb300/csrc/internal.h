@@ -65,6 +65,16 @@ struct AttnParams {
 };
 
 // ------------------------------------------------------------------ decision
+// Rows of the decision's scratch.  A sequence of n rows takes ceil(n / 8) whole
+// groups of 8 from scratch_row on: of the b sequences before it at most
+// min(b, r0) hold a row, and each of those ends in at most one part of a group.
+// A launch within max_rows and max_batch thus stays below scratch_rows, which
+// counts no more sequences than rows (65535 sequences of 4096 rows: 36864).
+__host__ __device__ inline int scratch_row(int r0, int b) { return 8 * (r0 / 8 + (b < r0 ? b : r0)); }
+inline int scratch_rows(int max_rows, int max_batch) {
+  return 8 * (max_rows / 8 + (max_batch < max_rows ? max_batch : max_rows));
+}
+
 struct RowsParams {
   int B, R, V, grid_lm;     // grid_lm: LM-head partials per row
   int features_in;          // 1: s_conf/s_ent/s_gap/s_arg are inputs
@@ -93,11 +103,11 @@ struct RowsParams {
   const uint4* mat;         // router image (rows_image.h)
   const float* vec;
   const float* tok_table;   // [V][64]
-  int cap_rows;             // rows of the scratch below: R rounded up to 32, and 32 per sequence
+  int cap_rows;             // rows of the scratch below (scratch_rows)
   __nv_bfloat16* kv;        // LBS keys and values [2 layers][2][planes][cap_rows][128]
-  __nv_bfloat16* kvp;       // LPS keys and values [2 blocks][2][planes][cap_rows][32]
-  float* z;                 // windows of more than 64 rows: LBS activations [cap_rows][128]
-  __nv_bfloat16* q;         // and queries [planes][cap_rows][128] between launches
+  __nv_bfloat16* kvp;       // windows of more than 64 rows: LPS keys and values [2 blocks][2][planes][cap_rows][32]
+  float* z;                 // and, between launches, LBS activations [cap_rows][128]
+  __nv_bfloat16* q;         // and queries [planes][cap_rows][128]
   float *O, *P;             // [cap_rows] LBS logits by rank in M, p_psi by rank in B n M
   int* status;
 };

@@ -1161,7 +1161,7 @@ __global__ void __launch_bounds__(kT, 1) lbs_wide_kernel(const RowsParams p) {
   const int r0 = p.cu_rows[b];
   int n = p.cu_rows[b + 1] - r0;
   if (n < 0 || n > CAP || r0 < 0 || r0 + n > p.R || n > p.gen_len) n = 0;  // reported by the decision
-  const int kbase = ((r0 + 31) & ~31) + 32 * b, capk = (n + 31) & ~31;
+  const int kbase = scratch_row(r0, b), capk = (n + 7) & ~7;
   bool m[RPT], f[RPT];
   int mrank[RPT], urank[RPT];
   if (PART == 0 && tid < 32) {
@@ -1280,8 +1280,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     if (rank == 0 && tid == 0) atomicCAS(p.status, 0, EBD_ERR_INVALID_ARG);
     n = 0;
   }
-  const int kbase = ((r0 + 31) & ~31) + 32 * b;  // this sequence's rows of the scratch
-  const int capk = (n + 31) & ~31;
+  const int kbase = scratch_row(r0, b), capk = (n + 7) & ~7;  // this sequence's rows of the scratch
   int meta_b = p.blk_meta[2 * b], meta_s = p.blk_meta[2 * b + 1];
   bool m[RPT], inb[RPT], f[RPT];
   int pos[RPT], mrank[RPT], urank[RPT];

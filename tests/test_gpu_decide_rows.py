@@ -33,7 +33,7 @@ def _stats(rng, n, vocab, eos):
 @pytest.mark.parametrize("bias", [0.0, 8.0])
 @pytest.mark.parametrize("batch,window", [(1, 64), (1, 13), (2, 9), (9, 64), (20, 57), (37, 64), (44, 40),
                                           (16, 32), (40, 24), (90, 32), (140, 16), (1, 65), (2, 129), (1, 512),
-                                          (3, 300)])
+                                          (3, 300), (400, 12), (60, 68)])
 def test_decide_launch_shapes(batch, window, bias):
     from paper_2609_16450_gb300 import _ebd as E
     from paper_2609_16450_gb300 import runtime as rt
