@@ -248,7 +248,7 @@ struct ebd_handle {
   // the decision
   uint8_t* d_rows = nullptr;        // its router image (rows_image.h)
   uint8_t* rows_scratch = nullptr;
-  int rows_slots[2] = {0, 0};       // its clusters of 8 and of 4 CTAs that fit the GPU
+  DecideSlots rows_slots{};         // its clusters that fit the GPU
   RowsParams rowsp{};               // image and scratch pointers, filled at create
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   int profile = 0;
@@ -523,7 +523,7 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   } else {
     const uint64_t cdims[5] = {64, Pm, NB, H, Bc}, wdims[4] = {64, R, NB, H};
     const uint64_t cstr[4] = {row, 128, head, Pm * row}, wstr[3] = {row, 128, head};
-    const uint32_t cbox[5] = {64, 64, static_cast<uint32_t>(NB), 1, 1}, wbox[4] = {64, 64, static_cast<uint32_t>(NB), 1};
+    const uint32_t nb = static_cast<uint32_t>(NB), cbox[5] = {64, 64, nb, 1, 1}, wbox[4] = {64, 64, nb, 1};
     ok = encode_bf16(&kc, kcp, 5, cdims, cstr, cbox) && encode_bf16(&vc, vcp, 5, cdims, cstr, cbox) &&
          encode_bf16(&kw, a->k_win, 4, wdims, wstr, wbox) && encode_bf16(&vw, a->v_win, 4, wdims, wstr, wbox);
   }

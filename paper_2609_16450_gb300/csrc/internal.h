@@ -128,9 +128,13 @@ cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const
                              bool pdl = false);
 // the decision, the rows of a sequence split over a cluster of CTAs
 // (k_decide.cu); cap: rows per sequence the launch has to hold (32, 64
-// or kMaxSeqRows).  slots: clusters of 8 and of 4 CTAs that fit the GPU at once
-cudaError_t decide_rows_configure(int (&slots)[2]);
-cudaError_t launch_decide_rows(const RowsParams& p, int cap, const int (&slots)[2], cudaStream_t st, bool pdl);
+// or kMaxSeqRows)
+struct DecideSlots {        // clusters that fit the GPU at once
+  int c8, c4;               // windows of up to 64 rows: of 8 and of 4 CTAs
+  int wide16, wide8, wide4; // of more: of 16, 8 and 4
+};
+cudaError_t decide_rows_configure(DecideSlots& n);
+cudaError_t launch_decide_rows(const RowsParams& p, int cap, const DecideSlots& n, cudaStream_t st, bool pdl);
 // vocabulary-parallel LM head: one state per row from a launch's partials,
 // and the statistics from the states of several shards (k_stats.cu)
 cudaError_t launch_shard_state(const float4* part_f, const int* part_i, int rows, int grid,

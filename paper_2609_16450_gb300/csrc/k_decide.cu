@@ -9,9 +9,9 @@
 // every row's keys and values (once per layer) and before the selection:
 // three cluster barriers.  Keys and values travel through an L2-resident
 // scratch.  Windows of more than 64 rows take their LBS through three launches
-// over the whole GPU instead (lbs_wide_kernel), ahead of the cluster.  The LPS router is small enough for a warp to take 8 rows of
-// B n M through it in registers; its warps meet for the keys and values of
-// its two attentions only.
+// over the whole GPU instead (lbs_wide_kernel), ahead of the cluster.  The LPS
+// router is small enough for a warp to take 8 rows of B n M through it in
+// registers; its warps meet for the keys and values of its two attentions only.
 //
 // Products run on mma.sync (m16n8k16) with the weights as the M = 16 operand
 // and the rows as N = 8.  The weights are bf16 values; an activation x is held
@@ -44,7 +44,13 @@ __device__ __forceinline__ void cluster_barrier() {
 // two consecutive rows by 8 lanes fall in different banks
 __device__ __host__ constexpr int row_bytes(int K) { return K == 32 ? 64 : 2 * K + 64; }
 
-template <int NR, int NP>
+// groups of 8 rows of a window of up to kMaxSeqRows that a warp of a cluster of
+// C CTAs takes through the LPS (C = 0: windows of up to 64 rows, one CTA)
+__device__ __host__ constexpr int lps_groups(int C) {
+  return C == 0 || C * kNW >= kMaxSeqRows / 8 ? 1 : kMaxSeqRows / 8 / (C * kNW);
+}
+
+template <int NR, int NP, int NG = 1>
 struct Lay {  // shared memory, byte offsets
   static constexpr int R = 8 * NR;                  // rows of a CTA
   static constexpr int P128 = R * row_bytes(128);   // one plane of R rows x 128
@@ -69,8 +75,8 @@ struct Lay {  // shared memory, byte offsets
   static constexpr int kLpsMat = 2 * MB_STRIDE;     // 16-byte units
   static constexpr int KV = W + kLpsMat * 16;
   static constexpr int kKvBlock = 64 * 64 * NP;     // elements of a block
-  static constexpr int ST = KV + (NP == 2 ? 2 * kKvBlock * 2 : 0);  // a warp's values between the parts
-  static constexpr int GL = ST + kNW * (16 + 4 * NP) * 32 * 4;      // LpsGlobal
+  static constexpr int ST = KV + (NP == 2 ? 2 * kKvBlock * 2 : 0);   // a group's values between the parts
+  static constexpr int GL = ST + NG * kNW * (16 + 4 * NP) * 32 * 4;  // LpsGlobal
   static constexpr int kLpsEnd = GL + 32;
   static constexpr int SLOT = kLbsEnd > kLpsEnd ? kLbsEnd : kLpsEnd;
   static constexpr int ROW = SLOT + 3 * 32 * 4;     // per-row arrays
@@ -620,7 +626,8 @@ __device__ __noinline__ void lbs_qkv(const LbsArgs a, int l) {
             split2<NP>(x0, x1, u);
             split2<NP>(y0, y1, v);
           }
-          __nv_bfloat16* const d0 = kind == 1 ? Kp + static_cast<size_t>(k) * 128 + c : Vp + static_cast<size_t>(c) * a.capk + k;
+          __nv_bfloat16* const d0 =
+              kind == 1 ? Kp + static_cast<size_t>(k) * 128 + c : Vp + static_cast<size_t>(c) * a.capk + k;
           const size_t step = kind == 1 ? 128 : a.capk;
 #pragma unroll
           for (int q = 0; q < NP; ++q) {
@@ -821,21 +828,29 @@ struct LpsGlobal {  // (GLOBAL; in shared memory, for all warps)
 };
 template <int NP>
 constexpr int kLpsWords = 8 + 4 * NP + 8;  // z, queries, attention output
+// a lane's words of them: of the warp's only group, or of group grp = rank +
+// C * (warp + kNW * pass)
+template <class L, int NP, int C>
+__device__ __forceinline__ float* lps_values(uint8_t* smem, int grp) {
+  const int slot = C > 0 ? grp / C : static_cast<int>(threadIdx.x >> 5);
+  return reinterpret_cast<float*>(smem + L::ST) + slot * kLpsWords<NP> * 32 + (threadIdx.x & 31);
+}
 
 // Linear(5 -> 32), LayerNorm, GELU (block 0); LN1, QKV
-template <int CAP, int NR, int NP, bool GLOBAL>
+template <int CAP, int NR, int NP, int C>
 __device__ __noinline__ void lps_qkv(int nb, int grp, int l) {
-  using L = Lay<NR, NP>;
+  using L = Lay<NR, NP, lps_groups(C)>;
   extern __shared__ __align__(16) uint8_t smem[];
   const float* const sv = reinterpret_cast<const float*>(smem + L::V);
   RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
-  float* const st = reinterpret_cast<float*>(smem + L::ST) + (threadIdx.x >> 5) * kLpsWords<NP> * 32 + (threadIdx.x & 31);
+  float* const st = lps_values<L, NP, C>(smem, grp);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const uint4* const wl = reinterpret_cast<const uint4*>(smem + L::W) + l * MB_STRIDE;
   const float* const vl = sv + V_BLOCK + l * VB_STRIDE;
   const LpsGlobal& gl = *reinterpret_cast<const LpsGlobal*>(smem + L::GL);
-  __nv_bfloat16* const K = GLOBAL ? gl.kv + l * gl.kv_stride : reinterpret_cast<__nv_bfloat16*>(smem + L::KV) + l * L::kKvBlock;
-  __nv_bfloat16* const V = K + (GLOBAL ? gl.v_off : L::kKvBlock / 2);
+  __nv_bfloat16* const K =
+      C > 0 ? gl.kv + l * gl.kv_stride : reinterpret_cast<__nv_bfloat16*>(smem + L::KV) + l * L::kKvBlock;
+  __nv_bfloat16* const V = K + (C > 0 ? gl.v_off : L::kKvBlock / 2);
   float z[2][4];
   if (l == 0) {
 #pragma unroll
@@ -887,15 +902,16 @@ __device__ __noinline__ void lps_qkv(int nb, int grp, int l) {
 }
 
 // softmax(q k^T / sqrt(8)) v
-template <int CAP, int NR, int NP, bool GLOBAL>
+template <int CAP, int NR, int NP, int C>
 __device__ __noinline__ void lps_attend(int nb, int grp, int l) {
-  using L = Lay<NR, NP>;
+  using L = Lay<NR, NP, lps_groups(C)>;
   extern __shared__ __align__(16) uint8_t smem[];
-  float* const st = reinterpret_cast<float*>(smem + L::ST) + (threadIdx.x >> 5) * kLpsWords<NP> * 32 + (threadIdx.x & 31);
+  float* const st = lps_values<L, NP, C>(smem, grp);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const LpsGlobal& gl = *reinterpret_cast<const LpsGlobal*>(smem + L::GL);
-  const __nv_bfloat16* const K = GLOBAL ? gl.kv + l * gl.kv_stride : reinterpret_cast<const __nv_bfloat16*>(smem + L::KV) + l * L::kKvBlock;
-  const __nv_bfloat16* const V = K + (GLOBAL ? gl.v_off : L::kKvBlock / 2);
+  const __nv_bfloat16* const K =
+      C > 0 ? gl.kv + l * gl.kv_stride : reinterpret_cast<const __nv_bfloat16*>(smem + L::KV) + l * L::kKvBlock;
+  const __nv_bfloat16* const V = K + (C > 0 ? gl.v_off : L::kKvBlock / 2);
   uint32_t qf[4][NP];
 #pragma unroll
   for (int h = 0; h < 4; ++h)
@@ -919,8 +935,8 @@ __device__ __noinline__ void lps_attend(int nb, int grp, int l) {
     for (int j = 0; j < 2; ++j) {
       const int key = k0 + 16 * j + g;
       uint32_t k0w[4 * NP], k1w[4 * NP];  // keys key, key + 8: dims 2 t, 2 t + 1
-      ld_kv<NP, GLOBAL>(K + ((key < n8 ? key : 0) * 4 + t) * (8 * NP), k0w);
-      ld_kv<NP, GLOBAL>(K + ((key + 8 < n8 ? key + 8 : 0) * 4 + t) * (8 * NP), k1w);
+      ld_kv<NP, (C > 0)>(K + ((key < n8 ? key : 0) * 4 + t) * (8 * NP), k0w);
+      ld_kv<NP, (C > 0)>(K + ((key + 8 < n8 ? key + 8 : 0) * 4 + t) * (8 * NP), k1w);
 #pragma unroll
       for (int h = 0; h < 4; ++h)
 #pragma unroll
@@ -958,7 +974,7 @@ __device__ __noinline__ void lps_attend(int nb, int grp, int l) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int key = k0 + 16 * j + 8 * u;
-        ld_kv<NP, GLOBAL>(V + (((key < n8 ? key : 0) / 2 + t) * 8 + g) * (8 * NP), va[u]);
+        ld_kv<NP, (C > 0)>(V + (((key < n8 ? key : 0) / 2 + t) * 8 + g) * (8 * NP), va[u]);
         if (key >= n8)
 #pragma unroll
           for (int i = 0; i < 4 * NP; ++i) va[u][i] = 0u;
@@ -1001,13 +1017,13 @@ __device__ __noinline__ void lps_attend(int nb, int grp, int l) {
 }
 
 // output projection, LN2, FFN; after block 1 the head and p_psi
-template <int CAP, int NR, int NP, bool GLOBAL>
+template <int CAP, int NR, int NP, int C>
 __device__ __noinline__ void lps_ffn(int nb, int grp, int l) {
-  using L = Lay<NR, NP>;
+  using L = Lay<NR, NP, lps_groups(C)>;
   extern __shared__ __align__(16) uint8_t smem[];
   const float* const sv = reinterpret_cast<const float*>(smem + L::V);
   RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
-  float* const st = reinterpret_cast<float*>(smem + L::ST) + (threadIdx.x >> 5) * kLpsWords<NP> * 32 + (threadIdx.x & 31);
+  float* const st = lps_values<L, NP, C>(smem, grp);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const uint4* const wl = reinterpret_cast<const uint4*>(smem + L::W) + l * MB_STRIDE;
   const float* const vl = sv + V_BLOCK + l * VB_STRIDE;
@@ -1052,23 +1068,26 @@ __device__ __noinline__ void lps_ffn(int nb, int grp, int l) {
         for (int u = 0; u < 2; ++u) s = fmaf(z[i][2 * u + c], sv[V_PHEADW + 16 * i + 8 * u + g], s);
       s = gsum(s) + sv[V_PHEADB];
       const int row = 8 * grp + 2 * t + c;
-      if (g == 0 && row < nb) (GLOBAL ? reinterpret_cast<const LpsGlobal*>(smem + L::GL)->prob : rs.prob)[row] = 1.0f / (1.0f + expf(-s));
+      float* const prob = C > 0 ? reinterpret_cast<const LpsGlobal*>(smem + L::GL)->prob : rs.prob;
+      if (g == 0 && row < nb) prob[row] = 1.0f / (1.0f + expf(-s));
     }
   }
 }
 
-// 8 rows of the nb per warp, group grp; meet(): every warp of the sequence
-// sees the others' keys and values
-template <int CAP, int NR, int NP, bool GLOBAL, class Meet>
-__device__ __forceinline__ void lps_router(int nb, int grp, Meet meet) {
-  const bool on = 8 * grp < nb;
+// Groups of 8 rows of the nb, the warp's first and every C * kNW-th one from
+// there; meet(): every warp of the sequence sees the others' keys and values
+template <int CAP, int NR, int NP, int C, class Meet>
+__device__ __forceinline__ void lps_router(int nb, int first, Meet meet) {
+  constexpr int NG = lps_groups(C);
 #pragma unroll 1
   for (int l = 0; l < 2; ++l) {
-    if (on) lps_qkv<CAP, NR, NP, GLOBAL>(nb, grp, l);
+#pragma unroll 1
+    for (int i = 0, grp = first; i < NG && 8 * grp < nb; ++i, grp += C * kNW) lps_qkv<CAP, NR, NP, C>(nb, grp, l);
     meet();
-    if (on) {
-      lps_attend<CAP, NR, NP, GLOBAL>(nb, grp, l);
-      lps_ffn<CAP, NR, NP, GLOBAL>(nb, grp, l);
+#pragma unroll 1
+    for (int i = 0, grp = first; i < NG && 8 * grp < nb; ++i, grp += C * kNW) {
+      lps_attend<CAP, NR, NP, C>(nb, grp, l);
+      lps_ffn<CAP, NR, NP, C>(nb, grp, l);
     }
   }
 }
@@ -1250,10 +1269,10 @@ __global__ void __launch_bounds__(kT, 1) lbs_wide_kernel(const RowsParams p) {
 
 template <int C, int NR, int NP, int CAP>
 __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) {
-  using L = Lay<NR, NP>;
   // windows of more than 64 rows: the LBS and the statistics come from
   // lbs_wide_kernel
   constexpr bool kWide = CAP > 64;
+  using L = Lay<NR, NP, kWide ? lps_groups(C) : 1>;
   static_assert(kWide || CAP == 8 * NR * C, "rows of the cluster's groups");
   constexpr int NC = CAP / 32, RPT = (NC + kNW - 1) / kNW;
   extern __shared__ __align__(16) uint8_t smem[];
@@ -1311,7 +1330,8 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   const bool run_lbs = p.mode == EBD_DECODE_EB && meta_s == 0 && nM > p.l_min;
   auto copy_lps = [&]() {
     for (int i = tid; i < L::kLpsMat; i += kT)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem + L::W + 16 * i)), "l"(p.mat + M_BLOCK + i)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem + L::W + 16 * i)),
+                   "l"(p.mat + M_BLOCK + i)
                    : "memory");
   };
   if (kWide) {
@@ -1366,11 +1386,11 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
       __syncthreads();
       if (warm) {
         if (warp % 3 == 0)
-          lps_qkv<CAP, NR, NP, false>(64, warp, 0);
+          lps_qkv<CAP, NR, NP, 0>(64, warp, 0);
         else if (warp % 3 == 1)
-          lps_attend<CAP, NR, NP, false>(64, warp, 0);
+          lps_attend<CAP, NR, NP, 0>(64, warp, 0);
         else
-          lps_ffn<CAP, NR, NP, false>(64, warp, 0);
+          lps_ffn<CAP, NR, NP, 0>(64, warp, 0);
       }
     } else if (warm && run_lbs && nr > 0) {
       lbs_input<NR, NP>(la);
@@ -1499,10 +1519,10 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
             LpsGlobal{p.kvp + static_cast<size_t>(kbase) * 64 * NP, static_cast<size_t>(p.cap_rows) * 64 * NP,
                       static_cast<size_t>(capk) * 32 * NP, p.P + kbase};
       __syncthreads();
-      lps_router<CAP, NR, NP, true>(nBM, rank + C * warp, [] { cluster_barrier(); });
+      lps_router<CAP, NR, NP, C>(nBM, rank + C * warp, [] { cluster_barrier(); });
       cluster_barrier();  // every row's p_psi is visible
     } else {
-      lps_router<CAP, NR, NP, false>(nBM, warp, [] { __syncthreads(); });
+      lps_router<CAP, NR, NP, 0>(nBM, warp, [] { __syncthreads(); });
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -1584,7 +1604,7 @@ constexpr int rows_cap() {
 }
 template <int C, int NR, int NP>
 constexpr int smem_bytes() {
-  return Lay<NR, NP>::ROW + static_cast<int>(sizeof(RowState<rows_cap<C, NR, NP>()>));
+  return Lay<NR, NP, NP == 3 ? lps_groups(C) : 1>::ROW + static_cast<int>(sizeof(RowState<rows_cap<C, NR, NP>()>));
 }
 constexpr int kWideSmem = Lay<1, 3>::ROW + static_cast<int>(sizeof(RowState<kMaxSeqRows>));
 
@@ -1630,29 +1650,41 @@ cudaError_t launch_wide(void (*k)(RowsParams), const RowsParams& p, int groups, 
 }
 }  // namespace
 
-cudaError_t decide_rows_configure(int (&slots)[2]) {
+cudaError_t decide_rows_configure(DecideSlots& n) {
   cudaError_t e;
   const RowsParams none{};
   const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if ((e = configure_one<8, 1, 2>()) != cudaSuccess || (e = configure_one<4, 2, 2>()) != cudaSuccess ||
       (e = configure_one<2, 4, 2>()) != cudaSuccess || (e = configure_one<4, 1, 2>()) != cudaSuccess ||
       (e = configure_one<2, 2, 2>()) != cudaSuccess || (e = configure_one<1, 4, 2>()) != cudaSuccess ||
-      (e = configure_one<16, 1, 3>()) != cudaSuccess ||
+      (e = configure_one<16, 1, 3>()) != cudaSuccess || (e = configure_one<8, 1, 3>()) != cudaSuccess ||
+      (e = configure_one<4, 1, 3>()) != cudaSuccess || (e = configure_one<2, 1, 3>()) != cudaSuccess ||
       (e = cudaFuncSetAttribute(lbs_wide_kernel<0>, smem, kWideSmem)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(lbs_wide_kernel<1>, smem, kWideSmem)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(lbs_wide_kernel<2>, smem, kWideSmem)) != cudaSuccess ||
-      (e = launch_one<8, 1, 2>(none, nullptr, false, &slots[0])) != cudaSuccess ||
-      (e = launch_one<4, 2, 2>(none, nullptr, false, &slots[1])) != cudaSuccess)
+      (e = launch_one<8, 1, 2>(none, nullptr, false, &n.c8)) != cudaSuccess ||
+      (e = launch_one<4, 2, 2>(none, nullptr, false, &n.c4)) != cudaSuccess ||
+      (e = launch_one<16, 1, 3>(none, nullptr, false, &n.wide16)) != cudaSuccess ||
+      (e = launch_one<8, 1, 3>(none, nullptr, false, &n.wide8)) != cudaSuccess ||
+      (e = launch_one<4, 1, 3>(none, nullptr, false, &n.wide4)) != cudaSuccess)
     return e;
   return cudaSuccess;
 }
 
-// Clusters per sequence: as many CTAs as leave all sequences resident at once
+// CTAs per sequence: as many as leave all sequences resident at once
 // (ebd_decide, us, 8 CTAs of one group / 4 of two / 2 of four: 8 x 64 rows 35
-// / 42 / 55, 16 x 64 49 / 41 / 55, 36 x 64 68 / 43 / 53, 40 x 64 68 / 66 / 53;
-// windows of up to 32 rows, 4 of one / 2 of two / 1 of four: 16 x 32 33 / 41 /
-// 53, 40 x 32 48 / 40 / 52, 128 x 32 98 / 73 / 54).
-cudaError_t launch_decide_rows(const RowsParams& p, int cap, const int (&slots)[2], cudaStream_t st, bool pdl) {
+// / 42 / 55, 16 x 64 49 / 41 / 55, 36 x 64 68 / 43 / 53, 40 x 64 68 / 66 / 53).
+// Windows of up to 32 rows, 4 of one / 2 of two / 1 of four: 16 x 32 33 / 41 /
+// 53, 40 x 32 48 / 40 / 52, 128 x 32 98 / 73 / 54, with the same limits, which
+// are those of the larger kernels above.
+// Windows of more than 64 rows, 16 CTAs / 8 / 4 (two passes over the LPS rows of
+// a 512-row window) / 2 (four), LBS and LPS: 1 x 512 77 / 78 / 100 / 129, 8 x 512
+// 168 / 151 / 172 / 200, 16 x 128 125 / 102 / 87 / 89, 60 x 65 319 / 227 / 188 /
+// 169; inside a block 1 x 512 25.0 / 25.1 / 25.4 / 26.7, 8 x 512 54 / 39 / 39 /
+// 40, 32 x 128 134 / 100 / 70 / 70, 60 x 65 234 / 155 / 122 / 106.  (16 CTAs
+// whatever the batch were slower inside a block than the chain of grid-wide
+// kernels before them, 32 x 128 107 us, 60 x 65 127.)
+cudaError_t launch_decide_rows(const RowsParams& p, int cap, const DecideSlots& n, cudaStream_t st, bool pdl) {
   if (p.B <= 0 || p.R <= 0) return cudaSuccess;
   if (cap > 64) {
     cudaError_t e = cudaSuccess;
@@ -1666,14 +1698,16 @@ cudaError_t launch_decide_rows(const RowsParams& p, int cap, const int (&slots)[
     if (lbs && ((e = launch_wide(lbs_wide_kernel<1>, p, groups, st, true)) != cudaSuccess ||
                 (e = launch_wide(lbs_wide_kernel<2>, p, groups, st, true)) != cudaSuccess))
       return e;
-    return launch_one<16, 1, 3>(p, st, pdl, nullptr);
+    if (p.B <= n.wide16) return launch_one<16, 1, 3>(p, st, pdl, nullptr);
+    if (p.B <= n.wide8) return launch_one<8, 1, 3>(p, st, pdl, nullptr);
+    return p.B <= n.wide4 ? launch_one<4, 1, 3>(p, st, pdl, nullptr) : launch_one<2, 1, 3>(p, st, pdl, nullptr);
   }
   if (cap > 32) {
-    if (p.B <= slots[0]) return launch_one<8, 1, 2>(p, st, pdl, nullptr);
-    return p.B <= slots[1] ? launch_one<4, 2, 2>(p, st, pdl, nullptr) : launch_one<2, 4, 2>(p, st, pdl, nullptr);
+    if (p.B <= n.c8) return launch_one<8, 1, 2>(p, st, pdl, nullptr);
+    return p.B <= n.c4 ? launch_one<4, 2, 2>(p, st, pdl, nullptr) : launch_one<2, 4, 2>(p, st, pdl, nullptr);
   }
-  if (p.B <= slots[1]) return launch_one<4, 1, 2>(p, st, pdl, nullptr);
-  return p.B <= 2 * slots[1] ? launch_one<2, 2, 2>(p, st, pdl, nullptr) : launch_one<1, 4, 2>(p, st, pdl, nullptr);
+  if (p.B <= n.c4) return launch_one<4, 1, 2>(p, st, pdl, nullptr);
+  return p.B <= 2 * n.c4 ? launch_one<2, 2, 2>(p, st, pdl, nullptr) : launch_one<1, 4, 2>(p, st, pdl, nullptr);
 }
 
 }  // namespace ebd

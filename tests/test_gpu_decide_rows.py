@@ -1,9 +1,10 @@
 """The decision's launch shapes at their boundaries, on statistics given to
 ebd_decide: clusters of 8, 4 and 2 CTAs for windows of up to 64 rows (picked by
-the batch), of 4, 2 and 1 for up to 32 rows in batches of 16 and more; a CTA
-per group of 8 rows above 64 rows; windows of a row, of whole groups of 8 rows
-and one more or one less, with nothing masked, and blocks of every masked row
-(the LPS over the whole window)."""
+the batch), of 4, 2 and 1 for up to 32 rows in batches of 16 and more; above 64
+rows a CTA per group of 8 rows, then clusters of 16, 8, 4 and 2 CTAs, also with
+one window of 512 rows among many short ones; windows of a row, of whole groups
+of 8 rows and one more or one less, with nothing masked, and blocks of every
+masked row (the LPS over the whole window)."""
 import dataclasses
 
 import numpy as np
@@ -33,16 +34,28 @@ def _stats(rng, n, vocab, eos):
 @pytest.mark.parametrize("bias", [0.0, 8.0])
 @pytest.mark.parametrize("batch,window", [(1, 64), (1, 13), (2, 9), (9, 64), (20, 57), (37, 64), (44, 40),
                                           (16, 32), (40, 24), (90, 32), (140, 16), (1, 65), (2, 129), (1, 512),
-                                          (3, 300), (400, 12), (60, 68)])
+                                          (3, 300), (400, 12), (9, 129), (20, 200), (60, 68)])
 def test_decide_launch_shapes(batch, window, bias):
-    from paper_2609_16450_gb300 import _ebd as E
-    from paper_2609_16450_gb300 import runtime as rt
     rng = np.random.default_rng(batch * 1000 + window)
     ws = np.minimum(rng.integers(0, window + 1, batch), window)
     ws[0] = window
     ws[rng.integers(0, batch, batch // 4)] = 8 * (window // 8)
     while ws.sum() > 4096:
         ws[int(np.argmax(ws))] //= 2
+    _check(rng, ws, window, bias)
+
+
+@pytest.mark.parametrize("bias", [0.0, 8.0])
+@pytest.mark.parametrize("batch", [7, 15, 36, 38])
+def test_one_long_window_among_short_ones(batch, bias):
+    rng = np.random.default_rng(batch)
+    _check(rng, np.concatenate([[512], rng.integers(0, 70, batch - 1)]), 512, bias)
+
+
+def _check(rng, ws, window, bias):
+    from paper_2609_16450_gb300 import _ebd as E
+    from paper_2609_16450_gb300 import runtime as rt
+    batch = len(ws)
     sh = synth.tiny.with_(name=f"dec_{batch}_{window}", batch=batch, windows=tuple(int(w) for w in ws),
                           gen_len=max(512, window), prefix=0, mask_frac=0.8, seed=batch + window)
     inp = synth.make_step_inputs(sh)
