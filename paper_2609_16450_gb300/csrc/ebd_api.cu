@@ -623,6 +623,14 @@ ebd_status run_lm(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, bool p
   return EBD_OK;
 }
 
+// Rows that the decision's launch holds per sequence.  Windows of up to 32
+// rows take half the CTAs per sequence where the batch is large (below that,
+// a sequence may bring more rows than the handle announced).
+int rows_cap(const ebd_handle* h, int batch) {
+  if (h->cfg.max_window > kMaxWindow) return kMaxSeqRows;
+  return h->cfg.max_window <= 32 && batch >= 16 ? 32 : 64;
+}
+
 // features_in: a's statistics are inputs (device), else the LM head's
 // partial states are merged into them
 RowsParams rows_params(ebd_handle* h, const ebd_step_args* a, bool features_in) {
@@ -633,6 +641,7 @@ RowsParams rows_params(ebd_handle* h, const ebd_step_args* a, bool features_in) 
   p.V = c.vocab;
   p.grid_lm = h->grid_lm;
   p.features_in = features_in ? 1 : 0;
+  p.cap = rows_cap(h, a->batch);
   p.strict = c.max_window <= kMaxWindow ? 1 : 0;
   p.mode = c.decode_mode;
   p.top_m = c.top_m;
@@ -671,14 +680,6 @@ RowsParams rows_params(ebd_handle* h, const ebd_step_args* a, bool features_in) 
   p.status = h->d_status;
   return p;
 }
-// Rows that the decision's launch holds per sequence.  Windows of up to 32
-// rows take half the CTAs per sequence where the batch is large (below that,
-// a sequence may bring more rows than the handle announced).
-int rows_cap(const ebd_handle* h, int batch) {
-  if (h->cfg.max_window > kMaxWindow) return kMaxSeqRows;
-  return h->cfg.max_window <= 32 && batch >= 16 ? 32 : 64;
-}
-
 }  // namespace
 
 extern "C" {
@@ -1143,7 +1144,7 @@ ebd_status step_seq(ebd_handle* h, const ebd_step_args* a, cudaStream_t st) {
   ebd_status s = run_lm(h, a, st);
   if (s != EBD_OK) return s;
   if (prof && (e = record(h->ev[1], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
-  if ((e = launch_decide_rows(rows_params(h, a, false), kMaxSeqRows, h->rows_slots, st, prof == 0)) != cudaSuccess)
+  if ((e = launch_decide_rows(rows_params(h, a, false), h->rows_slots, st, prof == 0)) != cudaSuccess)
     return cuda_fail(h, e, "decision launch");
   if (prof && (e = record(h->ev[2], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
   if (prof && (e = record(h->ev[3], st)) != cudaSuccess) return cuda_fail(h, e, "profile event");
@@ -1179,7 +1180,7 @@ ebd_status step_run(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, cons
     p.in_block_out = rt->in_block_out;
     p.blk_meta_out = rt->blk_meta_out;
   }
-  cudaError_t e = launch_decide_rows(p, rows_cap(h, a->batch), h->rows_slots, st, prof == 0);
+  cudaError_t e = launch_decide_rows(p, h->rows_slots, st, prof == 0);
   if (e != cudaSuccess) return cuda_fail(h, e, "decision launch");
   if (prof == 1 && (e0 = record(h->ev[2], st)) != cudaSuccess)
     return cuda_fail(h, e0, "profile event");
@@ -1227,8 +1228,7 @@ ebd_status ebd_decide(ebd_handle* h, const ebd_step_args* a, void* stream) {
     return fail(h, EBD_ERR_INVALID_ARG, "conf/ent_norm/gap/argmax inputs must be set");
   if (h->w_emb == nullptr) return fail(h, EBD_ERR_STATE, "bind the token embedding first");
   if (a->rows == 0 || a->batch == 0) return EBD_OK;
-  cudaError_t e = launch_decide_rows(rows_params(h, a, true), rows_cap(h, a->batch), h->rows_slots,
-                                     static_cast<cudaStream_t>(stream), false);
+  cudaError_t e = launch_decide_rows(rows_params(h, a, true), h->rows_slots, static_cast<cudaStream_t>(stream), false);
   if (e != cudaSuccess) return cuda_fail(h, e, "decision launch");
   return EBD_OK;
 }

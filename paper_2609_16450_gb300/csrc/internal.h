@@ -78,6 +78,7 @@ inline int scratch_rows(int max_rows, int max_batch) {
 struct RowsParams {
   int B, R, V, grid_lm;     // grid_lm: LM-head partials per row
   int features_in;          // 1: s_conf/s_ent/s_gap/s_arg are inputs
+  int cap;                  // rows per sequence the launch has to hold: 32, 64 or kMaxSeqRows
   int strict;               // cu_rows[B] has to be R
   int warm;                 // launched behind the LM head: first passes on stand-in rows
   int spare_row;            // a row of s_* that no window row uses
@@ -127,14 +128,13 @@ cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const
                              const CUtensorMap& vw, const AttnParams& p, cudaStream_t st,
                              bool pdl = false);
 // the decision, the rows of a sequence split over a cluster of CTAs
-// (k_decide.cu); cap: rows per sequence the launch has to hold (32, 64
-// or kMaxSeqRows)
+// (k_decide.cu)
 struct DecideSlots {        // clusters that fit the GPU at once
   int c8, c4;               // windows of up to 64 rows: of 8 and of 4 CTAs
   int wide16, wide8, wide4; // of more: of 16, 8 and 4
 };
 cudaError_t decide_rows_configure(DecideSlots& n);
-cudaError_t launch_decide_rows(const RowsParams& p, int cap, const DecideSlots& n, cudaStream_t st, bool pdl);
+cudaError_t launch_decide_rows(const RowsParams& p, const DecideSlots& n, cudaStream_t st, bool pdl);
 // vocabulary-parallel LM head: one state per row from a launch's partials,
 // and the statistics from the states of several shards (k_stats.cu)
 cudaError_t launch_shard_state(const float4* part_f, const int* part_i, int rows, int grid,

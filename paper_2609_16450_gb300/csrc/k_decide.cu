@@ -1267,17 +1267,23 @@ __global__ void __launch_bounds__(kT, 1) lbs_wide_kernel(const RowsParams p) {
   }
 }
 
-template <int C, int NR, int NP, int CAP>
+// RULE: the baselines' rules (Reading R20) on statistics that are there, which
+// use no router: one CTA per sequence without the cluster's meetings, weights
+// and activations.  ebd_decide under the threshold rule with a copy of its
+// state, us in a graph, here / the 8-CTA cluster / the kernels before it: 1 x 64
+// rows 3.4 / 5.1 / 7.0, 16 x 32 4.2 / 5.5 / 6.4, 64 x 64 3.9 / 5.6 / 28; 1 x 512
+// 4.2 / - / 14.4.  Call by call the host's launches bound it, 16 to 17 us.
+template <int C, int NR, int NP, int CAP, bool RULE = false>
 __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) {
   // windows of more than 64 rows: the LBS and the statistics come from
   // lbs_wide_kernel
   constexpr bool kWide = CAP > 64;
   using L = Lay<NR, NP, kWide ? lps_groups(C) : 1>;
-  static_assert(kWide || CAP == 8 * NR * C, "rows of the cluster's groups");
+  static_assert(kWide || RULE || CAP == 8 * NR * C, "rows of the cluster's groups");
   constexpr int NC = CAP / 32, RPT = (NC + kNW - 1) / kNW;
   extern __shared__ __align__(16) uint8_t smem[];
   float* const sv = reinterpret_cast<float*>(smem + L::V);
-  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + L::ROW);
+  RowState<CAP>& rs = *reinterpret_cast<RowState<CAP>*>(smem + (RULE ? 0 : L::ROW));
   Slots& sl = *reinterpret_cast<Slots*>(smem + L::SLOT);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = static_cast<int>(cluster_ctarank());
@@ -1286,14 +1292,15 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   // on the SMs this grid leaves free once every CTA of it is resident
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  if (p.mode == EBD_DECODE_EB)  // the baselines' rules use no router
+  const bool eb = !RULE && p.mode == EBD_DECODE_EB;
+  if (eb)  // the baselines' rules use no router
     for (int i = tid; i < kVecs / 4; i += kT)
       reinterpret_cast<float4*>(sv)[i] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
 
   // ------------------------------------------------------------ decode state
   const int r0 = p.cu_rows[b];
   int n = p.cu_rows[b + 1] - r0;
-  const bool bad_seq = n < 0 || n > CAP || r0 < 0 || r0 + n > p.R ||
+  const bool bad_seq = n < 0 || n > (RULE ? p.cap : CAP) || r0 < 0 || r0 + n > p.R ||
                        (p.strict ? p.cu_rows[p.B] != p.R : n > p.gen_len);
   if (bad_seq) {
     if (rank == 0 && tid == 0) atomicCAS(p.status, 0, EBD_ERR_INVALID_ARG);
@@ -1303,7 +1310,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   int meta_b = p.blk_meta[2 * b], meta_s = p.blk_meta[2 * b + 1];
   bool m[RPT], inb[RPT], f[RPT];
   int pos[RPT], mrank[RPT], urank[RPT];
-  if (tid < 32) {
+  if (!RULE && tid < 32) {
     sl.mrow[tid] = -1;
     sl.ent[tid] = 0.f;
     sl.arg[tid] = -1;
@@ -1326,15 +1333,18 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     f[i] = row && !m[i];
   }
   const int nM = rank_rows<CAP>(rs, m, mrank);
-  const int nU = kWide ? 0 : rank_rows<CAP>(rs, f, urank);
-  const bool run_lbs = p.mode == EBD_DECODE_EB && meta_s == 0 && nM > p.l_min;
+  const int nU = kWide || RULE ? 0 : rank_rows<CAP>(rs, f, urank);
+  const bool run_lbs = eb && meta_s == 0 && nM > p.l_min;
   auto copy_lps = [&]() {
     for (int i = tid; i < L::kLpsMat; i += kT)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem + L::W + 16 * i)),
                    "l"(p.mat + M_BLOCK + i)
                    : "memory");
   };
-  if (kWide) {
+  if constexpr (RULE) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __syncthreads();
+  } else if constexpr (kWide) {
     if (p.lps_enabled) copy_lps();
     // Rank 0 commits in place, and where no LPS follows nothing else stands
     // between a CTA's reads of the decode state above and that commit.  (In a
@@ -1368,7 +1378,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 
     // The LM head has streamed its weight through L2: bring the router's back
     // while its last CTAs run.
-    if (b == 0 && p.mode == EBD_DECODE_EB) {
+    if (b == 0 && eb) {
       const char* w = reinterpret_cast<const char*>(p.mat);
       for (int i = (run_lbs ? 0 : M_BLOCK / 8) + rank * kT + tid; i < M_TOTAL / 8; i += C * kT)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 128 * static_cast<size_t>(i)));
@@ -1379,7 +1389,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     // several times as much): meanwhile CTA 0 runs the LPS router, one part
     // per warp, the others the LBS input layers and the first QKV product, on
     // stand-in rows.
-    const bool warm = p.warm != 0 && C == 8 && p.mode == EBD_DECODE_EB;
+    const bool warm = p.warm != 0 && C == 8 && eb;
     if (apart && rank == 0 && p.lps_enabled) {
       copy_lps();
       asm volatile("cp.async.wait_all;" ::: "memory");
@@ -1449,7 +1459,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
       if (run_lbs && m[i]) lbs[i] = __ldcg(p.O + kbase + mrank[i]);
     }
   }
-  if (p.mode != EBD_DECODE_EB) {
+  if (!eb) {
 #pragma unroll
     for (int i = 0; i < RPT; ++i) sel[i] = 32 * (warp + kNW * i) + lane < n;  // the window is the block
   } else if (meta_s != 0) {
@@ -1496,10 +1506,10 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 #pragma unroll
   for (int i = 0; i < RPT; ++i) f[i] = sel[i] && m[i] && !bad[i];
   const int nBM = rank_rows<CAP>(rs, f, brank);
-  const bool run_lps = p.mode == EBD_DECODE_EB && p.lps_enabled && nBM > 0;
+  const bool run_lps = eb && p.lps_enabled && nBM > 0;
 
   // ------------------------------------------------------------ LPS
-  if (run_lps) {
+  if (!RULE && run_lps) {
     const float rho = static_cast<float>(nBM) / static_cast<float>(meta_s);
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
@@ -1513,7 +1523,8 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    if (kWide) {
+    if constexpr (RULE) {
+    } else if constexpr (kWide) {
       if (tid == 0)
         *reinterpret_cast<LpsGlobal*>(smem + L::GL) =
             LpsGlobal{p.kvp + static_cast<size_t>(kbase) * 64 * NP, static_cast<size_t>(p.cap_rows) * 64 * NP,
@@ -1525,7 +1536,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
       lps_router<CAP, NR, NP, 0>(nBM, warp, [] { __syncthreads(); });
     }
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (!RULE) asm volatile("cp.async.wait_all;" ::: "memory");
   if (rank != 0 || bad_seq) return;
 
   // ------------------------------------------------------------ accept, commit
@@ -1574,11 +1585,11 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
     m[i] = m[i] && !acc[i];
-    if (p.mode != EBD_DECODE_EB) sel[i] = inb[i];  // no block state
+    if (!eb) sel[i] = inb[i];  // no block state
     if (sel[i] && m[i]) rs.open = 1;
   }
   __syncthreads();
-  const bool resolve = p.mode == EBD_DECODE_EB && meta_s > 0 && !rs.open;
+  const bool resolve = eb && meta_s > 0 && !rs.open;
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
     const int j = 32 * (warp + kNW * i) + lane, r = r0 + j;
@@ -1635,6 +1646,21 @@ cudaError_t launch_one(const RowsParams& p, cudaStream_t st, bool pdl, int* slot
   if (slots != nullptr) return cudaOccupancyMaxActiveClusters(slots, k, &cfg);
   return cudaLaunchKernelEx(&cfg, k, p);
 }
+template <int CAP>
+cudaError_t launch_rule(const RowsParams& p, cudaStream_t st, bool pdl) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(p.B));
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = sizeof(RowState<CAP>);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  static_assert(sizeof(RowState<CAP>) <= 48 * 1024, "dynamic shared memory without an attribute");
+  return cudaLaunchKernelEx(&cfg, decide_rows_kernel<1, 1, 2, CAP, true>, p);
+}
 cudaError_t launch_wide(void (*k)(RowsParams), const RowsParams& p, int groups, cudaStream_t st, bool pdl) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(groups), static_cast<unsigned>(p.B));
@@ -1684,25 +1710,27 @@ cudaError_t decide_rows_configure(DecideSlots& n) {
 // 40, 32 x 128 134 / 100 / 70 / 70, 60 x 65 234 / 155 / 122 / 106.  (16 CTAs
 // whatever the batch were slower inside a block than the chain of grid-wide
 // kernels before them, 32 x 128 107 us, 60 x 65 127.)
-cudaError_t launch_decide_rows(const RowsParams& p, int cap, const DecideSlots& n, cudaStream_t st, bool pdl) {
+cudaError_t launch_decide_rows(const RowsParams& p, const DecideSlots& n, cudaStream_t st, bool pdl) {
   if (p.B <= 0 || p.R <= 0) return cudaSuccess;
-  if (cap > 64) {
+  const bool eb = p.mode == EBD_DECODE_EB;
+  if (p.cap > 64) {
     cudaError_t e = cudaSuccess;
-    const bool lbs = p.mode == EBD_DECODE_EB;
     // a sequence may bring more rows than announced, up to all of the step's
     const int most = p.gen_len < p.R ? p.gen_len : p.R, groups = ((most < kMaxSeqRows ? most : kMaxSeqRows) + 7) / 8;
-    if (lbs || !p.features_in) {
+    if (eb || !p.features_in) {
       if ((e = launch_wide(lbs_wide_kernel<0>, p, groups, st, pdl)) != cudaSuccess) return e;
       pdl = true;
     }
-    if (lbs && ((e = launch_wide(lbs_wide_kernel<1>, p, groups, st, true)) != cudaSuccess ||
-                (e = launch_wide(lbs_wide_kernel<2>, p, groups, st, true)) != cudaSuccess))
+    if (!eb) return launch_rule<kMaxSeqRows>(p, st, pdl);
+    if ((e = launch_wide(lbs_wide_kernel<1>, p, groups, st, true)) != cudaSuccess ||
+        (e = launch_wide(lbs_wide_kernel<2>, p, groups, st, true)) != cudaSuccess)
       return e;
     if (p.B <= n.wide16) return launch_one<16, 1, 3>(p, st, pdl, nullptr);
     if (p.B <= n.wide8) return launch_one<8, 1, 3>(p, st, pdl, nullptr);
     return p.B <= n.wide4 ? launch_one<4, 1, 3>(p, st, pdl, nullptr) : launch_one<2, 1, 3>(p, st, pdl, nullptr);
   }
-  if (cap > 32) {
+  if (!eb && p.features_in) return launch_rule<64>(p, st, pdl);
+  if (p.cap > 32) {
     if (p.B <= n.c8) return launch_one<8, 1, 2>(p, st, pdl, nullptr);
     return p.B <= n.c4 ? launch_one<4, 2, 2>(p, st, pdl, nullptr) : launch_one<2, 4, 2>(p, st, pdl, nullptr);
   }
