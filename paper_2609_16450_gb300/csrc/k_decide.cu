@@ -1293,8 +1293,10 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   // on the SMs this grid leaves free once every CTA of it is resident
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  const bool eb = !RULE && p.mode == EBD_DECODE_EB;
-  if (eb)  // the baselines' rules use no router
+  // (asked anew at each use: held in a register, which the kernels of 252 lack,
+  // 64 x 64 rows take 52.4 us instead of 51.4)
+  auto eb = [&]() { return !RULE && p.mode == EBD_DECODE_EB; };
+  if (eb())  // the baselines' rules use no router
     for (int i = tid; i < kVecs / 4; i += kT)
       reinterpret_cast<float4*>(sv)[i] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
 
@@ -1335,7 +1337,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
   }
   const int nM = rank_rows<CAP>(rs, m, mrank);
   const int nU = kWide || RULE ? 0 : rank_rows<CAP>(rs, f, urank);
-  const bool run_lbs = eb && meta_s == 0 && nM > p.l_min;
+  const bool run_lbs = eb() && meta_s == 0 && nM > p.l_min;
   auto copy_lps = [&]() {
     for (int i = tid; i < L::kLpsMat; i += kT)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem + L::W + 16 * i)),
@@ -1379,7 +1381,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 
     // The LM head has streamed its weight through L2: bring the router's back
     // while its last CTAs run.
-    if (b == 0 && eb) {
+    if (b == 0 && eb()) {
       const char* w = reinterpret_cast<const char*>(p.mat);
       for (int i = (run_lbs ? 0 : M_BLOCK / 8) + rank * kT + tid; i < M_TOTAL / 8; i += C * kT)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 128 * static_cast<size_t>(i)));
@@ -1390,7 +1392,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     // several times as much): meanwhile CTA 0 runs the LPS router, one part
     // per warp, the others the LBS input layers and the first QKV product, on
     // stand-in rows.
-    const bool warm = p.warm != 0 && C == 8 && eb;
+    const bool warm = p.warm != 0 && C == 8 && eb();
     if (apart && rank == 0 && p.lps_enabled) {
       copy_lps();
       asm volatile("cp.async.wait_all;" ::: "memory");
@@ -1460,7 +1462,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
       if (run_lbs && m[i]) lbs[i] = __ldcg(p.O + kbase + mrank[i]);
     }
   }
-  if (!eb) {
+  if (!eb()) {
 #pragma unroll
     for (int i = 0; i < RPT; ++i) sel[i] = 32 * (warp + kNW * i) + lane < n;  // the window is the block
   } else if (meta_s != 0) {
@@ -1507,7 +1509,7 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 #pragma unroll
   for (int i = 0; i < RPT; ++i) f[i] = sel[i] && m[i] && !bad[i];
   const int nBM = rank_rows<CAP>(rs, f, brank);
-  const bool run_lps = eb && p.lps_enabled && nBM > 0;
+  const bool run_lps = eb() && p.lps_enabled && nBM > 0;
 
   // ------------------------------------------------------------ LPS
   if (!RULE && run_lps) {
@@ -1606,11 +1608,11 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
     m[i] = m[i] && !acc[i];
-    if (!eb) sel[i] = inb[i];  // no block state
+    if (!eb()) sel[i] = inb[i];  // no block state
     if (sel[i] && m[i]) rs.open = 1;
   }
   __syncthreads();
-  const bool resolve = eb && meta_s > 0 && !rs.open;
+  const bool resolve = eb() && meta_s > 0 && !rs.open;
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
     const int j = 32 * (warp + kNW * i) + lane, r = r0 + j;
