@@ -706,17 +706,23 @@ void lm_plan(LmParams& p, int rows, int V, int d, int num_sms, bool pair) {
     p.grp_cols = p.grid;
   }
   p.ncols = p.grp_cols;  // partial states per row (a caller may raise it: neutral states)
-  // a second epilogue warpgroup (and its transpose buffer) only pays where
-  // the epilogue is exposed, i.e. with a single accumulator buffer; with two,
-  // one warpgroup keeps up with the MMAs and its buffer is worth more as
-  // pipeline stages (measured with 128-row tiles: 256 rows 270.7 -> 247.2 us)
-  p.nwg = p.nbuf == 1 ? 2 : 1;
+  // A second epilogue warpgroup (and its transpose buffer) pays where the
+  // epilogue is exposed: with a single accumulator buffer, and in row groups
+  // whose chunks' MMAs take less time than their epilogue, up to 1536 columns.
+  // Wider, one keeps up with the MMAs and the buffer is worth more as a pipeline
+  // stage.  57381 entries, packed, us, one / two: 336 columns 300 rows 47 / 37,
+  // 400 rows 61 / 46, 512 rows 69 / 54; 768 columns 400 rows 64 / 49; 1536
+  // columns 300 rows 57 / 53, 512 rows 78 / 78; 152064 entries, 2048 columns 432
+  // rows 207 / 195, 512 rows 241 / 255.  (One group of two N sub-tiles, with its
+  // single accumulator buffer and two warpgroups, took 45, 52 and 62 us at 336
+  // columns 300 and 400 rows and 768 columns 400 rows.)
+  p.nkb = (d + 63) / 64;
+  p.nwg = p.nbuf == 1 || (p.rgroups > 1 && p.nkb <= 24) ? 2 : 1;
   if (const char* env = getenv("EBD_LM_NWG")) p.nwg = atoi(env) == 2 ? 2 : 1;
   const uint32_t st_bytes = static_cast<uint32_t>(p.n_pad) * 20u;
   const uint32_t tail = kTBytes * static_cast<uint32_t>(p.nwg) + ((st_bytes + 7) / 8 * 8) +
                         (2 * 8 + 6) * 8 + 16;
   const uint32_t budget = 232448u - 1024u - tail;
-  p.nkb = (d + 63) / 64;
   // hidden bytes per k-box in one CTA: all rows, or half of them in a pair
   const uint32_t b_box = static_cast<uint32_t>(pair ? p.n_pad / 2 : p.n_pad) * 128u;
   // k-boxes (64 columns each) per pipeline stage, while keeping at least two

@@ -1,8 +1,8 @@
 """The LM head's launch shapes at their boundaries, every row against the
 oracle, through ebd_lm_stats: one CTA per SM below 65 rows, CTA pairs
-(cta_group::2) from 65 rows, two row groups above 432 rows, two N sub-tiles
-between 257 and 432 rows; a vocabulary that ends in a partial 64-row unit
-(4000 entries); both W layouts; and vocabulary shards so small that the odd
+(cta_group::2) from 65 rows, two row groups from 257 rows (with a second
+epilogue warpgroup up to 1536 columns); a vocabulary that ends in a partial
+64-row unit (4000 entries); both W layouts; and vocabulary shards so small that the odd
 CTA of a pair has no W rows in some chunks (ebd_lm_shard_state)."""
 import numpy as np
 import pytest
@@ -97,4 +97,13 @@ def test_spread_vocabulary_chunks(rows, units):
     """A row-major W of six chunks and more per owner (from 1824 units on for
     76 pairs): every nwork-th chunk, the last one of a single row."""
     rep = _run(_shape(rows, (units - 1) * 64 + 1).with_(d_model=128), "rowmajor")
+    assert rep["conf"] <= 2e-3
+
+
+@pytest.mark.parametrize("rows", [257, 300, 512])
+@pytest.mark.parametrize("d_model", [64, 1536, 1544])
+def test_epilogue_warpgroups(rows, d_model):
+    """Two epilogue warpgroups for row groups of up to 1536 columns, one above;
+    64 columns are a single k-box, so that the epilogue alone sets the pace."""
+    rep = _run(_shape(rows, 12000).with_(d_model=d_model), "packed" if rows % 2 else "rowmajor")
     assert rep["conf"] <= 2e-3
