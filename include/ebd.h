@@ -276,14 +276,15 @@ ebd_status ebd_lm_shard_state(ebd_handle* h, const ebd_step_args* a, int32_t v_o
 ebd_status ebd_merge_shard_states(ebd_handle* h, const float* states, int32_t shards,
                                   const ebd_step_args* a, void* stream);
 
-/* Only step 1 (window attention): writes a->attn_out.  The handle picks one
- * of two kernels when it is created: the tcgen05 kernel (S and O in tensor
- * memory, one CTA per SM) for long key ranges with few tiles or with query
- * tiles of more than 32 rows, the mma.sync kernel (two or three CTAs per SM)
- * otherwise; both compute the same attention.  The environment variables
- * EBD_ATTN_KERNEL = "tc" or "mma", EBD_ATTN_SPLITS (key splits per query
- * tile, 1..8) and EBD_ATTN_STAGES (ring of the mma.sync kernel: 2, three
- * CTAs per SM, or 3, two), read at ebd_create, override the choices. */
+/* Only step 1 (window attention): writes a->attn_out.  A call takes one of two
+ * kernels by its sequences and the handle's heads, max_window and max_prefix:
+ * the tcgen05 kernel (S and O in tensor memory, one CTA per SM) for long key
+ * ranges with few tiles or with query tiles of more than 32 rows, the mma.sync
+ * kernel (two or three CTAs per SM) otherwise; both compute the same attention.
+ * The environment variables EBD_ATTN_KERNEL = "tc" or "mma", EBD_ATTN_SPLITS
+ * (key splits per query tile, 1..8) and EBD_ATTN_STAGES (ring of the mma.sync
+ * kernel: 2, three CTAs per SM, or 3, two), read at ebd_create, override the
+ * choices. */
 ebd_status ebd_attention(ebd_handle* h, const ebd_step_args* a, void* stream);
 
 /* Synchronises `stream`, returns the first device-side failure recorded

@@ -38,7 +38,6 @@ using namespace ebd;
 namespace {
 
 constexpr uint64_t kLimitNs = 1000ull * 1000 * 1000;  // 1 s per device-side wait
-constexpr int kMaxSplits = kMaxAttnSplits;
 
 // ------------------------------------------------------------------ router layout
 struct TensorDesc {
@@ -238,9 +237,9 @@ struct ebd_handle {
   float* attn_part = nullptr;
   float* attn_part_ml = nullptr;
   int* tickets = nullptr;
-  int attn_splits = 1, attn_max_qtiles = 1;
-  int attn_stages = kAttnStages;
-  int attn_tc = 1;         // window attention on tcgen05 (else the mma.sync kernel)
+  int attn_max_qtiles = 1;
+  // EBD_ATTN_KERNEL (1: tcgen05, 0: mma.sync), _SPLITS and _STAGES, where set
+  int attn_force_tc = -1, attn_force_splits = 0, attn_force_stages = 0;
   int* d_status = nullptr;
   int* h_status = nullptr;  // pinned: where ebd_sync_status reads the word
   uint8_t* staging = nullptr;
@@ -497,6 +496,78 @@ ebd_status check_args(ebd_handle* h, const ebd_step_args* a, bool need_attn, boo
   return EBD_OK;
 }
 
+// How the window attention of `batch` sequences runs.
+struct AttnPlan {
+  int tc;      // 1: the tcgen05 kernel, 0: the mma.sync kernel
+  int slots;   // query tiles of 64 rows
+  int splits, split_from;  // key splits of each that has at least split_from chunks of keys
+  int stages;  // ring of the mma.sync kernel
+};
+AttnPlan attn_plan(const ebd_handle* h, int batch) {
+  const ebd_config& c = h->cfg;
+  // Both attention kernels take 64-row query tiles.  The tcgen05 kernel
+  // holds an SM alone (one CTA per SM) and pays a fixed setup and drain
+  // per CTA (TMEM, barriers, the query tile, its output), which long key
+  // ranges amortise; the mma.sync kernel runs two or three CTAs per SM, and
+  // with tiles of up to 32 rows it reads the cache as fast, its warps
+  // sharing each chunk's keys.  So, measured (attention alone, LLaDA-8B
+  // heads, us, mma.sync against tcgen05 in the better of their splits):
+  //   more tiles than SMs: 64 x 1024 x 32 rows 183 / 228, 64 x 4096 x 32
+  //     630 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 44 / 53; but tiles
+  //     of 33 to 64 rows over more than 8 chunks 62 / 62 (16 x 640 x 64), 298
+  //     / 235 (64 x 900 x 64), Dream-7B heads 51 / 43 (36 x 640 x 21), 120 /
+  //     86 (64 x 900 x 21), at 8 chunks 167 / 168 (64 x 400 x 64), 40 / 37
+  //     (36 x 400 x 21), below that 117 / 153 (64 x 250 x 64);
+  //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
+  //     47, 1 x 4096 x 32 26.5 / 21, but at 256 keys 10.8 / 12.2; with tiles
+  //     of 33 to 64 rows 14 / 13 at 250 keys (8 x 250 x 21, Dream-7B heads),
+  //     12.3 / 12.3 at 180, 10.8 / 12.2 at 120.
+  // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count,
+  // EBD_ATTN_STAGES the ring's stages (measurement sweeps).
+  // The tiles are the call's own.  Planned for the handle's largest batch
+  // instead, one sequence on a handle for 64 took, 4096 x 32 rows 70 us (now 22),
+  // 4096 x 8 50 (20), 1024 x 32 21 (12); with four sequences 4096 x 32 71 (47).
+  AttnPlan p{};
+  const int rows = (c.max_window < kMaxWindow ? c.max_window : kMaxWindow) * (c.n_heads_q / c.n_heads_kv);
+  const int nch = (c.max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
+  p.slots = batch * c.n_heads_kv * h->attn_max_qtiles;
+  const bool one_wave = p.slots <= h->num_sms;
+  p.tc = rows > 32 ? nch >= (one_wave ? 4 : 9) : (one_wave && nch >= 9);
+  if (h->attn_force_tc >= 0) p.tc = h->attn_force_tc;
+  // key splits per tile: as many as keep one wave of CTAs, of at least 4
+  // chunks each with the prefix at its longest (a CTA more than the SMs hold
+  // costs a second wave: 1 x 4096 x 8 rows on tcgen05 28.7 us with 5 splits, 18.7
+  // with 4).  On tcgen05, with its longer steps, a split's partials cost as much
+  // as it saves below 16 chunks (2 x 452 x 50 rows 14.5 us unsplit, 16.4 with 2; 2
+  // x 1024 x 50 18.6 either way, 2 x 2048 x 50 26.8 / 22.7); and five to seven are
+  // no better than four (Dream-7B heads 2 x 1600 x 16 16.5 with 4, 18.6 with 5 to
+  // 7; 2 x 2048 x 4 16.4 with 4, 14.5 with 8).  Sequences whose own keys stay
+  // below the first line are left whole (1 x 256 x 32 rows in a cache for 1024
+  // 11 us split, 9.8 whole).
+  p.split_from = p.tc ? 16 : 8;
+  p.splits = (p.tc ? h->num_sms : 2 * h->num_sms) / p.slots;
+  if (p.splits > nch / 4) p.splits = nch / 4;
+  if (nch < p.split_from) p.splits = 1;
+  if (p.tc && p.splits > 4 && p.splits < 8) p.splits = 4;
+  if (p.splits > kMaxAttnSplits) p.splits = kMaxAttnSplits;
+  if (p.splits < 1) p.splits = 1;
+  if (h->attn_force_splits != 0) {
+    p.splits = h->attn_force_splits < nch ? h->attn_force_splits : nch;
+    p.split_from = 0;
+  }
+  // CTAs per SM of the mma.sync kernel: two with a ring of three stages or
+  // three with two.  Three hide more of the CTAs' starts and ends and of the
+  // work between copies (us, two / three: 10 x 1024 x 8 rows 45 / 33, 12 x
+  // 4096 x 8 146 / 122, 24 x 1024 x 32 86 / 79, 64 x 256 x 32 81 / 69, 64 x
+  // 1024 x 32 193 / 183), but a wave of them takes longer: two where three
+  // would leave a last wave too empty (16 x 1024 x 8, 512 CTAs, 50 / 60; but
+  // 32 x 1024 x 8, 1024 CTAs, 94 / 95, x 32 rows 111 / 106).
+  auto waves = [&](int per_sm) { return (p.slots * p.splits + per_sm * h->num_sms - 1) / (per_sm * h->num_sms); };
+  p.stages = 6 * waves(3) <= 5 * waves(2) ? 2 : kAttnStages;
+  if (h->attn_force_stages != 0) p.stages = h->attn_force_stages;
+  return p;
+}
+
 ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
                          bool pdl = false, bool wait_prior = false, const unsigned* ready = nullptr,
                          unsigned ready_ticket = 0) {
@@ -514,7 +585,8 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   // all dims of a head for the mma.sync kernel, half by half (dim of the half,
   // key, half, head(, sequence))
   bool ok;
-  if (h->attn_tc) {
+  const AttnPlan plan = attn_plan(h, a->batch);
+  if (plan.tc) {
     const uint64_t cdims[4] = {static_cast<uint64_t>(D), H, Pm, Bc}, wdims[3] = {static_cast<uint64_t>(D), H, R};
     const uint64_t cstr[3] = {head, row, Pm * row}, wstr[2] = {head, row};
     const uint32_t cbox[4] = {64, 1, 64, 1}, wbox[3] = {64, 1, 64};
@@ -537,9 +609,10 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   p.group = c.n_heads_q / Hkv;
   p.max_prefix = c.max_prefix;
   p.max_qtiles = h->attn_max_qtiles;
-  p.splits = h->attn_splits;
-  p.stages = h->attn_stages;
-  p.tc = h->attn_tc;
+  p.splits = plan.splits;
+  p.split_from = plan.split_from;
+  p.stages = plan.stages;
+  p.tc = plan.tc;
   p.cu_rows = a->cu_rows;
   p.prefix_len = a->prefix_len;
   p.suffix = c.max_prefix > 0 ? a->suffix : nullptr;
@@ -815,66 +888,27 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     return bail(cuda_fail(h, e, "cudaMalloc(partials)"));
   // attention split-KV workspace
   {
-    // Both attention kernels take 64-row query tiles.  The tcgen05 kernel
-    // holds an SM alone (one CTA per SM) and pays a fixed setup and drain
-    // per CTA (TMEM, barriers, the query tile, its output), which long key
-    // ranges amortise; the mma.sync kernel runs two or three CTAs per SM, and
-    // with tiles of up to 32 rows it reads the cache as fast, its warps
-    // sharing each chunk's keys.  So, measured (attention alone, LLaDA-8B
-    // heads, us, mma.sync against tcgen05 in the better of their splits):
-    //   more tiles than SMs: 64 x 1024 x 32 rows 183 / 228, 64 x 4096 x 32
-    //     630 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 44 / 53; but tiles
-    //     of 33 to 64 rows over more than 8 chunks 62 / 62 (16 x 640 x 64), 298
-    //     / 235 (64 x 900 x 64), Dream-7B heads 51 / 43 (36 x 640 x 21), 120 /
-    //     86 (64 x 900 x 21), at 8 chunks 167 / 168 (64 x 400 x 64), 40 / 37
-    //     (36 x 400 x 21), below that 117 / 153 (64 x 250 x 64);
-    //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
-    //     47, 1 x 4096 x 32 26.5 / 21, but at 256 keys 10.8 / 12.2; with tiles
-    //     of 33 to 64 rows 14 / 13 at 250 keys (8 x 250 x 21, Dream-7B heads),
-    //     12.3 / 12.3 at 180, 10.8 / 12.2 at 120.
-    // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count,
-    // EBD_ATTN_STAGES the ring's stages (measurement sweeps).
     const int tile = 64;
-    const int group = cfg->n_heads_q / cfg->n_heads_kv;
     const int aw = cfg->max_window < kMaxWindow ? cfg->max_window : kMaxWindow;
-    h->attn_max_qtiles = (aw * group + tile - 1) / tile;
+    h->attn_max_qtiles = (aw * (cfg->n_heads_q / cfg->n_heads_kv) + tile - 1) / tile;
+    if (const char* env = getenv("EBD_ATTN_KERNEL")) h->attn_force_tc = strcmp(env, "mma") == 0 ? 0 : 1;
+    if (const char* env = getenv("EBD_ATTN_SPLITS")) {
+      const int n = atoi(env);
+      h->attn_force_splits = n < 1 ? 1 : n > kMaxAttnSplits ? kMaxAttnSplits : n;
+    }
+    if (const char* env = getenv("EBD_ATTN_STAGES")) h->attn_force_stages = atoi(env) == 2 ? 2 : kAttnStages;
+    // partials of the largest launch that splits its tiles, over all batches
     const int slots = cfg->max_batch * cfg->n_heads_kv * h->attn_max_qtiles;
-    const int nch = (cfg->max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
-    const bool one_wave = slots <= h->num_sms;
-    h->attn_tc = aw * group > 32 ? nch >= (one_wave ? 4 : 9) : (one_wave && nch >= 9);
-    if (const char* env = getenv("EBD_ATTN_KERNEL")) h->attn_tc = strcmp(env, "mma") == 0 ? 0 : 1;
-    // key splits per tile: as many as keep one wave of CTAs, of at least 4
-    // chunks each (a CTA more than the SMs hold costs a second wave: 1 x 4096
-    // x 8 rows on tcgen05 28.7 us with 5 splits, 18.7 with 4).  On tcgen05,
-    // with its longer steps, a split's partials cost as much as it saves below
-    // 16 chunks (2 x 452 x 50 rows 14.5 us unsplit, 16.4 with 2; 2 x 1024 x 50
-    // 18.6 either way, 2 x 2048 x 50 26.8 / 22.7); and five to seven are no
-    // better than four (Dream-7B heads 2 x 1600 x 16 16.5 with 4, 18.6 with 5 to
-    // 7; 2 x 2048 x 4 16.4 with 4, 14.5 with 8).
-    int splits = (h->attn_tc ? h->num_sms : 2 * h->num_sms) / slots;
-    if (splits > nch / 4) splits = nch / 4;
-    if (h->attn_tc && nch < 16) splits = 1;
-    if (h->attn_tc && splits > 4 && splits < 8) splits = 4;
-    if (const char* env = getenv("EBD_ATTN_SPLITS")) splits = atoi(env);
-    if (splits > kMaxSplits) splits = kMaxSplits;
-    if (splits > nch) splits = nch;
-    if (splits < 1) splits = 1;
-    h->attn_splits = splits;
-    // CTAs per SM of the mma.sync kernel: two with a ring of three stages or
-    // three with two.  Three hide more of the CTAs' starts and ends and of the
-    // work between copies (us, two / three: 10 x 1024 x 8 rows 45 / 33, 12 x
-    // 4096 x 8 146 / 122, 24 x 1024 x 32 86 / 79, 64 x 256 x 32 81 / 69, 64 x
-    // 1024 x 32 193 / 183), but a wave of them takes longer: two where three
-    // would leave a last wave too empty (16 x 1024 x 8, 512 CTAs, 50 / 60; but
-    // 32 x 1024 x 8, 1024 CTAs, 94 / 95, x 32 rows 111 / 106).
-    auto waves = [&](int per_sm) { return (slots * splits + per_sm * h->num_sms - 1) / (per_sm * h->num_sms); };
-    h->attn_stages = 6 * waves(3) <= 5 * waves(2) ? 2 : kAttnStages;
-    if (const char* env = getenv("EBD_ATTN_STAGES")) h->attn_stages = atoi(env) == 2 ? 2 : kAttnStages;
-    if (splits > 1) {
-      const size_t bytes = static_cast<size_t>(slots) * splits * tile * (cfg->head_dim + 2) * 4;
-      if ((e = cudaMalloc(&h->attn_part, bytes)) != cudaSuccess)
+    size_t parts = 0;
+    for (int b = 1; b <= cfg->max_batch; ++b) {
+      const AttnPlan p = attn_plan(h, b);
+      const size_t n = static_cast<size_t>(p.slots) * p.splits;
+      if (p.splits > 1 && n > parts) parts = n;
+    }
+    if (parts > 0) {
+      if ((e = cudaMalloc(&h->attn_part, parts * tile * (cfg->head_dim + 2) * 4)) != cudaSuccess)
         return bail(cuda_fail(h, e, "cudaMalloc(attention partials)"));
-      h->attn_part_ml = h->attn_part + static_cast<size_t>(slots) * splits * tile * cfg->head_dim;
+      h->attn_part_ml = h->attn_part + parts * tile * cfg->head_dim;
     }
     if ((e = cudaMalloc(&h->tickets, static_cast<size_t>(slots) * sizeof(int))) != cudaSuccess)
       return bail(cuda_fail(h, e, "cudaMalloc(tickets)"));

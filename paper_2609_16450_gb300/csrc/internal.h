@@ -46,7 +46,8 @@ struct AttnParams {
   int B, Hq, Hkv, D, group;
   int R;                    // rows of the step (extent of q and out)
   int max_prefix;
-  int max_qtiles, splits;
+  int max_qtiles, splits;   // key splits of a tile with at least
+  int split_from;           // split_from chunks of keys; the others have one
   int stages;               // ring of the mma.sync kernel: kAttnStages, or 2 for three CTAs per SM
   int tc;                   // 1: the tcgen05 kernel, 0: the mma.sync kernel (64-row tiles)
   const int* cu_rows;

@@ -182,8 +182,10 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
   }
   const int ncc = (P + kAttnChunk - 1) / kAttnChunk;
   const int nch = ncc + 1 + (S + kAttnChunk - 1) / kAttnChunk;
-  const int c0 = static_cast<int>((static_cast<long long>(split) * nch) / p.splits);
-  const int c1 = static_cast<int>((static_cast<long long>(split + 1) * nch) / p.splits);
+  const bool whole = p.splits == 1 || nch < p.split_from;  // the first split takes the keys
+  if (whole && split > 0) return;
+  const int c0 = whole ? 0 : static_cast<int>((static_cast<long long>(split) * nch) / p.splits);
+  const int c1 = whole ? nch : static_cast<int>((static_cast<long long>(split + 1) * nch) / p.splits);
   const int nmy = c1 - c0;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -398,7 +400,7 @@ __device__ __forceinline__ void attn_tile(const CUtensorMap& tm_kc, const CUtens
     const int hl = m / wb, r = m - hl * wb;
     return p.out + (static_cast<size_t>(r0 + r) * p.Hq + g * p.group + hl) * D;
   };
-  if (p.splits == 1) {
+  if (whole) {
     if (writer) {
       const float il = l_lo > 0.f ? 1.0f / l_lo : 0.f, ih = l_hi > 0.f ? 1.0f / l_hi : 0.f;
 #pragma unroll
@@ -568,8 +570,10 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
   }
   const int ncc = (P + kAttnChunk - 1) / kAttnChunk;
   const int nch = ncc + 1 + (S + kAttnChunk - 1) / kAttnChunk;
-  const int c0 = static_cast<int>((static_cast<long long>(split) * nch) / p.splits);
-  const int c1 = static_cast<int>((static_cast<long long>(split + 1) * nch) / p.splits);
+  const bool whole = p.splits == 1 || nch < p.split_from;  // the first split takes the keys
+  if (whole && split > 0) return;
+  const int c0 = whole ? 0 : static_cast<int>((static_cast<long long>(split) * nch) / p.splits);
+  const int c1 = whole ? nch : static_cast<int>((static_cast<long long>(split + 1) * nch) / p.splits);
   const int nmy = c1 - c0;              // 64-key chunks of this split
   const int nst = (nmy + 1) / 2;        // steps of two chunks
   const int slot = bg * p.max_qtiles + qt;
@@ -912,7 +916,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
           const float4 lv = *reinterpret_cast<const float4*>(comb + (64 + r) * LDC + 4 * lane);
           const float2 ml = *reinterpret_cast<const float2*>(rowinfo + 2 * r);
           float4 o4 = make_float4(hv.x + lv.x, hv.y + lv.y, hv.z + lv.z, hv.w + lv.w);
-          if (p.splits == 1) {
+          if (whole) {
             const float sc = ml.y > 0.f ? 1.0f / ml.y : 0.f;
             o4 = make_float4(o4.x * sc, o4.y * sc, o4.z * sc, o4.w * sc);
             const int m = qt * TR + r;
@@ -943,7 +947,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_kc, const CUt
     tc_fence_after();
     tmem_dealloc(tmem, kTcTmemCols);
   }
-  if (p.splits == 1 || *abort) return;
+  if (whole || *abort) return;
 
   // the last CTA of the slot combines the splits' partials, as in the
   // mma.sync kernel
