@@ -496,74 +496,95 @@ ebd_status check_args(ebd_handle* h, const ebd_step_args* a, bool need_attn, boo
   return EBD_OK;
 }
 
-// How the window attention of `batch` sequences runs.
+// How the window attention of a call runs.
 struct AttnPlan {
-  int tc;      // 1: the tcgen05 kernel, 0: the mma.sync kernel
-  int slots;   // query tiles of 64 rows
-  int splits, split_from;  // key splits of each that has at least split_from chunks of keys
-  int stages;  // ring of the mma.sync kernel
+  int tc;                  // 1: the tcgen05 kernel, 0: the mma.sync kernel
+  int splits, split_from;  // key splits of each tile that has at least split_from chunks of keys
+  int stages;              // ring of the mma.sync kernel
+  int two;                 // at most two of its CTAs per SM
 };
-AttnPlan attn_plan(const ebd_handle* h, int batch) {
+AttnPlan attn_plan(const ebd_handle* h, int batch, int rows) {
   const ebd_config& c = h->cfg;
-  // Both attention kernels take 64-row query tiles.  The tcgen05 kernel
-  // holds an SM alone (one CTA per SM) and pays a fixed setup and drain
-  // per CTA (TMEM, barriers, the query tile, its output), which long key
-  // ranges amortise; the mma.sync kernel runs two or three CTAs per SM, and
-  // with tiles of up to 32 rows it reads the cache as fast, its warps
-  // sharing each chunk's keys.  So, measured (attention alone, LLaDA-8B
-  // heads, us, mma.sync against tcgen05 in the better of their splits):
-  //   more tiles than SMs: 64 x 1024 x 32 rows 183 / 228, 64 x 4096 x 32
-  //     630 / 676, 8 x 1024 x 32 33 / 37, 12 x 1024 x 32 44 / 53; but tiles
-  //     of 33 to 64 rows over more than 8 chunks 62 / 62 (16 x 640 x 64), 298
-  //     / 235 (64 x 900 x 64), Dream-7B heads 51 / 43 (36 x 640 x 21), 120 /
-  //     86 (64 x 900 x 21), at 8 chunks 167 / 168 (64 x 400 x 64), 40 / 37
-  //     (36 x 400 x 21), below that 117 / 153 (64 x 250 x 64);
-  //   at most one tile per SM: 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50 /
-  //     47, 1 x 4096 x 32 26.5 / 21, but at 256 keys 10.8 / 12.2; with tiles
-  //     of 33 to 64 rows 14 / 13 at 250 keys (8 x 250 x 21, Dream-7B heads),
-  //     12.3 / 12.3 at 180, 10.8 / 12.2 at 120.
+  AttnPlan p{};
+  // Query tiles of 64 rows of (window row, query head of the group): the
+  // grid's, and those that hold rows.  The call's own: planned for the handle's
+  // largest batch, one sequence on a handle for 64 took, 4096 keys x 32 rows 70
+  // us (now 22), 4096 x 8 50 (20), 1024 x 32 21 (12.6).  Of ragged windows the
+  // host knows the sum, so it takes half a tile more per sequence than their
+  // rows fill.
+  const int window = c.max_window < kMaxWindow ? c.max_window : kMaxWindow;
+  const int group = c.n_heads_q / c.n_heads_kv, sms = h->num_sms;
+  const int grid = batch * c.n_heads_kv * h->attn_max_qtiles;
+  int tiles = grid;
+  if (rows < batch * window) {
+    const long long n = c.n_heads_kv * (2ll * rows * group + 64ll * batch) / 128;
+    tiles = n < grid ? static_cast<int>(n) : grid;
+    if (tiles < batch * c.n_heads_kv) tiles = batch * c.n_heads_kv;
+  }
+  const bool big = window * group > 32, one_wave = tiles <= sms;
+  const int nch = (c.max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
+  // The tcgen05 kernel holds an SM alone and pays a fixed setup and drain per
+  // CTA (TMEM, barriers, the query tile, its output), which long key ranges
+  // amortise; its steps take as long with 64-wide heads as with 128-wide ones.
+  // The mma.sync kernel runs two or more CTAs per SM, and with tiles of up to 32
+  // rows it reads the cache as fast, its warps sharing each chunk's keys.
+  // Measured (attention alone, us, mma.sync / tcgen05, each as it runs below):
+  //   tiles of up to 32 rows: one wave 4 x 1024 x 32 23 / 18.5, 4 x 4096 x 8 50
+  //     / 47, but 256 keys 10.8 / 12.2; more 64 x 1024 x 32 183 / 228, 64 x 4096
+  //     x 32 630 / 676;
+  //   larger ones, 128-wide: one wave 250 keys 14 / 13, 180 12.3 / 12.3, 120 10.8
+  //     / 12.2; up to three tiles per SM at 9 chunks 37 / 36, 43 / 36, 47 / 42;
+  //     more 93 / 96, 110 / 115, 165 / 178 there, at 16 chunks 83 / 76, 151 /
+  //     121, 265 / 231;
+  //   larger ones, 64-wide: one wave at 5 chunks 7.8 / 9.4, 9 11.5 / 11.2; more at
+  //     9 chunks 31 / 44, 49 / 75, 16 52 / 58, 81 / 97, 30 45 / 41.
+  if (!big)
+    p.tc = one_wave && nch >= 9;
+  else if (c.head_dim == 64)
+    p.tc = nch >= (one_wave ? 9 : 20);
+  else
+    p.tc = nch >= (one_wave ? 4 : tiles <= 3 * sms ? 9 : 12);
   // EBD_ATTN_KERNEL=tc|mma forces one, EBD_ATTN_SPLITS the split count,
   // EBD_ATTN_STAGES the ring's stages (measurement sweeps).
-  // The tiles are the call's own.  Planned for the handle's largest batch
-  // instead, one sequence on a handle for 64 took, 4096 x 32 rows 70 us (now 22),
-  // 4096 x 8 50 (20), 1024 x 32 21 (12); with four sequences 4096 x 32 71 (47).
-  AttnPlan p{};
-  const int rows = (c.max_window < kMaxWindow ? c.max_window : kMaxWindow) * (c.n_heads_q / c.n_heads_kv);
-  const int nch = (c.max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
-  p.slots = batch * c.n_heads_kv * h->attn_max_qtiles;
-  const bool one_wave = p.slots <= h->num_sms;
-  p.tc = rows > 32 ? nch >= (one_wave ? 4 : 9) : (one_wave && nch >= 9);
   if (h->attn_force_tc >= 0) p.tc = h->attn_force_tc;
-  // key splits per tile: as many as keep one wave of CTAs, of at least 4
+  // Key splits, on tcgen05: as many as keep one wave of CTAs, of at least 4
   // chunks each with the prefix at its longest (a CTA more than the SMs hold
-  // costs a second wave: 1 x 4096 x 8 rows on tcgen05 28.7 us with 5 splits, 18.7
-  // with 4).  On tcgen05, with its longer steps, a split's partials cost as much
-  // as it saves below 16 chunks (2 x 452 x 50 rows 14.5 us unsplit, 16.4 with 2; 2
-  // x 1024 x 50 18.6 either way, 2 x 2048 x 50 26.8 / 22.7); and five to seven are
-  // no better than four (Dream-7B heads 2 x 1600 x 16 16.5 with 4, 18.6 with 5 to
-  // 7; 2 x 2048 x 4 16.4 with 4, 14.5 with 8).  Sequences whose own keys stay
-  // below the first line are left whole (1 x 256 x 32 rows in a cache for 1024
-  // 11 us split, 9.8 whole).
-  p.split_from = p.tc ? 16 : 8;
-  p.splits = (p.tc ? h->num_sms : 2 * h->num_sms) / p.slots;
+  // costs a second wave: 1 x 4096 x 8 rows 28.7 us with 5 splits, 18.7 with 4).
+  // Two of them cost their partials as much as they save below 16 chunks (2 x 452
+  // x 50 rows 14.5 us unsplit, 16.4 with 2; 2 x 1024 x 50 18.6 either way), four
+  // from 11 on (9 chunks 12.5 unsplit, 13.3 with 4; 13 13.1 / 11.8); five to
+  // seven are no better than four (Dream-7B heads 2 x 1600 x 16 16.5 with 4, 18.6
+  // with 5 to 7; 2 x 2048 x 4 16.4 with 4, 14.5 with 8).  A sequence whose own
+  // keys stay below those lines is left whole (1 x 256 x 32 rows in a cache for
+  // 1024: 11.1 split, 9.8 whole).
+  p.splits = p.tc && nch >= 16 ? sms / tiles : 1;
   if (p.splits > nch / 4) p.splits = nch / 4;
-  if (nch < p.split_from) p.splits = 1;
-  if (p.tc && p.splits > 4 && p.splits < 8) p.splits = 4;
+  if (p.splits > kAttnParts * sms / grid) p.splits = kAttnParts * sms / grid;
+  if (p.splits > 4 && p.splits < 8) p.splits = 4;
   if (p.splits > kMaxAttnSplits) p.splits = kMaxAttnSplits;
   if (p.splits < 1) p.splits = 1;
+  p.split_from = p.splits >= 4 ? 11 : 16;
   if (h->attn_force_splits != 0) {
     p.splits = h->attn_force_splits < nch ? h->attn_force_splits : nch;
     p.split_from = 0;
   }
-  // CTAs per SM of the mma.sync kernel: two with a ring of three stages or
-  // three with two.  Three hide more of the CTAs' starts and ends and of the
-  // work between copies (us, two / three: 10 x 1024 x 8 rows 45 / 33, 12 x
-  // 4096 x 8 146 / 122, 24 x 1024 x 32 86 / 79, 64 x 256 x 32 81 / 69, 64 x
-  // 1024 x 32 193 / 183), but a wave of them takes longer: two where three
-  // would leave a last wave too empty (16 x 1024 x 8, 512 CTAs, 50 / 60; but
-  // 32 x 1024 x 8, 1024 CTAs, 94 / 95, x 32 rows 111 / 106).
-  auto waves = [&](int per_sm) { return (p.slots * p.splits + per_sm * h->num_sms - 1) / (per_sm * h->num_sms); };
-  p.stages = 6 * waves(3) <= 5 * waves(2) ? 2 : kAttnStages;
+  // CTAs per SM of the mma.sync kernel, with a ring of three stages two (64-wide
+  // heads: more, as shared memory allows), with one of two three.  Up to two
+  // tiles per SM, two: with room for more, CTAs crowd on some SMs as the grid's
+  // empty ones leave (ragged windows of 60 rows, Dream-7B heads 13 x 200 keys
+  // 14.2 us, 22.2 with three; 64-wide 24 x 450 15.9, 19.8).  Above that, three hide more of the
+  // starts and ends and of the work between copies where tiles have up to 32
+  // rows (two / three: 10 x 1024 x 8 rows 45 / 33, 12 x 4096 x 8 146 / 122, 24 x
+  // 1024 x 32 86 / 79, 64 x 256 x 32 81 / 69, 64 x 1024 x 32 193 / 183), unless a
+  // last wave of them would be too empty (16 x 1024 x 8, 512 CTAs, 50 / 60); larger
+  // tiles, with more work per chunk, gain from the deeper ring (64 x 200 x 60 rows
+  // 73 / 78, 24 x 200 x 60 49 / 53), but for a wave that just fits (448 tiles of 70
+  // keys 21.5 / 19.5).
+  const int ctas = tiles * p.splits;
+  auto waves = [&](int per_sm) { return (ctas + per_sm * sms - 1) / (per_sm * sms); };
+  p.two = ctas <= 2 * sms;
+  p.stages = kAttnStages;
+  if (!p.two && (big ? 10 * ctas > 27 * sms && ctas <= 3 * sms : 6 * waves(3) <= 5 * waves(2))) p.stages = 2;
   if (h->attn_force_stages != 0) p.stages = h->attn_force_stages;
   return p;
 }
@@ -585,7 +606,7 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   // all dims of a head for the mma.sync kernel, half by half (dim of the half,
   // key, half, head(, sequence))
   bool ok;
-  const AttnPlan plan = attn_plan(h, a->batch);
+  const AttnPlan plan = attn_plan(h, a->batch, a->rows);
   if (plan.tc) {
     const uint64_t cdims[4] = {static_cast<uint64_t>(D), H, Pm, Bc}, wdims[3] = {static_cast<uint64_t>(D), H, R};
     const uint64_t cstr[3] = {head, row, Pm * row}, wstr[2] = {head, row};
@@ -612,6 +633,7 @@ ebd_status run_attention(ebd_handle* h, const ebd_step_args* a, cudaStream_t st,
   p.splits = plan.splits;
   p.split_from = plan.split_from;
   p.stages = plan.stages;
+  p.two = plan.two;
   p.tc = plan.tc;
   p.cu_rows = a->cu_rows;
   p.prefix_len = a->prefix_len;
@@ -897,14 +919,11 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
       h->attn_force_splits = n < 1 ? 1 : n > kMaxAttnSplits ? kMaxAttnSplits : n;
     }
     if (const char* env = getenv("EBD_ATTN_STAGES")) h->attn_force_stages = atoi(env) == 2 ? 2 : kAttnStages;
-    // partials of the largest launch that splits its tiles, over all batches
+    // partials of any launch that splits its tiles
     const int slots = cfg->max_batch * cfg->n_heads_kv * h->attn_max_qtiles;
-    size_t parts = 0;
-    for (int b = 1; b <= cfg->max_batch; ++b) {
-      const AttnPlan p = attn_plan(h, b);
-      const size_t n = static_cast<size_t>(p.slots) * p.splits;
-      if (p.splits > 1 && n > parts) parts = n;
-    }
+    size_t parts = static_cast<size_t>(slots) * (h->attn_force_splits != 0 ? h->attn_force_splits : kMaxAttnSplits);
+    if (h->attn_force_splits == 0 && parts > static_cast<size_t>(kAttnParts) * h->num_sms)
+      parts = static_cast<size_t>(kAttnParts) * h->num_sms;
     if (parts > 0) {
       if ((e = cudaMalloc(&h->attn_part, parts * tile * (cfg->head_dim + 2) * 4)) != cudaSuccess)
         return bail(cuda_fail(h, e, "cudaMalloc(attention partials)"));

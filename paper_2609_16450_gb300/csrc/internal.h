@@ -38,6 +38,7 @@ constexpr int kAttnThreads = 128;
 constexpr int kAttnChunk = 64;        // keys per K/V tile
 constexpr int kAttnStages = 3;        // at most
 constexpr int kMaxAttnSplits = 8;
+constexpr int kAttnParts = 4;         // split tiles per SM that the attention's partials hold, at most
 constexpr int kAttnTcThreads = 352;   // tcgen05 attention: K and V load warps, MMA warp, 8 softmax warps
 constexpr int kAttnTcRows = 64;       // query rows per tile of the tcgen05 attention
 
@@ -49,6 +50,7 @@ struct AttnParams {
   int max_qtiles, splits;   // key splits of a tile with at least
   int split_from;           // split_from chunks of keys; the others have one
   int stages;               // ring of the mma.sync kernel: kAttnStages, or 2 for three CTAs per SM
+  int two;                  // at most two of its CTAs per SM, whatever they take
   int tc;                   // 1: the tcgen05 kernel, 0: the mma.sync kernel (64-row tiles)
   const int* cu_rows;
   const int* prefix_len;

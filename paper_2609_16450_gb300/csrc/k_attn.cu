@@ -12,10 +12,11 @@
 // a 128-byte swizzle.  The probabilities are split into a bf16 high part and
 // a bf16 remainder, so that P V keeps ~16 mantissa bits.
 //   attn_tc_kernel: the 5th-generation tensor cores (S and O in TMEM); one
-//     CTA per SM; for long key ranges and launches of few tiles.
+//     CTA per SM; for long key ranges.
 //   attn_kernel: mma.sync, 4 warps of 16 query rows, a K/V ring of two stages
-//     and three CTAs per SM, or of three and two; for launches of many tiles with short key ranges, where
-//     the tcgen05 kernel's per-CTA setup does not amortise.
+//     and three CTAs per SM, or of three and two; for launches of many tiles
+//     with short key ranges, where the tcgen05 kernel's per-CTA setup does not
+//     amortise, and for tiles of few rows.
 #include <type_traits>
 
 #include "internal.h"
@@ -28,6 +29,7 @@ namespace {
 // a stage of the mma.sync kernel: a chunk's K and V, 64-dim halves
 constexpr int attn_stage_bytes(int D) { return 2 * (D / 64) * 8192; }
 constexpr int attn_smem_bytes(int D, int stages) { return stages * attn_stage_bytes(D) + 1024 + 64; }
+constexpr int kAttnTwoBytes = 78 * 1024;  // more than a third of an SM's shared memory
 
 __device__ __forceinline__ void tma_load_5d(void* smem_dst, const void* tmap, uint64_t* bar, int32_t x,
                                             int32_t y, int32_t z, int32_t w, int32_t v) {
@@ -1099,7 +1101,7 @@ __global__ void __launch_bounds__(kAttnTcThreads, 1)
 cudaError_t attn_configure() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(attn_kernel<64, 2>, a, attn_smem_bytes(64, kAttnStages))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(attn_kernel<64, 2>, a, kAttnTwoBytes)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attn_kernel<64, 3>, a, attn_smem_bytes(64, 2))) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attn_kernel<128, 2>, a, attn_smem_bytes(128, kAttnStages))) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attn_kernel<128, 3>, a, attn_smem_bytes(128, 2))) != cudaSuccess) return e;
@@ -1115,6 +1117,8 @@ cudaError_t launch_attention(const CUtensorMap& kc, const CUtensorMap& vc, const
   cfg.blockDim = dim3(p.tc ? kAttnTcThreads : kAttnThreads, 1, 1);
   cfg.dynamicSmemBytes = p.tc ? (p.D == 64 ? TcMap<64>::kDyn : TcMap<128>::kDyn)
                               : attn_smem_bytes(p.D, p.stages);
+  if (!p.tc && p.two && p.stages == kAttnStages && cfg.dynamicSmemBytes < kAttnTwoBytes)
+    cfg.dynamicSmemBytes = kAttnTwoBytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
