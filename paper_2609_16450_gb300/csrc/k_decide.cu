@@ -1349,10 +1349,6 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     __syncthreads();
   } else if constexpr (kWide) {
     if (p.lps_enabled) copy_lps();
-    // Rank 0 commits in place, and where no LPS follows nothing else stands
-    // between a CTA's reads of the decode state above and that commit.  (In a
-    // step this meeting is over before the grids ahead are.)
-    cluster_barrier();
     // the statistics and the LBS logits of every row
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
@@ -1538,6 +1534,10 @@ __global__ void __launch_bounds__(kT, 1) decide_rows_kernel(const RowsParams p) 
     } else {
       lps_router<CAP, NR, NP, 0>(nBM, warp, [] { __syncthreads(); });
     }
+  } else if (kWide && !RULE) {
+    // Rank 0 commits in place over the decode state that every CTA has read:
+    // with no LPS, whose meetings stand between the two, they meet here.
+    cluster_barrier();
   }
   if (!RULE) asm volatile("cp.async.wait_all;" ::: "memory");
   if (rank != 0 || bad_seq) return;
