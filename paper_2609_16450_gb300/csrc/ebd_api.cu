@@ -582,9 +582,10 @@ AttnPlan attn_plan(const ebd_handle* h, int batch, int rows) {
   // keys 21.5 / 19.5).
   const int ctas = tiles * p.splits;
   auto waves = [&](int per_sm) { return (ctas + per_sm * sms - 1) / (per_sm * sms); };
-  p.two = ctas <= 2 * sms;
+  const bool few = ctas <= 2 * sms;
+  p.two = few && grid * p.splits > sms;  // a grid of one CTA per SM does not crowd
   p.stages = kAttnStages;
-  if (!p.two && (big ? 10 * ctas > 27 * sms && ctas <= 3 * sms : 6 * waves(3) <= 5 * waves(2))) p.stages = 2;
+  if (!few && (big ? 10 * ctas > 27 * sms && ctas <= 3 * sms : 6 * waves(3) <= 5 * waves(2))) p.stages = 2;
   if (h->attn_force_stages != 0) p.stages = h->attn_force_stages;
   return p;
 }
