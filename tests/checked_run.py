@@ -10,26 +10,20 @@ import numpy as np
 
 
 def run_cases():
-    import synth
     from paper_2609_16450_gb300 import _ebd as E
     from paper_2609_16450_gb300 import runtime as rt
     from tests import guards
-    from tests.test_gpu_guards import CASES, decide_kernel
+    from tests.test_gpu_guards import CASES, case_inputs
     res = {}
-    for name, state, attention, append, kernel in CASES:
-        sh = synth.SHAPES[name]
-        inp = synth.make_step_inputs(sh)
-        if state == "inblock":
-            synth.preset_in_block(inp, 20)
+    for name, state, attention, append in CASES:
+        sh, inp = case_inputs(name, state)
         w = rt.upload_weights(inp)
         h = rt.Handle(rt.config_for(sh), w.w_emb)
         try:
             if name != "tiny":
                 w = rt.pack_weights(h, w)
-            with decide_kernel(kernel):
-                status, out, g = guards.guarded_step(E, rt, h, inp, w, attention=attention,
-                                                     append=append)
-            key = f"{name}_{state}" + (f"_{kernel}" if kernel else "")
+            status, out, g = guards.guarded_step(E, rt, h, inp, w, attention=attention, append=append)
+            key = f"{name}_{state}"
             res[key + "/status"] = np.array(status)
             res[key + "/guards"] = np.array(all(v.intact() for v in g.values()))
             for k, v in out.items():

@@ -5,8 +5,8 @@
   cached prefix, a window with no masked row left, and one whose masked set
   is no larger than L_min (B = M without the LBS, Sec. 4.1).  The whole step
   (attention, statistics, routers, block, commit) against the oracle, with
-  no active block and inside one, decided by the cluster kernel and by the
-  grid-wide kernels.
+  no active block and inside one, decided by the cluster alone and behind the
+  grid-wide statistics and LBS (max_window > 64).
 * An empty step (rows = 0) returns EBD_OK and touches nothing.
 * A hidden state with NaN or Inf: the step reports EBD_ERR_NONFINITE, the
   row's argmax is -1 and it stays masked, and every other sequence's
@@ -70,7 +70,7 @@ def _step(sh, inp, max_window=None, attention=True, expect=0):
 @pytest.mark.parametrize("max_window", [64, 128])
 def test_degenerate_sequences_match_oracle(state, max_window):
     sh, inp = _ragged(state)
-    attention = max_window <= 64  # the grid-wide setting has no window attention
+    attention = max_window <= 64  # the full-sequence setting has no window attention
     gpu = _step(sh, inp, max_window=max_window, attention=attention)
     res = o.step(inp, _weights(sh), _prm(sh), attention=attention)
     parity.compare_stats(res.stats, gpu)

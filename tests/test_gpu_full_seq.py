@@ -1,7 +1,7 @@
 """The full-sequence setting on the GPU through the C ABI: every position of
 the response is a row of the step and the LBS sees every masked position
 (App. E algorithm with M = all masked positions; windows of up to 512 rows
-per sequence, decided by the grid-wide decision kernels).
+per sequence, their statistics and LBS over the whole GPU).
 
 * tiny shape, 3 sequences of 256, 100 and 40 rows: the whole step against
   the oracle (statistics of every row; routers, block, commit exact unless
@@ -139,8 +139,8 @@ def test_full_loop_tiny_matches_oracle():
 
 
 def test_small_window_same_decision_on_both_paths():
-    """The LLaDA-8B-shaped selection step (32 rows) decided by the cluster
-    kernel (max_window 64) and by the grid-wide kernels (max_window 128)."""
+    """The LLaDA-8B-shaped selection step (32 rows) decided by the cluster alone
+    (max_window 64) and behind the grid-wide statistics and LBS (max_window 128)."""
     sh = synth.llada
     inp = synth.make_step_inputs(sh)
     a = _gpu_step(sh, inp)
