@@ -66,7 +66,7 @@ def shape_for(name):
 
 def full_sequence(sh):
     """The full-sequence setting: windows of more than 64 rows (every
-    position of the response), decided by the grid-wide kernels, without
+    position of the response): statistics and LBS over the whole GPU, without
     the window attention."""
     import synth
     return int(np.max(synth.window_sizes(sh))) > 64

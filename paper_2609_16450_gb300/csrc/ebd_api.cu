@@ -232,7 +232,6 @@ struct ebd_handle {
   float4* part_f = nullptr;
   int* part_i = nullptr;
   int grid_lm = 0;       // LM-head partial states per row
-  int lm_ctas = 0;       // CTAs of the last LM-head launch (one SM each)
   int lm_units = 0;      // 64-row vocabulary units
   float* attn_part = nullptr;
   float* attn_part_ml = nullptr;
@@ -666,10 +665,7 @@ ebd_status run_lm(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, bool p
                   int v_off = 0, int v_count = -1) {
   const ebd_config& c = h->cfg;
   const int V = v_count < 0 ? c.vocab : v_count;
-  CUtensorMap tw;
   const bool packed = a->w_lm_layout == 1;
-  if (!encode_w_lm(&tw, a->w_lm, V, c.d_model, packed, 0))
-    return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (W_lm) failed");
   for (int g0 = 0; g0 < a->rows; g0 += kMaxGroupRows) {
     const int rows = a->rows - g0 < kMaxGroupRows ? a->rows - g0 : kMaxGroupRows;
     LmParams p{};
@@ -708,13 +704,11 @@ ebd_status run_lm(ebd_handle* h, const ebd_step_args* a, cudaStream_t st, bool p
       if (!encode_bf16(&th, a->hidden, 2, dims, str, box))
         return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (hidden) failed");
     }
-    CUtensorMap twp;  // the paired launches' view of W: one box per stage
-    const bool w_box = p.pair && (packed || p.boxed);
-    if (w_box && !encode_w_lm(&twp, a->w_lm, V, c.d_model, packed, p.kbs))
+    CUtensorMap tw;  // of W: one box per stage in paired launches
+    if (!encode_w_lm(&tw, a->w_lm, V, c.d_model, packed, p.pair && (packed || p.boxed) ? p.kbs : 0))
       return fail(h, EBD_ERR_CUDA, "cuTensorMapEncodeTiled (W_lm) failed");
-    cudaError_t e = launch_lm_stats(w_box ? twp : tw, th, p, st);
+    cudaError_t e = launch_lm_stats(tw, th, p, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "LM-head launch");
-    h->lm_ctas = p.grid;
   }
   return EBD_OK;
 }
@@ -1183,7 +1177,7 @@ struct StepRoute {
 }  // namespace
 
 namespace {
-// windows of more than kMaxWindow rows per sequence: the grid-wide decision
+// windows of more than kMaxWindow rows per sequence: the full-sequence setting
 bool seq_mode(const ebd_handle* h) { return h->cfg.max_window > kMaxWindow; }
 
 // LM head and decision

@@ -200,8 +200,8 @@ __device__ __forceinline__ bool epilogue_buffer(uint32_t taddr0, int wg, int nwg
 }  // namespace
 
 // PAIR (p.pair), PACKED (p.packed) and BOXED (p.boxed) are template
-// parameters: a runtime branch in the single-thread producer or MMA loop
-// costs measurable time.
+// parameters: a runtime branch in the producer or MMA loop costs measurable
+// time.
 //
 // PAIR: the CTAs of a cluster of 2 form a pair that runs cta_group::2 MMAs
 // of M = 256 vocabulary rows.  A vocabulary chunk is 4 units: the even CTA
@@ -567,8 +567,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
   } else {
     // ------------------------------------------------------------ epilogue
     // p.nwg warpgroups of 4 warps (one per TMEM lane quadrant) take the
-    // 32-row column slices of the accumulator in turn; a second warpgroup
-    // is used when the accumulator has a single buffer.
+    // 32-row column slices of the accumulator in turn.
     const int wg = (tid - 64) >> 7;
     const int et = (tid - 64) & 127;  // thread within the warpgroup
     const int quad = warp & 3;        // TMEM lane quadrant this warp may read

@@ -19,7 +19,7 @@ struct LmParams {
   int boxed;                // CTA pairs: a stage's hidden rows (and row-major W rows) come in
                             // as one 3-D box (d a multiple of 64)
   int stages, nbuf, acc_stride, tmem_cols;
-  int nwg;                  // epilogue warpgroups in use (2 with a single accumulator buffer)
+  int nwg;                  // epilogue warpgroups in use: 1 or 2 (lm_plan)
   int pair;                 // CTA pairs (clusters of 2) running cta_group::2 MMAs, M = 256
   int nwork;                // owners of vocabulary ranges per row group: CTAs, or pairs
   int rgroups;              // row groups of at most 256 rows (paired launches: 1 or 2), each

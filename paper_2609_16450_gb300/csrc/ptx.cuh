@@ -132,7 +132,7 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const void* tmap, ui
       "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
       : "memory");
 }
-// 4-D tiled load for a CTA pair (cta_group::2): the bytes are counted on the
+// 3-D and 4-D tiled loads for a CTA pair (cta_group::2): the bytes count on the
 // mbarrier at cluster address `bar_cluster`.  x as in tma_load_2d.
 __device__ __forceinline__ void tma_load_3d_pair(void* smem_dst, const void* tmap,
                                                  uint32_t bar_cluster, int32_t x, int32_t y,
