@@ -41,12 +41,13 @@
  *     rows of a step <= max_rows <= 4096.  Anything else returns
  *     EBD_ERR_UNSUPPORTED.
  *   - The decision runs as one thread-block cluster per sequence, of as many
- *     CTAs as suit the launch's sequences.  max_window > 64 (the
- *     full-sequence setting, where every position of the response is a row,
- *     App. E with M = all masked positions): the statistics and the LBS run
- *     over the whole GPU ahead of it, and a
- *     step takes no window attention (attn_out and kv_append must be unset:
- *     EBD_ERR_UNSUPPORTED otherwise).
+ *     CTAs as suit the launch's sequences (the baselines' rules on given
+ *     statistics: one CTA per sequence).  max_window > 64 (the full-sequence
+ *     setting, where every position of the response is a row, App. E with M =
+ *     all masked positions): the statistics and the LBS run over the whole GPU
+ *     ahead of it, the statistics of every row of the step, also of rows that no
+ *     accepted sequence holds; and a step takes no window attention (attn_out
+ *     and kv_append must be unset: EBD_ERR_UNSUPPORTED otherwise).
  *   - stream arguments are cudaStream_t values passed as void* (NULL = the
  *     legacy default stream).
  */

@@ -495,6 +495,11 @@ ebd_status check_args(ebd_handle* h, const ebd_step_args* a, bool need_attn, boo
   return EBD_OK;
 }
 
+// chunks of keys of a sequence with the prefix at its longest, and from how many
+// on the window attention splits its tiles
+int attn_chunks(const ebd_config& c) { return (c.max_prefix + kAttnChunk - 1) / kAttnChunk + 1; }
+constexpr int kAttnSplitChunks = 16;
+
 // How the window attention of a call runs.
 struct AttnPlan {
   int tc;                  // 1: the tcgen05 kernel, 0: the mma.sync kernel
@@ -521,7 +526,7 @@ AttnPlan attn_plan(const ebd_handle* h, int batch, int rows) {
     if (tiles < batch * c.n_heads_kv) tiles = batch * c.n_heads_kv;
   }
   const bool big = window * group > 32, one_wave = tiles <= sms;
-  const int nch = (c.max_prefix + kAttnChunk - 1) / kAttnChunk + 1;
+  const int nch = attn_chunks(c);
   // The tcgen05 kernel holds an SM alone and pays a fixed setup and drain per
   // CTA (TMEM, barriers, the query tile, its output), which long key ranges
   // amortise; its steps take as long with 64-wide heads as with 128-wide ones.
@@ -556,7 +561,7 @@ AttnPlan attn_plan(const ebd_handle* h, int batch, int rows) {
   // with 5 to 7; 2 x 2048 x 4 16.4 with 4, 14.5 with 8).  A sequence whose own
   // keys stay below those lines is left whole (1 x 256 x 32 rows in a cache for
   // 1024: 11.1 split, 9.8 whole).
-  p.splits = p.tc && nch >= 16 ? sms / tiles : 1;
+  p.splits = p.tc && nch >= kAttnSplitChunks ? sms / tiles : 1;
   if (p.splits > nch / 4) p.splits = nch / 4;
   if (p.splits > kAttnParts * sms / grid) p.splits = kAttnParts * sms / grid;
   if (p.splits > 4 && p.splits < 8) p.splits = 4;
@@ -917,8 +922,11 @@ ebd_status ebd_create(const ebd_config* cfg, ebd_handle** out) {
     // partials of any launch that splits its tiles
     const int slots = cfg->max_batch * cfg->n_heads_kv * h->attn_max_qtiles;
     size_t parts = static_cast<size_t>(slots) * (h->attn_force_splits != 0 ? h->attn_force_splits : kMaxAttnSplits);
-    if (h->attn_force_splits == 0 && parts > static_cast<size_t>(kAttnParts) * h->num_sms)
-      parts = static_cast<size_t>(kAttnParts) * h->num_sms;
+    if (h->attn_force_splits == 0) {
+      const size_t most = static_cast<size_t>(kAttnParts) * h->num_sms;
+      if (parts > most) parts = most;
+      if (attn_chunks(*cfg) < kAttnSplitChunks) parts = 0;
+    }
     if (parts > 0) {
       if ((e = cudaMalloc(&h->attn_part, parts * tile * (cfg->head_dim + 2) * 4)) != cudaSuccess)
         return bail(cuda_fail(h, e, "cudaMalloc(attention partials)"));
