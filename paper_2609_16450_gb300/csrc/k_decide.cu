@@ -818,9 +818,10 @@ __device__ __forceinline__ void ld_kv(const __nv_bfloat16* p, uint32_t (&w)[4 * 
 // side end before it.  (One function whose parts are skipped by branches ran
 // 1.5 times as long.)
 // C: CTAs of the cluster that share the rows, 0 where one CTA has them all.  Keys
-// and values of both blocks at kv + block * kv_stride (C = 0: in shared memory): K [key][dim pair][head][plane][2 dims] and, v_off further, V
-// [key pair][dim][head][plane][2 keys], so that a lane reads all heads and
-// planes of its key (pair) in NP 16-byte loads.
+// and values of both blocks at kv + block * kv_stride (C = 0: in shared memory):
+// K [key][dim pair][head][plane][2 dims] and, v_off further, V [key
+// pair][dim][head][plane][2 keys], so that a lane reads all heads and planes of
+// its key (pair) in NP 16-byte loads.
 struct LpsGlobal {  // (C > 0; itself in shared memory, for all warps)
   __nv_bfloat16* kv;
   size_t kv_stride, v_off;
